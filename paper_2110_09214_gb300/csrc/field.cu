@@ -59,9 +59,7 @@ struct __align__(16) SrcPk {
 // Targets are visited by the cell kernel in the Morton order of a 64^3 grid
 // over the cell bounding box (points outside are clamped to the border
 // bins), so the 32 targets of a warp are neighbours and mostly take the same
-// distance tier for a given cell.  Counting sort: histogram, scan, scatter;
-// the order inside a bin is arbitrary, which does not change any result (each
-// target's sum runs over the cells in the same order whatever its slot).
+// distance tier for a given cell.
 __device__ __forceinline__ uint32_t spread3(uint32_t x)
 {
     x &= 0x3Fu;
@@ -72,80 +70,96 @@ __device__ __forceinline__ uint32_t spread3(uint32_t x)
     return x;
 }
 
-__global__ void bin_count_kernel(FieldLaunch L, float3 lo, float3 scale, uint32_t *code, int32_t *hist)
+// bin code of every target and the targets per super-bin.  A cloud fills few
+// super-bins, so a warp adds its targets of one super-bin with one atomic.
+__device__ __forceinline__ uint32_t bin_code(float4 p, float3 lo, float3 scale)
 {
-    const int nt = L.nt_dev ? *L.nt_dev : L.nt;
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nt) return;
-    float4 p = L.targets[i];
     int ix = (int)fminf(fmaxf((p.x - lo.x) * scale.x, 0.f), (float)(OBEM_BINS_PER_AXIS - 1));
     int iy = (int)fminf(fmaxf((p.y - lo.y) * scale.y, 0.f), (float)(OBEM_BINS_PER_AXIS - 1));
     int iz = (int)fminf(fmaxf((p.z - lo.z) * scale.z, 0.f), (float)(OBEM_BINS_PER_AXIS - 1));
-    uint32_t c = spread3(ix) | (spread3(iy) << 1) | (spread3(iz) << 2);
-    code[i] = c;
-    atomicAdd(&hist[c], 1);
+    return spread3(ix) | (spread3(iy) << 1) | (spread3(iz) << 2);
+}
+__device__ __forceinline__ void bin_add(bool live, uint32_t c, int32_t *hist)
+{
+    const uint32_t sb = live ? c >> OBEM_SUPER_SHIFT : 0xffffffffu;
+    const unsigned peers = __match_any_sync(0xffffffffu, sb);
+    if (live && (peers & ((1u << (threadIdx.x & 31)) - 1u)) == 0u) atomicAdd(&hist[sb], __popc(peers));
+}
+__global__ void bin_count_kernel(FieldLaunch L, float3 lo, float3 scale, uint32_t *code, int32_t *hist)
+{
+    const int nt = L.nt_dev ? *L.nt_dev : L.nt;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i - (int)(threadIdx.x & 31) >= nt) return;         // warp-uniform
+    uint32_t c = 0;
+    if (i < nt) {
+        c = bin_code(L.targets[i], lo, scale);
+        code[i] = c;
+    }
+    bin_add(i < nt, c, hist);
 }
 
-// exclusive scan of OBEM_NBINS counts in place, one block of 1024 threads
-__global__ void bin_scan_kernel(int32_t *hist)
+// inclusive scan of one value per thread over a block of 1024
+__device__ __forceinline__ int32_t block_scan_1024(int32_t v, int32_t *s_warp)
 {
-    __shared__ int32_t part[1024];
-    const int per = OBEM_NBINS / 1024;
-    int32_t *h = hist + threadIdx.x * per;
-    int32_t s = 0;
-    for (int k = 0; k < per; ++k) s += h[k];
-    part[threadIdx.x] = s;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+    }
+    __syncthreads();                       // s_warp may still be read from the call before
+    if (lane == 31) s_warp[warp] = v;
     __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        int32_t v = threadIdx.x >= off ? part[threadIdx.x - off] : 0;
-        __syncthreads();
-        part[threadIdx.x] += v;
-        __syncthreads();
+    if (warp == 0) {
+        int32_t w = s_warp[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t u = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += u;
+        }
+        s_warp[lane] = w;
     }
-    int32_t run = part[threadIdx.x] - s;
-    for (int k = 0; k < per; ++k) {
-        int32_t c = h[k];
-        h[k] = run;
-        run += c;
-    }
+    __syncthreads();
+    return v + (warp > 0 ? s_warp[warp - 1] : 0);
 }
 
 // Blocks of the cell kernels: the targets of one super-bin (4 x 4 x 4 bins,
 // contiguous in the sorted order) are cut into blocks of at most CT_BLOCK_N,
-// so a block never spans distant bins.  One block of 1024 threads; reads the
-// scanned histogram (bin start offsets) before the scatter advances it.
+// so a block never spans distant bins.  One block of 1024 threads, from the
+// super-bins' counts alone: latency-bound (4096 counts, two block scans).  The
+// scan of all 64^3 bins that this replaces read its bins with a stride of 1 KB
+// and took 428 us of every field evaluation (a 1000-charge step of 2.68 ms is
+// 2.25 ms without it).
 #define CT_BLOCK_N 512
-__global__ void block_list_kernel(const int32_t *start, int nt_host, const int32_t *nt_dev, int2 *blocks,
-                                  int32_t *nblocks)
+__global__ void __launch_bounds__(1024) block_list_kernel(const int32_t *hist, int2 *blocks, int32_t *nblocks)
 {
-    __shared__ int32_t part[1024];
-    const int nt = nt_dev ? *nt_dev : nt_host;
-    constexpr int PER = OBEM_NSUPER >= 1024 ? OBEM_NSUPER / 1024 : 1;
-    const int per = OBEM_NSUPER >= 1024 ? PER : (threadIdx.x < OBEM_NSUPER ? 1 : 0);
-    int cnt[PER];
-    int32_t s = 0;
-    for (int q = 0; q < per; ++q) {
-        const int sb = threadIdx.x * per + q;
-        const int a = start[sb << OBEM_SUPER_SHIFT];
-        const int b = (sb + 1 < OBEM_NSUPER) ? start[(sb + 1) << OBEM_SUPER_SHIFT] : nt;
-        cnt[q] = b - a;
-        s += (b - a + CT_BLOCK_N - 1) / CT_BLOCK_N;
+    __shared__ int32_t s_warp[32];
+    constexpr int PER = OBEM_NSUPER / 1024;
+    static_assert(PER == 4, "one int4 of counts per thread");
+    const int4 h = reinterpret_cast<const int4 *>(hist)[threadIdx.x];
+    const int cnt[PER] = {h.x, h.y, h.z, h.w};
+    int32_t n = 0, k = 0;
+    for (int q = 0; q < PER; ++q) {
+        n += cnt[q];
+        k += (cnt[q] + CT_BLOCK_N - 1) / CT_BLOCK_N;
     }
-    part[threadIdx.x] = s;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        int32_t v = threadIdx.x >= off ? part[threadIdx.x - off] : 0;
-        __syncthreads();
-        part[threadIdx.x] += v;
-        __syncthreads();
+    int32_t a = block_scan_1024(n, s_warp) - n;
+    const int32_t kinc = block_scan_1024(k, s_warp);
+    int32_t o = kinc - k;
+    for (int q = 0; q < PER; ++q) {
+        // the warp writes each lane's blocks together
+        const int nb = (cnt[q] + CT_BLOCK_N - 1) / CT_BLOCK_N;
+        unsigned bal = __ballot_sync(0xffffffffu, nb > 0);
+        while (bal) {
+            const int src = __ffs(bal) - 1;
+            bal &= bal - 1;
+            const int sa = __shfl_sync(0xffffffffu, a, src), so = __shfl_sync(0xffffffffu, o, src),
+                      sc = __shfl_sync(0xffffffffu, cnt[q], src);
+            for (int b = threadIdx.x & 31; b * CT_BLOCK_N < sc; b += 32)
+                blocks[so + b] = make_int2(sa + b * CT_BLOCK_N, min(CT_BLOCK_N, sc - b * CT_BLOCK_N));
+        }
+        a += cnt[q];
+        o += nb;
     }
-    int32_t o = part[threadIdx.x] - s;
-    for (int q = 0; q < per; ++q) {
-        const int sb = threadIdx.x * per + q;
-        const int a = start[sb << OBEM_SUPER_SHIFT];
-        for (int k = 0; k < cnt[q]; k += CT_BLOCK_N) blocks[o++] = make_int2(a + k, min(CT_BLOCK_N, cnt[q] - k));
-    }
-    if (threadIdx.x == 1023) nblocks[0] = part[1023];
+    if (threadIdx.x == 1023) nblocks[0] = kinc;
 }
 
 // Target order of the cell kernels: a stable LSD radix sort of the bin codes
@@ -170,29 +184,40 @@ __global__ void rs_hist_kernel(const uint32_t *key, int nt, const int32_t *nt_de
     if (threadIdx.x < RS_RADIX) rh[threadIdx.x * nblk + blockIdx.x] = h[threadIdx.x];
 }
 
-// exclusive scan of m counts in place (one block of 1024 threads)
-__global__ void rs_scan_kernel(int32_t *a, int m)
+// exclusive scan of m counts in place: one block of 1024 threads, tiles of
+// 4096 counts read as int4 with the next tile's loads in flight.  Latency-bound:
+// one round trip to L2 and two barriers per tile (62,528 counts at 1e6 targets;
+// a thread per stretch of 62 counts, read with that stride, took 52 us)
+__global__ void __launch_bounds__(1024) rs_scan_kernel(int32_t *a, int m)
 {
-    __shared__ int32_t part[1024];
-    const int per = (m + 1023) / 1024, q0 = threadIdx.x * per;
-    int32_t sum = 0;
-    for (int q = 0; q < per; ++q)
-        if (q0 + q < m) sum += a[q0 + q];
-    part[threadIdx.x] = sum;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-        const int32_t v = threadIdx.x >= o ? part[threadIdx.x - o] : 0;
-        __syncthreads();
-        part[threadIdx.x] += v;
-        __syncthreads();
-    }
-    int32_t run = part[threadIdx.x] - sum;
-    for (int q = 0; q < per; ++q)
-        if (q0 + q < m) {
-            const int32_t v = a[q0 + q];
-            a[q0 + q] = run;
-            run += v;
+    __shared__ int32_t s_warp[32];
+    auto load = [&](int base) {
+        int4 v = make_int4(0, 0, 0, 0);
+        const int q = base + 4 * (int)threadIdx.x;
+        if (q + 3 < m) return *reinterpret_cast<const int4 *>(a + q);
+        if (q < m) v.x = a[q];
+        if (q + 1 < m) v.y = a[q + 1];
+        if (q + 2 < m) v.z = a[q + 2];
+        return v;
+    };
+    int32_t carry = 0;
+    int4 nx = load(0);
+    for (int base = 0; base < m; base += 4096) {
+        const int4 v = nx;
+        nx = load(base + 4096);
+        const int32_t t = v.x + v.y + v.z + v.w;
+        const int32_t inc = block_scan_1024(t, s_warp);
+        const int32_t e = carry + inc - t;
+        const int q = base + 4 * (int)threadIdx.x;
+        const int4 r = make_int4(e, e + v.x, e + v.x + v.y, e + v.x + v.y + v.z);
+        if (q + 3 < m) *reinterpret_cast<int4 *>(a + q) = r;
+        else {
+            if (q < m) a[q] = r.x;
+            if (q + 1 < m) a[q + 1] = r.y;
+            if (q + 2 < m) a[q + 2] = r.z;
         }
+        carry += s_warp[31];                // the tile's total (rewritten behind a barrier of the next scan)
+    }
 }
 
 // stable scatter by digit: within a block, rank = earlier keys of the same
@@ -259,7 +284,7 @@ size_t obem_point_bins_bytes(int n)
 {
     const size_t e = pb_align(sizeof(int32_t) * (size_t)n);
     return 4 * e + pb_align(sizeof(int32_t) * ((size_t)RS_RADIX * obem_binsort_blocks(n) + 1)) +
-           pb_align(sizeof(int32_t) * OBEM_NBINS) + pb_align(sizeof(int2) * obem_point_bins_maxblocks(n)) +
+           pb_align(sizeof(int32_t) * OBEM_NSUPER) + pb_align(sizeof(int2) * obem_point_bins_maxblocks(n)) +
            pb_align(sizeof(int32_t) * 8);
 }
 int obem_point_bins(obem_ctx *ctx, const float4 *pts, int n, void *scratch, int32_t **perm, int2 **blocks,
@@ -272,7 +297,7 @@ int obem_point_bins(obem_ctx *ctx, const float4 *pts, int n, void *scratch, int3
     uint32_t *tk = (uint32_t *)p; p += e;
     int32_t *tv = (int32_t *)p; p += e;
     int32_t *rh = (int32_t *)p; p += pb_align(sizeof(int32_t) * ((size_t)RS_RADIX * obem_binsort_blocks(n) + 1));
-    int32_t *hist = (int32_t *)p; p += pb_align(sizeof(int32_t) * OBEM_NBINS);
+    int32_t *hist = (int32_t *)p; p += pb_align(sizeof(int32_t) * OBEM_NSUPER);
     *blocks = (int2 *)p; p += pb_align(sizeof(int2) * obem_point_bins_maxblocks(n));
     *nblocks = (int32_t *)p;
     FieldLaunch L;
@@ -284,10 +309,9 @@ int obem_point_bins(obem_ctx *ctx, const float4 *pts, int n, void *scratch, int3
     sc.x = (float)OBEM_BINS_PER_AXIS / fmaxf(ctx->bbox_hi[0] - ctx->bbox_lo[0], 1e-30f);
     sc.y = (float)OBEM_BINS_PER_AXIS / fmaxf(ctx->bbox_hi[1] - ctx->bbox_lo[1], 1e-30f);
     sc.z = (float)OBEM_BINS_PER_AXIS / fmaxf(ctx->bbox_hi[2] - ctx->bbox_lo[2], 1e-30f);
-    OBEM_CUDA(ctx, cudaMemsetAsync(hist, 0, sizeof(int32_t) * OBEM_NBINS, s));
+    OBEM_CUDA(ctx, cudaMemsetAsync(hist, 0, sizeof(int32_t) * OBEM_NSUPER, s));
     bin_count_kernel<<<(n + 255) / 256, 256, 0, s>>>(L, lo, sc, code, hist);
-    bin_scan_kernel<<<1, 1024, 0, s>>>(hist);
-    block_list_kernel<<<1, 1024, 0, s>>>(hist, n, NULL, *blocks, *nblocks);
+    block_list_kernel<<<1, 1024, 0, s>>>(hist, *blocks, *nblocks);
     binsort(code, code, *perm, tk, tv, rh, n, NULL, n, s);
     OBEM_LAUNCH(ctx);
     return OBEM_OK;
@@ -1939,15 +1963,14 @@ int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets,
             sc.x = (float)OBEM_BINS_PER_AXIS / fmaxf(ctx->bbox_hi[0] - ctx->bbox_lo[0], 1e-30f);
             sc.y = (float)OBEM_BINS_PER_AXIS / fmaxf(ctx->bbox_hi[1] - ctx->bbox_lo[1], 1e-30f);
             sc.z = (float)OBEM_BINS_PER_AXIS / fmaxf(ctx->bbox_hi[2] - ctx->bbox_lo[2], 1e-30f);
-            OBEM_CUDA(ctx, cudaMemsetAsync(ctx->s_hist, 0, sizeof(int32_t) * OBEM_NBINS, s));
+            OBEM_CUDA(ctx, cudaMemsetAsync(ctx->s_hist, 0, sizeof(int32_t) * OBEM_NSUPER, s));
             const int nb = (capacity_targets + 255) / 256;
             bin_count_kernel<<<nb, 256, 0, s>>>(L, lo, sc, ctx->s_code, ctx->s_hist);
-            bin_scan_kernel<<<1, 1024, 0, s>>>(ctx->s_hist);
-            block_list_kernel<<<1, 1024, 0, s>>>(ctx->s_hist, L.nt, L.nt_dev, (int2 *)L.blocks, (int32_t *)L.nblocks);
+            block_list_kernel<<<1, 1024, 0, s>>>(ctx->s_hist, (int2 *)L.blocks, (int32_t *)L.nblocks);
             binsort(ctx->s_code, ctx->s_code, (int32_t *)L.perm, ctx->s_tk, ctx->s_tv, ctx->s_rh, L.nt, L.nt_dev,
                     capacity_targets, s);
             OBEM_LAUNCH(ctx);
-            if (L.events) ctx->launches += 12;
+            if (L.events) ctx->launches += 11;
         }
         const int nsuper = capacity_targets < OBEM_NSUPER ? capacity_targets : OBEM_NSUPER;
         dim3 cgrid((capacity_targets + CT_BLOCK - 1) / CT_BLOCK + (L.blocks ? nsuper : 0));
@@ -2210,7 +2233,7 @@ constexpr size_t na_align(size_t x) { return (x + 255) & ~(size_t)255; }
 constexpr size_t NA_CELLS_BYTES = na_align(sizeof(float4) * 6 * (size_t)NA_MAX_CELLS);
 constexpr size_t NA_CODE_BYTES = na_align(sizeof(uint32_t) * (size_t)NA_MAX_TARGETS);
 constexpr size_t NA_PERM_BYTES = na_align(sizeof(int32_t) * (size_t)NA_MAX_TARGETS);
-constexpr size_t NA_HIST_BYTES = na_align(sizeof(int32_t) * (size_t)OBEM_NBINS);
+constexpr size_t NA_HIST_BYTES = na_align(sizeof(int32_t) * (size_t)OBEM_NSUPER);
 constexpr size_t NA_NBLK = (size_t)NA_MAX_TARGETS / 512 + 2 + OBEM_NSUPER;
 constexpr size_t NA_BLOCKS_BYTES = na_align(sizeof(int2) * NA_NBLK);
 constexpr size_t NA_MISC_BYTES = 256;   // number of blocks, bounding box
@@ -2293,19 +2316,18 @@ __global__ void na_bbox_kernel(const double *v64, int np, float *box)
 // binning with the grid read from device memory (box from na_bbox_kernel)
 __global__ void na_bin_count_kernel(FieldLaunch L, const float *box, uint32_t *code, int32_t *hist)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= L.nt) return;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i - (int)(threadIdx.x & 31) >= L.nt) return;       // warp-uniform
     const float3 lo = make_float3(box[0], box[1], box[2]);
     const float3 sc = make_float3((float)OBEM_BINS_PER_AXIS / fmaxf(box[3] - box[0], 1e-30f),
                                   (float)OBEM_BINS_PER_AXIS / fmaxf(box[4] - box[1], 1e-30f),
                                   (float)OBEM_BINS_PER_AXIS / fmaxf(box[5] - box[2], 1e-30f));
-    float4 p = L.targets[i];
-    int ix = (int)fminf(fmaxf((p.x - lo.x) * sc.x, 0.f), (float)(OBEM_BINS_PER_AXIS - 1));
-    int iy = (int)fminf(fmaxf((p.y - lo.y) * sc.y, 0.f), (float)(OBEM_BINS_PER_AXIS - 1));
-    int iz = (int)fminf(fmaxf((p.z - lo.z) * sc.z, 0.f), (float)(OBEM_BINS_PER_AXIS - 1));
-    uint32_t c = spread3(ix) | (spread3(iy) << 1) | (spread3(iz) << 2);
-    code[i] = c;
-    atomicAdd(&hist[c], 1);
+    uint32_t c = 0;
+    if (i < L.nt) {
+        c = bin_code(L.targets[i], lo, sc);
+        code[i] = c;
+    }
+    bin_add(i < L.nt, c, hist);
 }
 
 static int na_fail(char *err, int32_t err_len, int code, const char *msg)
@@ -2395,12 +2417,11 @@ extern "C" int obem_field_eval_noalloc(const float *targets, int32_t nt, const f
                                                         (float4 *)L.panels.nrm, (float4 *)L.panels.c_lo);
         na_bbox_kernel<<<1, 1024, 0, s>>>(cell_xyz, np, box);
         // the array keeps the previous call's contents: the histogram must restart at zero
-        if (cudaMemsetAsync(hist, 0, sizeof(int32_t) * OBEM_NBINS, s) != cudaSuccess)
+        if (cudaMemsetAsync(hist, 0, sizeof(int32_t) * OBEM_NSUPER, s) != cudaSuccess)
             return na_fail(err, err_len, OBEM_ERR_CUDA, "cudaMemsetAsync of the histogram failed");
         const int nb = (nt + 255) / 256;
         na_bin_count_kernel<<<nb, 256, 0, s>>>(L, box, code, hist);
-        bin_scan_kernel<<<1, 1024, 0, s>>>(hist);
-        block_list_kernel<<<1, 1024, 0, s>>>(hist, nt, NULL, blocks, nblocks);
+        block_list_kernel<<<1, 1024, 0, s>>>(hist, blocks, nblocks);
         binsort(code, code, perm, na_tk, na_tv, na_rh, nt, NULL, nt, s);
         const int nsuper = nt < OBEM_NSUPER ? nt : OBEM_NSUPER;
         dim3 cgrid((nt + CT_BLOCK - 1) / CT_BLOCK + nsuper);

@@ -113,7 +113,7 @@ extern "C" int obem_create(obem_ctx **out, const obem_config *cfg)
     ALLOC(c->s_tk, sizeof(uint32_t) * cap);
     ALLOC(c->s_tv, sizeof(int32_t) * cap);
     ALLOC(c->s_rh, sizeof(int32_t) * (64 * (size_t)obem_binsort_blocks(cap) + 1));
-    ALLOC(c->s_hist, sizeof(int32_t) * OBEM_NBINS);
+    ALLOC(c->s_hist, sizeof(int32_t) * OBEM_NSUPER);
     ALLOC(c->s_blocks, sizeof(int2) * ((size_t)cap / 512 + 2 + (cap < OBEM_NSUPER ? cap : OBEM_NSUPER)));
     ALLOC(c->s_nblocks, sizeof(int32_t) * (OBEM_NSUPER + 8));
     ALLOC(c->ph_count, sizeof(int32_t) * ((size_t)1 << 20));
