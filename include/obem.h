@@ -456,12 +456,15 @@ int obem_selftest_waits(obem_ctx *ctx, int32_t which, obem_stream stream);
  * around its stages (up to 256 steps are kept; older ones are dropped) and
  * counting the evaluations below (the cell kernels then run in their counting
  * variants, a few per cent slower); obem_profile(ctx, OBEM_PROFILE_TIMES)
- * records the events only (counts[2..6] stay 0);
+ * records the events only (counts[2..6] stay 0; sets of up to about 1e5
+ * charges then take the single cell kernel, as without a profile, which has no
+ * separate near part);
  * obem_stage_times() waits for the recorded events and returns, summed over
  * the recorded steps:
  *   ms[0] cell field (binning + near + far kernels), ms[1] all-pairs field
  *   kernel, ms[2] step kernels (recombination, flight, compaction, moments),
- *   ms[3] whole obem_step, ms[4] the near-cell kernel alone (part of ms[0]);
+ *   ms[3] whole obem_step, ms[4] the near-cell kernels alone (part of ms[0];
+ *   0 for sets whose cell field is one kernel, see OBEM_PROFILE_TIMES);
  *   counts[0] steps recorded, counts[1] kernels launched by those steps,
  *   counts[2] charge pairs of the all-pairs kernel,
  *   counts[3..5] (block of targets, cell) pairs of the far-cell kernel by

@@ -19,6 +19,7 @@ COMMON = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", os.path
 UNITS = {
     "obem_api.cu": [],
     "field.cu": [],
+    "direct.cu": [],
     "step.cu": ["--fmad=false", "-prec-div=true", "-prec-sqrt=true"],
     "bem.cu": [],
     "backward.cu": [],

@@ -13,6 +13,9 @@
 // targets per thread as f32x2 packs, sources staged through shared memory as
 // duplicated pairs, compensated (TwoSum) folds of every tile.
 //
+// Few targets (direct.cu) and few charges take kernels whose lanes run over
+// the cells or charges instead; the rules stand at obem_launch_field.
+//
 // Cells.  Targets are ordered along a 64^3 Morton grid (stable radix sort) and
 // cut into blocks of <= 512; per block, cells near its box get the FP64
 // closed form (targets within h) and a 112- or 28-point rule, the others one
@@ -96,29 +99,6 @@ __global__ void bin_count_kernel(FieldLaunch L, float3 lo, float3 scale, uint32_
         code[i] = c;
     }
     bin_add(i < nt, c, hist);
-}
-
-// inclusive scan of one value per thread over a block of 1024
-__device__ __forceinline__ int32_t block_scan_1024(int32_t v, int32_t *s_warp)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int32_t u = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += u;
-    }
-    __syncthreads();                       // s_warp may still be read from the call before
-    if (lane == 31) s_warp[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        int32_t w = s_warp[lane];
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t u = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += u;
-        }
-        s_warp[lane] = w;
-    }
-    __syncthreads();
-    return v + (warp > 0 ? s_warp[warp - 1] : 0);
 }
 
 // Blocks of the cell kernels: the targets of one super-bin (4 x 4 x 4 bins,
@@ -1948,6 +1928,28 @@ __global__ void const_field_kernel(FieldLaunch L)
     if (i < nt) L.E_out[i] = make_float4(L.e_ext.x, L.e_ext.y, L.e_ext.z, 0.f);
 }
 
+// Which kernels evaluate a set of targets (by its capacity: the live count is
+// on the device).  Cells: the direct kernel up to about 1e5 targets, twice that
+// for a mesh of 49k cells and more, where the few blocks of the block kernels
+// run longer: measured block / direct (ms) at 60k and 200k targets, plates of
+// 1024 cells 2.9 / 1.9 and 5.0 / 6.3, plates of 4096 2.9 / 1.7 and 5.3 / 5.4,
+// GEM of 5952 9.8 / 7.2 and 15.7 / 23.2, GEM of 59,968 in groups 40.7 / 13.3
+// and 51.4 / 43.5.
+static bool direct_cells_rule(int targets, int cells)
+{
+    return targets <= 98304 + 2 * (cells < 49152 ? cells : 49152);
+}
+// Charges at themselves: the symmetric kernel takes over between 16,000
+// (558 us, direct 200 us) and 32,000 charges (657 and 714 us).  Charges at
+// other points: the one-sided kernel from 64,000 points on (20,000 charges:
+// 967 and 875 us at 64,000, 1438 and 1733 us at 128,000), with few charges,
+// whose tiles it reads once per 512 points, from 32,000 (1000 charges: 55 and
+// 84 us at 64,000).
+static bool direct_pairs_rule(bool self, int targets, int sources)
+{
+    return self ? targets <= 24576 : targets <= (sources < 4096 ? 32768 : 65536);
+}
+
 int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets, cudaStream_t s)
 {
     if (capacity_targets <= 0) return OBEM_OK;
@@ -1955,7 +1957,12 @@ int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets,
     const bool cells = L.sigma != NULL && L.panels.np > 0;
     const bool charges = L.sources != NULL;
     const bool add = cells || L.add_init;      // E_out holds a field the all-pairs sum adds to
-    if (cells) {
+    const bool direct_cells = cells && !L.counters && direct_cells_rule(capacity_targets, L.panels.np);
+    if (direct_cells) {
+        if (L.events) { cudaEventRecord(L.events[4], s); cudaEventRecord(L.events[5], s); ctx->launches++; }
+        const int rc = obem_launch_direct_cells(ctx, L, NULL, capacity_targets, s);
+        if (rc != OBEM_OK) return rc;
+    } else if (cells) {
         if (L.perm) {
             // spatial order of the targets for the cell kernel
             float3 lo = make_float3(ctx->bbox_lo[0], ctx->bbox_lo[1], ctx->bbox_lo[2]);
@@ -2017,7 +2024,9 @@ int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets,
         }
         // self_exclude: the targets are the sources (same charges, nt == ns)
         const bool nn = L.nn_grid > 0 && L.self_exclude && !L.shard;
-        const bool sym = !nn && ctx->sym_jpart && L.self_exclude && !L.shard && capacity_targets <= ctx->sym_cap;
+        const bool self = L.self_exclude && !L.shard;
+        const bool direct = !nn && direct_pairs_rule(self, capacity_targets, L.ns);
+        const bool sym = !nn && !direct && ctx->sym_jpart && self && capacity_targets <= ctx->sym_cap;
         if (nn) {
             int rc = obem_launch_nbody_nn(ctx, L.sources, L.nt_dev, capacity_targets, L.nn_grid, L.eps2, L.E_out,
                                           L.e_ext, add ? 1 : 0, s);
@@ -2086,6 +2095,9 @@ int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets,
                 OBEM_LAUNCH(ctx);
             }
             if (L.events) ctx->launches += 4 + 2 * npass;
+        } else if (direct) {
+            const int rc = obem_launch_direct_pairs(ctx, L, NULL, capacity_targets, add ? 1 : 0, s);
+            if (rc != OBEM_OK) return rc;
         } else if (L.want_v) {
             if (add) nbody_kernel<true, true><<<grid, FT_THREADS, 0, s>>>(L);
             else nbody_kernel<true, false><<<grid, FT_THREADS, 0, s>>>(L);
@@ -2158,6 +2170,9 @@ __global__ void bt_const_field_kernel(FieldBatch F, float4 *E_out)
     E_out[i] = make_float4(F.e_ext.x, F.e_ext.y, F.e_ext.z, 0.f);
 }
 
+// Batches of at most this many slots take the direct cell kernel: their block
+// kernels have no more parallel work than one set of as many targets.
+#define BT_DIRECT_SLOTS 98304
 int obem_launch_field_batch(obem_ctx *ctx, const FieldBatch &F, const float4 *pos_q, float4 *E_out, cudaStream_t s)
 {
     if (F.cut < 32 || F.cut > CT_BLOCK) return obem_fail(ctx, OBEM_ERR_ARG, "batch: cell block size outside 32..512");
@@ -2178,13 +2193,18 @@ int obem_launch_field_batch(obem_ctx *ctx, const FieldBatch &F, const float4 *po
         L.nblocks = F.nblocks;
         L.block_cham = F.block_cham;
         L.cham_pan = F.cham_pan;
-        bt_blocks_kernel<<<1, 1024, 0, s>>>(F, F.blocks, F.block_cham, F.nblocks);
-        OBEM_LAUNCH(ctx);
-        const dim3 cg(F.max_blocks);
-        near_closed_kernel<false, false><<<cg, CT_THREADS, 0, s>>>(L);
-        near_quad_kernel<false, false><<<cg, CT_THREADS, 0, s>>>(L);
-        cell_kernel<false, false, true><<<cg, CT_THREADS, 0, s>>>(L);
-        OBEM_LAUNCH(ctx);
+        if (F.slots <= BT_DIRECT_SLOTS) {
+            const int rc = obem_launch_direct_cells(ctx, L, &F.sym, F.slots, s);
+            if (rc != OBEM_OK) return rc;
+        } else {
+            bt_blocks_kernel<<<1, 1024, 0, s>>>(F, F.blocks, F.block_cham, F.nblocks);
+            OBEM_LAUNCH(ctx);
+            const dim3 cg(F.max_blocks);
+            near_closed_kernel<false, false><<<cg, CT_THREADS, 0, s>>>(L);
+            near_quad_kernel<false, false><<<cg, CT_THREADS, 0, s>>>(L);
+            cell_kernel<false, false, true><<<cg, CT_THREADS, 0, s>>>(L);
+            OBEM_LAUNCH(ctx);
+        }
     }
     if (F.charges) {
         const int nsb = F.slots / SP_BLOCK;

@@ -60,6 +60,29 @@ __device__ __forceinline__ void two_sum_acc(float &s, float &c, float b)
     c = __fadd_rn(c, e);
 }
 
+// inclusive scan of one value per thread over a block of 1024
+__device__ __forceinline__ int32_t block_scan_1024(int32_t v, int32_t *s_warp)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+    }
+    __syncthreads();                       // s_warp may still be read from the call before
+    if (lane == 31) s_warp[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        int32_t w = s_warp[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t u = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += u;
+        }
+        s_warp[lane] = w;
+    }
+    __syncthreads();
+    return v + (warp > 0 ? s_warp[warp - 1] : 0);
+}
+
 // ------------------------------------------------------------------ FP64 closed form
 // Potential and field of a unit uniform density on a flat triangle at r:
 // phi = sum_i p0_i L_i - h Omega,  F = Omega n + sum_i u_i L_i, with the edge

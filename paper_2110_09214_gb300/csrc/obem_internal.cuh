@@ -368,6 +368,11 @@ struct FieldBatch {
 };
 int obem_launch_field_batch(obem_ctx *ctx, const FieldBatch &F, const float4 *pos_q, float4 *E_out,
                             cudaStream_t s);
+// direct.cu: the cell field (E_out = e_ext + cells) and the charges' field of
+// few targets; SB: the batch of chambers, or NULL; slots: capacity of the targets
+int obem_launch_direct_cells(obem_ctx *ctx, const FieldLaunch &L, const SymBatch *SB, int slots, cudaStream_t s);
+int obem_launch_direct_pairs(obem_ctx *ctx, const FieldLaunch &L, const SymBatch *SB, int slots, int add,
+                             cudaStream_t s);
 size_t obem_sym_sizes(int capacity, size_t *ipart_floats);
 int obem_cell_layout(const double *tri, const int32_t *kind, int np, float4 *ca, float4 *g0, float4 *g1,
                      float4 *g2, float4 *nr, float4 *cl);
