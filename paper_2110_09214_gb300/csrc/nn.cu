@@ -11,16 +11,25 @@
 //   - far: every other cell contributes its positive and its negative charge
 //     separately, each as the total charge at its charge-weighted centre.
 // Pipeline: bounding box (min/max reductions on order-preserving integer
-// images of the floats), cell of every charge + counts, exclusive scan,
-// counting-sort scatter, per-cell aggregates (FP64 sums), then one thread per
-// charge in cell order (so a warp walks the same neighbour lists) for the near
-// sum and the far sum over all cells' aggregates staged in shared memory.
+// images of the floats), cell of every charge + counts, exclusive scans
+// (charges, occupied cells, groups of 8 charges), counting-sort scatter of the
+// positions, per-cell aggregates of the occupied cells (FP64 sums), and the
+// field.
+//
+// Field: a warp takes up to 8 charges of one cell (four f32x2 packs) and its
+// lanes run over the sources.  The 27 cells around are 9 contiguous runs of
+// the sorted charges (three cells in x each), and their centres 9 runs of the
+// list of occupied cells' centres, so the far cells are the stretches between
+// those runs: both sums are coalesced reads with no test per source.  Bound:
+// FP32 issue (12 lane-operations and one rsqrt per charge and source); the four
+// warps of a block mostly share their cell, so their sources hit in L1.
 #include "obem_internal.cuh"
-#include "field_common.cuh"
+#include "direct_common.cuh"
 
 #define NN_THREADS 256
-#define NN_AGG_TILE 256            // cells per shared-memory tile of the far sum
-#define NN_CHUNK 32                // pair terms summed in FP32 before each FP64 add
+#define NN_T 8                     // targets per warp
+#define NN_FW 4                    // warps per block of the field kernel
+#define NN_AT 128                  // threads per cell of the aggregates
 
 // float <-> integer with the same order (for atomic min / max)
 __device__ __forceinline__ int nn_ford(float f)
@@ -51,11 +60,19 @@ __global__ void nn_bbox_kernel(const float4 *pos, const int32_t *n_dev, int n, i
             mn[a] = fminf(mn[a], __shfl_xor_sync(0xffffffffu, mn[a], o));
             mx[a] = fmaxf(mx[a], __shfl_xor_sync(0xffffffffu, mx[a], o));
         }
-    if ((threadIdx.x & 31) == 0 && mn[0] <= mx[0]) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            atomicMin(&bb[a], nn_ford(mn[a]));
-            atomicMax(&bb[3 + a], nn_ford(mx[a]));
+    // one atomic per block and bound (per warp they serialised on six words)
+    __shared__ float red[6][NN_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane == 0)
+        for (int a = 0; a < 3; ++a) { red[a][warp] = mn[a]; red[3 + a][warp] = mx[a]; }
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        float v = red[threadIdx.x][0];
+        for (int w = 1; w < NN_THREADS / 32; ++w)
+            v = threadIdx.x < 3 ? fminf(v, red[threadIdx.x][w]) : fmaxf(v, red[threadIdx.x][w]);
+        if (threadIdx.x < 3 ? v < INFINITY : v > -INFINITY) {
+            if (threadIdx.x < 3) atomicMin(&bb[threadIdx.x], nn_ford(v));
+            else atomicMax(&bb[threadIdx.x], nn_ford(v));
         }
     }
 }
@@ -102,152 +119,153 @@ __global__ void nn_cell_kernel(const float4 *pos, const int32_t *n_dev, int n, c
     atomicAdd(&count[(cz * G + cy) * G + cx], 1);
 }
 
-// start = exclusive scan of count[0..nc) (nc <= 1024 * 256), start[nc] = total; cursor = start
-__global__ void __launch_bounds__(1024) nn_scan_kernel(const int32_t *count, int nc, int32_t *start, int32_t *cursor)
+// exclusive scans over the cells, nc + 1 entries each: start (charges; cursor
+// is a copy), occ (occupied cells), grp (groups of up to NN_T charges)
+__global__ void __launch_bounds__(1024) nn_scan_kernel(const int32_t *count, int nc, int32_t *start, int32_t *cursor,
+                                                       int32_t *occ, int32_t *grp)
 {
-    __shared__ int32_t s_sum[1024];
-    const int per = (nc + 1023) / 1024;
-    const int t = threadIdx.x, b0 = t * per;
-    int32_t acc = 0;
-    for (int k = 0; k < per && b0 + k < nc; ++k) acc += count[b0 + k];
-    s_sum[t] = acc;
-    __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-        const int32_t v = t >= o ? s_sum[t - o] : 0;
-        __syncthreads();
-        s_sum[t] += v;
-        __syncthreads();
+    __shared__ int32_t s_warp[32];
+    int32_t carry[3] = {0, 0, 0};
+    for (int base = 0; base < nc; base += 1024) {
+        const int q = base + threadIdx.x;
+        const int32_t n = q < nc ? count[q] : 0;
+        const int32_t v[3] = {n, n > 0, (n + NN_T - 1) / NN_T};
+        int32_t *const out[3] = {start, occ, grp};
+        for (int k = 0; k < 3; ++k) {
+            const int32_t inc = block_scan_1024(v[k], s_warp);
+            if (q < nc) out[k][q] = carry[k] + inc - v[k];
+            if (k == 0 && q < nc) cursor[q] = carry[0] + inc - v[0];
+            carry[k] += s_warp[31];
+        }
     }
-    int32_t run = s_sum[t] - acc;
-    for (int k = 0; k < per && b0 + k < nc; ++k) {
-        start[b0 + k] = run;
-        cursor[b0 + k] = run;
-        run += count[b0 + k];
+    if (threadIdx.x == 0) {
+        start[nc] = carry[0];
+        occ[nc] = carry[1];
+        grp[nc] = carry[2];
     }
-    if (t == 1023) start[nc] = s_sum[1023];
 }
 
-__global__ void nn_scatter_kernel(const int32_t *n_dev, int n, const int32_t *cell, int G, int32_t *cursor,
-                                  int32_t *sorted)
+__global__ void nn_scatter_kernel(const float4 *pos, const int32_t *n_dev, int n, const int32_t *cell, int G,
+                                  int32_t *cursor, int32_t *sorted, float4 *spos)
 {
     const int nn = n_dev ? *n_dev : n;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nn) return;
     const int32_t c = cell[i];
     const int idx = (((c >> 20) & 1023) * G + ((c >> 10) & 1023)) * G + (c & 1023);
-    sorted[atomicAdd(&cursor[idx], 1)] = i;
+    const int k = atomicAdd(&cursor[idx], 1);
+    sorted[k] = i;
+    spos[k] = pos[i];
 }
 
-// per cell: positive and negative charge centres (x, y, z, k_C Q)
-__global__ void nn_agg_kernel(const float4 *pos, const int32_t *start, const int32_t *sorted, int nc, float4 *agg)
+// per occupied cell: positive and negative charge centres (x, y, z, k_C Q) at
+// agg[2 occ], agg[2 occ + 1] (no charge of a sign: weight 0), and the cell's
+// groups (cell, first sorted charge).  One block per cell: a thread per cell
+// took 11.7 ms at 3e5 charges, the densest cell's serial FP64 sum.
+__global__ void __launch_bounds__(NN_AT) nn_agg_kernel(const float4 *spos, const int32_t *start, const int32_t *occ,
+                                                       const int32_t *grp, float4 *agg, int2 *groups)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= nc) return;
-    double sp[4] = {0.0, 0.0, 0.0, 0.0}, sn[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int k = start[c]; k < start[c + 1]; ++k) {
-        const float4 p = pos[sorted[k]];
-        double *s = p.w >= 0.0f ? sp : sn;
+    __shared__ double red[NN_AT / 32][8];
+    const int c = blockIdx.x;
+    const int k0 = start[c], k1 = start[c + 1];
+    if (k0 == k1) return;
+    double s[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int k = k0 + threadIdx.x; k < k1; k += NN_AT) {
+        const float4 p = spos[k];
         const double q = (double)p.w;
-        s[0] += q * p.x; s[1] += q * p.y; s[2] += q * p.z; s[3] += q;
+        if (p.w >= 0.0f) { s[0] += q * p.x; s[1] += q * p.y; s[2] += q * p.z; s[3] += q; }
+        else { s[4] += q * p.x; s[5] += q * p.y; s[6] += q * p.z; s[7] += q; }
     }
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-    if (sp[3] != 0.0) a = make_float4((float)(sp[0] / sp[3]), (float)(sp[1] / sp[3]), (float)(sp[2] / sp[3]),
-                                      (float)(OBEM_KC * sp[3]));
-    if (sn[3] != 0.0) b = make_float4((float)(sn[0] / sn[3]), (float)(sn[1] / sn[3]), (float)(sn[2] / sn[3]),
-                                      (float)(OBEM_KC * sn[3]));
-    agg[2 * c] = a;
-    agg[2 * c + 1] = b;
-}
-
-// softened point-charge field term w (x - y) / (|x - y|^2 + eps^2)^(3/2)
-__device__ __forceinline__ void nn_term(float4 x, float4 y, float w, float eps2, float &ax, float &ay, float &az)
-{
-    const float dx = x.x - y.x, dy = x.y - y.y, dz = x.z - y.z;
-    const float r2 = fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, eps2)));
-    if (!(r2 > 0.f)) return;
-    const float inv = rsq(r2);
-    const float s3 = w * inv * inv * inv;
-    ax = fmaf(dx, s3, ax);
-    ay = fmaf(dy, s3, ay);
-    az = fmaf(dz, s3, az);
-}
-
-// field at every charge (one thread per charge, in cell order); E_out adds to
-// its initial value when add is set, else starts from e_ext
-__global__ void __launch_bounds__(NN_THREADS) nn_field_kernel(const float4 *pos, const int32_t *n_dev, int n,
-                                                              const int32_t *cell, const int32_t *start,
-                                                              const int32_t *sorted, const float4 *agg, int G,
-                                                              float eps2, float4 *E_out, float3 e_ext, int add)
-{
-    __shared__ float4 s_agg[2 * NN_AGG_TILE];
-    const int nn = n_dev ? *n_dev : n;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const bool live = t < nn;
-    const int i = live ? sorted[t] : 0;
-    const float4 x = live ? pos[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const int32_t ci = live ? cell[i] : 0;
-    const int cx = ci & 1023, cy = (ci >> 10) & 1023, cz = (ci >> 20) & 1023;
-    const float kC = (float)OBEM_KC;
-    double e[3] = {0.0, 0.0, 0.0};
-    if (live) {
-        // near: charges of the 27 cells around
-        for (int dz = -1; dz <= 1; ++dz) {
-            const int z = cz + dz;
-            if (z < 0 || z >= G) continue;
-            for (int dy = -1; dy <= 1; ++dy) {
-                const int y = cy + dy;
-                if (y < 0 || y >= G) continue;
-                for (int dx = -1; dx <= 1; ++dx) {
-                    const int xx = cx + dx;
-                    if (xx < 0 || xx >= G) continue;
-                    const int c = (z * G + y) * G + xx;
-                    const int k1 = start[c + 1];
-                    for (int k0 = start[c]; k0 < k1; k0 += NN_CHUNK) {
-                        float ax = 0.f, ay = 0.f, az = 0.f;
-                        for (int k = k0; k < min(k1, k0 + NN_CHUNK); ++k) {
-                            const int j = sorted[k];
-                            if (j == i) continue;
-                            const float4 y4 = pos[j];
-                            nn_term(x, y4, kC * y4.w, eps2, ax, ay, az);
-                        }
-                        e[0] += ax; e[1] += ay; e[2] += az;
-                    }
-                }
-            }
+#pragma unroll
+    for (int f = 0; f < 8; ++f)
+        for (int o = 16; o; o >>= 1) s[f] += __shfl_xor_sync(0xffffffffu, s[f], o);
+    if ((threadIdx.x & 31) == 0)
+        for (int f = 0; f < 8; ++f) red[threadIdx.x >> 5][f] = s[f];
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        double t[4];
+        for (int f = 0; f < 4; ++f) {
+            t[f] = red[0][4 * threadIdx.x + f];
+            for (int w = 1; w < NN_AT / 32; ++w) t[f] += red[w][4 * threadIdx.x + f];
         }
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (t[3] != 0.0) a = make_float4((float)(t[0] / t[3]), (float)(t[1] / t[3]), (float)(t[2] / t[3]),
+                                         (float)(OBEM_KC * t[3]));
+        agg[2 * occ[c] + threadIdx.x] = a;
     }
-    // far: charge centres of every cell outside the 27
+    const int g0 = grp[c];
+    for (int g = threadIdx.x; g * NN_T < k1 - k0; g += NN_AT) groups[g0 + g] = make_int2(c, k0 + g * NN_T);
+}
+
+// Field at every charge: warp g takes group g.  E_out adds to its initial
+// value when add is set, else starts from e_ext.  A pair at zero distance
+// gives no term: eps2 (x 2^80) is at least that of 1e-19 m.
+__global__ void __launch_bounds__(32 * NN_FW, 4)
+nn_field_kernel(const int32_t *start, const int32_t *occ, const int32_t *grp, const int2 *groups, const int32_t *sorted,
+                const float4 *spos, const float4 *agg, int G, float eps2, float4 *E_out, float3 e_ext, int add)
+{
+    constexpr int NP = NN_T / 2;
+    __shared__ DfShared<NP, NN_FW> sh;
     const int nc = G * G * G;
-    for (int cb = 0; cb < nc; cb += NN_AGG_TILE) {
-        __syncthreads();
-        for (int l = threadIdx.x; l < 2 * NN_AGG_TILE; l += blockDim.x) {
-            const int c = cb + l / 2;
-            s_agg[l] = c < nc ? agg[2 * cb + l] : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        __syncthreads();
-        if (!live) continue;
-        const int cn = min(NN_AGG_TILE, nc - cb);
-        for (int l0 = 0; l0 < cn; l0 += NN_CHUNK / 2) {
-            float ax = 0.f, ay = 0.f, az = 0.f;
-            for (int l = l0; l < min(cn, l0 + NN_CHUNK / 2); ++l) {
-                const int c = cb + l;
-                const int ux = c % G, uy = (c / G) % G, uz = c / (G * G);
-                if (abs(ux - cx) <= 1 && abs(uy - cy) <= 1 && abs(uz - cz) <= 1) continue;
-                const float4 a = s_agg[2 * l], b = s_agg[2 * l + 1];
-                if (a.w != 0.f) nn_term(x, a, a.w, eps2, ax, ay, az);
-                if (b.w != 0.f) nn_term(x, b, b.w, eps2, ax, ay, az);
+    const int lane = threadIdx.x & 31;
+    const int g = blockIdx.x * NN_FW + (threadIdx.x >> 5);
+    if (g >= grp[nc]) return;                               // warp-uniform; only warp barriers below
+    const int2 gr = groups[g];
+    const int c = gr.x, base = gr.y;
+    const int n = min(NN_T, start[c + 1] - base);
+    u64 TX[NP], TY[NP], TZ[NP], A[4][NP];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        const float4 a = spos[base + min(2 * p, n - 1)], b = spos[base + min(2 * p + 1, n - 1)];
+        TX[p] = pk(a.x * DF_XS, b.x * DF_XS);
+        TY[p] = pk(a.y * DF_XS, b.y * DF_XS);
+        TZ[p] = pk(a.z * DF_XS, b.z * DF_XS);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) A[k][p] = 0ull;
+    }
+#pragma unroll
+    for (int v = 0; v < 4 * NN_T; ++v) { sh.S[v][threadIdx.x] = 0.f; sh.C[v][threadIdx.x] = 0.f; }
+    const float4 none = make_float4(1e6f, 1e6f, 1e6f, 0.f);
+    int since = 0;
+    // the sources [b, e) of src with weights kC w
+    auto run = [&](const float4 *src, int b, int e, float kC) {
+        float4 nx = b + lane < e ? src[b + lane] : none;
+        for (int ib = b; ib < e; ib += 32) {
+            const float4 x = nx;
+            nx = ib + 32 + lane < e ? src[ib + 32 + lane] : none;
+            if (src == spos && ib + 32 > base && ib < base + NN_T)
+                df_source<false, true>(TX, TY, TZ, x, kC, eps2, ib + lane - base, A);
+            else
+                df_source<false, false>(TX, TY, TZ, x, kC, eps2, 0, A);
+            if (++since == DF_FOLD) {
+                df_fold<false>(sh, A, 1.f);
+                since = 0;
             }
-            e[0] += ax; e[1] += ay; e[2] += az;
         }
+    };
+    const int cx = c % G, cy = (c / G) % G, cz = c / (G * G);
+    const int x0 = max(cx - 1, 0), x1 = min(cx + 1, G - 1);
+    int fe = 0;                                             // centres before fe are done
+    for (int z = max(cz - 1, 0); z <= min(cz + 1, G - 1); ++z)
+        for (int y = max(cy - 1, 0); y <= min(cy + 1, G - 1); ++y) {
+            const int r = (z * G + y) * G;
+            run(agg, fe, 2 * occ[r + x0], DF_QS);
+            fe = 2 * occ[r + x1 + 1];
+            run(spos, start[r + x0], start[r + x1 + 1], (float)OBEM_KC * DF_QS);
+        }
+    run(agg, fe, 2 * occ[nc], DF_QS);
+    df_fold<false>(sh, A, 1.f);
+    float s[4 * NN_T], cc[4 * NN_T];
+#pragma unroll
+    for (int v = 0; v < 4 * NN_T; ++v) { s[v] = sh.S[v][threadIdx.x]; cc[v] = sh.C[v][threadIdx.x]; }
+    df_reduce<4 * NN_T>(s, cc);                             // lane l: component l % 4 of target l / 4
+    const int t = lane >> 2, k = lane & 3;
+    if (t < n) {
+        float *out = reinterpret_cast<float *>(E_out + sorted[base + t]) + k;
+        float e0 = k == 0 ? e_ext.x : k == 1 ? e_ext.y : e_ext.z;
+        if (add) e0 = *out;
+        *out = k < 3 ? (float)((double)s[0] + (double)cc[0] + (double)e0) : 0.f;
     }
-    if (!live) return;
-    if (add) {
-        const float4 q = E_out[i];
-        e[0] += q.x; e[1] += q.y; e[2] += q.z;
-    } else {
-        e[0] += e_ext.x; e[1] += e_ext.y; e[2] += e_ext.z;
-    }
-    E_out[i] = make_float4((float)e[0], (float)e[1], (float)e[2], 0.f);
 }
 
 int obem_launch_nbody_nn(obem_ctx *c, const float4 *pos, const int32_t *n_dev, int n, int G, float eps2,
@@ -261,11 +279,13 @@ int obem_launch_nbody_nn(obem_ctx *c, const float4 *pos, const int32_t *n_dev, i
     nn_bbox_kernel<<<nb < 1024 ? nb : 1024, NN_THREADS, 0, s>>>(pos, n_dev, n, c->nn_bbox);
     OBEM_CUDA(c, cudaMemsetAsync(c->nn_count, 0, sizeof(int32_t) * nc, s));
     nn_cell_kernel<<<nb, NN_THREADS, 0, s>>>(pos, n_dev, n, c->nn_bbox, G, c->nn_cell, c->nn_count);
-    nn_scan_kernel<<<1, 1024, 0, s>>>(c->nn_count, nc, c->nn_start, c->nn_cursor);
-    nn_scatter_kernel<<<nb, NN_THREADS, 0, s>>>(n_dev, n, c->nn_cell, G, c->nn_cursor, c->nn_sorted);
-    nn_agg_kernel<<<(nc + 255) / 256, 256, 0, s>>>(pos, c->nn_start, c->nn_sorted, nc, c->nn_agg);
-    nn_field_kernel<<<nb, NN_THREADS, 0, s>>>(pos, n_dev, n, c->nn_cell, c->nn_start, c->nn_sorted, c->nn_agg, G,
-                                             eps2, E_out, e_ext, add);
+    nn_scan_kernel<<<1, 1024, 0, s>>>(c->nn_count, nc, c->nn_start, c->nn_cursor, c->nn_occ, c->nn_grp);
+    nn_scatter_kernel<<<nb, NN_THREADS, 0, s>>>(pos, n_dev, n, c->nn_cell, G, c->nn_cursor, c->nn_sorted, c->nn_spos);
+    nn_agg_kernel<<<nc, NN_AT, 0, s>>>(c->nn_spos, c->nn_start, c->nn_occ, c->nn_grp, c->nn_agg, c->nn_groups);
+    const int ng = n / NN_T + (n < nc ? n : nc);
+    nn_field_kernel<<<(ng + NN_FW - 1) / NN_FW, 32 * NN_FW, 0, s>>>(
+        c->nn_start, c->nn_occ, c->nn_grp, c->nn_groups, c->nn_sorted, c->nn_spos, c->nn_agg, G,
+        fmaxf(eps2 * DF_QS, 1e-14f), E_out, e_ext, add);
     OBEM_LAUNCH(c);
     return OBEM_OK;
 }

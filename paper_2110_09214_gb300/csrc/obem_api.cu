@@ -127,6 +127,11 @@ extern "C" int obem_create(obem_ctx **out, const obem_config *cfg)
     ALLOC(c->nn_cell, sizeof(int32_t) * cap);
     ALLOC(c->nn_sorted, sizeof(int32_t) * cap);
     ALLOC(c->nn_count, sizeof(int32_t) * (size_t)OBEM_NN_GMAX * OBEM_NN_GMAX * OBEM_NN_GMAX);
+    ALLOC(c->nn_spos, sizeof(float4) * cap);
+    ALLOC(c->nn_groups, sizeof(int2) * ((size_t)cap / 8 + (cap < OBEM_NN_GMAX * OBEM_NN_GMAX * OBEM_NN_GMAX
+                                                            ? cap : OBEM_NN_GMAX * OBEM_NN_GMAX * OBEM_NN_GMAX)));
+    ALLOC(c->nn_occ, sizeof(int32_t) * ((size_t)OBEM_NN_GMAX * OBEM_NN_GMAX * OBEM_NN_GMAX + 1));
+    ALLOC(c->nn_grp, sizeof(int32_t) * ((size_t)OBEM_NN_GMAX * OBEM_NN_GMAX * OBEM_NN_GMAX + 1));
     ALLOC(c->nn_start, sizeof(int32_t) * ((size_t)OBEM_NN_GMAX * OBEM_NN_GMAX * OBEM_NN_GMAX + 1));
     ALLOC(c->nn_cursor, sizeof(int32_t) * (size_t)OBEM_NN_GMAX * OBEM_NN_GMAX * OBEM_NN_GMAX);
     ALLOC(c->nn_agg, sizeof(float4) * 2 * (size_t)OBEM_NN_GMAX * OBEM_NN_GMAX * OBEM_NN_GMAX);
@@ -187,7 +192,8 @@ extern "C" void obem_destroy(obem_ctx *c)
     free_dev(c->fm.nodes);
     free_dev(c->s_hit);
     free_dev(c->nn_bbox); free_dev(c->nn_cell); free_dev(c->nn_sorted); free_dev(c->nn_count);
-    free_dev(c->nn_start); free_dev(c->nn_cursor); free_dev(c->nn_agg);
+    free_dev(c->nn_start); free_dev(c->nn_cursor); free_dev(c->nn_agg); free_dev(c->nn_spos);
+    free_dev(c->nn_groups); free_dev(c->nn_occ); free_dev(c->nn_grp);
     if (c->cublas) cublasDestroy(c->cublas);
     if (c->prof_ev) {
         for (int i = 0; i < OBEM_PROF_EV * OBEM_PROF_MAX; ++i) cudaEventDestroy(c->prof_ev[i]);

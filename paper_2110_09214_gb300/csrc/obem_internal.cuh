@@ -217,10 +217,13 @@ struct obem_ctx {
     long long *d_deposit;
     int32_t *s_hit;
     // approximate N-body: bounding box, cell of each charge, cell counts /
-    // starts / cursors, charges sorted by cell, per-cell charge centres
+    // starts / cursors, occupied cells and groups of 8 charges before each
+    // cell, charges sorted by cell (indices, positions), charge centres of the
+    // occupied cells, groups (cell, first sorted charge)
     int *nn_bbox;
-    int32_t *nn_cell, *nn_sorted, *nn_count, *nn_start, *nn_cursor;
-    float4 *nn_agg;
+    int32_t *nn_cell, *nn_sorted, *nn_count, *nn_start, *nn_cursor, *nn_occ, *nn_grp;
+    float4 *nn_agg, *nn_spos;
+    int2 *nn_groups;
     int *sym_counter;
     uint32_t *s_tk;          // stable bin sort scratch: keys, values, digit counts
     int32_t *s_tv, *s_rh;
