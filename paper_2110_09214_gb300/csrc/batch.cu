@@ -76,7 +76,7 @@ extern "C" void obem_batch_destroy(obem_batch *b)
     BtScratch &W = b->W;
     bfree(W.prop); bfree(W.ionkey); bfree(W.keep); bfree(W.nsp); bfree(W.blk); bfree(W.o_pos); bfree(W.o_vel);
     bfree(W.o_id); bfree(W.o_birth); bfree(W.o_sp); bfree(W.ph_bucket); bfree(W.ph_count); bfree(W.ph_start);
-    bfree(W.ph_cursor); bfree(W.ph_sorted); bfree(W.ph_bsum); bfree(W.mpart);
+    bfree(W.ph_cursor); bfree(W.ph_sorted); bfree(W.ph_bsum); bfree(W.mpart); bfree(W.rec);
     if (b->graph) cudaGraphExecDestroy(b->graph);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
     delete b;
@@ -156,7 +156,7 @@ extern "C" int obem_batch_create(obem_batch **out, obem_ctx *ctx, int32_t n_cham
     BUP(b->d_joff, joff.data(), sizeof(long long) * nb);
     BUP(b->d_ioff, ioff.data(), sizeof(long long) * nb);
     BALLOC(b->d_ctl, sizeof(StepCtl) * nb);
-    BALLOC(b->d_abort, sizeof(int32_t));
+    BALLOC(b->d_abort, sizeof(int32_t) * 2);
     BALLOC(b->d_cham_pan, sizeof(int2) * nb);
     BALLOC(b->d_E, sizeof(float4) * S);
     BALLOC(b->d_blocks, sizeof(int2) * max_blocks);
@@ -176,7 +176,8 @@ extern "C" int obem_batch_create(obem_batch **out, obem_ctx *ctx, int32_t n_cham
     BALLOC(W.ionkey, sizeof(unsigned long long) * S);
     BALLOC(W.keep, sizeof(int32_t) * S);
     BALLOC(W.nsp, sizeof(int32_t) * S);
-    BALLOC(W.blk, sizeof(int32_t) * 2 * (S / 256));
+    BALLOC(W.blk, sizeof(int32_t) * 2 * (S / 32));
+    BALLOC(W.rec, sizeof(float4) * OBEM_REC_F4 * (S / 2));
     BALLOC(W.o_pos, sizeof(float4) * S);
     BALLOC(W.o_vel, sizeof(float4) * S);
     BALLOC(W.o_id, sizeof(uint32_t) * S);
@@ -188,7 +189,7 @@ extern "C" int obem_batch_create(obem_batch **out, obem_ctx *ctx, int32_t n_cham
     BALLOC(W.ph_cursor, sizeof(int32_t) * OBEM_PH_BUCKETS);
     BALLOC(W.ph_sorted, sizeof(int32_t) * S);
     BALLOC(W.ph_bsum, sizeof(int32_t) * (OBEM_PH_BUCKETS / 1024 + 1));
-    BALLOC(W.mpart, sizeof(double) * 13 * (S / 256));
+    BALLOC(W.mpart, sizeof(double) * 13 * (S / 1024));
     if (rc == OBEM_OK) {
         std::vector<int2> pan(nb, make_int2(0, 0));
         if (cudaMemcpy(b->d_cham_pan, pan.data(), sizeof(int2) * nb, cudaMemcpyHostToDevice) != cudaSuccess)
@@ -388,6 +389,7 @@ extern "C" int obem_batch_step(obem_batch *b, const obem_state *st, const float 
     B.stats = stats;
     B.ctl = b->d_ctl;
     B.abort = b->d_abort;
+    B.n_rec = b->d_abort + 1;
     B.step = step;
     return obem_launch_step_batch(b->ctx, st, B, b->W, E, s);
 }

@@ -100,7 +100,8 @@ extern "C" int obem_create(obem_ctx **out, const obem_config *cfg)
     ALLOC(c->s_ionkey, sizeof(unsigned long long) * cap);
     ALLOC(c->s_keep, sizeof(int32_t) * cap);
     ALLOC(c->s_nsp, sizeof(int32_t) * cap);
-    ALLOC(c->s_blk, sizeof(int32_t) * 4 * max_blocks);
+    ALLOC(c->s_blk, sizeof(int32_t) * 2 * ((size_t)cap / 32 + 8));
+    ALLOC(c->s_rec, sizeof(float4) * OBEM_REC_F4 * ((size_t)cap / 2 + 1));
     ALLOC(c->s_mpart, sizeof(double) * 13 * max_blocks);
     ALLOC(c->s_ctl, sizeof(StepCtl));
     ALLOC(c->o_pos, sizeof(float4) * cap);
@@ -179,9 +180,9 @@ extern "C" void obem_destroy(obem_ctx *c)
 {
     if (!c) return;
     free_mesh(c);
-    free_dev(c->d_egrid); free_dev(c->d_xs);
+    free_dev(c->d_egrid); free_dev(c->d_xs); free_dev(c->d_elut);
     free_dev(c->s_E); free_dev(c->s_prop); free_dev(c->s_ionkey); free_dev(c->s_keep);
-    free_dev(c->s_nsp); free_dev(c->s_blk); free_dev(c->s_ctl); free_dev(c->o_pos); free_dev(c->s_mpart);
+    free_dev(c->s_nsp); free_dev(c->s_blk); free_dev(c->s_ctl); free_dev(c->o_pos); free_dev(c->s_mpart); free_dev(c->s_rec);
     free_dev(c->o_vel); free_dev(c->o_id); free_dev(c->o_birth); free_dev(c->o_sp);
     free_dev(c->s_code); free_dev(c->s_perm); free_dev(c->s_hist); free_dev(c->s_blocks); free_dev(c->s_nblocks);
     free_dev(c->s_tk); free_dev(c->s_tv); free_dev(c->s_rh);
@@ -282,6 +283,34 @@ static void derive_gas(obem_ctx *c)
     g.rc2 = (float)(rc * rc);
 }
 
+// For every value k of a binary32 number's leading 14 bits: lo | hi << 16 with
+// grid[lo] <= e < grid[hi] for each energy e of those bits inside the grid.
+void obem_energy_lut(const float *grid, int n, uint32_t *lut)
+{
+    auto last = [&](float x) {                     // last grid point <= x, -1 if none
+        int lo = -1, hi = n;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) / 2;
+            if (grid[mid] <= x) lo = mid; else hi = mid;
+        }
+        return lo;
+    };
+    for (uint32_t k = 0; k < OBEM_ELUT; ++k) {
+        int lo = 0, hi = n - 1;
+        const uint32_t b0 = k << OBEM_ELUT_SHIFT, b1 = (k + 1) << OBEM_ELUT_SHIFT;
+        if (b1 <= 0x7f800000u) {                   // finite energies (the others keep the whole grid)
+            float f0, f1;
+            memcpy(&f0, &b0, 4);
+            memcpy(&f1, &b1, 4);
+            lo = last(f0);
+            hi = last(f1) + 1;
+            lo = lo < 0 ? 0 : (lo > n - 2 ? n - 2 : lo);
+            hi = hi < lo + 1 ? lo + 1 : (hi > n - 1 ? n - 1 : hi);
+        }
+        lut[k] = (uint32_t)lo | ((uint32_t)hi << 16);
+    }
+}
+
 extern "C" int obem_gas_load(obem_ctx *c, const obem_gas *gs)
 {
     if (!c || !gs) return OBEM_ERR_ARG;
@@ -299,16 +328,34 @@ extern "C" int obem_gas_load(obem_ctx *c, const obem_gas *gs)
     if (!(gs->N >= 0.0) || !(gs->T >= 0.0) || !(gs->nu_ion >= 0.0))
         return obem_fail(c, OBEM_ERR_ARG, "gas: negative N, T or nu_ion");
     int ne = gs->n_energy, npr = gs->n_proc;
-    free_dev(c->d_egrid); free_dev(c->d_xs);
-    c->d_egrid = NULL; c->d_xs = NULL;
+    free_dev(c->d_egrid); free_dev(c->d_xs); free_dev(c->d_elut);
+    c->d_egrid = NULL; c->d_xs = NULL; c->d_elut = NULL;
     OBEM_CUDA(c, cudaMalloc((void **)&c->d_egrid, sizeof(float) * ne));
     OBEM_CUDA(c, cudaMalloc((void **)&c->d_xs, sizeof(float) * ne * npr));
+    OBEM_CUDA(c, cudaMalloc((void **)&c->d_elut, sizeof(uint32_t) * OBEM_ELUT));
     OBEM_CUDA(c, cudaMemcpy(c->d_egrid, gs->energy_eV, sizeof(float) * ne, cudaMemcpyHostToDevice));
-    OBEM_CUDA(c, cudaMemcpy(c->d_xs, gs->sigma_m2, sizeof(float) * ne * npr, cudaMemcpyHostToDevice));
+    {
+        float *xt = (float *)malloc(sizeof(float) * ne * npr);
+        uint32_t *lut = (uint32_t *)malloc(sizeof(uint32_t) * OBEM_ELUT);
+        cudaError_t e = xt && lut ? cudaSuccess : cudaErrorMemoryAllocation;
+        if (e == cudaSuccess) {
+            for (int i = 0; i < ne; ++i)
+                for (int j = 0; j < npr; ++j) xt[(size_t)i * npr + j] = gs->sigma_m2[(size_t)j * ne + i];
+            obem_energy_lut(gs->energy_eV, ne, lut);
+            e = cudaMemcpy(c->d_xs, xt, sizeof(float) * ne * npr, cudaMemcpyHostToDevice);
+        }
+        if (e == cudaSuccess) e = cudaMemcpy(c->d_elut, lut, sizeof(uint32_t) * OBEM_ELUT, cudaMemcpyHostToDevice);
+        free(xt);
+        free(lut);
+        OBEM_CUDA(c, e);
+    }
     GasDev &g = c->gas;
     memset(&g, 0, sizeof g);
     g.egrid = c->d_egrid;
     g.xs = c->d_xs;
+    g.elut = c->d_elut;
+    g.e_first = gs->energy_eV[0];
+    g.e_last = gs->energy_eV[ne - 1];
     g.n_proc = npr;
     g.n_e = ne;
     c->gas_T = gs->T; c->gas_N = gs->N; c->gas_M_amu = gs->M_amu; c->gas_nu_ion = gs->nu_ion;

@@ -24,12 +24,20 @@
 #define OBEM_MAX_TRIALS 256
 #define OBEM_NCOUNTERS 7      // evaluation counters of the profiling variants of the field kernels
 
+// grid-segment bounds by the leading bits of a binary32 energy (sign, exponent,
+// 5 of the fraction)
+#define OBEM_ELUT_SHIFT 18
+#define OBEM_ELUT 8192
+#define OBEM_REC_F4 4          // float4 per record of a spawned pair (step.cu)
+
 // ---------------------------------------------------------------- gas constants
 // Everything the step kernels need, passed by value.  The float members are
 // derived in FP64 on the host and rounded once.
 struct GasDev {
     const float *egrid;   // [n_e]
-    const float *xs;      // [n_proc][n_e]
+    const float *xs;      // [n_e][n_proc]: the processes of a grid point together
+    const uint32_t *elut; // [OBEM_ELUT]: bounds lo | hi << 16 of the grid segment by an energy's leading bits
+    float e_first, e_last;
     int n_proc, n_e;
     int kind[OBEM_MAX_PROC];
     int mode[OBEM_MAX_PROC];
@@ -86,6 +94,7 @@ struct StepCtl {
     int32_t n_keep;       // survivors
     int32_t n_spawn;      // spawned pairs
     int32_t trial_overflow;
+    int32_t n_rec;        // records of spawned pairs
 };
 
 // What differs between the chambers of a batch in the tracking step: Philox
@@ -107,6 +116,7 @@ struct StepBatch {
     obem_step_stats *stats;      // [nb]
     StepCtl *ctl;                // [nb]
     int32_t *abort;              // [1]
+    int32_t *n_rec;              // [1] records of spawned pairs, all chambers
     uint32_t *step;              // [1] step index, advanced when the batch commits
 };
 
@@ -118,7 +128,8 @@ struct BtScratch {
     uint32_t *o_id, *o_birth;
     uint8_t *o_sp;
     int32_t *ph_bucket, *ph_count, *ph_start, *ph_cursor, *ph_sorted, *ph_bsum;
-    double *mpart;           // per-block partial moments (13 per block of 256 slots)
+    double *mpart;           // per-block partial moments (13 per block of 1024 slots)
+    float4 *rec;             // records of spawned pairs, OBEM_REC_F4 float4 each, one per two slots
 };
 
 struct obem_ctx {
@@ -129,6 +140,7 @@ struct obem_ctx {
     int gas_loaded;
     GasDev gas;
     float *d_egrid, *d_xs;
+    uint32_t *d_elut;
     float gas_thr_ioni;
     double gas_T, gas_N, gas_M_amu, gas_nu_ion;
     // mesh
@@ -184,8 +196,9 @@ struct obem_ctx {
     float4 *s_E;
     unsigned long long *s_prop, *s_ionkey;
     int32_t *s_keep, *s_nsp;
-    int32_t *s_blk;       // per-block sums / offsets (2 * max_blocks)
-    double *s_mpart;      // per-block partial moments (13 * max_blocks)
+    int32_t *s_blk;       // per-chunk (survivors, spawned pairs), then those before the chunk
+    double *s_mpart;      // per-block partial moments (13 per 1024 charges)
+    float4 *s_rec;        // records of spawned pairs, OBEM_REC_F4 float4 each, one per two charges
     StepCtl *s_ctl;
     float4 *o_pos, *o_vel;
     uint32_t *o_id, *o_birth;
@@ -379,6 +392,7 @@ int obem_launch_direct_pairs(obem_ctx *ctx, const FieldLaunch &L, const SymBatch
 size_t obem_sym_sizes(int capacity, size_t *ipart_floats);
 int obem_cell_layout(const double *tri, const int32_t *kind, int np, float4 *ca, float4 *g0, float4 *g1,
                      float4 *g2, float4 *nr, float4 *cl);
+void obem_energy_lut(const float *grid, int n, uint32_t *lut);
 void obem_cell_geo64(const double *tri, int np, double *geo);
 size_t obem_sym_jpart_floats(int capacity);
 size_t obem_sym_pass_jpart_floats(int capacity);

@@ -11,17 +11,22 @@
 //   init      zero the stats and the control block
 //   partners  nearest eligible cation of every electron (spatial hash, ph_*)
 //   resolve   each proposing electron atomicMin's (d^2, e) into its cation
-//   count     simulate every charge without writing: survivors, spawn counts,
-//             per-block totals for the scan
-//   scan      one block: block offsets, totals, capacity check (all-or-nothing)
-//   write     simulate again (same counters, same draws) and write survivors
-//             and spawned charges to their final slots in scratch
-//   commit    copy scratch to the caller's arrays, update n and next_id
-//   moments   species counts and cloud moments of the new state
+//   count     simulate every charge: its new state to scratch at its own
+//             index, ionisation products to a list of records, survivors and
+//             spawned pairs per chunk of charges
+//   scan      one block: chunk offsets, totals, capacity check (all-or-nothing)
+//   write     survivors and spawned charges from scratch to their final slots
+//   moments   species counts and cloud moments of the new state, then the
+//             blocks' partial sums folded and n, next_id updated
 // The bt_* kernels at the end run the same passes for a batch of chambers.
 #include "obem_internal.cuh"
 
 #define ST_THREADS 256
+#define ST_CT 128                  // threads of the count and write kernels (4 warps, a chunk of charges each)
+#define ST_CHUNK_S 32              // charges per chunk: contexts of at most ST_SMALL charges, so that few charges
+#define ST_CHUNK_L 256             // still fill the SMs; larger ones refill a warp's idle lanes from its chunk
+#define ST_SMALL 65536
+#define ST_MB 1024                 // charges per block of the moments
 
 typedef unsigned long long u64;
 
@@ -124,14 +129,18 @@ __device__ __forceinline__ float next_toward(float x, float dir)
     return __int_as_float(up == pos ? b + 1 : b - 1);
 }
 
-// grid segment and weight of energy eps (linear interpolation in energy)
+// grid segment and weight of energy eps (linear interpolation in energy): the
+// segment is the last grid point <= eps, searched between the bounds that
+// elut holds for eps's leading bits (the 2000-point grid: 2 steps, not 11)
 __device__ __forceinline__ void egrid_locate(const GasDev &g, float eps, int &lo, float &w)
 {
-    int hi = g.n_e - 1;
     lo = 0;
-    if (eps < __ldg(&g.egrid[0])) { lo = 0; w = 0.0f; }
-    else if (eps >= __ldg(&g.egrid[g.n_e - 1])) { lo = g.n_e - 2; w = 1.0f; }
+    if (eps < g.e_first) { lo = 0; w = 0.0f; }
+    else if (eps >= g.e_last) { lo = g.n_e - 2; w = 1.0f; }
     else {
+        const uint32_t b = __ldg(&g.elut[(__float_as_uint(eps) >> OBEM_ELUT_SHIFT) & (OBEM_ELUT - 1)]);
+        lo = (int)(b & 0xffffu);
+        int hi = (int)(b >> 16);
         while (hi - lo > 1) {
             int mid = (lo + hi) / 2;
             if (__ldg(&g.egrid[mid]) <= eps) lo = mid; else hi = mid;
@@ -141,16 +150,17 @@ __device__ __forceinline__ void egrid_locate(const GasDev &g, float eps, int &lo
     }
 }
 
-// collision frequency of process j (zero below its threshold)
+// collision frequency of process j (zero below its threshold); the table
+// holds every process of a grid point together
 __device__ __forceinline__ float nu_proc(const GasDev &g, int j, float eps, float Ns, int lo, float w)
 {
     if (g.mode[j] == OBEM_MODE_CONST) return g.nuc[j];
-    const float *row = g.xs + (size_t)j * g.n_e;
-    float s0 = __ldg(&row[lo]);
-    float s1 = __ldg(&row[lo + 1]);
+    if (eps < g.thr[j]) return Ns * 0.0f;
+    const float *row = g.xs + (size_t)lo * g.n_proc + j;
+    float s0 = __ldg(row);
+    float s1 = __ldg(row + g.n_proc);
     float ds = s1 - s0;
     float sg = s0 + w * ds;
-    if (eps < g.thr[j]) sg = 0.0f;
     return Ns * sg;
 }
 
@@ -165,16 +175,26 @@ __device__ __forceinline__ ChamberP chamber_of(const GasDev &g)
 struct FlightOut {
     int dead, attached, nsp, collisions, trials, overflow;
     int hit_cell;         // cell that absorbed the charge, or -1
+    int rec;              // record of its last spawned pair, or -1
+};
+
+// Records of the spawned pairs (OBEM_REC_F4 float4 each, in the order of the
+// race: only the links matter): electron position and the previous record of
+// the same parent, electron velocity, cation position, cation velocity.  A step
+// that commits spawns at most half the capacity; later records are dropped.
+struct SpawnRec {
+    float4 *rec;
+    int *count;
+    int max;
 };
 
 // One collision trial at the charge's current state: with x uniform in
 // [0, scale), process j is taken when x < nu_1 + ... + nu_j (none: null).
 // Returns 0 when nothing happened (null, or ionisation without the energy),
 // 1 after a collision, 2 when the flight ends (attachment).
-template <bool EMIT>
-__device__ int collide(const GasDev &g, const ChamberP &cp, uint32_t id, uint32_t step, uint32_t k, const uint4 &r, float x,
-                       float3 &p, float3 &v, uint8_t &sp, FlightOut &fo, float4 *o_pos, float4 *o_vel,
-                       uint32_t *o_id, uint32_t *o_birth, uint8_t *o_sp, int sbase, uint32_t id_base)
+__device__ __forceinline__ int collide(const GasDev &g, const ChamberP &cp, uint32_t id, uint32_t step, uint32_t k,
+                                       const uint4 &r, float x, float3 &p, float3 &v, uint8_t &sp, FlightOut &fo,
+                                       const SpawnRec &R)
 {
     float v2 = v.x * v.x + v.y * v.y + v.z * v.z;
     float speed = sqrtf(v2);
@@ -229,20 +249,16 @@ __device__ int collide(const GasDev &g, const ChamberP &cp, uint32_t id, uint32_
                 else if (axi == 1) { pn.y = next_toward(p.y, d.y); pp.y = next_toward(p.y, -d.y); }
                 else { pn.z = next_toward(p.z, d.z); pp.z = next_toward(p.z, -d.z); }
             }
-            if (EMIT) {
+            const int slot = atomicAdd(R.count, 1);
+            if (slot < R.max) {
                 uint4 r2 = philox4x32_10(make_uint4(id, step, k, 1u), cp.seed_lo, cp.seed_hi);
                 float3 di = isotropic(r2.x, r2.y);
-                int slot = sbase + 2 * fo.nsp;
-                o_pos[slot] = make_float4(pn.x, pn.y, pn.z, -(float)OBEM_QE);
-                o_vel[slot] = make_float4(sn * d.x, sn * d.y, sn * d.z, 0.0f);
-                o_id[slot] = id_base + (uint32_t)(2 * fo.nsp);
-                o_birth[slot] = step + 1u;
-                o_sp[slot] = OBEM_ELECTRON;
-                o_pos[slot + 1] = make_float4(p.x, p.y, p.z, (float)OBEM_QE);
-                o_vel[slot + 1] = make_float4(g.v_th_ion * di.x, g.v_th_ion * di.y, g.v_th_ion * di.z, 0.0f);
-                o_id[slot + 1] = id_base + (uint32_t)(2 * fo.nsp + 1);
-                o_birth[slot + 1] = step + 1u;
-                o_sp[slot + 1] = OBEM_CATION;
+                float4 *o = R.rec + (size_t)OBEM_REC_F4 * slot;
+                o[0] = make_float4(pn.x, pn.y, pn.z, __int_as_float(fo.rec));
+                o[1] = make_float4(sn * d.x, sn * d.y, sn * d.z, 0.0f);
+                o[2] = make_float4(p.x, p.y, p.z, 0.0f);
+                o[3] = make_float4(g.v_th_ion * di.x, g.v_th_ion * di.y, g.v_th_ion * di.z, 0.0f);
+                fo.rec = slot;
             }
             p = pp;
             v = make_float3(-sn * d.x, -sn * d.y, -sn * d.z);
@@ -333,35 +349,40 @@ __device__ __forceinline__ bool flight(const GasDev &g, const ChamberP &cp, floa
     return p.z <= cp.z_lo || p.z >= cp.z_hi;
 }
 
-// Flight of charge i over one step under the field E (Euler in the field,
-// exact ballistic motion between trials).  Collision sampling: null-collision
-// trials at exponential waiting times -ln(U)/nu_max, process j with
-// probability nu_j(eps)/nu_max (coll_mode 0); or the paper's per-step scheme
-// (coll_mode 1): flight over the whole step, then one interaction when
+// A charge in flight
+struct Fly {
+    float3 p, v;
+    float ax, ay, az;
+    float t;              // time since the start of the step
+    uint32_t id, k;       // id, trials drawn
+    uint8_t s0, sp;       // species at the start of the step, now
+    FlightOut fo;
+};
+
+// One part of a charge's flight over the step under its step-start field
+// (Euler in the field, exact ballistic motion between trials); returns true
+// when the charge is done.  Collision sampling: null-collision trials at
+// exponential waiting times -ln(U)/nu_max, process j with probability
+// nu_j(eps)/nu_max (coll_mode 0; a call is one trial); or the paper's per-step
+// scheme (coll_mode 1): flight over the whole step, then one interaction when
 // -ln(U) < nu_tot(eps) dt, of type j with probability nu_j/nu_tot.
 // Ionisation products at the distance of Eq. (distIoni).  A charge is
 // absorbed where a sub-flight's chord crosses a cell (g.hit_on: charging-up)
-// or where it ends beyond a plane z_lo / z_hi.  When EMIT is set,
-// spawned pairs are written to o_* at slots sbase, sbase+1...
-template <bool EMIT>
-__device__ void fly(const GasDev &g, const ChamberP &cp, uint32_t id, uint32_t step, float3 &p, float3 &v, uint8_t &sp,
-                    float3 E, FlightOut &fo, float4 *o_pos, float4 *o_vel, uint32_t *o_id,
-                    uint32_t *o_birth, uint8_t *o_sp, int sbase, uint32_t id_base)
+// or where it ends beyond a plane z_lo / z_hi.
+__device__ __forceinline__ bool fly_part(const GasDev &g, const ChamberP &cp, uint32_t step, Fly &f, const SpawnRec &R)
 {
-    const int s = sp;
-    const float qm = g.qm[s];
-    const float ax = qm * E.x, ay = qm * E.y, az = qm * E.z;
-    const float hx = 0.5f * ax, hy = 0.5f * ay, hz = 0.5f * az;
+    const int s = f.s0;
+    const float hx = 0.5f * f.ax, hy = 0.5f * f.ay, hz = 0.5f * f.az;
     if (g.coll_mode == 1) {
-        const float3 p0 = p;
-        const bool crossed = flight(g, cp, p, v, ax, ay, az, hx, hy, hz, g.dt);
-        if (g.hit_on && (fo.hit_cell = seg_hit(g, p0, p)) >= 0) { fo.dead = 1; return; }
-        if (crossed) { fo.dead = 1; return; }
-        const uint4 r = philox4x32_10(make_uint4(id, step, 1u, 0u), cp.seed_lo, cp.seed_hi);
-        fo.trials += 1;
+        const float3 p0 = f.p;
+        const bool crossed = flight(g, cp, f.p, f.v, f.ax, f.ay, f.az, hx, hy, hz, g.dt);
+        if (g.hit_on && (f.fo.hit_cell = seg_hit(g, p0, f.p)) >= 0) { f.fo.dead = 1; return true; }
+        if (crossed) { f.fo.dead = 1; return true; }
+        const uint4 r = philox4x32_10(make_uint4(f.id, step, 1u, 0u), cp.seed_lo, cp.seed_hi);
+        f.fo.trials += 1;
         float nu_tot;
         if (s == OBEM_ELECTRON) {
-            float v2 = v.x * v.x + v.y * v.y + v.z * v.z;
+            float v2 = f.v.x * f.v.x + f.v.y * f.v.y + f.v.z * f.v.z;
             float speed = sqrtf(v2);
             float eps = g.K_e * v2;
             int lo;
@@ -374,38 +395,31 @@ __device__ void fly(const GasDev &g, const ChamberP &cp, uint32_t id, uint32_t s
             nu_tot = g.nu_ion;
         }
         float pr = nu_tot * g.dt;
-        if (!(neg_log_unif(r.x) < pr)) return;
-        collide<EMIT>(g, cp, id, step, 1u, r, unif01(r.y) * nu_tot, p, v, sp, fo, o_pos, o_vel, o_id, o_birth,
-                      o_sp, sbase, id_base);
-        return;
+        if (!(neg_log_unif(r.x) < pr)) return true;
+        collide(g, cp, f.id, step, 1u, r, unif01(r.y) * nu_tot, f.p, f.v, f.sp, f.fo, R);
+        return true;
     }
     const float numax = (s == OBEM_ELECTRON) ? g.nu_max_e : g.nu_ion;
-    float t = 0.0f;
-    uint32_t k = 0;
-    for (;;) {
-        float tau;
-        uint4 r = make_uint4(0u, 0u, 0u, 0u);
-        if (numax > 0.0f) {
-            k += 1u;
-            if ((int)k > g.trial_cap) { fo.overflow = 1; return; }
-            r = philox4x32_10(make_uint4(id, step, k, 0u), cp.seed_lo, cp.seed_hi);
-            tau = neg_log_unif(r.x) / numax;
-        } else {
-            tau = __int_as_float(0x7f800000);
-        }
-        float tn = t + tau;
-        float fl = (tn >= g.dt) ? (g.dt - t) : tau;
-        const float3 p0 = p;
-        const bool crossed = flight(g, cp, p, v, ax, ay, az, hx, hy, hz, fl);
-        if (g.hit_on && (fo.hit_cell = seg_hit(g, p0, p)) >= 0) { fo.dead = 1; return; }
-        if (crossed) { fo.dead = 1; return; }
-        if (tn >= g.dt) return;
-        t = tn;
-        fo.trials += 1;
-        if (collide<EMIT>(g, cp, id, step, k, r, unif01(r.y) * numax, p, v, sp, fo, o_pos, o_vel, o_id, o_birth,
-                          o_sp, sbase, id_base) == 2)
-            return;
+    float tau;
+    uint4 r = make_uint4(0u, 0u, 0u, 0u);
+    if (numax > 0.0f) {
+        f.k += 1u;
+        if ((int)f.k > g.trial_cap) { f.fo.overflow = 1; return true; }
+        r = philox4x32_10(make_uint4(f.id, step, f.k, 0u), cp.seed_lo, cp.seed_hi);
+        tau = neg_log_unif(r.x) / numax;
+    } else {
+        tau = __int_as_float(0x7f800000);
     }
+    float tn = f.t + tau;
+    float fl = (tn >= g.dt) ? (g.dt - f.t) : tau;
+    const float3 p0 = f.p;
+    const bool crossed = flight(g, cp, f.p, f.v, f.ax, f.ay, f.az, hx, hy, hz, fl);
+    if (g.hit_on && (f.fo.hit_cell = seg_hit(g, p0, f.p)) >= 0) { f.fo.dead = 1; return true; }
+    if (crossed) { f.fo.dead = 1; return true; }
+    if (tn >= g.dt) return true;
+    f.t = tn;
+    f.fo.trials += 1;
+    return collide(g, cp, f.id, step, f.k, r, unif01(r.y) * numax, f.p, f.v, f.sp, f.fo, R) == 2;
 }
 
 // ------------------------------------------------------------------ kernels
@@ -422,15 +436,17 @@ __global__ void init_kernel(obem_step_stats *stats, StepCtl *ctl, const obem_sta
 
 // ---------------------------------------------------------------- partner search
 // Nearest eligible cation within R_c for every electron, by spatial hashing:
-// cells of edge h = R_c (1 + 1e-5) are hashed into PH_BUCKETS buckets, the
+// cells of edge h = 2 R_c (1 + 1e-5) are hashed into PH_BUCKETS buckets, the
 // eligible cations (not created in the previous step) are counting-sorted by
-// bucket, and each electron scans the buckets of its 27 neighbouring cells,
-// keeping the smallest (binary32 d^2, index) key with d^2 <= R_c^2.  Every
-// cation within R_c lies in one of those cells and hash collisions only add
-// candidates that the distance test rejects, so the result is the exact
-// minimum over all cations (the same key as a brute-force scan, whatever the
-// order in a bucket).  Cell coordinates are computed in FP64 (exact floor to
-// ~1e-8 of a cell at metre-scale positions).
+// bucket, and each electron scans the buckets of the 8 cells that the cube of
+// half-edge R_c around it can touch (its own and, per axis, the neighbour on
+// its side of the cell's middle; cells of R_c took 27), keeping the smallest
+// (binary32 d^2, index) key with d^2 <= R_c^2.  Every cation within R_c lies in
+// one of those cells and hash collisions only add candidates that the
+// distance test rejects, so the result is the exact minimum over all cations
+// (the same key as a brute-force scan, whatever the order in a bucket).  Cell
+// coordinates are computed in FP64 (exact to ~1e-8 of a cell at metre-scale
+// positions, against the margin of 5e-6 of a cell).
 #define PH_BUCKETS (1 << 20)
 
 __device__ __forceinline__ uint32_t ph_hash(long long cx, long long cy, long long cz)
@@ -449,6 +465,13 @@ __device__ __forceinline__ void ph_cell(float4 p, double inv_h, long long &cx, l
     cx = ph_coord(p.x, inv_h);
     cy = ph_coord(p.y, inv_h);
     cz = ph_coord(p.z, inv_h);
+}
+// x's cell in c[0], the neighbour on x's side of its middle in c[1]
+__device__ __forceinline__ void ph_coord2(float x, double inv_h, long long (&c)[2])
+{
+    const double t = (double)x * inv_h, k = floor(t);
+    c[0] = (long long)fmin(fmax(k, -4.0e18), 4.0e18);
+    c[1] = c[0] + (t - k < 0.5 ? -1 : 1);
 }
 
 __global__ void ph_count_kernel(const obem_state st, uint32_t step, double inv_h, int32_t *bucket_of,
@@ -542,13 +565,20 @@ __global__ void ph_query_kernel(const obem_state st, GasDev g, double inv_h, con
     u64 best = ~0ull;
     if (st.species[i] == OBEM_ELECTRON) {
         const float4 pe = reinterpret_cast<const float4 *>(st.pos_q)[i];
-        long long cx, cy, cz;
-        ph_cell(pe, inv_h, cx, cy, cz);
-        for (int dz = -1; dz <= 1; ++dz)
-            for (int dy = -1; dy <= 1; ++dy)
-                for (int dx = -1; dx <= 1; ++dx) {
-                    const uint32_t h = ph_hash(cx + dx, cy + dy, cz + dz);
-                    for (int k = start[h]; k < start[h + 1]; ++k) {
+        long long cx[2], cy[2], cz[2];
+        ph_coord2(pe.x, inv_h, cx);
+        ph_coord2(pe.y, inv_h, cy);
+        ph_coord2(pe.z, inv_h, cz);
+        int k0[8], k1[8];                      // the eight buckets' loads in flight together
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            const uint32_t h = ph_hash(cx[m & 1], cy[(m >> 1) & 1], cz[m >> 2]);
+            k0[m] = start[h];
+            k1[m] = start[h + 1];
+        }
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+                    for (int k = k0[m]; k < k1[m]; ++k) {
                         const int c = sorted[k];
                         const float4 pc = reinterpret_cast<const float4 *>(st.pos_q)[c];
                         const float ex = pe.x - pc.x, ey = pe.y - pc.y, ez = pe.z - pc.z;
@@ -600,96 +630,195 @@ __device__ __forceinline__ T block_sum(T v, T *sh)
     return t;   // valid in thread 0
 }
 
-__global__ void __launch_bounds__(ST_THREADS)
-count_kernel(const obem_state st, GasDev g, const float4 *E, uint32_t step, const u64 *prop,
-             const u64 *ionkey, int32_t *keep, int32_t *nsp, int32_t *blk, obem_step_stats *stats,
-             StepCtl *ctl, int32_t *s_hit)
+// ---------------------------------------------------------------- simulate
+// The new state of a chunk of charges, in scratch at the charges' own indices.
+struct StepScratch {
+    float4 *pos, *vel;
+    uint32_t *id, *birth;
+    uint8_t *sp;
+    int32_t *keep;         // spawned pairs << 1 | survives
+    int32_t *rec;          // last record of its spawned pairs, or -1
+    int32_t *blk;          // (survivors, spawned pairs) per chunk; after the scan, those before it
+    int32_t *hit;          // charging-up: cell << 1 | positive, or -1
+    SpawnRec R;
+};
+
+struct StepCounts {
+    int absorbed, attached, coll, rec, trials, ovf;
+};
+
+// Simulates the charges [i0, i0 + m), m <= WC, one warp.  The warp lists its
+// charges, electrons first, and its lanes take them from the list: a lane whose
+// charge is done takes the next one (once a quarter of the lanes are idle), so
+// that lanes do not wait for the charge with the most trials of 32, nor ions
+// (hardly a trial per step) for electrons (a dozen).  With 11.65 trials per
+// electron and half the charges ions, 36 % of the lane slots are busy in array
+// order and 84 % with the list (counted for Poisson trials, chunks of 256).
+// Measured with the one simulation per step (it was simulated again to write):
+// tracking of 1e6 charges 2124 to 725 us.
+template <int WC>
+__device__ __forceinline__ void step_chunk(const obem_state &st, const GasDev &g, const ChamberP &cp, const float4 *E,
+                                           uint32_t step, const u64 *prop, const u64 *ionkey, int i0, int m,
+                                           const StepScratch &W, uint8_t *list, int &nkeep, int &nspawn, StepCounts &n)
 {
-    __shared__ long long sh[ST_THREADS / 32];
-    const int n = cur_n(st);
-    int i = blockIdx.x * ST_THREADS + threadIdx.x;
-    int kp = 0, ns = 0, absorbed = 0, attached = 0, coll = 0, rec = 0, ovf = 0;
-    int hit = -1;
-    long long trials = 0;
-    if (i < n) {
-        uint8_t s = st.species[i];
-        if (recombined(i, s, prop, ionkey, g.recomb_on)) {
-            rec = (s == OBEM_CATION);
-        } else {
-            float4 pq = reinterpret_cast<const float4 *>(st.pos_q)[i];
-            float4 vv = reinterpret_cast<const float4 *>(st.vel)[i];
-            float4 e = E[i];
-            float3 p = make_float3(pq.x, pq.y, pq.z), v = make_float3(vv.x, vv.y, vv.z);
-            FlightOut fo = {0, 0, 0, 0, 0, 0, -1};
-            fly<false>(g, chamber_of(g), st.id[i], step, p, v, s, make_float3(e.x, e.y, e.z), fo, NULL, NULL, NULL,
-                       NULL, NULL, 0, 0u);
-            if (g.hit_on) hit = fo.hit_cell >= 0 ? (fo.hit_cell << 1) | (pq.w > 0.0f ? 1 : 0) : -1;
-            kp = !fo.dead;
-            ns = fo.nsp;
-            absorbed = fo.dead;
-            attached = fo.attached;
-            coll = fo.collisions;
-            trials = fo.trials;
-            ovf = fo.overflow;
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    int ne = 0, ni = 0;
+    for (int q = 0; q < m; q += 32) {
+        const int i = i0 + q + lane;
+        const bool in = q + lane < m;
+        uint8_t s = 0;
+        bool fly = false;
+        if (in) {
+            s = st.species[i];
+            W.id[i] = st.id[i];
+            W.birth[i] = st.birth[i];
+            fly = true;
+            if (recombined(i, s, prop, ionkey, g.recomb_on)) {
+                fly = false;
+                n.rec += s == OBEM_CATION;
+                W.keep[i] = 0;
+                if (g.hit_on) W.hit[i] = -1;
+            }
         }
-        keep[i] = kp;
-        nsp[i] = ns;
-        if (g.hit_on) s_hit[i] = hit;
+        const unsigned be = __ballot_sync(0xffffffffu, fly && s == OBEM_ELECTRON);
+        const unsigned bi = __ballot_sync(0xffffffffu, fly && s != OBEM_ELECTRON);
+        if ((be >> lane) & 1u) list[ne + __popc(be & below)] = (uint8_t)(q + lane);
+        if ((bi >> lane) & 1u) list[WC - 1 - ni - __popc(bi & below)] = (uint8_t)(q + lane);
+        ne += __popc(be);
+        ni += __popc(bi);
     }
-    long long t;
-    t = block_sum<long long>(kp, sh);
-    if (threadIdx.x == 0) blk[2 * blockIdx.x] = (int32_t)t;
-    t = block_sum<long long>(ns, sh);
-    if (threadIdx.x == 0) blk[2 * blockIdx.x + 1] = (int32_t)t;
-    t = block_sum<long long>(absorbed, sh);
-    if (threadIdx.x == 0 && t) atomicAdd(&stats->absorbed, (int)t);
-    t = block_sum<long long>(attached, sh);
-    if (threadIdx.x == 0 && t) atomicAdd(&stats->attached, (int)t);
-    t = block_sum<long long>(coll, sh);
-    if (threadIdx.x == 0 && t) atomicAdd(&stats->collisions, (int)t);
-    t = block_sum<long long>(rec, sh);
-    if (threadIdx.x == 0 && t) atomicAdd(&stats->recombined_pairs, (int)t);
-    t = block_sum<long long>(trials, sh);
-    if (threadIdx.x == 0 && t) atomicAdd((unsigned long long *)&stats->trials, (unsigned long long)t);
-    t = block_sum<long long>(ovf, sh);
-    if (threadIdx.x == 0 && t) atomicOr(&ctl->trial_overflow, 1);
+    __syncwarp();
+    const int total = ne + ni;
+    int head = 0, cur = -1;
+    Fly f;
+    nkeep = nspawn = 0;
+    for (;;) {
+        const unsigned idle = __ballot_sync(0xffffffffu, cur < 0);
+        if (idle && head < total && (__popc(idle) >= 8 || WC == 32)) {
+            const int e = head + __popc(idle & below);
+            if (cur < 0 && e < total) {
+                cur = i0 + list[e < ne ? e : WC - 1 - (e - ne)];
+                const float4 pq = reinterpret_cast<const float4 *>(st.pos_q)[cur];
+                const float4 vv = reinterpret_cast<const float4 *>(st.vel)[cur];
+                const float4 ee = E[cur];
+                f.id = st.id[cur];
+                f.s0 = f.sp = st.species[cur];
+                f.p = make_float3(pq.x, pq.y, pq.z);
+                f.v = make_float3(vv.x, vv.y, vv.z);
+                const float qm = g.qm[f.s0];
+                f.ax = qm * ee.x;
+                f.ay = qm * ee.y;
+                f.az = qm * ee.z;
+                f.t = 0.0f;
+                f.k = 0u;
+                f.fo = {0, 0, 0, 0, 0, 0, -1, -1};
+            }
+            head = min(total, head + __popc(idle));
+        }
+        if (!__any_sync(0xffffffffu, cur >= 0)) {
+            if (head >= total) break;
+            continue;
+        }
+        if (cur >= 0 && fly_part(g, cp, step, f, W.R)) {
+            const int i = cur;
+            cur = -1;
+            const int kp = !f.fo.dead;
+            if (kp) {
+                W.pos[i] = make_float4(f.p.x, f.p.y, f.p.z, st.pos_q[4 * (size_t)i + 3]);
+                W.vel[i] = make_float4(f.v.x, f.v.y, f.v.z, st.vel[4 * (size_t)i + 3]);
+                W.sp[i] = f.sp;
+            }
+            W.keep[i] = (f.fo.nsp << 1) | kp;
+            if (f.fo.nsp) W.rec[i] = f.fo.rec;
+            if (g.hit_on)
+                W.hit[i] = f.fo.hit_cell >= 0 ? (f.fo.hit_cell << 1) | (st.pos_q[4 * (size_t)i + 3] > 0.0f ? 1 : 0) : -1;
+            nkeep += kp;
+            nspawn += f.fo.nsp;
+            n.absorbed += f.fo.dead;
+            n.attached += f.fo.attached;
+            n.coll += f.fo.collisions;
+            n.trials += f.fo.trials;
+            n.ovf |= f.fo.overflow;
+        }
+    }
+    nkeep = (int)__reduce_add_sync(0xffffffffu, (unsigned)nkeep);
+    nspawn = (int)__reduce_add_sync(0xffffffffu, (unsigned)nspawn);
 }
 
-// single block: exclusive scan of the per-block (keep, spawn) totals
-__global__ void scan_kernel(const obem_state st, int32_t *blk, obem_step_stats *stats, StepCtl *ctl,
-                            int cap)
+// the block's counts to the stats (every thread calls it)
+__device__ __forceinline__ void step_counts(const StepCounts &n, obem_step_stats *stats, StepCtl *ctl)
 {
-    __shared__ int32_t sk[1024], ss[1024];
-    __shared__ int32_t carry_k, carry_s;
-    const int n = cur_n(st);
-    const int nb = (n + ST_THREADS - 1) / ST_THREADS;
-    if (threadIdx.x == 0) { carry_k = 0; carry_s = 0; }
+    __shared__ int s_n[6];
+    if (threadIdx.x < 6) s_n[threadIdx.x] = 0;
     __syncthreads();
-    for (int c0 = 0; c0 < nb; c0 += 1024) {
-        int b = c0 + threadIdx.x;
-        int vk = b < nb ? blk[2 * b] : 0;
-        int vs = b < nb ? blk[2 * b + 1] : 0;
-        sk[threadIdx.x] = vk;
-        ss[threadIdx.x] = vs;
-        __syncthreads();
-        for (int off = 1; off < 1024; off <<= 1) {
-            int ak = threadIdx.x >= off ? sk[threadIdx.x - off] : 0;
-            int as = threadIdx.x >= off ? ss[threadIdx.x - off] : 0;
-            __syncthreads();
-            sk[threadIdx.x] += ak;
-            ss[threadIdx.x] += as;
-            __syncthreads();
-        }
-        if (b < nb) {
-            blk[2 * b] = carry_k + sk[threadIdx.x] - vk;      // exclusive
-            blk[2 * b + 1] = carry_s + ss[threadIdx.x] - vs;
-        }
-        __syncthreads();
-        if (threadIdx.x == 1023) { carry_k += sk[1023]; carry_s += ss[1023]; }
-        __syncthreads();
+    const int v[6] = {n.absorbed, n.attached, n.coll, n.rec, n.trials, n.ovf};
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        const int t = (int)__reduce_add_sync(0xffffffffu, (unsigned)v[k]);
+        if ((threadIdx.x & 31) == 0 && t) atomicAdd(&s_n[k], t);
     }
+    __syncthreads();
+    const int k = threadIdx.x;
+    const int t = k < 6 ? s_n[k] : 0;
+    if (t) {
+        if (k == 0) atomicAdd(&stats->absorbed, t);
+        else if (k == 1) atomicAdd(&stats->attached, t);
+        else if (k == 2) atomicAdd(&stats->collisions, t);
+        else if (k == 3) atomicAdd(&stats->recombined_pairs, t);
+        else if (k == 4) atomicAdd((unsigned long long *)&stats->trials, (unsigned long long)t);
+        else atomicOr(&ctl->trial_overflow, 1);
+    }
+}
+
+template <int WC>
+__global__ void __launch_bounds__(ST_CT) count_kernel(const obem_state st, GasDev g, const float4 *E, uint32_t step,
+                                                      const u64 *prop, const u64 *ionkey, StepScratch W,
+                                                      obem_step_stats *stats, StepCtl *ctl)
+{
+    __shared__ uint8_t s_list[ST_CT / 32][WC];
+    const int n = cur_n(st);
+    if (blockIdx.x * (WC * (ST_CT / 32)) >= n) return;
+    const int ch = blockIdx.x * (ST_CT / 32) + (threadIdx.x >> 5);
+    StepCounts sc = {0, 0, 0, 0, 0, 0};
+    if (ch * WC < n) {                                   // warp-uniform
+        int nk, ns;
+        step_chunk<WC>(st, g, chamber_of(g), E, step, prop, ionkey, ch * WC, min(WC, n - ch * WC), W,
+                       s_list[threadIdx.x >> 5], nk, ns, sc);
+        if ((threadIdx.x & 31) == 0) { W.blk[2 * ch] = nk; W.blk[2 * ch + 1] = ns; }
+    }
+    step_counts(sc, stats, ctl);
+}
+
+// exclusive scan of the (survivors, spawned pairs) of nb chunks, one block of
+// 1024; returns the totals
+__device__ __forceinline__ void step_scan(int32_t *blk, int nb, int32_t &tk, int32_t &ts)
+{
+    __shared__ int32_t s_warp[32];
+    tk = ts = 0;
+    for (int c0 = 0; c0 < nb; c0 += 1024) {
+        const int b = c0 + threadIdx.x;
+        const int2 v = b < nb ? reinterpret_cast<const int2 *>(blk)[b] : make_int2(0, 0);
+        const int32_t ik = ph_block_scan(v.x, s_warp);
+        const int32_t wk = s_warp[31];
+        __syncthreads();
+        const int32_t is = ph_block_scan(v.y, s_warp);
+        const int32_t ws = s_warp[31];
+        __syncthreads();
+        if (b < nb) reinterpret_cast<int2 *>(blk)[b] = make_int2(tk + ik - v.x, ts + is - v.y);
+        tk += wk;
+        ts += ws;
+    }
+}
+
+// single block: chunk offsets, totals, capacity and trial checks
+__global__ void __launch_bounds__(1024) scan_kernel(const obem_state st, int32_t *blk, int chunk,
+                                                    obem_step_stats *stats, StepCtl *ctl, int cap)
+{
+    const int n = cur_n(st);
+    int32_t nk, nsp;
+    step_scan(blk, (n + chunk - 1) / chunk, nk, nsp);
     if (threadIdx.x == 0) {
-        int nk = carry_k, nsp = carry_s;
         long long total = (long long)nk + 2ll * nsp;
         ctl->n_keep = nk;
         ctl->n_spawn = nsp;
@@ -706,85 +835,76 @@ __global__ void scan_kernel(const obem_state st, int32_t *blk, obem_step_stats *
     }
 }
 
-__global__ void __launch_bounds__(ST_THREADS)
-write_kernel(const obem_state st, GasDev g, const float4 *E, uint32_t step, const u64 *prop,
-             const u64 *ionkey, const int32_t *keep, const int32_t *nsp, const int32_t *blk,
-             const StepCtl *ctl, float4 *o_pos, float4 *o_vel, uint32_t *o_id, uint32_t *o_birth,
-             uint8_t *o_sp)
+// Survivors of a chunk to their slots (in order from `off`), the pairs its
+// charges spawned to theirs (parents in order, a parent's pairs in trial
+// order: its records are linked last to first), the charges its cells
+// absorbed to the cells' counts.  Scratch is the only input: the state's
+// arrays can be written in place.
+template <int WC>
+__device__ __forceinline__ void write_chunk(const obem_state &st, uint32_t step, int i0, int m, int off, int n_keep,
+                                            uint32_t id0, const int32_t *blk, const StepScratch &W,
+                                            unsigned long long *deposit)
 {
-    __shared__ int32_t wk[ST_THREADS / 32], ws[ST_THREADS / 32];
-    if (ctl->abort) return;
-    const int n = cur_n(st);
-    int i = blockIdx.x * ST_THREADS + threadIdx.x;
-    int kp = 0, ns = 0;
-    if (i < n) { kp = keep[i]; ns = nsp[i]; }
-    // block-local exclusive scan
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int ik = kp, is = ns;
-    for (int o = 1; o < 32; o <<= 1) {
-        int a = __shfl_up_sync(0xffffffffu, ik, o);
-        int b = __shfl_up_sync(0xffffffffu, is, o);
-        if (lane >= o) { ik += a; is += b; }
-    }
-    if (lane == 31) { wk[warp] = ik; ws[warp] = is; }
-    __syncthreads();
-    int pk_ = 0, ps_ = 0;
-    for (int w = 0; w < warp; ++w) { pk_ += wk[w]; ps_ += ws[w]; }
-    const int out_keep = blk[2 * blockIdx.x] + pk_ + ik - kp;
-    const int out_spawn = blk[2 * blockIdx.x + 1] + ps_ + is - ns;
-    if (i >= n || (!kp && !ns)) return;
-    uint8_t s = st.species[i];
-    float4 pq = reinterpret_cast<const float4 *>(st.pos_q)[i];
-    float4 vv = reinterpret_cast<const float4 *>(st.vel)[i];
-    float4 e = E[i];
-    float3 p = make_float3(pq.x, pq.y, pq.z), v = make_float3(vv.x, vv.y, vv.z);
-    FlightOut fo = {0, 0, 0, 0, 0, 0, -1};
-    const int sbase = ctl->n_keep + 2 * out_spawn;
-    const uint32_t id_base = *st.next_id + (uint32_t)(2 * out_spawn);
-    fly<true>(g, chamber_of(g), st.id[i], step, p, v, s, make_float3(e.x, e.y, e.z), fo, o_pos, o_vel, o_id, o_birth,
-              o_sp, sbase, id_base);
-    if (kp) {
-        o_pos[out_keep] = make_float4(p.x, p.y, p.z, pq.w);
-        o_vel[out_keep] = make_float4(v.x, v.y, v.z, vv.w);
-        o_id[out_keep] = st.id[i];
-        o_birth[out_keep] = st.birth[i];
-        o_sp[out_keep] = s;
+    const int lane = threadIdx.x & 31;
+    int ok = blk[0], os = blk[1];
+    for (int q = 0; q < m; q += 32) {
+        const int i = i0 + q + lane;
+        const bool in = q + lane < m;
+        const int32_t v = in ? W.keep[i] : 0;
+        const bool kp = v & 1;
+        const int ns = v >> 1;
+        const unsigned bk = __ballot_sync(0xffffffffu, kp);
+        if (kp) {
+            const int o = off + ok + __popc(bk & ((1u << lane) - 1u));
+            reinterpret_cast<float4 *>(st.pos_q)[o] = W.pos[i];
+            reinterpret_cast<float4 *>(st.vel)[o] = W.vel[i];
+            st.id[o] = W.id[i];
+            st.birth[o] = W.birth[i];
+            st.species[o] = W.sp[i];
+        }
+        ok += __popc(bk);
+        if (__any_sync(0xffffffffu, ns > 0)) {
+            int is = ns;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, is, o);
+                if (lane >= o) is += u;
+            }
+            int r = ns ? W.rec[i] : -1;
+            for (int k = ns - 1; k >= 0; --k) {
+                const int pair = os + is - ns + k;
+                const float4 *e = W.R.rec + (size_t)OBEM_REC_F4 * r;
+                const float4 a = e[0], b = e[1], c = e[2], d = e[3];
+                const int o = off + n_keep + 2 * pair;
+                reinterpret_cast<float4 *>(st.pos_q)[o] = make_float4(a.x, a.y, a.z, -(float)OBEM_QE);
+                reinterpret_cast<float4 *>(st.vel)[o] = b;
+                st.id[o] = id0 + (uint32_t)(2 * pair);
+                st.birth[o] = step + 1u;
+                st.species[o] = OBEM_ELECTRON;
+                reinterpret_cast<float4 *>(st.pos_q)[o + 1] = make_float4(c.x, c.y, c.z, (float)OBEM_QE);
+                reinterpret_cast<float4 *>(st.vel)[o + 1] = d;
+                st.id[o + 1] = id0 + (uint32_t)(2 * pair + 1);
+                st.birth[o + 1] = step + 1u;
+                st.species[o + 1] = OBEM_CATION;
+                r = __float_as_int(a.w);
+            }
+            os += __shfl_sync(0xffffffffu, is, 31);
+        }
+        if (deposit && in) {
+            const int32_t h = W.hit[i];
+            if (h >= 0) atomicAdd(&deposit[h >> 1], (h & 1) ? 1ull : ~0ull);   // +1 or -1 (two's complement)
+        }
     }
 }
 
-__global__ void commit_kernel(const obem_state st, const StepCtl *ctl, const float4 *o_pos,
-                              const float4 *o_vel, const uint32_t *o_id, const uint32_t *o_birth,
-                              const uint8_t *o_sp)
-{
-    if (ctl->abort) return;
-    const int m = ctl->n_keep + 2 * ctl->n_spawn;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-        reinterpret_cast<float4 *>(st.pos_q)[i] = o_pos[i];
-        reinterpret_cast<float4 *>(st.vel)[i] = o_vel[i];
-        st.id[i] = o_id[i];
-        st.birth[i] = o_birth[i];
-        st.species[i] = o_sp[i];
-    }
-}
-
-__global__ void finish_kernel(const obem_state st, const StepCtl *ctl)
-{
-    if (threadIdx.x != 0 || ctl->abort) return;
-    *st.n = ctl->n_keep + 2 * ctl->n_spawn;
-    *st.next_id = *st.next_id + (uint32_t)(2 * ctl->n_spawn);
-}
-
-// charges absorbed by cells this step: deposits[cell] += +-1 (units of e),
-// only when the step commits (run before the count of charges is updated)
-__global__ void deposit_kernel(const obem_state st, const StepCtl *ctl, const int32_t *s_hit,
-                               unsigned long long *deposit)
+template <int WC>
+__global__ void __launch_bounds__(ST_CT) write_kernel(const obem_state st, uint32_t step, StepScratch W,
+                                                      const StepCtl *ctl, unsigned long long *deposit)
 {
     if (ctl->abort) return;
     const int n = cur_n(st);
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int32_t h = s_hit[i];
-    if (h >= 0) atomicAdd(&deposit[h >> 1], (h & 1) ? 1ull : ~0ull);   // +1 or -1 (two's complement)
+    const int ch = blockIdx.x * (ST_CT / 32) + (threadIdx.x >> 5);
+    if (ch * WC >= n) return;
+    write_chunk<WC>(st, step, ch * WC, min(WC, n - ch * WC), 0, ctl->n_keep, *st.next_id, W.blk + 2 * ch, W, deposit);
 }
 
 // free surface density of Eq. (charge-up): e * deposits / area on dielectric
@@ -805,81 +925,117 @@ int obem_launch_surface_sigma(obem_ctx *c, float *sigma_free, cudaStream_t s)
 }
 
 // Cloud moments of the new state.  Counts go to the stats by integer atomics
-// (exact in any order); the FP64 sums are reduced per block and the blocks'
-// partial sums added by moments_fold_kernel in block order, so the moments
-// are the same on every run.
+// (exact in any order); the FP64 sums are formed per thread over four charges,
+// reduced per block of ST_MB charges and the blocks' partial sums added by
+// moments_fold in block order, so the moments are the same on every run.
+// Bound: the FP64 pipe (2 FMAs per SM and clock): thirteen sums per charge
+// reduced by shuffles over every 256 charges took 213 us at 1e6 charges.
 #define NMOM 13    // sum_e[3], sum2_e[3], sum_i[3], sum2_i[3], sum_energy_e
 
-__device__ void moments_block(const obem_state &st, int i, bool live, obem_step_stats *stats, double *part)
+// charges i0 + threadIdx.x + ST_THREADS k below end; part[f * stride]
+__device__ __forceinline__ void moments_block(const obem_state &st, int i0, int end, obem_step_stats *stats,
+                                              double *part, int stride)
 {
-    __shared__ double shd[ST_THREADS / 32];
-    __shared__ long long shl[ST_THREADS / 32];
-    int ne = 0, nc = 0, na = 0;
-    double v[NMOM];
+    __shared__ double red[ST_THREADS / 32][16];
+    __shared__ int cnt[3];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x < 3) cnt[threadIdx.x] = 0;
+    __syncthreads();
+    double v[16];
 #pragma unroll
-    for (int f = 0; f < NMOM; ++f) v[f] = 0.0;
-    if (live) {
-        const uint8_t s = st.species[i];
-        const float4 p = reinterpret_cast<const float4 *>(st.pos_q)[i];
-        const double x[3] = {p.x, p.y, p.z};
+    for (int f = 0; f < 16; ++f) v[f] = 0.0;
+    int ne = 0, nc = 0, na = 0;
+#pragma unroll
+    for (int q = 0; q < ST_MB / ST_THREADS; ++q) {
+        const int i = i0 + q * ST_THREADS + threadIdx.x;
+        const uint8_t s = i < end ? st.species[i] : 255;
+        const float4 p = i < end ? reinterpret_cast<const float4 *>(st.pos_q)[i] : make_float4(0.f, 0.f, 0.f, 0.f);
         if (s == OBEM_ELECTRON) {
-            ne = 1;
-            for (int c = 0; c < 3; ++c) { v[c] = x[c]; v[3 + c] = x[c] * x[c]; }
             const float4 u = reinterpret_cast<const float4 *>(st.vel)[i];
-            const double v2 = (double)u.x * u.x + (double)u.y * u.y + (double)u.z * u.z;
-            v[12] = 0.5 * OBEM_ME * v2 / OBEM_QE;
-        } else {
-            if (s == OBEM_CATION) nc = 1; else na = 1;
-            for (int c = 0; c < 3; ++c) { v[6 + c] = x[c]; v[9 + c] = x[c] * x[c]; }
+            const double x = p.x, y = p.y, z = p.z;
+            v[0] += x; v[1] += y; v[2] += z;
+            v[3] += x * x; v[4] += y * y; v[5] += z * z;
+            v[12] += (double)u.x * u.x + (double)u.y * u.y + (double)u.z * u.z;
+        } else if (s != 255) {
+            const double x = p.x, y = p.y, z = p.z;
+            v[6] += x; v[7] += y; v[8] += z;
+            v[9] += x * x; v[10] += y * y; v[11] += z * z;
+        }
+        ne += __popc(__ballot_sync(0xffffffffu, s == OBEM_ELECTRON));
+        nc += __popc(__ballot_sync(0xffffffffu, s == OBEM_CATION));
+        na += __popc(__ballot_sync(0xffffffffu, s != OBEM_ELECTRON && s != OBEM_CATION && s != 255));
+    }
+    v[12] *= 0.5 * OBEM_ME / OBEM_QE;
+    if (lane == 0) {
+        if (ne) atomicAdd(&cnt[0], ne);
+        if (nc) atomicAdd(&cnt[1], nc);
+        if (na) atomicAdd(&cnt[2], na);
+    }
+    // sums over the lanes, a step halves the values a lane holds: lane l ends
+    // with value l >> 1
+    int o = 16;
+#pragma unroll
+    for (int k = 8; k > 0; k >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int f = 0; f < k; ++f) {
+            const double send = up ? v[f] : v[f + k], keep = up ? v[f + k] : v[f];
+            v[f] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
     }
-    long long t;
-    t = block_sum<long long>(ne, shl); if (threadIdx.x == 0 && t) atomicAdd(&stats->n_electron, (int)t);
-    t = block_sum<long long>(nc, shl); if (threadIdx.x == 0 && t) atomicAdd(&stats->n_cation, (int)t);
-    t = block_sum<long long>(na, shl); if (threadIdx.x == 0 && t) atomicAdd(&stats->n_anion, (int)t);
-    for (int f = 0; f < NMOM; ++f) {
-        const double d = block_sum<double>(v[f], shd);
-        if (threadIdx.x == 0) part[f] = d;
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    if ((lane & 1) == 0) red[warp][lane >> 1] = v[0];
+    __syncthreads();
+    if (threadIdx.x < NMOM) {
+        double t = red[0][threadIdx.x];
+        for (int w = 1; w < ST_THREADS / 32; ++w) t += red[w][threadIdx.x];
+        part[(size_t)threadIdx.x * stride] = t;
     }
+    if (threadIdx.x < 3 && cnt[threadIdx.x])
+        atomicAdd(threadIdx.x == 0 ? &stats->n_electron : threadIdx.x == 1 ? &stats->n_cation : &stats->n_anion,
+                  cnt[threadIdx.x]);
+}
+
+// charges after the step
+__device__ __forceinline__ int step_n(const obem_state &st, const StepCtl *ctl)
+{
+    return ctl->abort ? *st.n : ctl->n_keep + 2 * ctl->n_spawn;
 }
 
 __global__ void __launch_bounds__(ST_THREADS)
-moments_kernel(const obem_state st, obem_step_stats *stats, double *part)
+moments_kernel(const obem_state st, const StepCtl *ctl, obem_step_stats *stats, double *part, int stride)
 {
-    const int n = cur_n(st);
-    const int i = blockIdx.x * ST_THREADS + threadIdx.x;
-    if (blockIdx.x * ST_THREADS >= n) return;            // a block with no charge adds nothing
-    moments_block(st, i, i < n, stats, part + (size_t)NMOM * blockIdx.x);
+    const int n = step_n(st, ctl);
+    const int i0 = blockIdx.x * ST_MB;
+    if (i0 >= n) return;                                 // a block with no charge adds nothing
+    moments_block(st, i0, n, stats, part + blockIdx.x, stride);
 }
 
-// sum of the nb blocks' partial sums from part (NMOM per block), in block
-// order within each thread's stride and a fixed tree across threads (1024)
-__device__ void moments_fold(const double *part, int nb, obem_step_stats *stats)
+// sums of the nb blocks' partial sums part[f * stride + b]: warp f adds moment
+// f, its lanes' strides in block order and a fixed butterfly
+__device__ __forceinline__ void moments_fold(const double *part, int stride, int nb, obem_step_stats *stats)
 {
-    __shared__ double red[1024];
-    double *dst[NMOM] = {&stats->sum_e[0], &stats->sum_e[1], &stats->sum_e[2], &stats->sum2_e[0],
-                         &stats->sum2_e[1], &stats->sum2_e[2], &stats->sum_i[0], &stats->sum_i[1],
-                         &stats->sum_i[2], &stats->sum2_i[0], &stats->sum2_i[1], &stats->sum2_i[2],
-                         &stats->sum_energy_e};
-    for (int f = 0; f < NMOM; ++f) {
-        double acc = 0.0;
-        for (int b = threadIdx.x; b < nb; b += blockDim.x) acc += part[(size_t)NMOM * b + f];
-        red[threadIdx.x] = acc;
-        __syncthreads();
-        for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-            if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) *dst[f] = red[0];
-        __syncthreads();
+    const int f = threadIdx.x >> 5;
+    if (f >= NMOM) return;
+    double *const dst = f < 3 ? &stats->sum_e[f] : f < 6 ? &stats->sum2_e[f - 3] : f < 9 ? &stats->sum_i[f - 6]
+                      : f < 12 ? &stats->sum2_i[f - 9] : &stats->sum_energy_e;
+    double acc = 0.0;
+    for (int b = threadIdx.x & 31; b < nb; b += 32) acc += part[(size_t)f * stride + b];
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) *dst = acc;
+}
+
+// the fold, and the new counts
+__global__ void __launch_bounds__(32 * NMOM) finish_kernel(const obem_state st, const StepCtl *ctl, const double *part,
+                                                           int stride, obem_step_stats *stats)
+{
+    const int n = step_n(st, ctl);
+    moments_fold(part, stride, (n + ST_MB - 1) / ST_MB, stats);
+    __syncthreads();                                     // every thread has read the old count
+    if (threadIdx.x == 0 && !ctl->abort) {
+        *st.next_id = *st.next_id + (uint32_t)(2 * ctl->n_spawn);
+        *st.n = n;
     }
-}
-
-__global__ void __launch_bounds__(1024) moments_fold_kernel(const obem_state st, const double *part,
-                                                            obem_step_stats *stats)
-{
-    const int n = cur_n(st);
-    moments_fold(part, (n + ST_THREADS - 1) / ST_THREADS, stats);
 }
 
 // ====================================================================
@@ -904,13 +1060,20 @@ __global__ void sh_query_kernel(const obem_state st, const obem_state G, GasDev 
     u64 best = ~0ull, best_idx = 0;
     if (st.species[i] == OBEM_ELECTRON) {
         const float4 pe = reinterpret_cast<const float4 *>(st.pos_q)[i];
-        long long cx, cy, cz;
-        ph_cell(pe, inv_h, cx, cy, cz);
-        for (int dz = -1; dz <= 1; ++dz)
-            for (int dy = -1; dy <= 1; ++dy)
-                for (int dx = -1; dx <= 1; ++dx) {
-                    const uint32_t h = ph_hash(cx + dx, cy + dy, cz + dz);
-                    for (int k = start[h]; k < start[h + 1]; ++k) {
+        long long cx[2], cy[2], cz[2];
+        ph_coord2(pe.x, inv_h, cx);
+        ph_coord2(pe.y, inv_h, cy);
+        ph_coord2(pe.z, inv_h, cz);
+        int k0[8], k1[8];                      // the eight buckets' loads in flight together
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            const uint32_t h = ph_hash(cx[m & 1], cy[(m >> 1) & 1], cz[m >> 2]);
+            k0[m] = start[h];
+            k1[m] = start[h + 1];
+        }
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+                    for (int k = k0[m]; k < k1[m]; ++k) {
                         const int c = sorted[k];
                         const float4 pc = reinterpret_cast<const float4 *>(G.pos_q)[c];
                         const float ex = pe.x - pc.x, ey = pe.y - pc.y, ez = pe.z - pc.z;
@@ -980,6 +1143,44 @@ static GasDev step_gas(obem_ctx *c)
     return g;
 }
 
+// the context's scratch as the count and write kernels see it
+static StepScratch step_scratch(obem_ctx *c)
+{
+    StepScratch W;
+    W.pos = c->o_pos; W.vel = c->o_vel; W.id = c->o_id; W.birth = c->o_birth; W.sp = c->o_sp;
+    W.keep = c->s_keep; W.rec = c->s_nsp; W.blk = c->s_blk; W.hit = c->s_hit;
+    W.R.rec = c->s_rec; W.R.count = &c->s_ctl->n_rec; W.R.max = c->cap / 2;
+    return W;
+}
+// charges per chunk, by the context's capacity
+static int step_chunk_size(const obem_ctx *c) { return c->cap <= ST_SMALL ? ST_CHUNK_S : ST_CHUNK_L; }
+
+static void launch_count(obem_ctx *c, const obem_state &st, const GasDev &g, const float4 *E, uint32_t step,
+                         obem_step_stats *stats, cudaStream_t s)
+{
+    const StepScratch W = step_scratch(c);
+    const int ch = step_chunk_size(c), per = ch * (ST_CT / 32), nb = (st.capacity + per - 1) / per;
+    if (ch == ST_CHUNK_S)
+        count_kernel<ST_CHUNK_S><<<nb, ST_CT, 0, s>>>(st, g, E, step, c->s_prop, c->s_ionkey, W, stats, c->s_ctl);
+    else
+        count_kernel<ST_CHUNK_L><<<nb, ST_CT, 0, s>>>(st, g, E, step, c->s_prop, c->s_ionkey, W, stats, c->s_ctl);
+    scan_kernel<<<1, 1024, 0, s>>>(st, c->s_blk, ch, stats, c->s_ctl, st.capacity < c->cap ? st.capacity : c->cap);
+}
+
+// write, moments, fold and the new counts
+static void launch_write(obem_ctx *c, const obem_state &st, const GasDev &g, uint32_t step, obem_step_stats *stats,
+                         cudaStream_t s)
+{
+    const StepScratch W = step_scratch(c);
+    const int ch = step_chunk_size(c), per = ch * (ST_CT / 32), nb = (st.capacity + per - 1) / per;
+    unsigned long long *dep = g.hit_on ? (unsigned long long *)c->d_deposit : NULL;
+    if (ch == ST_CHUNK_S) write_kernel<ST_CHUNK_S><<<nb, ST_CT, 0, s>>>(st, step, W, c->s_ctl, dep);
+    else write_kernel<ST_CHUNK_L><<<nb, ST_CT, 0, s>>>(st, step, W, c->s_ctl, dep);
+    const int mb = (st.capacity + ST_MB - 1) / ST_MB;
+    moments_kernel<<<mb, ST_THREADS, 0, s>>>(st, c->s_ctl, stats, c->s_mpart, mb);
+    finish_kernel<<<1, 32 * NMOM, 0, s>>>(st, c->s_ctl, c->s_mpart, mb, stats);
+}
+
 int obem_launch_shard_propose(obem_ctx *c, const obem_state *stp, const obem_state *Gp, uint32_t step,
                               unsigned long long *ionkey, cudaStream_t s)
 {
@@ -995,7 +1196,7 @@ int obem_launch_shard_propose(obem_ctx *c, const obem_state *stp, const obem_sta
         return OBEM_OK;
     }
     // spatial hash of the gathered cations, queried by the local electrons
-    const double inv_h = 1.0 / (sqrt((double)g.rc2) * (1.0 + 1e-5));
+    const double inv_h = 0.5 / (sqrt((double)g.rc2) * (1.0 + 1e-5));
     OBEM_CUDA(c, cudaMemsetAsync(c->ph_count, 0, sizeof(int32_t) * PH_BUCKETS, s));
     ph_count_kernel<<<gblk, ST_THREADS, 0, s>>>(G, step, inv_h, c->ph_bucket, c->ph_count);
     ph_blocksum_kernel<<<PH_NBLK, PH_BLK, 0, s>>>(c->ph_count, c->ph_bsum);
@@ -1012,8 +1213,7 @@ int obem_launch_shard_count(obem_ctx *c, const obem_state *stp, const float4 *E,
                             const unsigned long long *ionkey, int self_off, obem_step_stats *stats, cudaStream_t s)
 {
     const obem_state st = *stp;
-    const int cap = st.capacity;
-    const int nblk = (cap + ST_THREADS - 1) / ST_THREADS;
+    const int nblk = (st.capacity + ST_THREADS - 1) / ST_THREADS;
     const GasDev g = step_gas(c);
     init_kernel<<<1, 32, 0, s>>>(stats, c->s_ctl, st);
     OBEM_LAUNCH(c);
@@ -1021,10 +1221,7 @@ int obem_launch_shard_count(obem_ctx *c, const obem_state *stp, const float4 *E,
         sh_localize_kernel<<<nblk, ST_THREADS, 0, s>>>(st, ionkey, self_off, c->s_prop, c->s_ionkey);
         OBEM_LAUNCH(c);
     }
-    count_kernel<<<nblk, ST_THREADS, 0, s>>>(st, g, E, step, c->s_prop, c->s_ionkey, c->s_keep,
-                                             c->s_nsp, c->s_blk, stats, c->s_ctl, c->s_hit);
-    OBEM_LAUNCH(c);
-    scan_kernel<<<1, 1024, 0, s>>>(st, c->s_blk, stats, c->s_ctl, cap < c->cap ? cap : c->cap);
+    launch_count(c, st, g, E, step, stats, s);
     OBEM_LAUNCH(c);
     return OBEM_OK;
 }
@@ -1048,30 +1245,15 @@ int obem_launch_shard_commit(obem_ctx *c, const obem_state *stp, const float4 *E
                              int commit, obem_step_stats *stats, cudaStream_t s)
 {
     const obem_state st = *stp;
-    const int cap = st.capacity;
-    const int nblk = (cap + ST_THREADS - 1) / ST_THREADS;
     const GasDev g = step_gas(c);
+    (void)E;                             // the flights were simulated by obem_launch_shard_count
     if (!commit) {
         sh_abort_kernel<<<1, 32, 0, s>>>(c->s_ctl, stats);
         OBEM_LAUNCH(c);
         return OBEM_OK;
     }
     sh_set_id_kernel<<<1, 32, 0, s>>>(st.next_id, id_base);
-    write_kernel<<<nblk, ST_THREADS, 0, s>>>(st, g, E, step, c->s_prop, c->s_ionkey, c->s_keep,
-                                             c->s_nsp, c->s_blk, c->s_ctl, c->o_pos, c->o_vel,
-                                             c->o_id, c->o_birth, c->o_sp);
-    OBEM_LAUNCH(c);
-    commit_kernel<<<nblk, ST_THREADS, 0, s>>>(st, c->s_ctl, c->o_pos, c->o_vel, c->o_id, c->o_birth,
-                                              c->o_sp);
-    OBEM_LAUNCH(c);
-    if (g.hit_on) {
-        deposit_kernel<<<nblk, ST_THREADS, 0, s>>>(st, c->s_ctl, c->s_hit, (unsigned long long *)c->d_deposit);
-        OBEM_LAUNCH(c);
-    }
-    finish_kernel<<<1, 32, 0, s>>>(st, c->s_ctl);
-    OBEM_LAUNCH(c);
-    moments_kernel<<<nblk, ST_THREADS, 0, s>>>(st, stats, c->s_mpart);
-    moments_fold_kernel<<<1, 1024, 0, s>>>(st, c->s_mpart, stats);
+    launch_write(c, st, g, step, stats, s);
     OBEM_LAUNCH(c);
     return OBEM_OK;
 }
@@ -1082,20 +1264,12 @@ int obem_launch_step(obem_ctx *c, const obem_state *stp, const float4 *E, uint32
     const obem_state st = *stp;
     const int cap = st.capacity;
     const int nblk = (cap + ST_THREADS - 1) / ST_THREADS;
-    GasDev g = c->gas;
-    g.hit_on = (c->cfg.flags & OBEM_STEP_SURFACE_HITS) && c->np > 0 && c->d_tri9;
-    if (g.hit_on) {
-        g.tri9 = c->d_tri9;
-        g.hstart = c->d_hstart;
-        g.htri = c->d_htri;
-        for (int k = 0; k < 3; ++k) { g.hlo[k] = c->h_hlo[k]; g.hdim[k] = c->h_hdim[k]; }
-        g.hinv = c->h_hinv;
-    }
+    const GasDev g = step_gas(c);
     init_kernel<<<1, 32, 0, s>>>(stats, c->s_ctl, st);
     OBEM_LAUNCH(c);
     if (g.recomb_on) {
         if (g.rc2 > 0.f) {
-            const double inv_h = 1.0 / (sqrt((double)g.rc2) * (1.0 + 1e-5));
+            const double inv_h = 0.5 / (sqrt((double)g.rc2) * (1.0 + 1e-5));
             OBEM_CUDA(c, cudaMemsetAsync(c->ph_count, 0, sizeof(int32_t) * PH_BUCKETS, s));
             ph_count_kernel<<<nblk, ST_THREADS, 0, s>>>(st, step, inv_h, c->ph_bucket, c->ph_count);
             ph_blocksum_kernel<<<PH_NBLK, PH_BLK, 0, s>>>(c->ph_count, c->ph_bsum);
@@ -1111,28 +1285,11 @@ int obem_launch_step(obem_ctx *c, const obem_state *stp, const float4 *E, uint32
         resolve_kernel<<<nblk, ST_THREADS, 0, s>>>(st, c->s_prop, c->s_ionkey);
         OBEM_LAUNCH(c);
     }
-    count_kernel<<<nblk, ST_THREADS, 0, s>>>(st, g, E, step, c->s_prop, c->s_ionkey, c->s_keep,
-                                             c->s_nsp, c->s_blk, stats, c->s_ctl, c->s_hit);
+    launch_count(c, st, g, E, step, stats, s);
     OBEM_LAUNCH(c);
-    scan_kernel<<<1, 1024, 0, s>>>(st, c->s_blk, stats, c->s_ctl, cap < c->cap ? cap : c->cap);
+    launch_write(c, st, g, step, stats, s);
     OBEM_LAUNCH(c);
-    write_kernel<<<nblk, ST_THREADS, 0, s>>>(st, g, E, step, c->s_prop, c->s_ionkey, c->s_keep,
-                                             c->s_nsp, c->s_blk, c->s_ctl, c->o_pos, c->o_vel,
-                                             c->o_id, c->o_birth, c->o_sp);
-    OBEM_LAUNCH(c);
-    commit_kernel<<<nblk, ST_THREADS, 0, s>>>(st, c->s_ctl, c->o_pos, c->o_vel, c->o_id, c->o_birth,
-                                              c->o_sp);
-    OBEM_LAUNCH(c);
-    if (g.hit_on) {
-        deposit_kernel<<<nblk, ST_THREADS, 0, s>>>(st, c->s_ctl, c->s_hit, (unsigned long long *)c->d_deposit);
-        OBEM_LAUNCH(c);
-    }
-    finish_kernel<<<1, 32, 0, s>>>(st, c->s_ctl);
-    OBEM_LAUNCH(c);
-    moments_kernel<<<nblk, ST_THREADS, 0, s>>>(st, stats, c->s_mpart);
-    moments_fold_kernel<<<1, 1024, 0, s>>>(st, c->s_mpart, stats);
-    OBEM_LAUNCH(c);
-    if (c->prof_on) c->launches += 9 + (g.recomb_on ? 7 : 0) + (g.hit_on ? 1 : 0);
+    if (c->prof_on) c->launches += 6 + (g.recomb_on ? 7 : 0);
     return OBEM_OK;
 }
 
@@ -1165,7 +1322,7 @@ __device__ __forceinline__ BtSlot bt_slot(const StepBatch &B)
 __global__ void bt_init_kernel(StepBatch B)
 {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c == 0) *B.abort = 0;
+    if (c == 0) { *B.abort = 0; *B.n_rec = 0; }
     if (c >= B.nb) return;
     memset(&B.stats[c], 0, sizeof(obem_step_stats));
     memset(&B.ctl[c], 0, sizeof(StepCtl));
@@ -1214,13 +1371,20 @@ __global__ void bt_ph_query_kernel(const obem_state st, StepBatch B, GasDev g, d
     u64 best = ~0ull;
     if (st.species[i] == OBEM_ELECTRON) {
         const float4 pe = reinterpret_cast<const float4 *>(st.pos_q)[i];
-        long long cx, cy, cz;
-        ph_cell(pe, inv_h, cx, cy, cz);
-        for (int dz = -1; dz <= 1; ++dz)
-            for (int dy = -1; dy <= 1; ++dy)
-                for (int dx = -1; dx <= 1; ++dx) {
-                    const uint32_t h = bt_hash(cx + dx, cy + dy, cz + dz, q.c);
-                    for (int k = start[h]; k < start[h + 1]; ++k) {
+        long long cx[2], cy[2], cz[2];
+        ph_coord2(pe.x, inv_h, cx);
+        ph_coord2(pe.y, inv_h, cy);
+        ph_coord2(pe.z, inv_h, cz);
+        int k0[8], k1[8];                      // the eight buckets' loads in flight together
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            const uint32_t h = bt_hash(cx[m & 1], cy[(m >> 1) & 1], cz[m >> 2], q.c);
+            k0[m] = start[h];
+            k1[m] = start[h + 1];
+        }
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+                    for (int k = k0[m]; k < k1[m]; ++k) {
                         const int c = sorted[k];
                         if (c < q.off || c >= q.off + q.n) continue;      // another chamber
                         const float4 pc = reinterpret_cast<const float4 *>(st.pos_q)[c];
@@ -1246,96 +1410,47 @@ __global__ void bt_resolve_kernel(const obem_state st, StepBatch B, const u64 *p
     atomicMin(&ionkey[ion], (pr & 0xFFFFFFFF00000000ull) | (u64)(uint32_t)i);
 }
 
-__global__ void __launch_bounds__(ST_THREADS)
-bt_count_kernel(const obem_state st, StepBatch B, GasDev g, const float4 *E, const u64 *prop, const u64 *ionkey,
-                int32_t *keep, int32_t *nsp, int32_t *blk)
+// chunk of a batch: WC slots of one chamber (segments are multiples of 1024);
+// m: its live charges
+struct BtChunk {
+    int ch, c, off, i0, m;
+};
+template <int WC>
+__device__ __forceinline__ BtChunk bt_chunk(const StepBatch &B)
 {
-    __shared__ long long sh[ST_THREADS / 32];
-    const BtSlot q = bt_slot(B);
-    const uint32_t step = *B.step;
-    int kp = 0, ns = 0, absorbed = 0, attached = 0, coll = 0, rec = 0, ovf = 0;
-    long long trials = 0;
-    if (q.li < q.n) {
-        const int i = q.off + q.li;
-        const uint8_t s = st.species[i];
-        if (recombined(i, s, prop, ionkey, g.recomb_on)) {
-            rec = (s == OBEM_CATION);
-        } else {
-            const float4 pq = reinterpret_cast<const float4 *>(st.pos_q)[i];
-            const float4 vv = reinterpret_cast<const float4 *>(st.vel)[i];
-            const float4 e = E[i];
-            float3 p = make_float3(pq.x, pq.y, pq.z), v = make_float3(vv.x, vv.y, vv.z);
-            uint8_t sp = s;
-            FlightOut fo = {0, 0, 0, 0, 0, 0, -1};
-            fly<false>(g, B.cham[q.c], st.id[i], step, p, v, sp, make_float3(e.x, e.y, e.z), fo, NULL, NULL, NULL,
-                       NULL, NULL, 0, 0u);
-            kp = !fo.dead;
-            ns = fo.nsp;
-            absorbed = fo.dead;
-            attached = fo.attached;
-            coll = fo.collisions;
-            trials = fo.trials;
-            ovf = fo.overflow;
-        }
-        keep[i] = kp;
-        nsp[i] = ns;
+    BtChunk r;
+    r.ch = blockIdx.x * (ST_CT / 32) + (threadIdx.x >> 5);
+    r.i0 = r.ch * WC;
+    r.c = B.blk_cham[r.i0 / ST_THREADS];
+    r.off = B.seg_off[r.c];
+    r.m = min(WC, r.off + B.n[r.c] - r.i0);
+    return r;
+}
+
+template <int WC>
+__global__ void __launch_bounds__(ST_CT)
+bt_count_kernel(const obem_state st, StepBatch B, GasDev g, const float4 *E, const u64 *prop, const u64 *ionkey,
+                StepScratch W)
+{
+    __shared__ uint8_t s_list[ST_CT / 32][WC];
+    const BtChunk q = bt_chunk<WC>(B);
+    StepCounts sc = {0, 0, 0, 0, 0, 0};
+    if (q.m > 0) {                                       // warp-uniform
+        int nk, ns;
+        step_chunk<WC>(st, g, B.cham[q.c], E, *B.step, prop, ionkey, q.i0, q.m, W, s_list[threadIdx.x >> 5], nk, ns, sc);
+        if ((threadIdx.x & 31) == 0) { W.blk[2 * q.ch] = nk; W.blk[2 * q.ch + 1] = ns; }
     }
-    obem_step_stats *stt = &B.stats[q.c];
-    long long t;
-    t = block_sum<long long>(kp, sh);
-    if (threadIdx.x == 0) blk[2 * blockIdx.x] = (int32_t)t;
-    t = block_sum<long long>(ns, sh);
-    if (threadIdx.x == 0) blk[2 * blockIdx.x + 1] = (int32_t)t;
-    t = block_sum<long long>(absorbed, sh);
-    if (threadIdx.x == 0 && t) atomicAdd(&stt->absorbed, (int)t);
-    t = block_sum<long long>(attached, sh);
-    if (threadIdx.x == 0 && t) atomicAdd(&stt->attached, (int)t);
-    t = block_sum<long long>(coll, sh);
-    if (threadIdx.x == 0 && t) atomicAdd(&stt->collisions, (int)t);
-    t = block_sum<long long>(rec, sh);
-    if (threadIdx.x == 0 && t) atomicAdd(&stt->recombined_pairs, (int)t);
-    t = block_sum<long long>(trials, sh);
-    if (threadIdx.x == 0 && t) atomicAdd((unsigned long long *)&stt->trials, (unsigned long long)t);
-    t = block_sum<long long>(ovf, sh);
-    if (threadIdx.x == 0 && t) atomicOr(&B.ctl[q.c].trial_overflow, 1);
+    step_counts(sc, &B.stats[q.c], &B.ctl[q.c]);         // the block's chunks are of one chamber
 }
 
 // one block per chamber: exclusive scan of its blocks' (keep, spawn) totals,
 // capacity and trial checks
-__global__ void bt_scan_kernel(StepBatch B, int32_t *blk)
+__global__ void __launch_bounds__(1024) bt_scan_kernel(StepBatch B, int32_t *blk, int chunk)
 {
-    __shared__ int32_t sk[1024], ss[1024];
-    __shared__ int32_t carry_k, carry_s;
     const int c = blockIdx.x;
-    const int n = B.n[c];
-    const int b0 = B.seg_off[c] / ST_THREADS;
-    const int nb = (n + ST_THREADS - 1) / ST_THREADS;
     const int cap = B.seg_off[c + 1] - B.seg_off[c];
-    if (threadIdx.x == 0) { carry_k = 0; carry_s = 0; }
-    __syncthreads();
-    for (int c0 = 0; c0 < nb; c0 += 1024) {
-        const int b = c0 + threadIdx.x;
-        const int vk = b < nb ? blk[2 * (b0 + b)] : 0;
-        const int vs = b < nb ? blk[2 * (b0 + b) + 1] : 0;
-        sk[threadIdx.x] = vk;
-        ss[threadIdx.x] = vs;
-        __syncthreads();
-        for (int o = 1; o < 1024; o <<= 1) {
-            const int ak = threadIdx.x >= o ? sk[threadIdx.x - o] : 0;
-            const int as = threadIdx.x >= o ? ss[threadIdx.x - o] : 0;
-            __syncthreads();
-            sk[threadIdx.x] += ak;
-            ss[threadIdx.x] += as;
-            __syncthreads();
-        }
-        if (b < nb) {
-            blk[2 * (b0 + b)] = carry_k + sk[threadIdx.x] - vk;
-            blk[2 * (b0 + b) + 1] = carry_s + ss[threadIdx.x] - vs;
-        }
-        __syncthreads();
-        if (threadIdx.x == 1023) { carry_k += sk[1023]; carry_s += ss[1023]; }
-        __syncthreads();
-    }
+    int32_t carry_k, carry_s;
+    step_scan(blk + 2 * (B.seg_off[c] / chunk), (B.n[c] + chunk - 1) / chunk, carry_k, carry_s);
     if (threadIdx.x == 0) {
         StepCtl *ctl = &B.ctl[c];
         obem_step_stats *stt = &B.stats[c];
@@ -1354,66 +1469,13 @@ __global__ void bt_scan_kernel(StepBatch B, int32_t *blk)
     }
 }
 
-__global__ void __launch_bounds__(ST_THREADS)
-bt_write_kernel(const obem_state st, StepBatch B, GasDev g, const float4 *E, const u64 *prop, const u64 *ionkey,
-                const int32_t *keep, const int32_t *nsp, const int32_t *blk, float4 *o_pos, float4 *o_vel,
-                uint32_t *o_id, uint32_t *o_birth, uint8_t *o_sp)
-{
-    __shared__ int32_t wk[ST_THREADS / 32], ws[ST_THREADS / 32];
-    if (*B.abort) return;
-    const BtSlot q = bt_slot(B);
-    const uint32_t step = *B.step;
-    const int i = q.off + q.li;
-    int kp = 0, ns = 0;
-    if (q.li < q.n) { kp = keep[i]; ns = nsp[i]; }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int ik = kp, is = ns;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int a = __shfl_up_sync(0xffffffffu, ik, o);
-        const int b = __shfl_up_sync(0xffffffffu, is, o);
-        if (lane >= o) { ik += a; is += b; }
-    }
-    if (lane == 31) { wk[warp] = ik; ws[warp] = is; }
-    __syncthreads();
-    int pk_ = 0, ps_ = 0;
-    for (int w = 0; w < warp; ++w) { pk_ += wk[w]; ps_ += ws[w]; }
-    if (q.li >= q.n || (!kp && !ns)) return;
-    const int out_keep = blk[2 * blockIdx.x] + pk_ + ik - kp;
-    const int out_spawn = blk[2 * blockIdx.x + 1] + ps_ + is - ns;
-    const uint8_t s = st.species[i];
-    const float4 pq = reinterpret_cast<const float4 *>(st.pos_q)[i];
-    const float4 vv = reinterpret_cast<const float4 *>(st.vel)[i];
-    const float4 e = E[i];
-    float3 p = make_float3(pq.x, pq.y, pq.z), v = make_float3(vv.x, vv.y, vv.z);
-    uint8_t sp = s;
-    FlightOut fo = {0, 0, 0, 0, 0, 0, -1};
-    const int sbase = q.off + B.ctl[q.c].n_keep + 2 * out_spawn;
-    const uint32_t id_base = B.next_id[q.c] + (uint32_t)(2 * out_spawn);
-    fly<true>(g, B.cham[q.c], st.id[i], step, p, v, sp, make_float3(e.x, e.y, e.z), fo, o_pos, o_vel, o_id,
-              o_birth, o_sp, sbase, id_base);
-    if (kp) {
-        const int o = q.off + out_keep;
-        o_pos[o] = make_float4(p.x, p.y, p.z, pq.w);
-        o_vel[o] = make_float4(v.x, v.y, v.z, vv.w);
-        o_id[o] = st.id[i];
-        o_birth[o] = st.birth[i];
-        o_sp[o] = sp;                    // after the flight (attachment makes an anion)
-    }
-}
-
-__global__ void bt_commit_kernel(const obem_state st, StepBatch B, const float4 *o_pos, const float4 *o_vel,
-                                 const uint32_t *o_id, const uint32_t *o_birth, const uint8_t *o_sp)
+template <int WC>
+__global__ void __launch_bounds__(ST_CT) bt_write_kernel(const obem_state st, StepBatch B, StepScratch W)
 {
     if (*B.abort) return;
-    const BtSlot q = bt_slot(B);
-    const StepCtl &ctl = B.ctl[q.c];
-    if (q.li >= ctl.n_keep + 2 * ctl.n_spawn) return;
-    const int i = q.off + q.li;
-    reinterpret_cast<float4 *>(st.pos_q)[i] = o_pos[i];
-    reinterpret_cast<float4 *>(st.vel)[i] = o_vel[i];
-    st.id[i] = o_id[i];
-    st.birth[i] = o_birth[i];
-    st.species[i] = o_sp[i];
+    const BtChunk q = bt_chunk<WC>(B);
+    if (q.m <= 0) return;
+    write_chunk<WC>(st, *B.step, q.i0, q.m, q.off, B.ctl[q.c].n_keep, B.next_id[q.c], W.blk + 2 * q.ch, W, NULL);
 }
 
 // per chamber: new counts (or, when any chamber failed, the chambers that did
@@ -1438,19 +1500,20 @@ __global__ void bt_finish_kernel(StepBatch B)
 }
 
 __global__ void __launch_bounds__(ST_THREADS)
-bt_moments_kernel(const obem_state st, StepBatch B, double *part)
+bt_moments_kernel(const obem_state st, StepBatch B, double *part, int stride)
 {
-    const BtSlot q = bt_slot(B);
-    if (q.li - (int)threadIdx.x >= q.n) return;          // a block past the chamber's charges
-    moments_block(st, q.off + q.li, q.li < q.n, &B.stats[q.c], part + (size_t)NMOM * blockIdx.x);
+    const int i0 = blockIdx.x * ST_MB;
+    const int c = B.blk_cham[i0 / ST_THREADS];
+    const int end = B.seg_off[c] + B.n[c];
+    if (i0 >= end) return;                               // a block past the chamber's charges
+    moments_block(st, i0, end, &B.stats[c], part + blockIdx.x, stride);
 }
 
 // one block per chamber: its blocks' partial sums in block order
-__global__ void __launch_bounds__(1024) bt_moments_fold_kernel(StepBatch B, const double *part)
+__global__ void __launch_bounds__(32 * NMOM) bt_moments_fold_kernel(StepBatch B, const double *part, int stride)
 {
     const int c = blockIdx.x;
-    const int b0 = B.seg_off[c] / ST_THREADS;
-    moments_fold(part + (size_t)NMOM * b0, (B.n[c] + ST_THREADS - 1) / ST_THREADS, &B.stats[c]);
+    moments_fold(part + B.seg_off[c] / ST_MB, stride, (B.n[c] + ST_MB - 1) / ST_MB, &B.stats[c]);
 }
 
 // The whole batched step on stream s.  Scratch (BtScratch) is sized for the
@@ -1468,7 +1531,7 @@ int obem_launch_step_batch(obem_ctx *c, const obem_state *stp, const StepBatch &
     OBEM_LAUNCH(c);
     if (g.recomb_on) {
         if (g.rc2 > 0.f) {
-            const double inv_h = 1.0 / (sqrt((double)g.rc2) * (1.0 + 1e-5));
+            const double inv_h = 0.5 / (sqrt((double)g.rc2) * (1.0 + 1e-5));
             OBEM_CUDA(c, cudaMemsetAsync(W.ph_count, 0, sizeof(int32_t) * PH_BUCKETS, s));
             bt_ph_count_kernel<<<nblk, ST_THREADS, 0, s>>>(st, B, inv_h, W.ph_bucket, W.ph_count);
             ph_blocksum_kernel<<<PH_NBLK, PH_BLK, 0, s>>>(W.ph_count, W.ph_bsum);
@@ -1484,19 +1547,24 @@ int obem_launch_step_batch(obem_ctx *c, const obem_state *stp, const StepBatch &
         bt_resolve_kernel<<<nblk, ST_THREADS, 0, s>>>(st, B, W.prop, W.ionkey);
         OBEM_LAUNCH(c);
     }
-    bt_count_kernel<<<nblk, ST_THREADS, 0, s>>>(st, B, g, E, W.prop, W.ionkey, W.keep, W.nsp, W.blk);
+    StepScratch SW;
+    SW.pos = W.o_pos; SW.vel = W.o_vel; SW.id = W.o_id; SW.birth = W.o_birth; SW.sp = W.o_sp;
+    SW.keep = W.keep; SW.rec = W.nsp; SW.blk = W.blk; SW.hit = NULL;
+    SW.R.rec = W.rec; SW.R.count = B.n_rec; SW.R.max = slots / 2;
+    const int ch = slots <= ST_SMALL ? ST_CHUNK_S : ST_CHUNK_L, cb2 = slots / (ch * (ST_CT / 32));
+    const bool small = ch == ST_CHUNK_S;
+    if (small) bt_count_kernel<ST_CHUNK_S><<<cb2, ST_CT, 0, s>>>(st, B, g, E, W.prop, W.ionkey, SW);
+    else bt_count_kernel<ST_CHUNK_L><<<cb2, ST_CT, 0, s>>>(st, B, g, E, W.prop, W.ionkey, SW);
     OBEM_LAUNCH(c);
-    bt_scan_kernel<<<B.nb, 1024, 0, s>>>(B, W.blk);
+    bt_scan_kernel<<<B.nb, 1024, 0, s>>>(B, W.blk, ch);
     OBEM_LAUNCH(c);
-    bt_write_kernel<<<nblk, ST_THREADS, 0, s>>>(st, B, g, E, W.prop, W.ionkey, W.keep, W.nsp, W.blk, W.o_pos,
-                                                W.o_vel, W.o_id, W.o_birth, W.o_sp);
-    OBEM_LAUNCH(c);
-    bt_commit_kernel<<<nblk, ST_THREADS, 0, s>>>(st, B, W.o_pos, W.o_vel, W.o_id, W.o_birth, W.o_sp);
+    if (small) bt_write_kernel<ST_CHUNK_S><<<cb2, ST_CT, 0, s>>>(st, B, SW);
+    else bt_write_kernel<ST_CHUNK_L><<<cb2, ST_CT, 0, s>>>(st, B, SW);
     OBEM_LAUNCH(c);
     bt_finish_kernel<<<cb, 256, 0, s>>>(B);
     OBEM_LAUNCH(c);
-    bt_moments_kernel<<<nblk, ST_THREADS, 0, s>>>(st, B, W.mpart);
-    bt_moments_fold_kernel<<<B.nb, 1024, 0, s>>>(B, W.mpart);
+    bt_moments_kernel<<<slots / ST_MB, ST_THREADS, 0, s>>>(st, B, W.mpart, slots / ST_MB);
+    bt_moments_fold_kernel<<<B.nb, 32 * NMOM, 0, s>>>(B, W.mpart, slots / ST_MB);
     OBEM_LAUNCH(c);
     return OBEM_OK;
 }
