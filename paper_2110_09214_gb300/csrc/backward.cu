@@ -14,20 +14,24 @@
 // (tiers by centroid distance in units of the longest edge h) and through the
 // FP64 closed form of F and of its Jacobian near the cell.
 //
-// Pair arithmetic is FP32 (rsqrt.approx); partial sums of at most BW_CHUNK
-// pair terms (or of one target's quadrature points) are added into FP64
-// accumulators, so cancelling terms of both signs lose no more than ~16 ulps
+// Pair arithmetic is FP32 (rsqrt.approx), two targets per f32x2 instruction;
+// partial sums of a few terms are folded into compensated (TwoSum) binary32
+// accumulators, so cancelling terms of both signs lose no more than a few ulps
 // of the largest term.  Pairs at zero distance, and the pair t == p when
 // self_exclude is set, are skipped.
+//
+// All three kernels put few rows on a block and split the sum over its lanes
+// or warps: a few thousand probe points then fill the GPU, a far cell's rule
+// is evaluated without divergence, and no FP64 instruction is left but the
+// closed forms.  Bound: FP32 issue.
 #include "obem_internal.cuh"
-#include "field_common.cuh"
+#include "direct_common.cuh"
 
-#define BW_THREADS 128
-#define BW_TILE 128            // points staged per shared-memory tile
-#define BW_CHUNK 16            // pair terms summed in FP32 before each FP64 add
-#define BS_WARPS 8
-#define BS_PANELS 32           // cells per block of the dL/dsigma kernel
-#define BS_TILE 256            // targets staged per tile of the dL/dsigma kernel
+#define BW_NP 2                // target packs per block of the dL/dx kernel (4 targets)
+#define BW_NW 4                // its warps
+#define BR_WARPS 8             // warps of the dL/dsigma and dL/dy kernels: 32 rows, one per lane, each
+                               // warp an eighth of the targets
+#define BR_TILE 256            // targets staged per tile
 
 // Jacobian tiers (squared centroid distance in units of h^2); each keeps the
 // per-cell relative error of dF/dr below ~2e-6
@@ -81,6 +85,27 @@ __device__ __forceinline__ float dens_term(float dx, float dy, float dz, float w
     const float inv = rsq(r2);
     const float dg = fmaf(dz, g.z, fmaf(dy, g.y, dx * g.x));
     return w * inv * fmaf(dg, inv * inv, g.w);
+}
+
+// 1 / r of a pack, 0 where r2 is 0
+__device__ __forceinline__ u64 inv_or_0(u64 r2)
+{
+    float a, b;
+    upk(r2, a, b);
+    return pk(a > 0.f ? rsq(a) : 0.f, b > 0.f ? rsq(b) : 0.f);
+}
+
+// the target-side terms of a pack of targets (offsets d, 1/r, g) for weight w
+__device__ __forceinline__ void tgt_term2(u64 dx, u64 dy, u64 dz, u64 inv, u64 w, u64 gx, u64 gy, u64 gz, u64 gv,
+                                          u64 &ax, u64 &ay, u64 &az)
+{
+    const u64 inv2 = mul2(inv, inv);
+    const u64 c1 = mul2(mul2(w, inv), inv2);
+    const u64 dg = fma2(dz, gz, fma2(dy, gy, mul2(dx, gx)));
+    const u64 c2 = mul2(c1, fma2(mul2(pk(-3.0f, -3.0f), dg), inv2, mul2(pk(-1.0f, -1.0f), gv)));   // -c2
+    ax = fma2(c1, gx, fma2(c2, dx, ax));
+    ay = fma2(c1, gy, fma2(c2, dy, ay));
+    az = fma2(c1, gz, fma2(c2, dz, az));
 }
 
 // dF/dr (row-major) and F of a unit uniform density on a flat triangle, FP64.
@@ -157,11 +182,6 @@ __device__ __noinline__ void tri_closed_jac(const double *v, double rx, double r
 
 // number of quadrature points of a tier (0: closed form) for squared
 // centroid distance d2 and squared longest edge h2
-__device__ __forceinline__ int jac_tier(float d2, float h2)
-{
-    return d2 >= BJ_1PT * h2 ? 1 : d2 >= BJ_3PT * h2 ? 3 : d2 >= BJ_7PT * h2 ? 7 : d2 >= BJ_28PT * h2 ? 28
-         : d2 >= BJ_112PT * h2 ? 112 : 0;
-}
 __device__ __forceinline__ int fld_tier(float d2, float h2)
 {
     return d2 >= BF_1PT * h2 ? 1 : d2 >= BF_3PT * h2 ? 3 : d2 >= BF_7PT * h2 ? 7 : d2 >= BF_28PT * h2 ? 28
@@ -181,164 +201,398 @@ __device__ __forceinline__ void tier_point(int n, int k, float3 g0, float3 g1, f
     rule_point(n == 7 ? 0 : (n == 28 ? 1 : 2), k, g0, g1, g2, off, wf);
 }
 
-// ---------------------------------------------------------------- dL/dx
-// One warp per target: the lanes take every 32nd charge and every 32nd cell
-// (a target's sums are split across 32 lanes, so a few thousand probe points
-// fill the GPU), each lane summing in FP64 partial sums of at most BW_CHUNK
-// FP32 charge terms or one cell's quadrature points; the lanes' sums are
-// added by a fixed butterfly of shuffles (deterministic).
-__global__ void __launch_bounds__(BW_THREADS) bw_targets_kernel(BwLaunch B)
+// barycentric offsets (coefficients of the vertex offsets g0, g1, g2) and weight
+// of point k of the 112- (k < 112) and the 28-point rule (112 <= k < 140)
+#define BW_NBARY 140
+__device__ __forceinline__ float4 bary_point(int k)
 {
-    const int t = (blockIdx.x * BW_THREADS + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (t >= B.nt) return;                              // warp-uniform
-    const float4 x = B.targets[t];
-    const float4 g = B.g[t];
-    double acc[3] = {0.0, 0.0, 0.0};
-    const float kC = (float)OBEM_KC;
+    float3 off;
+    float wf;
+    rule_point(k < 112 ? 2 : 1, k < 112 ? k : k - 112, make_float3(1.f, 0.f, 0.f), make_float3(0.f, 1.f, 0.f),
+               make_float3(0.f, 0.f, 1.f), off, wf);
+    return make_float4(off.x, off.y, off.z, wf);
+}
+
+// ---------------------------------------------------------------- dL/dx
+// A block holds 2 BW_NP targets and its lanes run over the charges, then over
+// the cells.  A cell's rule is that of the block's nearest target (1, 3 or 7
+// points, evaluated as c, c + a g_k, c + b g_k without divergence); pairs
+// closer than 4 h are taken by the warp together, a lane per quadrature point
+// (28 points, 112 below 2 h), and those closer than 1.5 h queue for the FP64
+// Jacobian, 32 at a time.
+__global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
+{
+    constexpr int NP = BW_NP, T = 2 * NP, TH = 32 * BW_NW;
+    __shared__ DfShared<NP, BW_NW> sh;
+    __shared__ float4 s_g[T];
+    __shared__ float4 s_b[BW_NBARY];
+    __shared__ uint32_t s_q[BW_NW][32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int base = blockIdx.x * T;
+    const int n = min(T, B.nt - base);
+    if (tid < T) {
+        sh.t[tid] = B.targets[base + min(tid, n - 1)];
+        s_g[tid] = B.g[base + min(tid, n - 1)];
+    }
+    for (int k = tid; k < BW_NBARY; k += TH) s_b[k] = bary_point(k);
+#pragma unroll
+    for (int v = 0; v < 4 * T; ++v) { sh.S[v][tid] = 0.f; sh.C[v][tid] = 0.f; }
+    __syncthreads();
+    u64 TX[NP], TY[NP], TZ[NP], GX[NP], GY[NP], GZ[NP], GV[NP], A[4][NP];
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+        const float4 a = sh.t[2 * p], b = sh.t[2 * p + 1], ga = s_g[2 * p], gb = s_g[2 * p + 1];
+        TX[p] = pk(a.x, b.x); TY[p] = pk(a.y, b.y); TZ[p] = pk(a.z, b.z);
+        GX[p] = pk(ga.x, gb.x); GY[p] = pk(ga.y, gb.y); GZ[p] = pk(ga.z, gb.z); GV[p] = pk(ga.w, gb.w);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) A[c][p] = 0ull;
+    }
+    int since = 0;
     // point charges
-    for (int p0 = 0; p0 < B.ns; p0 += 32 * BW_CHUNK) {
-        float ax = 0.f, ay = 0.f, az = 0.f;
-        const int p1 = min(B.ns, p0 + 32 * BW_CHUNK);
-        for (int p = p0 + lane; p < p1; p += 32) {
-            if (B.self_exclude && p == t) continue;
-            const float4 s = B.sources[p];
-            tgt_term(x.x - s.x, x.y - s.y, x.z - s.z, kC * s.w, g, ax, ay, az);
+    const float kC = (float)OBEM_KC;
+    const float4 none = make_float4(1e6f, 1e6f, 1e6f, 0.f);
+    float4 nx = tid < B.ns ? B.sources[tid] : none;
+    for (int ib = 32 * warp; ib < B.ns; ib += TH) {
+        const float4 y = nx;
+        const int i = ib + lane;
+        nx = i + TH < B.ns ? B.sources[i + TH] : none;
+        const bool mine = B.self_exclude && ib + 32 > base && ib < base + T;     // warp-uniform
+        const u64 YX = pk(y.x, y.x), YY = pk(y.y, y.y), YZ = pk(y.z, y.z), W = pk(kC * y.w, kC * y.w);
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const u64 dx = sub2(TX[p], YX), dy = sub2(TY[p], YY), dz = sub2(TZ[p], YZ);
+            u64 inv = inv_or_0(fma2(dz, dz, fma2(dy, dy, mul2(dx, dx))));
+            if (mine) {
+                float a, b;
+                upk(inv, a, b);
+                inv = pk(i == base + 2 * p ? 0.f : a, i == base + 2 * p + 1 ? 0.f : b);
+            }
+            tgt_term2(dx, dy, dz, inv, W, GX[p], GY[p], GZ[p], GV[p], A[0][p], A[1][p], A[2][p]);
         }
-        acc[0] += ax; acc[1] += ay; acc[2] += az;
+        if (++since == DF_FOLD) { df_fold<false>(sh, A, 1.f); since = 0; }
     }
     // cells
+    int nq = 0;
+    auto flush = [&](int m) {
+        __syncwarp();
+        if (lane < m) {
+            const uint32_t e = s_q[warp][lane];
+            const int j = (int)(e >> 3), t = (int)(e & 7u);
+            const float4 x = sh.t[t], g = s_g[t];
+            double J[9], F[3];
+            tri_closed_jac(B.panels.v64 + 9 * (size_t)j, (double)x.x, (double)x.y, (double)x.z, J, F);
+            const double q = OBEM_KC * (double)B.sigma[j];
+            for (int b = 0; b < 3; ++b)
+                df_put(sh, 4 * t + b, (float)(q * (J[b] * g.x + J[3 + b] * g.y + J[6 + b] * g.z - (double)g.w * F[b])));
+        }
+        __syncwarp();
+    };
     if (B.sigma) {
         const PanelsDev &P = B.panels;
-        for (int j = lane; j < P.np; j += 32) {
-            const float4 ca = P.c_a[j], cl = P.c_lo[j], g0 = P.g0_h[j];
-            // exact target - centroid: x - c_hi is exact for nearby targets
-            const float ex = (x.x - ca.x) - cl.x, ey = (x.y - ca.y) - cl.y, ez = (x.z - ca.z) - cl.z;
-            const float d2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
-            const int n = jac_tier(d2, g0.w);
-            const float sg = B.sigma[j];
-            if (n > 0) {
-                const float4 g1 = P.g1[j], g2 = P.g2[j];
-                const float3 G0 = make_float3(g0.x, g0.y, g0.z), G1 = make_float3(g1.x, g1.y, g1.z),
-                             G2 = make_float3(g2.x, g2.y, g2.z);
-                const float wq = ca.w * sg;
-                float ax = 0.f, ay = 0.f, az = 0.f;
-                for (int k = 0; k < n; ++k) {
-                    float3 off;
-                    float wf;
-                    tier_point(n, k, G0, G1, G2, off, wf);
-                    tgt_term(ex - off.x, ey - off.y, ez - off.z, wq * wf, g, ax, ay, az);
-                }
-                acc[0] += ax; acc[1] += ay; acc[2] += az;
-            } else {
-                double J[9], F[3];
-                tri_closed_jac(P.v64 + 9 * (size_t)j, (double)x.x, (double)x.y, (double)x.z, J, F);
-                const double s = OBEM_KC * (double)sg;
-                for (int b = 0; b < 3; ++b)
-                    acc[b] += s * (J[b] * g.x + J[3 + b] * g.y + J[6 + b] * g.z - (double)g.w * F[b]);
-            }
-        }
-    }
+        for (int jb = 32 * warp; jb < P.np; jb += TH) {
+            const bool live = jb + lane < P.np;
+            const int j = live ? jb + lane : jb;
+            const float4 ca = P.c_a[j], cl = P.c_lo[j], g0 = P.g0_h[j], g1 = P.g1[j], g2 = P.g2[j];
+            const float q = live ? ca.w * B.sigma[j] : 0.f, h2 = g0.w;
+            u64 D[3][NP], EP[NP];
+            unsigned nm = 0u;
+            float dmin = 3e38f;
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
-        for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
-    if (lane == 0) B.dtargets[t] = make_float4((float)acc[0], (float)acc[1], (float)acc[2], 0.f);
+            for (int p = 0; p < NP; ++p) {
+                // exact target - centroid: x - c_hi is exact for nearby targets
+                D[0][p] = sub2(sub2(TX[p], pk(ca.x, ca.x)), pk(cl.x, cl.x));
+                D[1][p] = sub2(sub2(TY[p], pk(ca.y, ca.y)), pk(cl.y, cl.y));
+                D[2][p] = sub2(sub2(TZ[p], pk(ca.z, ca.z)), pk(cl.z, cl.z));
+                float da, db;
+                upk(fma2(D[2][p], D[2][p], fma2(D[1][p], D[1][p], mul2(D[0][p], D[0][p]))), da, db);
+                dmin = fminf(dmin, fminf(da, db));
+                const bool na = da < BJ_7PT * h2, nb = db < BJ_7PT * h2;
+                nm |= (na ? 1u << (2 * p) : 0u) | (nb ? 2u << (2 * p) : 0u);
+                EP[p] = pk(na ? 1e30f : 0.f, nb ? 1e30f : 0.f);     // near pairs: no term here
+            }
+            if (!live) nm = 0u;
+            nm &= (1u << n) - 1u;
+            const bool t1 = dmin >= BJ_1PT * h2, t3 = dmin >= BJ_3PT * h2;
+            const float w0 = t1 ? 1.f : t3 ? 0.f : D7_W0, wa = t1 ? 0.f : t3 ? 1.0f / 3.0f : D7_W1,
+                        sa = t1 ? 0.f : t3 ? 0.5f : D7_T1, wb = t3 ? 0.f : D7_W2, sb = t3 ? 0.f : D7_T2;
+            auto point = [&](float ox, float oy, float oz, float w) {
+                const u64 OX = pk(ox, ox), OY = pk(oy, oy), OZ = pk(oz, oz), W = pk(w, w);
+#pragma unroll
+                for (int p = 0; p < NP; ++p) {
+                    const u64 dx = sub2(D[0][p], OX), dy = sub2(D[1][p], OY), dz = sub2(D[2][p], OZ);
+                    float ra, rb;
+                    upk(fma2(dz, dz, fma2(dy, dy, fma2(dx, dx, EP[p]))), ra, rb);
+                    tgt_term2(dx, dy, dz, pk(rsq(ra), rsq(rb)), W, GX[p], GY[p], GZ[p], GV[p], A[0][p], A[1][p],
+                              A[2][p]);
+                }
+            };
+            if (__any_sync(0xffffffffu, w0 != 0.f)) point(0.f, 0.f, 0.f, q * w0);
+            if (__any_sync(0xffffffffu, wa != 0.f)) {
+                const float w = q * wa;
+                point(sa * g0.x, sa * g0.y, sa * g0.z, w);
+                point(sa * g1.x, sa * g1.y, sa * g1.z, w);
+                point(sa * g2.x, sa * g2.y, sa * g2.z, w);
+            }
+            if (__any_sync(0xffffffffu, wb != 0.f)) {
+                const float w = q * wb;
+                point(sb * g0.x, sb * g0.y, sb * g0.z, w);
+                point(sb * g1.x, sb * g1.y, sb * g1.z, w);
+                point(sb * g2.x, sb * g2.y, sb * g2.z, w);
+            }
+            if (__any_sync(0xffffffffu, nm != 0u)) {
+                for (int t = 0; t < n; ++t) {
+                    unsigned bal = __ballot_sync(0xffffffffu, (nm >> t) & 1u);
+                    if (!bal) continue;
+                    const float4 x = sh.t[t], g = s_g[t];
+                    float ax = 0.f, ay = 0.f, az = 0.f;
+                    while (bal) {
+                        const int jj = jb + __ffs(bal) - 1;            // warp-uniform
+                        bal &= bal - 1;
+                        const float4 c = P.c_a[jj], l = P.c_lo[jj], v0 = P.g0_h[jj];
+                        const float ex = (x.x - c.x) - l.x, ey = (x.y - c.y) - l.y, ez = (x.z - c.z) - l.z;
+                        const float d2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
+                        if (d2 < BJ_112PT * v0.w) {
+                            if (lane == 0) s_q[warp][nq] = ((uint32_t)jj << 3) | (uint32_t)t;
+                            if (++nq == 32) { flush(32); nq = 0; }
+                            continue;
+                        }
+                        const float4 v1 = P.g1[jj], v2 = P.g2[jj];
+                        const float qq = c.w * B.sigma[jj];
+                        const bool coarse = d2 >= BJ_28PT * v0.w;
+                        for (int k = coarse ? 112 + lane : lane; k < (coarse ? 140 : 112); k += 32) {
+                            const float4 b = s_b[k];
+                            tgt_term(ex - fmaf(b.z, v2.x, fmaf(b.y, v1.x, b.x * v0.x)),
+                                     ey - fmaf(b.z, v2.y, fmaf(b.y, v1.y, b.x * v0.y)),
+                                     ez - fmaf(b.z, v2.z, fmaf(b.y, v1.z, b.x * v0.z)), qq * b.w, g, ax, ay, az);
+                        }
+                    }
+                    df_put(sh, 4 * t, ax);
+                    df_put(sh, 4 * t + 1, ay);
+                    df_put(sh, 4 * t + 2, az);
+                }
+            }
+            if (++since == DF_FOLD) { df_fold<false>(sh, A, 1.f); since = 0; }
+        }
+        if (nq > 0) flush(nq);
+    }
+    df_fold<false>(sh, A, 1.f);
+    float s[4 * T], c[4 * T];
+#pragma unroll
+    for (int v = 0; v < 4 * T; ++v) { s[v] = sh.S[v][tid]; c[v] = sh.C[v][tid]; }
+    df_reduce<4 * T>(s, c);
+    constexpr int per = 32 / (4 * T);
+    if (lane % per == 0) { sh.red[0][warp][lane / per] = s[0]; sh.red[1][warp][lane / per] = c[0]; }
+    __syncthreads();
+    if (tid < 4 * n) {
+        float S = 0.f, C = 0.f;
+        for (int w = 0; w < BW_NW; ++w) df_add(S, C, sh.red[0][w][tid], sh.red[1][w][tid]);
+        reinterpret_cast<float *>(B.dtargets + base)[tid] = (tid & 3) < 3 ? (float)((double)S + (double)C) : 0.f;
+    }
+}
+
+// ---------------------------------------------------------------- rows of 32
+// The targets [tb, tb + BR_TILE) as packs in shared memory (positions and g;
+// padding: the last target's position, g = 0)
+struct BrTile {
+    u64 x[3][BR_TILE / 2], g[4][BR_TILE / 2];
+};
+__device__ __forceinline__ void br_load(const BwLaunch &B, BrTile &t, int tb)
+{
+    __syncthreads();
+    for (int l = threadIdx.x; l < BR_TILE / 2; l += blockDim.x) {
+        const int a = tb + 2 * l, b = a + 1, last = B.nt - 1;
+        const float4 xa = B.targets[min(a, last)], xb = B.targets[min(b, last)];
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 ga = a <= last ? B.g[a] : z, gb = b <= last ? B.g[b] : z;
+        t.x[0][l] = pk(xa.x, xb.x); t.x[1][l] = pk(xa.y, xb.y); t.x[2][l] = pk(xa.z, xb.z);
+        t.g[0][l] = pk(ga.x, gb.x); t.g[1][l] = pk(ga.y, gb.y); t.g[2][l] = pk(ga.z, gb.z); t.g[3][l] = pk(ga.w, gb.w);
+    }
+    __syncthreads();
+}
+__device__ __forceinline__ void br_fold(u64 &a, float &s, float &c)
+{
+    float x, y;
+    upk(a, x, y);
+    two_sum_acc(s, c, x);
+    two_sum_acc(s, c, y);
+    a = 0ull;
 }
 
 // ---------------------------------------------------------------- dL/dy, dL/dq
-__global__ void __launch_bounds__(BW_THREADS) bw_sources_kernel(BwLaunch B)
+// A lane per source, a warp per eighth of the targets.
+__global__ void __launch_bounds__(32 * BR_WARPS) bw_sources_kernel(BwLaunch B)
 {
-    __shared__ float4 s_x[BW_TILE], s_g[BW_TILE];
-    const int p = blockIdx.x * BW_THREADS + threadIdx.x;
+    __shared__ BrTile st;
+    __shared__ float s_red[2][4][BR_WARPS][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int p0 = blockIdx.x * 32, p = p0 + lane;
     const bool live = p < B.ns;
-    const float4 y = live ? B.sources[p] : make_float4(0.f, 0.f, 0.f, 0.f);
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int tb = 0; tb < B.nt; tb += BW_TILE) {
-        __syncthreads();
-        for (int l = threadIdx.x; l < BW_TILE; l += BW_THREADS) {
-            const int t = tb + l;
-            s_x[l] = t < B.nt ? B.targets[t] : make_float4(0.f, 0.f, 0.f, 0.f);
-            s_g[l] = t < B.nt ? B.g[t] : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        __syncthreads();
-        const int n = min(BW_TILE, B.nt - tb);
-        for (int l0 = 0; l0 < n; l0 += BW_CHUNK) {
-            float ax = 0.f, ay = 0.f, az = 0.f, aq = 0.f;
-            for (int l = l0; l < min(n, l0 + BW_CHUNK); ++l) {
-                if (B.self_exclude && tb + l == p) continue;
-                const float4 x = s_x[l], g = s_g[l];
-                const float dx = x.x - y.x, dy = x.y - y.y, dz = x.z - y.z;
-                tgt_term(dx, dy, dz, 1.0f, g, ax, ay, az);
-                aq += dens_term(dx, dy, dz, 1.0f, g);
+    const float4 y = B.sources[live ? p : p0];
+    const u64 YX = pk(y.x, y.x), YY = pk(y.y, y.y), YZ = pk(y.z, y.z), ONE = pk(1.f, 1.f);
+    u64 A[4] = {0ull, 0ull, 0ull, 0ull};
+    float S[4] = {0.f, 0.f, 0.f, 0.f}, C[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int tb = 0; tb < B.nt; tb += BR_TILE) {
+        br_load(B, st, tb);
+        const int np = (min(BR_TILE, B.nt - tb) + 1) / 2;
+        int since = 0;
+        for (int l = warp; l < np; l += BR_WARPS) {
+            const u64 dx = sub2(st.x[0][l], YX), dy = sub2(st.x[1][l], YY), dz = sub2(st.x[2][l], YZ);
+            const u64 gx = st.g[0][l], gy = st.g[1][l], gz = st.g[2][l], gv = st.g[3][l];
+            u64 inv = inv_or_0(fma2(dz, dz, fma2(dy, dy, mul2(dx, dx))));
+            const int t = tb + 2 * l;
+            if (B.self_exclude && t + 1 >= p0 && t < p0 + 32) {             // warp-uniform
+                float a, b;
+                upk(inv, a, b);
+                inv = pk(t == p ? 0.f : a, t + 1 == p ? 0.f : b);
             }
-            acc[0] += ax; acc[1] += ay; acc[2] += az; acc[3] += aq;
+            tgt_term2(dx, dy, dz, inv, ONE, gx, gy, gz, gv, A[0], A[1], A[2]);
+            const u64 dg = fma2(dz, gz, fma2(dy, gy, mul2(dx, gx)));
+            A[3] = fma2(inv, fma2(dg, mul2(inv, inv), gv), A[3]);
+            if (++since == 8) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) br_fold(A[c], S[c], C[c]);
+                since = 0;
+            }
         }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) br_fold(A[c], S[c], C[c]);
     }
-    if (live) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) { s_red[0][c][warp][lane] = S[c]; s_red[1][c][warp][lane] = C[c]; }
+    __syncthreads();
+    if (warp == 0 && live) {
+        double r[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            float a = 0.f, b = 0.f;
+            for (int w = 0; w < BR_WARPS; ++w) df_add(a, b, s_red[0][c][w][lane], s_red[1][c][w][lane]);
+            r[c] = (double)a + (double)b;
+        }
         const double kq = OBEM_KC * (double)y.w;
-        B.dsources[p] = make_float4((float)(-kq * acc[0]), (float)(-kq * acc[1]), (float)(-kq * acc[2]),
-                                    (float)(OBEM_KC * acc[3]));
+        B.dsources[p] = make_float4((float)(-kq * r[0]), (float)(-kq * r[1]), (float)(-kq * r[2]),
+                                    (float)(OBEM_KC * r[3]));
     }
 }
 
 // ---------------------------------------------------------------- dL/dsigma
-// Block: BS_PANELS cells, warp w takes cells w, w + 8, ...; lanes stride over
-// a tile of BS_TILE targets staged in shared memory.
-__global__ void __launch_bounds__(BS_WARPS * 32) bw_sigma_kernel(BwLaunch B)
+// A lane per cell, a warp per eighth of the targets; far targets two at a
+// time with the rule of the nearer one (1, 3 or 7 points, as in dL/dx); pairs
+// closer than 3 h are taken by the warp together, a lane per quadrature point,
+// and those within h queue for the FP64 closed form.
+__global__ void __launch_bounds__(32 * BR_WARPS) bw_sigma_kernel(BwLaunch B)
 {
-    __shared__ float4 s_x[BS_TILE], s_g[BS_TILE];
-    constexpr int PER_WARP = BS_PANELS / BS_WARPS;
+    __shared__ BrTile st;
+    __shared__ float s_red[2][BR_WARPS][32];
+    __shared__ float4 s_b[BW_NBARY];
+    __shared__ int s_q[BR_WARPS][2][32];                // closed-form queue: target, lane of the cell
+    __shared__ float s_v[BR_WARPS][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const PanelsDev &P = B.panels;
-    double acc[PER_WARP];
-#pragma unroll
-    for (int i = 0; i < PER_WARP; ++i) acc[i] = 0.0;
-    for (int tb = 0; tb < B.nt; tb += BS_TILE) {
-        __syncthreads();
-        for (int l = threadIdx.x; l < BS_TILE; l += BS_WARPS * 32) {
-            const int t = tb + l;
-            s_x[l] = t < B.nt ? B.targets[t] : make_float4(0.f, 0.f, 0.f, 0.f);
-            s_g[l] = t < B.nt ? B.g[t] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const int j0 = blockIdx.x * 32;
+    const bool live = j0 + lane < P.np;
+    const int j = live ? j0 + lane : j0;
+    const float4 ca = P.c_a[j], cl = P.c_lo[j], g0 = P.g0_h[j], g1 = P.g1[j], g2 = P.g2[j];
+    const float h2 = g0.w;
+    for (int k = threadIdx.x; k < BW_NBARY; k += blockDim.x) s_b[k] = bary_point(k);
+    u64 A = 0ull;
+    float S = 0.f, C = 0.f;
+    int nq = 0;
+    auto flush = [&](int m) {
+        __syncwarp();
+        if (lane < m) {
+            const int t = s_q[warp][0][lane];
+            const float4 x = B.targets[t], g = B.g[t];
+            double phi, fx, fy, fz;
+            tri_closed_form(P.v64 + 9 * (size_t)(j0 + s_q[warp][1][lane]), (double)x.x, (double)x.y, (double)x.z, phi, fx,
+                            fy, fz);
+            s_v[warp][lane] =
+                (float)(OBEM_KC * ((double)g.x * fx + (double)g.y * fy + (double)g.z * fz + (double)g.w * phi));
         }
-        __syncthreads();
-        const int n = min(BS_TILE, B.nt - tb);
-#pragma unroll
-        for (int i = 0; i < PER_WARP; ++i) {
-            const int j = blockIdx.x * BS_PANELS + warp + BS_WARPS * i;
-            if (j >= P.np) continue;
-            const float4 ca = P.c_a[j], cl = P.c_lo[j], g0 = P.g0_h[j], g1 = P.g1[j], g2 = P.g2[j];
-            const float3 G0 = make_float3(g0.x, g0.y, g0.z), G1 = make_float3(g1.x, g1.y, g1.z),
-                         G2 = make_float3(g2.x, g2.y, g2.z);
-            double ad = 0.0;
-            for (int l = lane; l < n; l += 32) {
-                float a = 0.f;
-                const float4 x = s_x[l], g = s_g[l];
-                const float ex = (x.x - ca.x) - cl.x, ey = (x.y - ca.y) - cl.y, ez = (x.z - ca.z) - cl.z;
-                const float d2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
-                const int nq = fld_tier(d2, g0.w);
-                if (nq > 0) {
-                    for (int k = 0; k < nq; ++k) {
-                        float3 off;
-                        float wf;
-                        tier_point(nq, k, G0, G1, G2, off, wf);
-                        a += dens_term(ex - off.x, ey - off.y, ez - off.z, ca.w * wf, g);
-                    }
-                } else {
-                    double phi, fx, fy, fz;
-                    tri_closed_form(P.v64 + 9 * (size_t)j, (double)x.x, (double)x.y, (double)x.z, phi, fx, fy, fz);
-                    ad += OBEM_KC * ((double)g.x * fx + (double)g.y * fy + (double)g.z * fz + (double)g.w * phi);
-                }
-                ad += (double)a;   // one target's quadrature points in FP32, targets summed in FP64
+        __syncwarp();
+        for (int e = 0; e < m; ++e)
+            if (s_q[warp][1][e] == lane) two_sum_acc(S, C, s_v[warp][e]);
+        __syncwarp();
+    };
+    for (int tb = 0; tb < B.nt; tb += BR_TILE) {
+        br_load(B, st, tb);
+        const int np = (min(BR_TILE, B.nt - tb) + 1) / 2;
+        int since = 0;
+        for (int l = warp; l < np; l += BR_WARPS) {
+            const u64 DX = sub2(sub2(st.x[0][l], pk(ca.x, ca.x)), pk(cl.x, cl.x)),
+                      DY = sub2(sub2(st.x[1][l], pk(ca.y, ca.y)), pk(cl.y, cl.y)),
+                      DZ = sub2(sub2(st.x[2][l], pk(ca.z, ca.z)), pk(cl.z, cl.z));
+            const u64 gx = st.g[0][l], gy = st.g[1][l], gz = st.g[2][l], gv = st.g[3][l];
+            float da, db;
+            upk(fma2(DZ, DZ, fma2(DY, DY, mul2(DX, DX))), da, db);
+            const int t = tb + 2 * l;
+            const bool na = da < BF_7PT * h2, nb = db < BF_7PT * h2;
+            const u64 EP = pk(na ? 1e30f : 0.f, nb ? 1e30f : 0.f);          // near pairs: no term here
+            const float dmin = fminf(da, db);
+            const bool t1 = dmin >= BF_1PT * h2, t3 = dmin >= BF_3PT * h2;
+            const float w0 = t1 ? 1.f : t3 ? 0.f : D7_W0, wa = t1 ? 0.f : t3 ? 1.0f / 3.0f : D7_W1,
+                        sa = t1 ? 0.f : t3 ? 0.5f : D7_T1, wb = t3 ? 0.f : D7_W2, sb = t3 ? 0.f : D7_T2;
+            auto point = [&](float ox, float oy, float oz, float w) {
+                const u64 dx = sub2(DX, pk(ox, ox)), dy = sub2(DY, pk(oy, oy)), dz = sub2(DZ, pk(oz, oz));
+                float ra, rb;
+                upk(fma2(dz, dz, fma2(dy, dy, fma2(dx, dx, EP))), ra, rb);
+                const u64 inv = pk(rsq(ra), rsq(rb));
+                const u64 dg = fma2(dz, gz, fma2(dy, gy, mul2(dx, gx)));
+                A = fma2(mul2(pk(w, w), inv), fma2(dg, mul2(inv, inv), gv), A);
+            };
+            if (__any_sync(0xffffffffu, w0 != 0.f)) point(0.f, 0.f, 0.f, ca.w * w0);
+            if (__any_sync(0xffffffffu, wa != 0.f)) {
+                const float w = ca.w * wa;
+                point(sa * g0.x, sa * g0.y, sa * g0.z, w);
+                point(sa * g1.x, sa * g1.y, sa * g1.z, w);
+                point(sa * g2.x, sa * g2.y, sa * g2.z, w);
             }
-            acc[i] += ad;
-        }
-    }
+            if (__any_sync(0xffffffffu, wb != 0.f)) {
+                const float w = ca.w * wb;
+                point(sb * g0.x, sb * g0.y, sb * g0.z, w);
+                point(sb * g1.x, sb * g1.y, sb * g1.z, w);
+                point(sb * g2.x, sb * g2.y, sb * g2.z, w);
+            }
 #pragma unroll
-    for (int i = 0; i < PER_WARP; ++i) {
-        double v = acc[i];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        const int j = blockIdx.x * BS_PANELS + warp + BS_WARPS * i;
-        if (lane == 0 && j < P.np) B.dsigma[j] = (float)v;
+            for (int half = 0; half < 2; ++half) {
+                unsigned bal = __ballot_sync(0xffffffffu, live && t + half < B.nt && (half ? nb : na));
+                if (!bal) continue;
+                const float4 x = B.targets[t + half], g = B.g[t + half];
+                while (bal) {
+                    const int own = __ffs(bal) - 1, jj = j0 + own;          // warp-uniform
+                    bal &= bal - 1;
+                    const float4 c = P.c_a[jj], lo = P.c_lo[jj], v0 = P.g0_h[jj];
+                    const float ex = (x.x - c.x) - lo.x, ey = (x.y - c.y) - lo.y, ez = (x.z - c.z) - lo.z;
+                    const float d2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
+                    if (d2 < BF_112PT * v0.w) {
+                        if (lane == 0) { s_q[warp][0][nq] = t + half; s_q[warp][1][nq] = own; }
+                        if (++nq == 32) { flush(32); nq = 0; }
+                        continue;
+                    }
+                    const float4 v1 = P.g1[jj], v2 = P.g2[jj];
+                    const bool coarse = d2 >= BF_28PT * v0.w;
+                    float a = 0.f;
+                    for (int k = coarse ? 112 + lane : lane; k < (coarse ? 140 : 112); k += 32) {
+                        const float4 b = s_b[k];
+                        a += dens_term(ex - fmaf(b.z, v2.x, fmaf(b.y, v1.x, b.x * v0.x)),
+                                       ey - fmaf(b.z, v2.y, fmaf(b.y, v1.y, b.x * v0.y)),
+                                       ez - fmaf(b.z, v2.z, fmaf(b.y, v1.z, b.x * v0.z)), c.w * b.w, g);
+                    }
+                    for (int o = 16; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+                    if (lane == own) two_sum_acc(S, C, a);
+                }
+            }
+            if (++since == 4) { br_fold(A, S, C); since = 0; }
+        }
+        br_fold(A, S, C);
+    }
+    if (nq > 0) flush(nq);
+    s_red[0][warp][lane] = S;
+    s_red[1][warp][lane] = C;
+    __syncthreads();
+    if (warp == 0 && live) {
+        float a = 0.f, b = 0.f;
+        for (int w = 0; w < BR_WARPS; ++w) df_add(a, b, s_red[0][w][lane], s_red[1][w][lane]);
+        B.dsigma[j] = (float)((double)a + (double)b);
     }
 }
 
@@ -927,15 +1181,15 @@ int obem_launch_backward(obem_ctx *ctx, const BwArgs &A, cudaStream_t s)
     B.dtargets = (float4 *)A.dL_dtargets;
     B.dsources = (float4 *)A.dL_dsources;
     if (B.dtargets && B.nt > 0) {
-        bw_targets_kernel<<<(unsigned)(((long long)B.nt * 32 + BW_THREADS - 1) / BW_THREADS), BW_THREADS, 0, s>>>(B);
+        bw_targets_kernel<<<(B.nt + 2 * BW_NP - 1) / (2 * BW_NP), 32 * BW_NW, 0, s>>>(B);
         OBEM_LAUNCH(ctx);
     }
     if (B.dsources && B.ns > 0) {
-        bw_sources_kernel<<<(B.ns + BW_THREADS - 1) / BW_THREADS, BW_THREADS, 0, s>>>(B);
+        bw_sources_kernel<<<(B.ns + 31) / 32, 32 * BR_WARPS, 0, s>>>(B);
         OBEM_LAUNCH(ctx);
     }
     if (B.dsigma && B.panels.np > 0) {
-        bw_sigma_kernel<<<(B.panels.np + BS_PANELS - 1) / BS_PANELS, BS_WARPS * 32, 0, s>>>(B);
+        bw_sigma_kernel<<<(B.panels.np + 31) / 32, 32 * BR_WARPS, 0, s>>>(B);
         OBEM_LAUNCH(ctx);
     }
     return OBEM_OK;
