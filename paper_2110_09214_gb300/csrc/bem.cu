@@ -904,21 +904,40 @@ __global__ void __launch_bounds__(256) residual_kernel(const float *A, const flo
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if (lane == 0) r[row] = b[row] - v;
 }
-__global__ void norms_kernel(const double *r, const double *x, const double *b, int n, double *out)
+// out[q] = max |r|, |x|, |b|: one block of 1024, the magnitudes compared as
+// integers (a single SM's FP64 pipe took 155 us at 60k entries; a NaN counts as
+// 0, as fmax does)
+__device__ __forceinline__ unsigned long long abs_bits(double v)
 {
-    __shared__ double s[3][256];
-    double a0 = 0, a1 = 0, a2 = 0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        a0 = fmax(a0, fabs(r[i])); a1 = fmax(a1, fabs(x[i])); a2 = fmax(a2, fabs(b[i]));
+    const unsigned long long k = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+    return k > 0x7ff0000000000000ull ? 0ull : k;
+}
+__global__ void __launch_bounds__(1024) norms_kernel(const double *r, const double *x, const double *b, int n,
+                                                     double *out)
+{
+    __shared__ unsigned long long s[3][32];
+    unsigned long long m[3] = {0ull, 0ull, 0ull};
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += 1024) {
+        const unsigned long long a0 = abs_bits(r[i]), a1 = abs_bits(x[i]), a2 = abs_bits(b[i]);
+        m[0] = a0 > m[0] ? a0 : m[0];
+        m[1] = a1 > m[1] ? a1 : m[1];
+        m[2] = a2 > m[2] ? a2 : m[2];
     }
-    s[0][threadIdx.x] = a0; s[1][threadIdx.x] = a1; s[2][threadIdx.x] = a2;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        for (int o = 16; o; o >>= 1) {
+            const unsigned long long v = __shfl_xor_sync(0xffffffffu, m[q], o);
+            m[q] = v > m[q] ? v : m[q];
+        }
+        if ((threadIdx.x & 31) == 0) s[q][threadIdx.x >> 5] = m[q];
+    }
     __syncthreads();
-    for (int o = blockDim.x / 2; o; o >>= 1) {
-        if (threadIdx.x < o)
-            for (int q = 0; q < 3; ++q) s[q][threadIdx.x] = fmax(s[q][threadIdx.x], s[q][threadIdx.x + o]);
-        __syncthreads();
+    if (threadIdx.x < 3) {
+        unsigned long long v = s[threadIdx.x][0];
+        for (int w = 1; w < 32; ++w) v = s[threadIdx.x][w] > v ? s[threadIdx.x][w] : v;
+        out[threadIdx.x] = __longlong_as_double((long long)v);
     }
-    if (threadIdx.x == 0) { out[0] = s[0][0]; out[1] = s[1][0]; out[2] = s[2][0]; }
 }
 
 // y = P r / sc in FP32 (sc = max |r|): the factorisation's row swaps as one
@@ -955,16 +974,23 @@ __global__ void to_float_kernel(const double *x, float *a, float *b, int n)
 // in one launch.  Block row i of TS_R rows is taken by the thread block that
 // draws ticket i (in dependency order: i = 0 is the first block row of L,
 // the last of U), so every block row it depends on belongs to a thread block
-// that started before it, whatever the scheduling.  Each warp owns TS_R / 8
-// rows and runs over the solved blocks of y in dependency order; the loads
-// of y wait for that block's flag to show the launch's epoch.  The block row
-// then multiplies its right-hand side, less the solved part, by the inverse
-// of its diagonal block (computed once after the factorisation) and
-// publishes its y values and flag.  A wait on a flag is bounded
-// (TS_WAIT_NS): one that runs out records OBEM_ERR_TIMEOUT and goes on, so
-// that the launch always ends.
+// that started before it, whatever the scheduling.  A thread block runs over
+// the solved blocks of y in dependency order, then multiplies its right-hand
+// side, less the solved part, by the inverse of its diagonal block (computed
+// once after the factorisation) and publishes its y values.
+//
+// Bound: at 60k cells the factor's 7.2 GB (1.06 ms) and a chain of 469 steps.
+// A published value carries the launch's epoch in its upper half, so a step
+// waits for the data itself (one round trip to L2, no flag before it and no
+// fence after it); the block's matrix entries are in flight before the wait;
+// one warp polls, the more rarely the farther its block row is from its turn
+// (every warp polling flags, the matrix read after them: 4.05 ms; now 1.45 ms,
+// and 0.515 to 0.17 ms at 11,008 cells).
+// A wait is bounded (TS_WAIT_NS): one that runs out records OBEM_ERR_TIMEOUT
+// and the block waits no more, so that the launch always ends.
 #define TS_WAIT_NS 2000000000ull
-#define TS_SMEM (sizeof(float) * (TS_R * (TS_R + 1) + TS_R))
+#define TS_TH 256
+#define TS_SMEM (sizeof(float) * TS_R * TS_R)
 #define TS_INV_SMEM (sizeof(float) * 2 * TS_R * (TS_R + 1))
 
 __device__ __forceinline__ unsigned long long ts_now()
@@ -973,23 +999,24 @@ __device__ __forceinline__ unsigned long long ts_now()
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
-__device__ __forceinline__ int ts_ld_acquire(const int *p)
+__device__ __forceinline__ unsigned long long ts_ld(const unsigned long long *p)
 {
-    int v;
-    asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
-__device__ __forceinline__ void ts_st_release(int *p, int v)
+__device__ __forceinline__ void ts_st(unsigned long long *p, unsigned long long v)
 {
-    asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
 struct TsArgs {
     const float *LU;
     const float *dinv;  // inverses of the diagonal blocks (inv_diag_kernel)
     float *y;           // right-hand side in, solution out
-    int n, lower, epoch;
-    int *flags;         // [nbk] epoch of the last launch that solved the block row
+    unsigned long long *z;   // [n] published values: launch epoch << 32 | y
+    int n, lower;
+    unsigned epoch;
     int *ticket;        // zero before the launch
     int *err;
 };
@@ -1028,11 +1055,77 @@ __global__ void __launch_bounds__(TS_R) inv_diag_kernel(const float *LU, int n, 
     for (int e = c; e < TS_R * TS_R; e += TS_R) D[e] = X[(e / TS_R) * TS_LD + e % TS_R];
 }
 
-__global__ void __launch_bounds__(256) trsv_chain_kernel(TsArgs a)
+// Inverse of a diagonal block in shared memory, column c of row r at c ^
+// ts_swz(r, c): the two halves of 16 rows are read without bank conflicts
+__device__ __forceinline__ int ts_swz(int r, int c) { return c ^ ((r & 15) | ((c >> 6) << 4)); }
+__device__ __forceinline__ void ts_load_inv(const TsArgs &a, int blk, int upper, float *D)
 {
-    extern __shared__ float ts_sm[];
-    float *D = ts_sm;                        // [TS_R][TS_LD] inverse of the diagonal block
-    float *s_b = ts_sm + TS_R * TS_LD;       // [TS_R] right-hand side minus the solved part
+    const float *g = a.dinv + (size_t)(2 * blk + upper) * TS_R * TS_R;
+    for (int e = threadIdx.x; e < TS_R * TS_R; e += TS_TH) {
+        const int r = e / TS_R;
+        D[r * TS_R + ts_swz(r, e % TS_R)] = g[e];
+    }
+}
+
+// Warp 0: the values of block [c0, c0 + cols) into zs once they carry the
+// launch's epoch; `behind`: block rows between this one and its turn.  `gave`:
+// a wait ran out before (then nothing is waited for).
+__device__ __forceinline__ void ts_wait(const TsArgs &a, int c0, int cols, int behind, float *zs, bool &gave)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned long long t0 = ts_now();
+    for (unsigned it = 0;; ++it) {
+        unsigned long long v[TS_R / 32];
+        bool ok = true;
+#pragma unroll
+        for (int q = 0; q < TS_R / 32; ++q) {
+            const int c = lane + 32 * q;
+            v[q] = c < cols ? ts_ld(a.z + c0 + c) : (unsigned long long)a.epoch << 32;
+            ok = ok && (unsigned)(v[q] >> 32) == a.epoch;
+        }
+        const bool all = __all_sync(0xffffffffu, ok);
+        if (!all && !gave && (it & 63u) == 63u && ts_now() - t0 > TS_WAIT_NS) {
+            gave = true;
+            if (lane == 0) atomicExch(a.err, OBEM_ERR_TIMEOUT);
+        }
+        gave = __shfl_sync(0xffffffffu, (int)gave, 0) != 0;
+        if (all || gave) {
+#pragma unroll
+            for (int q = 0; q < TS_R / 32; ++q)
+                zs[lane + 32 * q] = lane + 32 * q < cols ? __uint_as_float((unsigned)v[q]) : 0.f;
+            return;
+        }
+        if (behind > 1) __nanosleep(behind < 32 ? 32u * behind : 1000u);
+    }
+}
+
+// the block's solution: its inverse (trans: transposed) times s_b; thread
+// (row, half) = (tid / 2, tid % 2).  s_b: entries 0..63, then 64..127 from 80 on
+__device__ __forceinline__ void ts_publish(const TsArgs &a, const float *D, const float *s_b, bool trans, int r0,
+                                           int rows)
+{
+    const int row = threadIdx.x >> 1, half = threadIdx.x & 1;
+    const float *sb = s_b + 80 * half;
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int k = 0; k < 64; k += 4)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int c = 64 * half + k + u;
+            v[u] = fmaf(trans ? D[c * TS_R + ts_swz(c, row)] : D[row * TS_R + ts_swz(row, c)], sb[k + u], v[u]);
+        }
+    float t = (v[0] + v[1]) + (v[2] + v[3]);
+    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    if (half == 0 && row < rows) {
+        ts_st(a.z + r0 + row, (unsigned long long)a.epoch << 32 | __float_as_uint(t));
+        a.y[r0 + row] = t;
+    }
+}
+
+__global__ void __launch_bounds__(TS_TH) trsv_chain_kernel(TsArgs a)
+{
+    extern __shared__ float ts_sm[];         // [TS_R][TS_R] inverse of the diagonal block
+    __shared__ float s_b[144], s_z[2][TS_R];
     __shared__ int s_t;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     constexpr int RW = TS_R / 8;             // rows per warp
@@ -1042,157 +1135,98 @@ __global__ void __launch_bounds__(256) trsv_chain_kernel(TsArgs a)
     const int t = s_t;
     const int blk = a.lower ? t : nbk - 1 - t;
     const int r0 = blk * TS_R, rows = min(TS_R, n - r0);
-    {
-        const float *g = a.dinv + (size_t)(2 * blk + (a.lower ? 0 : 1)) * TS_R * TS_R;
-        for (int e = tid; e < TS_R * TS_R; e += 256) D[(e / TS_R) * TS_LD + e % TS_R] = g[e];
-    }
+    ts_load_inv(a, blk, a.lower ? 0 : 1, ts_sm);
     float acc[RW];
 #pragma unroll
     for (int r = 0; r < RW; ++r) acc[r] = 0.f;
-    int ready = 0;          // dependency steps this warp knows to be solved
+    // lane's row after the sum over the lanes, and its right-hand side
+    const int mine = RW * w + (lane >> 1);
+    const float rhs = mine < rows ? a.y[r0 + mine] : 0.f;
+    bool gave = false;
     for (int st = 0; st < t; ++st) {
         const int j = a.lower ? st : nbk - 1 - st;
         const int c0 = j * TS_R, cols = min(TS_R, n - c0);
-        if (st >= ready) {
-            // flags of steps st .. st + 31, until step st is solved
-            const unsigned long long t0 = ts_now();
-            for (unsigned it = 0;; ++it) {
-                const int q = st + lane;
-                const int f = q < t ? ts_ld_acquire(a.flags + (a.lower ? q : nbk - 1 - q)) : 0;
-                const unsigned ok = __ballot_sync(0xffffffffu, q < t && f == a.epoch);
-                if (ok & 1u) {
-                    ready = st + (~ok ? __ffs(~ok) - 1 : 32);
-                    break;
-                }
-                if ((it & 63u) == 63u && ts_now() - t0 > TS_WAIT_NS) {
-                    if (lane == 0) atomicExch(a.err, OBEM_ERR_TIMEOUT);
-                    ready = st + 1;
-                    break;
-                }
-                __nanosleep(32);
-            }
-            __syncwarp();
+        float l[RW][4];
+#pragma unroll
+        for (int r = 0; r < RW; ++r) {
+            const int row = RW * w + r;
+            const float *arow = a.LU + (size_t)(r0 + (row < rows ? row : 0)) * n + c0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) l[r][q] = lane + 32 * q < cols ? arow[lane + 32 * q] : 0.f;
         }
+        float *z = s_z[st & 1];
+        if (w == 0) ts_wait(a, c0, cols, t - st, z, gave);
+        __syncthreads();
+        float zz[4];
 #pragma unroll
-        for (int h = 0; h < TS_R; h += 64) {
-            float l0[RW], l1[RW];
+        for (int q = 0; q < 4; ++q) zz[q] = z[lane + 32 * q];
 #pragma unroll
-            for (int r = 0; r < RW; ++r) {
-                const int row = RW * w + r;
-                const float *arow = a.LU + (size_t)(r0 + row) * n + c0 + h;
-                l0[r] = (row < rows && h + lane < cols) ? arow[lane] : 0.f;
-                l1[r] = (row < rows && h + lane + 32 < cols) ? arow[lane + 32] : 0.f;
-            }
-            const float y0 = h + lane < cols ? __ldcg(a.y + c0 + h + lane) : 0.f;
-            const float y1 = h + lane + 32 < cols ? __ldcg(a.y + c0 + h + lane + 32) : 0.f;
+        for (int r = 0; r < RW; ++r)
 #pragma unroll
-            for (int r = 0; r < RW; ++r) acc[r] = fmaf(l0[r], y0, fmaf(l1[r], y1, acc[r]));
+            for (int q = 0; q < 4; ++q) acc[r] = fmaf(l[r][q], zz[q], acc[r]);
+    }
+    // sums over the lanes: each step halves the rows a lane holds; lanes 2 r,
+    // 2 r + 1 end with row r
+    int o = 16;
+#pragma unroll
+    for (int k = RW / 2; k > 0; k >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int r = 0; r < k; ++r) {
+            const float send = up ? acc[r] : acc[r + k], keep = up ? acc[r + k] : acc[r];
+            acc[r] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
     }
-#pragma unroll
-    for (int r = 0; r < RW; ++r) {
-        float v = acc[r];
-        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        const int row = RW * w + r;
-        if (lane == 0) s_b[row] = row < rows ? a.y[r0 + row] - v : 0.f;
-    }
+    const float sum = acc[0] + __shfl_xor_sync(0xffffffffu, acc[0], 1);
+    if ((lane & 1) == 0) s_b[mine + (mine >= 64 ? 16 : 0)] = mine < rows ? rhs - sum : 0.f;
     __syncthreads();
-    if (tid < rows) {
-        const float *d = D + tid * TS_LD;
-        float v = 0.f;
-        for (int k = 0; k < rows; ++k) v = fmaf(d[k], s_b[k], v);
-        a.y[r0 + tid] = v;
-        __threadfence();
-    }
-    __syncthreads();
-    if (tid == 0) ts_st_release(a.flags + blk, a.epoch);
+    ts_publish(a, ts_sm, s_b, false, r0, rows);
 }
 
 // The transposed substitutions of the adjoint solve, A^T x = b with
 // P A = L U: U^T (lower, forward; lower = 1) and L^T (unit upper, backward;
-// lower = 0) in one launch each, with the same tickets and flags.  Block row
-// i of U^T (L^T) is block column i of U (L): thread (c, half) sums column c
-// over every other row of each solved block j, whose y values warp 0 puts in
-// shared memory (double-buffered, one barrier per block); the diagonal block
-// uses the transposed inverse.
-#define TS_T_SMEM (sizeof(float) * (TS_R * (TS_R + 1) + 4 * TS_R))
-__global__ void __launch_bounds__(256) trsv_chain_t_kernel(TsArgs a)
+// lower = 0) in one launch each, with the same tickets and published values.
+// Block row i of U^T (L^T) is block column i of U (L): thread (c, half) sums
+// column c over half the rows of each solved block; the diagonal block uses
+// the transposed inverse.
+__global__ void __launch_bounds__(TS_TH) trsv_chain_t_kernel(TsArgs a)
 {
     extern __shared__ float ts_sm[];
-    float *D = ts_sm;                        // [TS_R][TS_LD]
-    float *s_b = D + TS_R * TS_LD;           // [TS_R]
-    float *s_z = s_b + TS_R;                 // [2][TS_R]
-    float *s_h = s_z + 2 * TS_R;             // [TS_R]
+    __shared__ float s_b[144], s_z[2][TS_R], s_h[TS_R];
     __shared__ int s_t;
-    const int tid = threadIdx.x, lane = tid & 31, c = tid & (TS_R - 1), half = tid / TS_R;
+    const int tid = threadIdx.x, c = tid & (TS_R - 1), half = tid / TS_R;
     const int n = a.n, nbk = (n + TS_R - 1) / TS_R;
     if (tid == 0) s_t = atomicAdd(a.ticket, 1);
     __syncthreads();
     const int t = s_t;
     const int blk = a.lower ? t : nbk - 1 - t;
     const int i0 = blk * TS_R, ni = min(TS_R, n - i0);
-    {
-        const float *g = a.dinv + (size_t)(2 * blk + (a.lower ? 1 : 0)) * TS_R * TS_R;
-        for (int e = tid; e < TS_R * TS_R; e += 256) D[(e / TS_R) * TS_LD + e % TS_R] = g[e];
-    }
-    float acc = 0.f;
-    int ready = 0;
+    ts_load_inv(a, blk, a.lower ? 1 : 0, ts_sm);
+    const float rhs = c < ni ? a.y[i0 + c] : 0.f;
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    bool gave = false;
     for (int st = 0; st < t; ++st) {
         const int j = a.lower ? st : nbk - 1 - st;
         const int j0 = j * TS_R, nj = min(TS_R, n - j0);
-        float *z = s_z + (st & 1) * TS_R;
-        if (tid < 32) {
-            if (st >= ready) {
-                const unsigned long long t0 = ts_now();
-                for (unsigned it = 0;; ++it) {
-                    const int q = st + lane;
-                    const int f = q < t ? ts_ld_acquire(a.flags + (a.lower ? q : nbk - 1 - q)) : 0;
-                    const unsigned ok = __ballot_sync(0xffffffffu, q < t && f == a.epoch);
-                    if (ok & 1u) {
-                        ready = st + (~ok ? __ffs(~ok) - 1 : 32);
-                        break;
-                    }
-                    if ((it & 63u) == 63u && ts_now() - t0 > TS_WAIT_NS) {
-                        if (lane == 0) atomicExch(a.err, OBEM_ERR_TIMEOUT);
-                        ready = st + 1;
-                        break;
-                    }
-                    __nanosleep(32);
-                }
-                __syncwarp();
-            }
+        const float *col = a.LU + (size_t)j0 * n + i0 + c;
+        float v[TS_R / 2];
 #pragma unroll
-            for (int q = 0; q < TS_R / 32; ++q) {
-                const int r = lane + 32 * q;
-                z[r] = r < nj ? __ldcg(a.y + j0 + r) : 0.f;
-            }
+        for (int u = 0; u < TS_R / 2; ++u) {
+            const int r = half * (TS_R / 2) + u;
+            v[u] = c < ni && r < nj ? col[(size_t)r * n] : 0.f;
         }
+        float *z = s_z[st & 1];
+        if (tid < 32) ts_wait(a, j0, nj, t - st, z, gave);
         __syncthreads();
-        if (c < ni) {
-            const float *col = a.LU + (size_t)j0 * n + i0 + c;
-            int r = half;
-            for (; r + 14 < nj; r += 16) {
-                float v[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = col[(size_t)(r + 2 * u) * n];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) acc = fmaf(v[u], z[r + 2 * u], acc);
-            }
-            for (; r < nj; r += 2) acc = fmaf(col[(size_t)r * n], z[r], acc);
-        }
+        for (int u = 0; u < TS_R / 2; ++u) acc[u & 3] = fmaf(v[u], z[half * (TS_R / 2) + u], acc[u & 3]);
     }
-    if (half == 1) s_h[c] = acc;
+    const float sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    if (half == 1) s_h[c] = sum;
     __syncthreads();
-    if (half == 0) s_b[c] = c < ni ? a.y[i0 + c] - (acc + s_h[c]) : 0.f;
+    if (half == 0) s_b[c + (c >= 64 ? 16 : 0)] = c < ni ? rhs - (sum + s_h[c]) : 0.f;
     __syncthreads();
-    if (tid < ni) {
-        float v = 0.f;
-        for (int k = 0; k < ni; ++k) v = fmaf(D[k * TS_LD + tid], s_b[k], v);
-        a.y[i0 + tid] = v;
-        __threadfence();
-    }
-    __syncthreads();
-    if (tid == 0) ts_st_release(a.flags + blk, a.epoch);
+    ts_publish(a, ts_sm, s_b, true, i0, ni);
 }
 
 // ------------------------------------------------------------------ host drivers
@@ -1387,7 +1421,8 @@ static int alloc_system(obem_ctx *c, int n)
     for (void *q : bufs)
         if (q) cudaFree(q);
     c->d_A = c->d_LU = NULL;
-    c->d_piv = c->d_flag = c->d_perm = c->d_trsv = NULL;
+    c->d_piv = c->d_flag = c->d_perm = NULL;
+    c->d_trsv = NULL;
     c->d_dinv = NULL;
     c->d_rowscale = c->d_work64 = NULL;
     c->d_work32 = c->d_panel = NULL;
@@ -1403,8 +1438,9 @@ static int alloc_system(obem_ctx *c, int n)
     OBEM_CUDA(c, cudaMalloc((void **)&c->d_panel,
                             sizeof(float) * (PAN_SCRATCH_FLOATS + PAN_PLAN_FLOATS + 2 * (size_t)LU_NB * n)));
     OBEM_CUDA(c, cudaMalloc((void **)&c->d_perm, sizeof(int) * n));
-    OBEM_CUDA(c, cudaMalloc((void **)&c->d_trsv, sizeof(int) * ((size_t)n / TS_R + 16)));
-    OBEM_CUDA(c, cudaMemset(c->d_trsv, 0, sizeof(int) * ((size_t)n / TS_R + 16)));
+    // published values of the substitutions (no epoch yet), tickets and status
+    OBEM_CUDA(c, cudaMalloc((void **)&c->d_trsv, sizeof(unsigned long long) * ((size_t)n + 4)));
+    OBEM_CUDA(c, cudaMemset(c->d_trsv, 0, sizeof(unsigned long long) * ((size_t)n + 4)));
     c->trsv_epoch = 0;
     OBEM_CUDA(c, cudaMalloc((void **)&c->d_dinv, sizeof(float) * 2 * TS_R * TS_R * (size_t)((n + TS_R - 1) / TS_R)));
     c->nsys_alloc = n;
@@ -1548,7 +1584,7 @@ static int factor_system(obem_ctx *c, int precision, cudaStream_t s)
 static int lu_solve(obem_ctx *c, float *y, cudaStream_t s)
 {
     const int n = c->nsys, nbk = (n + TS_R - 1) / TS_R;
-    int *ticket = c->d_trsv + nbk, *err = ticket + 2;
+    int *ticket = (int *)(c->d_trsv + n), *err = ticket + 2;
     OBEM_CUDA(c, cudaMemsetAsync(ticket, 0, sizeof(int) * 3, s));
     for (int lower = 1; lower >= 0; --lower) {
         TsArgs a;
@@ -1558,10 +1594,10 @@ static int lu_solve(obem_ctx *c, float *y, cudaStream_t s)
         a.n = n;
         a.lower = lower;
         a.epoch = ++c->trsv_epoch;
-        a.flags = c->d_trsv;
+        a.z = c->d_trsv;
         a.ticket = ticket + (lower ? 0 : 1);
         a.err = err;
-        trsv_chain_kernel<<<nbk, 256, TS_SMEM, s>>>(a);
+        trsv_chain_kernel<<<nbk, TS_TH, TS_SMEM, s>>>(a);
         OBEM_LAUNCH(c);
     }
     int h = 0;
@@ -1580,7 +1616,7 @@ int obem_selftest_solve_wait(obem_ctx *c, cudaStream_t s)
     if (!c->factored || c->nsys < 2 * TS_R)
         return obem_fail(c, OBEM_ERR_STATE, "wait self-test: needs the factors of a system of >= %d rows", 2 * TS_R);
     const int n = c->nsys, nbk = (n + TS_R - 1) / TS_R;
-    int *ticket = c->d_trsv + nbk, *err = ticket + 2;
+    int *ticket = (int *)(c->d_trsv + n), *err = ticket + 2;
     const int one = 1;
     OBEM_CUDA(c, cudaMemsetAsync(ticket, 0, sizeof(int) * 3, s));
     OBEM_CUDA(c, cudaMemcpyAsync(ticket, &one, sizeof(int), cudaMemcpyHostToDevice, s));
@@ -1591,10 +1627,10 @@ int obem_selftest_solve_wait(obem_ctx *c, cudaStream_t s)
     a.n = n;
     a.lower = 1;
     a.epoch = ++c->trsv_epoch;
-    a.flags = c->d_trsv;
+    a.z = c->d_trsv;
     a.ticket = ticket;
     a.err = err;
-    trsv_chain_kernel<<<1, 256, TS_SMEM, s>>>(a);
+    trsv_chain_kernel<<<1, TS_TH, TS_SMEM, s>>>(a);
     OBEM_LAUNCH(c);
     int h = 0;
     OBEM_CUDA(c, cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -1619,9 +1655,14 @@ static int refine(obem_ctx *c, int &it, int &status, double &be, cudaStream_t s)
     status = OBEM_ERR_NOT_CONVERGED;
     const int max_it = 30;
     for (; it <= max_it; ++it) {
-        split_kernel<<<(n + 255) / 256, 256, 0, s>>>(x, y, y + n, n);
-        residual_kernel<<<(n + 7) / 8, 256, 0, s>>>(c->d_A, y, y + n, b, r, n);
-        norms_kernel<<<1, 256, 0, s>>>(r, x, b, n, nrm);
+        if (it == 0) {
+            // x = 0: the residual is b (no pass over the matrix)
+            OBEM_CUDA(c, cudaMemcpyAsync(r, b, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
+        } else {
+            split_kernel<<<(n + 255) / 256, 256, 0, s>>>(x, y, y + n, n);
+            residual_kernel<<<(n + 7) / 8, 256, 0, s>>>(c->d_A, y, y + n, b, r, n);
+        }
+        norms_kernel<<<1, 1024, 0, s>>>(r, x, b, n, nrm);
         OBEM_LAUNCH(c);
         double h[3];
         OBEM_CUDA(c, cudaMemcpyAsync(h, nrm, sizeof h, cudaMemcpyDeviceToHost, s));
@@ -1764,13 +1805,33 @@ __global__ void residual_t_fold_kernel(const double *part, const double *b, doub
     r[j] = b[j] - s;
 }
 
-// colsum[j] = sum_i |At[i][j]|  (for the transposed system's infinity norm)
-__global__ void colsum_kernel(const float *A, double *colsum, int n)
+// column sums of |A| over a share of the rows (for the transposed system's
+// infinity norm), compensated; HBM-bound (one thread per column over all rows
+// in FP64 took 1.65 ms at 11,008 cells)
+__global__ void colsum_kernel(const float *A, double *part, int n)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    const int s = blockIdx.y;
+    const int i0 = (int)((long long)n * s / ADJ_SPLIT), i1 = (int)((long long)n * (s + 1) / ADJ_SPLIT);
+    if (j >= n) return;
+    float sm = 0.f, cm = 0.f;
+    int i = i0;
+    for (; i + 7 < i1; i += 8) {
+        float av[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) av[u] = __ldcs(A + (size_t)(i + u) * n + j);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) two_sum_acc(sm, cm, fabsf(av[u]));
+    }
+    for (; i < i1; ++i) two_sum_acc(sm, cm, fabsf(A[(size_t)i * n + j]));
+    part[(size_t)s * n + j] = (double)sm + (double)cm;
+}
+__global__ void colsum_fold_kernel(const double *part, double *colsum, int n)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
     double s = 0.0;
-    for (int i = 0; i < n; ++i) s += fabs((double)A[(size_t)i * n + j]);
+    for (int q = 0; q < ADJ_SPLIT; ++q) s += part[(size_t)q * n + j];
     colsum[j] = s;
 }
 
@@ -1821,11 +1882,11 @@ __global__ void axpy_unpermute_kernel(double *x, const float *y, const int *perm
 static int lu_solve_t(obem_ctx *c, float *y, cudaStream_t s)
 {
     const int n = c->nsys, nbk = (n + TS_R - 1) / TS_R;
-    int *ticket = c->d_trsv + nbk, *err = ticket + 2;
+    int *ticket = (int *)(c->d_trsv + n), *err = ticket + 2;
     static unsigned long long attr = 0;   // devices done (a bit each)
     if (!(attr >> (c->device & 63) & 1ull)) {
         OBEM_CUDA(c, cudaFuncSetAttribute(trsv_chain_t_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)TS_T_SMEM));
+                                          (int)TS_SMEM));
         attr |= 1ull << (c->device & 63);
     }
     OBEM_CUDA(c, cudaMemsetAsync(ticket, 0, sizeof(int) * 3, s));
@@ -1837,10 +1898,10 @@ static int lu_solve_t(obem_ctx *c, float *y, cudaStream_t s)
         a.n = n;
         a.lower = lower;
         a.epoch = ++c->trsv_epoch;
-        a.flags = c->d_trsv;
+        a.z = c->d_trsv;
         a.ticket = ticket + (lower ? 0 : 1);
         a.err = err;
-        trsv_chain_t_kernel<<<nbk, 256, TS_T_SMEM, s>>>(a);
+        trsv_chain_t_kernel<<<nbk, TS_TH, TS_SMEM, s>>>(a);
         OBEM_LAUNCH(c);
     }
     int h = 0;
@@ -1873,16 +1934,22 @@ int obem_solve_adjoint(obem_ctx *c, const float *g, double *dL_dgv, float *dL_db
     } while (0)
     ADJ_CUDA(cudaMalloc((void **)&part, sizeof(double) * (size_t)ADJ_SPLIT * n));
     ADJ_CUDA(cudaMalloc((void **)&col, sizeof(double) * ((size_t)n + 1)));
-    colsum_kernel<<<(n + 255) / 256, 256, 0, s>>>(c->d_A, col, n);
+    colsum_kernel<<<dim3((n + 255) / 256, ADJ_SPLIT), 256, 0, s>>>(c->d_A, part, n);
+    colsum_fold_kernel<<<(n + 255) / 256, 256, 0, s>>>(part, col, n);
     max_kernel<<<1, 256, 0, s>>>(col, n, col + n);
     load_adjoint_kernel<<<(n + 255) / 256, 256, 0, s>>>(g, b, x, n);
     ADJ_CUDA(cudaGetLastError());
     ADJ_CUDA(cudaMemcpyAsync(&a1, col + n, sizeof(double), cudaMemcpyDeviceToHost, s));
     for (; it <= 30; ++it) {
-        split_kernel<<<(n + 255) / 256, 256, 0, s>>>(x, y, y + n, n);
-        residual_t_part_kernel<<<dim3((n + 255) / 256, ADJ_SPLIT), 256, 0, s>>>(c->d_A, y, y + n, part, n);
-        residual_t_fold_kernel<<<(n + 255) / 256, 256, 0, s>>>(part, b, r, n);
-        norms_kernel<<<1, 256, 0, s>>>(r, x, b, n, nrm);
+        if (it == 0) {
+            // x = 0: the residual is b (no pass over the matrix)
+            ADJ_CUDA(cudaMemcpyAsync(r, b, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
+        } else {
+            split_kernel<<<(n + 255) / 256, 256, 0, s>>>(x, y, y + n, n);
+            residual_t_part_kernel<<<dim3((n + 255) / 256, ADJ_SPLIT), 256, 0, s>>>(c->d_A, y, y + n, part, n);
+            residual_t_fold_kernel<<<(n + 255) / 256, 256, 0, s>>>(part, b, r, n);
+        }
+        norms_kernel<<<1, 1024, 0, s>>>(r, x, b, n, nrm);
         ADJ_CUDA(cudaGetLastError());
         double h[3];
         ADJ_CUDA(cudaMemcpyAsync(h, nrm, sizeof h, cudaMemcpyDeviceToHost, s));
