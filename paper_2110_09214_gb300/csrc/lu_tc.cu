@@ -300,35 +300,70 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                      : "memory");
 }
 
-// out[i * ldo + k] = bf16(A[i * lda + k]), i < M, k < K: blockDim.x threads
-// across a row (a multiple of 32, not above K's), blockDim.y rows per pass,
-// grid-stride in both
-__global__ void tc_cvt_rows_kernel(const float *__restrict__ A, long long lda, int M, int K,
-                                   __nv_bfloat16 *__restrict__ out, int ldo)
+// Both operands of a GEMM to BF16 in one launch: blocks [0, na) round 64 x 64
+// tiles of A (Ab[i][k] = bf16(A[i][k])), the others round and transpose tiles of
+// B (Bb[j][k] = bf16(B[k][j])) through shared memory.  Eight values per 16-byte
+// store; VEC: float4 loads (both matrices 16-byte aligned with row pitches of
+// multiples of 4).  Columns K .. ldo - 1 are written as zeros.  HBM-bound for the
+// large operands (6 bytes per element); most of the factorisation's 2,729
+// GEMMs are small and paid the launch of a second kernel and 2- and 4-byte
+// accesses: 50.3 ms of conversions at order 59,968 in two kernels.
+#define CV_T 64
+template <bool VEC>
+__global__ void __launch_bounds__(256) tc_cvt_kernel(const float *__restrict__ A, long long lda, int M, int K,
+                                                     __nv_bfloat16 *__restrict__ Ab, const float *__restrict__ B,
+                                                     long long ldb, int N, __nv_bfloat16 *__restrict__ Bb, int ldo,
+                                                     int na, int nk)
 {
-    for (int i = blockIdx.y * blockDim.y + threadIdx.y; i < M; i += gridDim.y * blockDim.y)
-        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < K; k += gridDim.x * blockDim.x)
-            out[(size_t)i * ldo + k] = __float2bfloat16_rn(A[(size_t)i * lda + k]);
-}
-
-// out[j * ldo + k] = bf16(B[k * ldb + j]), j < N, k < K (transpose through
-// a 32 x 32 shared tile: both sides coalesced)
-__global__ void tc_cvt_trans_kernel(const float *__restrict__ B, long long ldb, int K, int N,
-                                    __nv_bfloat16 *__restrict__ out, int ldo)
-{
-    __shared__ float t[32][33];
-    const int j0 = blockIdx.x * 32;
-    for (int k0 = blockIdx.y * 32; k0 < K; k0 += gridDim.y * 32) {
-        for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-            const int k = k0 + r, j = j0 + threadIdx.x;
-            t[r][threadIdx.x] = (k < K && j < N) ? B[(size_t)k * ldb + j] : 0.f;
+    __shared__ float t[CV_T][CV_T + 1];
+    const int tid = threadIdx.x;
+    union Pack { __nv_bfloat162 h[4]; uint4 u; };
+    auto load8 = [](const float *p, int left, float (&v)[8]) {
+        if (VEC && left >= 8) {
+            const float4 x = *reinterpret_cast<const float4 *>(p), y = *reinterpret_cast<const float4 *>(p + 4);
+            v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w; v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+        } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = q < left ? p[q] : 0.f;
         }
-        __syncthreads();
-        for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-            const int j = j0 + r, k = k0 + threadIdx.x;
-            if (j < N && k < K) out[(size_t)j * ldo + k] = __float2bfloat16_rn(t[threadIdx.x][r]);
+    };
+    auto store8 = [](__nv_bfloat16 *p, const float (&v)[8]) {
+        Pack o;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) o.h[q] = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
+        *reinterpret_cast<uint4 *>(p) = o.u;
+    };
+    const bool isA = (int)blockIdx.x < na;
+    const int tile = isA ? blockIdx.x : blockIdx.x - na;
+    const int k0 = (tile % nk) * CV_T, i0 = (tile / nk) * CV_T;
+    if (isA) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int i = i0 + (tid >> 3) + 32 * q, k = k0 + (tid & 7) * 8;
+            if (i >= M || k >= ldo) continue;
+            float v[8];
+            load8(A + (size_t)i * lda + k, K - k, v);
+            store8(Ab + (size_t)i * ldo + k, v);
         }
-        __syncthreads();
+        return;
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int r = (tid >> 3) + 32 * q, c = (tid & 7) * 8;
+        float v[8];
+        load8(B + (size_t)(k0 + r) * ldb + i0 + c, k0 + r < K ? N - i0 - c : 0, v);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) t[r][c + e] = v[e];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int c = (tid >> 3) + 32 * q, r = (tid & 7) * 8;
+        if (i0 + c >= N || k0 + r >= ldo) continue;
+        float v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = t[r + e][c];
+        store8(Bb + (size_t)(i0 + c) * ldo + k0 + r, v);
     }
 }
 
@@ -409,13 +444,12 @@ int obem_tc_gemm_sub(obem_ctx *c, float *C, long long ldc, const float *A, long 
     if (rc != OBEM_OK) return rc;
     __nv_bfloat16 *Ab = (__nv_bfloat16 *)c->tc_a, *Bb = (__nv_bfloat16 *)c->tc_b;
     {
-        // skinny operands (K of 64 against tall M) get several rows per block
-        const int tx = K >= 256 ? 256 : (K + 31) / 32 * 32, ty = 256 / tx;
-        const int gx = K >= 256 ? ((K + 255) / 256 < 64 ? (K + 255) / 256 : 64) : 1;
-        const int gyn = (M + ty - 1) / ty, gy = gyn < 4096 ? gyn : 4096;
-        tc_cvt_rows_kernel<<<dim3(gx, gy), dim3(tx, ty), 0, s>>>(A, lda, M, K, Ab, ldk);
-        dim3 gt((N + 31) / 32, (K + 31) / 32 < 65535 ? (K + 31) / 32 : 65535);
-        tc_cvt_trans_kernel<<<gt, dim3(32, 8), 0, s>>>(B, ldb, K, N, Bb, ldk);
+        const int nk = (ldk + CV_T - 1) / CV_T;
+        const long long na = (long long)((M + CV_T - 1) / CV_T) * nk, nb = (long long)((N + CV_T - 1) / CV_T) * nk;
+        if (na + nb > 0x7fffffffll) return obem_fail(c, OBEM_ERR_ARG, "tensor-core GEMM: operands exceed the grid");
+        const bool vec = (((uintptr_t)A | (uintptr_t)B) & 15) == 0 && ((lda | ldb) & 3) == 0;
+        if (vec) tc_cvt_kernel<true><<<(unsigned)(na + nb), 256, 0, s>>>(A, lda, M, K, Ab, B, ldb, N, Bb, ldk, (int)na, nk);
+        else tc_cvt_kernel<false><<<(unsigned)(na + nb), 256, 0, s>>>(A, lda, M, K, Ab, B, ldb, N, Bb, ldk, (int)na, nk);
         OBEM_LAUNCH(c);
     }
     CUtensorMap ma, mb;
