@@ -503,8 +503,9 @@ __global__ void __launch_bounds__(32 * BR_WARPS) bw_sigma_kernel(BwLaunch B)
             const int t = s_q[warp][0][lane];
             const float4 x = B.targets[t], g = B.g[t];
             double phi, fx, fy, fz;
-            tri_closed_form(P.v64 + 9 * (size_t)(j0 + s_q[warp][1][lane]), (double)x.x, (double)x.y, (double)x.z, phi, fx,
-                            fy, fz);
+            const size_t jc = (size_t)(j0 + s_q[warp][1][lane]);
+            tri_closed_form_g(P.v64 + 9 * jc, P.geo + OBEM_GEO64 * jc, (double)x.x, (double)x.y, (double)x.z, phi, fx, fy,
+                              fz);
             s_v[warp][lane] =
                 (float)(OBEM_KC * ((double)g.x * fx + (double)g.y * fy + (double)g.z * fz + (double)g.w * phi));
         }
@@ -942,7 +943,8 @@ __device__ __forceinline__ void if_closed(const PanelsDev &P, int j, const float
     if (lane < n) {
         const float4 x = cq[lane];
         double phi, fx, fy, fz;
-        tri_closed_form(P.v64 + 9 * (size_t)j, (double)x.x, (double)x.y, (double)x.z, phi, fx, fy, fz);
+        tri_closed_form_g(P.v64 + 9 * (size_t)j, P.geo + (size_t)OBEM_GEO64 * j, (double)x.x, (double)x.y, (double)x.z,
+                          phi, fx, fy, fz);
         const double qk = (double)x.w * OBEM_KC;
         v[0] += (float)(qk * phi); v[1] += (float)(qk * fx);
         v[2] += (float)(qk * fy); v[3] += (float)(qk * fz);

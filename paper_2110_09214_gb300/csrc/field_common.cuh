@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "closed_form.cuh"
+
 typedef unsigned long long u64;
 
 // ------------------------------------------------------------------ packed f32x2
@@ -89,21 +91,21 @@ __device__ __forceinline__ int32_t block_scan_1024(int32_t v, int32_t *s_warp)
 // integrals L_i = ln((R+ + l+)/(R- + l-)) evaluated without cancellation and
 // Omega the signed solid angle (Van Oosterom & Strackee); principal value in
 // the cell's plane.
-static __device__ __noinline__ void tri_closed_form(const double *v, double rx, double ry, double rz, double &phi,
+static __host__ __device__ __noinline__ void tri_closed_form(const double *v, double rx, double ry, double rz, double &phi,
                                 double &Fx, double &Fy, double &Fz)
 {
     double e1x = v[3] - v[0], e1y = v[4] - v[1], e1z = v[5] - v[2];
     double e2x = v[6] - v[0], e2y = v[7] - v[1], e2z = v[8] - v[2];
     double nx = e1y * e2z - e1z * e2y, ny = e1z * e2x - e1x * e2z, nz = e1x * e2y - e1y * e2x;
-    double a2 = sqrt(nx * nx + ny * ny + nz * nz);
-    nx /= a2; ny /= a2; nz /= a2;
+    const double a2 = cf_sqrt(nx * nx + ny * ny + nz * nz), ia = 1.0 / a2;
+    nx *= ia; ny *= ia; nz *= ia;
     double ax[3], ay[3], az[3], R[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         ax[i] = v[3 * i] - rx;
         ay[i] = v[3 * i + 1] - ry;
         az[i] = v[3 * i + 2] - rz;
-        R[i] = sqrt(ax[i] * ax[i] + ay[i] * ay[i] + az[i] * az[i]);
+        R[i] = cf_sqrt(ax[i] * ax[i] + ay[i] * ay[i] + az[i] * az[i]);
     }
     double h = -(ax[0] * nx + ay[0] * ny + az[0] * nz);
     double ps = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;
@@ -111,23 +113,23 @@ static __device__ __noinline__ void tri_closed_form(const double *v, double rx, 
     for (int i = 0; i < 3; ++i) {
         int j = (i + 1) % 3;
         double dx = v[3 * j] - v[3 * i], dy = v[3 * j + 1] - v[3 * i + 1], dz = v[3 * j + 2] - v[3 * i + 2];
-        double len = sqrt(dx * dx + dy * dy + dz * dz);
-        dx /= len; dy /= len; dz /= len;
+        const double il = 1.0 / cf_sqrt(dx * dx + dy * dy + dz * dz);
+        dx *= il; dy *= il; dz *= il;
         double ux = dy * nz - dz * ny, uy = dz * nx - dx * nz, uz = dx * ny - dy * nx;
         double lm = ax[i] * dx + ay[i] * dy + az[i] * dz;
         double lp = ax[j] * dx + ay[j] * dy + az[j] * dz;
         double p0 = ax[i] * ux + ay[i] * uy + az[i] * uz;
-        double L;
-        if (lm >= 0.0) L = log((R[j] + lp) / (R[i] + lm));
-        else if (lp <= 0.0) L = log((R[i] - lm) / (R[j] - lp));
-        else L = log((R[j] + lp) * (R[i] - lm) / (p0 * p0 + h * h));
+        const bool fwd = lm >= 0.0, bwd = lp <= 0.0;
+        const double num = fwd ? R[j] + lp : bwd ? R[i] - lm : (R[j] + lp) * (R[i] - lm);
+        const double den = fwd ? R[i] + lm : bwd ? R[j] - lp : p0 * p0 + h * h;
+        const double L = cf_log_ratio(num, den);
         if (p0 != 0.0) ps += p0 * L;
         fx += ux * L; fy += uy * L; fz += uz * L;
     }
     double D = R[0] * R[1] * R[2] + (ax[0] * ax[1] + ay[0] * ay[1] + az[0] * az[1]) * R[2]
              + (ax[0] * ax[2] + ay[0] * ay[2] + az[0] * az[2]) * R[1]
              + (ax[1] * ax[2] + ay[1] * ay[2] + az[1] * az[2]) * R[0];
-    double Om = (h == 0.0) ? 0.0 : 2.0 * atan2(a2 * h, D);
+    double Om = (h == 0.0) ? 0.0 : 2.0 * cf_atan2(a2 * h, D);
     phi = ps - h * Om;
     Fx = fx + Om * nx;
     Fy = fy + Om * ny;
@@ -138,7 +140,7 @@ static __device__ __noinline__ void tri_closed_form(const double *v, double rx, 
 // normal, twice the area, unit edge vectors and in-plane edge normals, the
 // layout of OBEM_GEO64): per evaluation only the vertex offsets, their
 // lengths, the edge logarithms and the solid angle remain.
-static __device__ __noinline__ void tri_closed_form_g(const double *v, const double *g, double rx, double ry,
+static __host__ __device__ __noinline__ void tri_closed_form_g(const double *v, const double *g, double rx, double ry,
                                                       double rz, double &phi, double &Fx, double &Fy, double &Fz)
 {
     const double nx = g[0], ny = g[1], nz = g[2], a2 = g[3];
@@ -148,7 +150,7 @@ static __device__ __noinline__ void tri_closed_form_g(const double *v, const dou
         ax[i] = v[3 * i] - rx;
         ay[i] = v[3 * i + 1] - ry;
         az[i] = v[3 * i + 2] - rz;
-        R[i] = sqrt(ax[i] * ax[i] + ay[i] * ay[i] + az[i] * az[i]);
+        R[i] = cf_sqrt(ax[i] * ax[i] + ay[i] * ay[i] + az[i] * az[i]);
     }
     const double h = -(ax[0] * nx + ay[0] * ny + az[0] * nz);
     double ps = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;
@@ -160,17 +162,17 @@ static __device__ __noinline__ void tri_closed_form_g(const double *v, const dou
         const double lm = ax[i] * dx + ay[i] * dy + az[i] * dz;
         const double lp = ax[j] * dx + ay[j] * dy + az[j] * dz;
         const double p0 = ax[i] * ux + ay[i] * uy + az[i] * uz;
-        double L;
-        if (lm >= 0.0) L = log((R[j] + lp) / (R[i] + lm));
-        else if (lp <= 0.0) L = log((R[i] - lm) / (R[j] - lp));
-        else L = log((R[j] + lp) * (R[i] - lm) / (p0 * p0 + h * h));
+        const bool fwd = lm >= 0.0, bwd = lp <= 0.0;
+        const double num = fwd ? R[j] + lp : bwd ? R[i] - lm : (R[j] + lp) * (R[i] - lm);
+        const double den = fwd ? R[i] + lm : bwd ? R[j] - lp : p0 * p0 + h * h;
+        const double L = cf_log_ratio(num, den);
         if (p0 != 0.0) ps += p0 * L;
         fx += ux * L; fy += uy * L; fz += uz * L;
     }
     const double D = R[0] * R[1] * R[2] + (ax[0] * ax[1] + ay[0] * ay[1] + az[0] * az[1]) * R[2]
                    + (ax[0] * ax[2] + ay[0] * ay[2] + az[0] * az[2]) * R[1]
                    + (ax[1] * ax[2] + ay[1] * ay[2] + az[1] * az[2]) * R[0];
-    const double Om = (h == 0.0) ? 0.0 : 2.0 * atan2(a2 * h, D);
+    const double Om = (h == 0.0) ? 0.0 : 2.0 * cf_atan2(a2 * h, D);
     phi = ps - h * Om;
     Fx = fx + Om * nx;
     Fy = fy + Om * ny;
