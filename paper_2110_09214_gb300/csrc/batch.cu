@@ -20,6 +20,7 @@ struct obem_batch {
     std::vector<std::vector<float>> sig;   // densities per chamber
     int cells_dirty;
     int cut;                               // cell-kernel block size
+    int ch;                                // items per work unit of the all-pairs kernel
     // device tables
     int32_t *d_seg_off, *d_blk_cham, *d_slot_cham;
     ChamberP *d_cham;
@@ -118,6 +119,9 @@ extern "C" int obem_batch_create(obem_batch **out, obem_ctx *ctx, int32_t n_cham
     std::vector<int32_t> blk_cham(S / 256), slot_cham(S / OBEM_SEG_ALIGN);
     std::vector<ChamberP> cham(nb);
     std::vector<long long> joff(nb), ioff(nb);
+    long long items = 0;
+    for (int c = 0; c < nb; ++c) items += obem_sym_items(off[c + 1] - off[c]);
+    b->ch = obem_sym_batch_ch(items);
     long long jt = 0, it = 0;
     int max_blocks = 0;
     for (int c = 0; c < nb; ++c) {
@@ -130,7 +134,7 @@ extern "C" int obem_batch_create(obem_batch **out, obem_ctx *ctx, int32_t n_cham
         // a chamber may fill its whole segment: everything is sized by its length
         const int seg = off[c + 1] - off[c];
         size_t ipf;
-        const size_t jpf = obem_sym_sizes(seg, &ipf);
+        const size_t jpf = obem_sym_sizes(seg, b->ch, &ipf);
         joff[c] = jt;
         ioff[c] = it;
         jt += (long long)jpf;
@@ -348,6 +352,7 @@ static FieldBatch field_args(obem_batch *b, const obem_state *st)
     F.tileq = b->d_tileq;
     F.counter = b->d_counter;
     F.sym_grid = b->sym_grid;
+    F.ch = b->ch;
     return F;
 }
 

@@ -305,16 +305,15 @@ direct_pairs_kernel(FieldLaunch L, SymBatch SB, int add)
 }
 
 // Targets per block: 8 (four packs, 4 warps), 2 (8 warps) for fewer than
-// DF_WIDE targets: 2000 targets are 250 blocks of 8, hardly a warp per
+// OBEM_DIRECT_WIDE targets: 2000 targets are 250 blocks of 8, hardly a warp per
 // scheduler, and the cells of a block of 2 cost one iteration per 256.
-#define DF_WIDE 4096
 
 int obem_launch_direct_cells(obem_ctx *ctx, const FieldLaunch &L, const SymBatch *SB, int slots, cudaStream_t s)
 {
     SymBatch none;
     memset(&none, 0, sizeof none);
     const SymBatch &B = SB ? *SB : none;
-    if (slots >= DF_WIDE || SB) {
+    if (slots >= OBEM_DIRECT_WIDE || SB) {
         const int g = (slots + 7) / 8;
         if (SB) direct_cells_kernel<false, true, 4, 4><<<g, 128, 0, s>>>(L, B);
         else if (L.want_v) direct_cells_kernel<true, false, 4, 4><<<g, 128, 0, s>>>(L, B);
@@ -334,7 +333,7 @@ int obem_launch_direct_pairs(obem_ctx *ctx, const FieldLaunch &L, const SymBatch
     SymBatch none;
     memset(&none, 0, sizeof none);
     const SymBatch &B = SB ? *SB : none;
-    if (slots >= DF_WIDE || SB) {
+    if (slots >= OBEM_DIRECT_WIDE || SB) {
         const int g = (slots + 7) / 8;
         if (SB) direct_pairs_kernel<false, true, 4, 4><<<g, 128, 0, s>>>(L, B, add);
         else if (L.want_v) direct_pairs_kernel<true, false, 4, 4><<<g, 128, 0, s>>>(L, B, add);

@@ -1495,6 +1495,7 @@ __global__ void sym_tileq_kernel(const float4 *sorted, int nt, const int32_t *nt
 }
 
 // units of every chamber of a batch and their offsets (one block)
+template <int CH>
 __global__ void sym_units_kernel(SymBatch SB)
 {
     __shared__ int32_t carry;
@@ -1504,7 +1505,7 @@ __global__ void sym_units_kernel(SymBatch SB)
         const int c = c0 + threadIdx.x;
         int32_t u = 0;
         if (c < SB.nb && SB.n[c] > 0) {
-            const SymGeom G = sym_geom(SB.n[c]);
+            const SymGeom G = sym_geom_ch<CH>(SB.n[c]);
             u = G.n * G.nch;
         }
         // inclusive block scan
@@ -1526,6 +1527,8 @@ __global__ void sym_units_kernel(SymBatch SB)
 }
 
 template <bool B> struct SyBool { static constexpr bool value = B; };
+template <int I> struct SyInt { static constexpr int value = I; };
+static_assert(SY_NP == 4, "four packs of targets per thread (diagonal item)");
 
 template <bool WANT_V, bool BATCH, int CH = SY_CH>
 __global__ void __launch_bounds__(SY_THREADS, SY_MINB)
@@ -1642,45 +1645,65 @@ nbsym_kernel(FieldLaunch L, float *jpart, float *ipart, int *counter, const floa
                         s_src[l] = sp;
                     }
                     __syncthreads();
-                    float part[SY_NI][4];
+                    // 128 sources at a time: their own targets are slot seg of
+                    // the threads, so one pack of targets masks its own pair
+                    u64 X[SY_NP], Y[SY_NP], Z[SY_NP], W[SY_NP];
 #pragma unroll
-                    for (int k = 0; k < SY_NI; ++k) part[k][0] = part[k][1] = part[k][2] = part[k][3] = 0.f;
-                    for (int jj = 0; jj < SY_DTILE; ++jj) {
-                        const int j = jb + sb + jj;
-                        float sx, sy, sz, sq, dum;
-                        upk(s_src[jj].xx, sx, dum); upk(s_src[jj].yy, sy, dum);
-                        upk(s_src[jj].zz, sz, dum); upk(s_src[jj].qq, sq, dum);
+                    for (int p = 0; p < SY_NP; ++p) X[p] = Y[p] = Z[p] = W[p] = 0ull;
+                    auto segment = [&](int l0, int half, auto pack_c) {
+                        constexpr int PO = decltype(pack_c)::value;
+#pragma unroll 2
+                        for (int jj = 0; jj < SY_THREADS; ++jj) {
+                            const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(&s_src[l0 + jj].xx);
+                            const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(&s_src[l0 + jj].zz);
+                            const bool own = jj == tid;
 #pragma unroll
-                        for (int k = 0; k < SY_NI; ++k) {
-                            const int i = base + k * SY_THREADS + tid;
-                            if (j == i) continue;
-                            float txk, tyk, tzk, t2;
-                            if (k & 1) { upk(TX[k >> 1], t2, txk); upk(TY[k >> 1], t2, tyk); upk(TZ[k >> 1], t2, tzk); }
-                            else { upk(TX[k >> 1], txk, t2); upk(TY[k >> 1], tyk, t2); upk(TZ[k >> 1], tzk, t2); }
-                            const float dx = __fsub_rn(txk, sx), dy = __fsub_rn(tyk, sy), dz = __fsub_rn(tzk, sz);
-                            const float r2 = fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, L.eps2)));
-                            const float inv = rsq(r2);
-                            const float s = sq * inv;
-                            const float s3 = s * (inv * inv);
-                            part[k][0] = fmaf(dx, s3, part[k][0]);
-                            part[k][1] = fmaf(dy, s3, part[k][1]);
-                            part[k][2] = fmaf(dz, s3, part[k][2]);
-                            part[k][3] += s;
+                            for (int p = 0; p < SY_NP; ++p) {
+                                const u64 dx = sub2(TX[p], a.x), dy = sub2(TY[p], a.y), dz = sub2(TZ[p], b.x);
+                                const u64 r2 = fma2(dz, dz, fma2(dy, dy, fma2(dx, dx, EPS2)));
+                                float ra, rb;
+                                upk(r2, ra, rb);
+                                float ia = rsq(ra), ib = rsq(rb);
+                                if (p == PO) {
+                                    ia = own && half == 0 ? 0.f : ia;
+                                    ib = own && half == 1 ? 0.f : ib;
+                                }
+                                const u64 inv = pk(ia, ib);
+                                const u64 sq = mul2(b.y, inv);
+                                const u64 s3 = mul2(sq, mul2(inv, inv));
+                                X[p] = fma2(dx, s3, X[p]);
+                                Y[p] = fma2(dy, s3, Y[p]);
+                                Z[p] = fma2(dz, s3, Z[p]);
+                                if (WANT_V) W[p] = add2(W[p], sq);
+                            }
+                        }
+                    };
+                    for (int h = 0; h < SY_DTILE / SY_THREADS; ++h) {
+                        const int seg = sb / SY_THREADS + h;
+                        switch (seg >> 1) {
+                        case 0: segment(h * SY_THREADS, seg & 1, SyInt<0>{}); break;
+                        case 1: segment(h * SY_THREADS, seg & 1, SyInt<1>{}); break;
+                        case 2: segment(h * SY_THREADS, seg & 1, SyInt<2>{}); break;
+                        default: segment(h * SY_THREADS, seg & 1, SyInt<3>{}); break;
                         }
                     }
-                    if (WANT_V) {
 #pragma unroll
-                        for (int k = 0; k < SY_NI; ++k) part[k][3] *= SY_VS;
-                    }
-#pragma unroll
-                    for (int k = 0; k < SY_NI; ++k)
+                    for (int p = 0; p < SY_NP; ++p) {
+                        float a[4], b[4];
+                        upk(X[p], a[0], b[0]); upk(Y[p], a[1], b[1]); upk(Z[p], a[2], b[2]);
+                        if (WANT_V) { upk(W[p], a[3], b[3]); a[3] *= SY_VS; b[3] *= SY_VS; }
 #pragma unroll
                         for (int c = 0; c < NC; ++c) {
-                            float sv = s_S[c][k][tid], cv = s_C[c][k][tid];
-                            two_sum_acc(sv, cv, part[k][c]);
-                            s_S[c][k][tid] = sv;
-                            s_C[c][k][tid] = cv;
+                            float sv = s_S[c][2 * p][tid], cv = s_C[c][2 * p][tid];
+                            two_sum_acc(sv, cv, a[c]);
+                            s_S[c][2 * p][tid] = sv;
+                            s_C[c][2 * p][tid] = cv;
+                            sv = s_S[c][2 * p + 1][tid]; cv = s_C[c][2 * p + 1][tid];
+                            two_sum_acc(sv, cv, b[c]);
+                            s_S[c][2 * p + 1][tid] = sv;
+                            s_C[c][2 * p + 1][tid] = cv;
                         }
+                    }
                 }
                 continue;
             }
@@ -1899,10 +1922,11 @@ int obem_sym_grid(int device)
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
     void (*ks[])(FieldLaunch, float *, float *, int *, const float *, SymBatch, SymPass) = {
         nbsym_kernel<true, false>, nbsym_kernel<false, false>, nbsym_kernel<false, true>,
+        nbsym_kernel<false, true, 1>, nbsym_kernel<false, true, 4>,
         nbsym_kernel<true, false, SY_CH_SMALL>, nbsym_kernel<false, false, SY_CH_SMALL>,
         nbsym_kernel<true, false, SY_CH_MID>, nbsym_kernel<false, false, SY_CH_MID>};
-    const size_t sm[] = {sym_smem(4), sym_smem(3), sym_smem(3), sym_smem(4), sym_smem(3), sym_smem(4), sym_smem(3)};
-    for (int q = 0; q < 7; ++q) {
+    const size_t sm[] = {sym_smem(4), sym_smem(3), sym_smem(3), sym_smem(3), sym_smem(3), sym_smem(4), sym_smem(3), sym_smem(4), sym_smem(3)};
+    for (int q = 0; q < 9; ++q) {
         if (cudaFuncSetAttribute(ks[q], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm[q]) != cudaSuccess)
             return 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ks[q], SY_THREADS, sm[q]) != cudaSuccess) return 0;
@@ -2122,9 +2146,20 @@ int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets,
 // ====================================================================
 // Batch of chambers.
 
-size_t obem_sym_sizes(int capacity, size_t *ipart_floats)
+// Items per work unit of a batch whose chambers' tile pairs are `items` in all:
+// single items while they are few blocks' worth each (the longest unit then
+// decides: 64 chambers of up to 30,000 charges, 2,700 items, 3.9 ms in units of
+// 16), larger units where their target-side sums (32 KB each) would add up.
+int obem_sym_batch_ch(long long items) { return items <= 16384 ? 1 : items <= 65536 ? 4 : SY_CH; }
+long long obem_sym_items(int capacity)
 {
-    *ipart_floats = obem_sym_ipart_floats(capacity);
+    const SymGeom g = sym_geom(capacity);
+    return (long long)g.n * (g.hmax + 1);
+}
+size_t obem_sym_sizes(int capacity, int ch, size_t *ipart_floats)
+{
+    const SymGeom g = sym_geom(capacity);
+    *ipart_floats = (size_t)g.n * ((g.hmax + ch) / ch) * 8 * SY_T;
     return obem_sym_jpart_floats(capacity);
 }
 
@@ -2213,18 +2248,25 @@ int obem_launch_field_batch(obem_ctx *ctx, const FieldBatch &F, const float4 *po
         sym_part_scatter_kernel<<<nsb, SP_BLOCK, 0, s>>>(pos_q, pos_q, 0, NULL, F.sym, F.bcnt, F.sym.negtot, F.sorted,
                                                         F.perm);
         sym_tileq_kernel<<<nsb, 256, 0, s>>>(F.sorted, 0, NULL, F.sym, F.tileq);
-        sym_units_kernel<<<1, 1024, 0, s>>>(F.sym);
+        if (F.ch == 1) sym_units_kernel<1><<<1, 1024, 0, s>>>(F.sym);
+        else if (F.ch == 4) sym_units_kernel<4><<<1, 1024, 0, s>>>(F.sym);
+        else sym_units_kernel<SY_CH><<<1, 1024, 0, s>>>(F.sym);
         OBEM_LAUNCH(ctx);
         FieldLaunch Ls = L;
         Ls.targets = F.sorted;
         Ls.sources = F.sorted;
         Ls.eps2 = L.eps2 * SY_QS;                        // the sorted copy's positions are x 2^40
         OBEM_CUDA(ctx, cudaMemsetAsync(F.counter, 0, sizeof(int), s));
-        nbsym_kernel<false, true><<<F.sym_grid, SY_THREADS, sym_smem(3), s>>>(Ls, F.jpart, F.ipart, F.counter, F.tileq,
-                                                                       F.sym, SymPass{0, 0, 0, 1, 1, NULL});
+        const SymPass PS{0, 0, 0, 1, 1, NULL};
+        typedef void (*SymK)(FieldLaunch, float *, float *, int *, const float *, SymBatch, SymPass);
+        typedef void (*FoldK)(FieldLaunch, const float *, const float *, int, const int32_t *, SymBatch, SymPass);
+        const SymK kern = F.ch == 1 ? nbsym_kernel<false, true, 1> : F.ch == 4 ? nbsym_kernel<false, true, 4>
+                                                                               : nbsym_kernel<false, true>;
+        const FoldK fold = F.ch == 1 ? nbsym_fold_kernel<false, 1> : F.ch == 4 ? nbsym_fold_kernel<false, 4>
+                                                                               : nbsym_fold_kernel<false>;
+        kern<<<F.sym_grid, SY_THREADS, sym_smem(3), s>>>(Ls, F.jpart, F.ipart, F.counter, F.tileq, F.sym, PS);
         OBEM_LAUNCH(ctx);
-        nbsym_fold_kernel<false><<<F.slots / 256, 256, 0, s>>>(L, F.jpart, F.ipart, F.cells ? 1 : 0, F.perm, F.sym,
-                                                               SymPass{0, 0, 0, 1, 1, NULL});
+        fold<<<F.slots / 256, 256, 0, s>>>(L, F.jpart, F.ipart, F.cells ? 1 : 0, F.perm, F.sym, PS);
         OBEM_LAUNCH(ctx);
     }
     if (!F.cells && !F.charges) {

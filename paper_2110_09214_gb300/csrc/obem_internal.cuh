@@ -381,15 +381,19 @@ struct FieldBatch {
     float *tileq;
     int *counter;
     int sym_grid;
+    int ch;                      // items per work unit of the all-pairs kernel
 };
 int obem_launch_field_batch(obem_ctx *ctx, const FieldBatch &F, const float4 *pos_q, float4 *E_out,
                             cudaStream_t s);
+#define OBEM_DIRECT_WIDE 4096     // direct kernels: targets from which a block takes 8 of them
 // direct.cu: the cell field (E_out = e_ext + cells) and the charges' field of
 // few targets; SB: the batch of chambers, or NULL; slots: capacity of the targets
 int obem_launch_direct_cells(obem_ctx *ctx, const FieldLaunch &L, const SymBatch *SB, int slots, cudaStream_t s);
 int obem_launch_direct_pairs(obem_ctx *ctx, const FieldLaunch &L, const SymBatch *SB, int slots, int add,
                              cudaStream_t s);
-size_t obem_sym_sizes(int capacity, size_t *ipart_floats);
+int obem_sym_batch_ch(long long items);
+long long obem_sym_items(int capacity);
+size_t obem_sym_sizes(int capacity, int ch, size_t *ipart_floats);
 int obem_cell_layout(const double *tri, const int32_t *kind, int np, float4 *ca, float4 *g0, float4 *g1,
                      float4 *g2, float4 *nr, float4 *cl);
 void obem_energy_lut(const float *grid, int n, uint32_t *lut);
