@@ -227,6 +227,7 @@ __global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
     __shared__ float4 s_g[T];
     __shared__ float4 s_b[BW_NBARY];
     __shared__ uint32_t s_q[BW_NW][32];
+    __shared__ int s_nq[BW_NW];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int base = blockIdx.x * T;
     const int n = min(T, B.nt - base);
@@ -273,19 +274,14 @@ __global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
     }
     // cells
     int nq = 0;
-    auto flush = [&](int m) {
-        __syncwarp();
-        if (lane < m) {
-            const uint32_t e = s_q[warp][lane];
-            const int j = (int)(e >> 3), t = (int)(e & 7u);
-            const float4 x = sh.t[t], g = s_g[t];
-            double J[9], F[3];
-            tri_closed_jac(B.panels.v64 + 9 * (size_t)j, (double)x.x, (double)x.y, (double)x.z, J, F);
-            const double q = OBEM_KC * (double)B.sigma[j];
-            for (int b = 0; b < 3; ++b)
-                df_put(sh, 4 * t + b, (float)(q * (J[b] * g.x + J[3 + b] * g.y + J[6 + b] * g.z - (double)g.w * F[b])));
-        }
-        __syncwarp();
+    auto closed_pair = [&](uint32_t e) {
+        const int j = (int)(e >> 3), t = (int)(e & 7u);
+        const float4 x = sh.t[t], g = s_g[t];
+        double J[9], F[3];
+        tri_closed_jac(B.panels.v64 + 9 * (size_t)j, (double)x.x, (double)x.y, (double)x.z, J, F);
+        const double q = OBEM_KC * (double)B.sigma[j];
+        for (int b = 0; b < 3; ++b)
+            df_put(sh, 4 * t + b, (float)(q * (J[b] * g.x + J[3 + b] * g.y + J[6 + b] * g.z - (double)g.w * F[b])));
     };
     if (B.sigma) {
         const PanelsDev &P = B.panels;
@@ -353,7 +349,12 @@ __global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
                         const float d2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
                         if (d2 < BJ_112PT * v0.w) {
                             if (lane == 0) s_q[warp][nq] = ((uint32_t)jj << 3) | (uint32_t)t;
-                            if (++nq == 32) { flush(32); nq = 0; }
+                            if (++nq == 32) {
+                                __syncwarp();
+                                closed_pair(s_q[warp][lane]);
+                                __syncwarp();
+                                nq = 0;
+                            }
                             continue;
                         }
                         const float4 v1 = P.g1[jj], v2 = P.g2[jj];
@@ -373,9 +374,16 @@ __global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
             }
             if (++since == DF_FOLD) { df_fold<false>(sh, A, 1.f); since = 0; }
         }
-        if (nq > 0) flush(nq);
     }
     df_fold<false>(sh, A, 1.f);
+    // what is left in the warps' queues, together (in warp order)
+    if (lane == 0) s_nq[warp] = nq;
+    __syncthreads();
+    {
+        int e = tid, w = 0;
+        while (w < BW_NW && e >= s_nq[w]) e -= s_nq[w++];
+        if (w < BW_NW) closed_pair(s_q[w][e]);
+    }
     float s[4 * T], c[4 * T];
 #pragma unroll
     for (int v = 0; v < 4 * T; ++v) { s[v] = sh.S[v][tid]; c[v] = sh.C[v][tid]; }
@@ -486,6 +494,7 @@ __global__ void __launch_bounds__(32 * BR_WARPS) bw_sigma_kernel(BwLaunch B)
     __shared__ float4 s_b[BW_NBARY];
     __shared__ int s_q[BR_WARPS][2][32];                // closed-form queue: target, lane of the cell
     __shared__ float s_v[BR_WARPS][32];
+    __shared__ int s_nq[BR_WARPS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const PanelsDev &P = B.panels;
     const int j0 = blockIdx.x * 32;
@@ -497,22 +506,19 @@ __global__ void __launch_bounds__(32 * BR_WARPS) bw_sigma_kernel(BwLaunch B)
     u64 A = 0ull;
     float S = 0.f, C = 0.f;
     int nq = 0;
-    auto flush = [&](int m) {
-        __syncwarp();
-        if (lane < m) {
-            const int t = s_q[warp][0][lane];
-            const float4 x = B.targets[t], g = B.g[t];
-            double phi, fx, fy, fz;
-            const size_t jc = (size_t)(j0 + s_q[warp][1][lane]);
-            tri_closed_form_g(P.v64 + 9 * jc, P.geo + OBEM_GEO64 * jc, (double)x.x, (double)x.y, (double)x.z, phi, fx, fy,
-                              fz);
-            s_v[warp][lane] =
-                (float)(OBEM_KC * ((double)g.x * fx + (double)g.y * fy + (double)g.z * fz + (double)g.w * phi));
-        }
-        __syncwarp();
+    auto closed_pair = [&](int w, int k) {
+        const int t = s_q[w][0][k];
+        const float4 x = B.targets[t], g = B.g[t];
+        double phi, fx, fy, fz;
+        const size_t jc = (size_t)(j0 + s_q[w][1][k]);
+        tri_closed_form_g(P.v64 + 9 * jc, P.geo + OBEM_GEO64 * jc, (double)x.x, (double)x.y, (double)x.z, phi, fx, fy,
+                          fz);
+        s_v[w][k] = (float)(OBEM_KC * ((double)g.x * fx + (double)g.y * fy + (double)g.z * fz + (double)g.w * phi));
+    };
+    // the warp's m queued pairs, evaluated, to their cells' lanes in order
+    auto take = [&](int m) {
         for (int e = 0; e < m; ++e)
             if (s_q[warp][1][e] == lane) two_sum_acc(S, C, s_v[warp][e]);
-        __syncwarp();
     };
     for (int tb = 0; tb < B.nt; tb += BR_TILE) {
         br_load(B, st, tb);
@@ -566,7 +572,14 @@ __global__ void __launch_bounds__(32 * BR_WARPS) bw_sigma_kernel(BwLaunch B)
                     const float d2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
                     if (d2 < BF_112PT * v0.w) {
                         if (lane == 0) { s_q[warp][0][nq] = t + half; s_q[warp][1][nq] = own; }
-                        if (++nq == 32) { flush(32); nq = 0; }
+                        if (++nq == 32) {
+                            __syncwarp();
+                            closed_pair(warp, lane);
+                            __syncwarp();
+                            take(32);
+                            __syncwarp();
+                            nq = 0;
+                        }
                         continue;
                     }
                     const float4 v1 = P.g1[jj], v2 = P.g2[jj];
@@ -586,7 +599,16 @@ __global__ void __launch_bounds__(32 * BR_WARPS) bw_sigma_kernel(BwLaunch B)
         }
         br_fold(A, S, C);
     }
-    if (nq > 0) flush(nq);
+    // what is left in the warps' queues, together (in warp order)
+    if (lane == 0) s_nq[warp] = nq;
+    __syncthreads();
+    {
+        int e = threadIdx.x, w = 0;
+        while (w < BR_WARPS && e >= s_nq[w]) e -= s_nq[w++];
+        if (w < BR_WARPS) closed_pair(w, e);
+    }
+    __syncthreads();
+    take(nq);
     s_red[0][warp][lane] = S;
     s_red[1][warp][lane] = C;
     __syncthreads();

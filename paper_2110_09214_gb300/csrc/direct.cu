@@ -1,5 +1,5 @@
 // Field at few targets: one launch for the cells and one for the charges, no
-// spatial sort of the targets, no block list.
+// block list; the cells' targets in spatial order from OBEM_DIRECT_WIDE on.
 //
 // The block kernels of field.cu give a thread block 512 neighbouring targets
 // and let it run over all cells (or all charges): at a few thousand targets,
@@ -43,7 +43,7 @@ __device__ __forceinline__ bool df_targets(const FieldLaunch &L, const SymBatch 
 
 // E_out of the block's targets from the threads' slots
 template <bool WANT_V, int NP, int NW>
-__device__ __forceinline__ void df_finish(const FieldLaunch &L, DfShared<NP, NW> &sh, int base, int n, int add)
+__device__ __forceinline__ void df_finish(const FieldLaunch &L, DfShared<NP, NW> &sh, int n, int add)
 {
     constexpr int V = DfShared<NP, NW>::V;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -58,7 +58,7 @@ __device__ __forceinline__ void df_finish(const FieldLaunch &L, DfShared<NP, NW>
         float S = 0.f, C = 0.f;
         for (int w = 0; w < NW; ++w) df_add(S, C, sh.red[0][w][tid], sh.red[1][w][tid]);
         const int k = tid & 3;
-        float *out = reinterpret_cast<float *>(L.E_out + base) + tid;
+        float *out = reinterpret_cast<float *>(L.E_out + sh.ti[tid >> 2]) + k;
         float e0 = k == 0 ? L.e_ext.x : k == 1 ? L.e_ext.y : k == 2 ? L.e_ext.z : 0.f;
         if (add) e0 = *out;
         *out = (k < 3 || WANT_V) ? (float)((double)S + (double)C + (double)e0) : 0.f;
@@ -75,15 +75,29 @@ __device__ __forceinline__ void df_finish(const FieldLaunch &L, DfShared<NP, NW>
 // the warp evaluates them together, a lane per quadrature point (28 points,
 // 112 below 1.5 h), and pairs within h go to a per-warp queue of the FP64
 // closed form, 32 at a time.  All sums are formed in a fixed order.
-template <bool WANT_V, bool BATCH, int NP, int NW>
+// perm: order of the targets (spatial, so that a block's targets are neighbours
+// and share few near cells: 1e4 targets in a GEM of 5952 cells 1592 to 677 us),
+// or NULL.
+// GRP: cells in groups of 32.  A warp takes 32 groups at a time, a lane each
+// tests whether the group is far from the block's targets; the far ones enter
+// as their equivalent charges, a lane per charge of the list of all of them
+// (1.5 points per lane and group, where the cells cost a point and its
+// distances and weights), the others cell by cell: 60,000 targets in a GEM of
+// 59,968 cells 14.8 to 11.6 ms.
+template <bool WANT_V, bool BATCH, bool GRP, int NP, int NW>
 __global__ void __launch_bounds__(32 * NW, NP == 1 ? 2 : 4)
-direct_cells_kernel(FieldLaunch L, SymBatch SB)
+direct_cells_kernel(FieldLaunch L, SymBatch SB, const int32_t *perm, CellGroups G)
 {
     constexpr int T = 2 * NP, TH = 32 * NW;
     __shared__ DfShared<NP, NW> sh;
     __shared__ float4 s_b[DF_NBARY];          // near rules: barycentric offsets of the points, weight
     __shared__ uint32_t s_q[NW][32 + T];      // closed-form queue: cell * 8 + target
     __shared__ u64 s_tp[3][NP];               // target packs
+    __shared__ int s_nq[NW];
+    constexpr int GW = GRP ? NW : 1, GL = GRP ? 32 : 1, GM = GRP ? OBEM_GRP_M : 1;
+    __shared__ float4 s_u[GM], s_c[GW][GL];   // GRP: charges' directions; far groups' centres from target 0, radii
+    __shared__ int s_g[GW][GL];               // and numbers
+    __shared__ u64 s_rp[3][NP];               // target packs from target 0
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned below = (1u << lane) - 1u;
     int base, n, lo, hi, cham;
@@ -95,7 +109,11 @@ direct_cells_kernel(FieldLaunch L, SymBatch SB)
         np = r.y;
     }
     const PanelsDev &P = L.panels;
-    if (tid < T) sh.t[tid] = L.targets[base + min(tid, n - 1)];
+    if (tid < T) {
+        const int i = base + min(tid, n - 1);
+        sh.ti[tid] = !BATCH && perm ? perm[i] : i;
+        sh.t[tid] = L.targets[sh.ti[tid]];
+    }
     for (int k = tid; k < DF_NBARY; k += TH) {
         float3 off;
         float wf;
@@ -111,7 +129,15 @@ direct_cells_kernel(FieldLaunch L, SymBatch SB)
         s_tp[0][tid] = pk(a.x, b.x);
         s_tp[1][tid] = pk(a.y, b.y);
         s_tp[2][tid] = pk(a.z, b.z);
+        if (GRP) {
+            const float4 o = sh.t[0];
+            s_rp[0][tid] = pk(a.x - o.x, b.x - o.x);
+            s_rp[1][tid] = pk(a.y - o.y, b.y - o.y);
+            s_rp[2][tid] = pk(a.z - o.z, b.z - o.z);
+        }
     }
+    if (GRP)
+        for (int k = tid; k < OBEM_GRP_M; k += TH) s_u[k] = G.u[k];
     __syncthreads();
     u64 A[4][NP];
 #pragma unroll
@@ -119,35 +145,46 @@ direct_cells_kernel(FieldLaunch L, SymBatch SB)
 #pragma unroll
         for (int p = 0; p < NP; ++p) A[c][p] = 0ull;
     int nq = 0;                               // queued pairs (warp-uniform, < 32)
-    auto flush = [&](int m) {
-        __syncwarp();
-        if (lane < m) {
-            const uint32_t e = s_q[warp][lane];
-            const int j = (int)(e >> 3), t = (int)(e & 7u);
-            const float4 x = sh.t[t];
-            double phi, Fx, Fy, Fz;
-            if (P.geo)
-                tri_closed_form_g(P.v64 + 9 * (size_t)j, P.geo + (size_t)OBEM_GEO64 * j, (double)x.x, (double)x.y,
-                                  (double)x.z, phi, Fx, Fy, Fz);
-            else
-                tri_closed_form(P.v64 + 9 * (size_t)j, (double)x.x, (double)x.y, (double)x.z, phi, Fx, Fy, Fz);
-            const double kq = OBEM_KC * (double)L.sigma[j];
-            df_put(sh, 4 * t, (float)(kq * Fx));
-            df_put(sh, 4 * t + 1, (float)(kq * Fy));
-            df_put(sh, 4 * t + 2, (float)(kq * Fz));
-            if (WANT_V) df_put(sh, 4 * t + 3, (float)(kq * phi));
+    auto closed_pair = [&](uint32_t e) {
+        const int j = (int)(e >> 3), t = (int)(e & 7u);
+        const float4 x = sh.t[t];
+        double phi, Fx, Fy, Fz;
+        if (P.geo)
+            tri_closed_form_g(P.v64 + 9 * (size_t)j, P.geo + (size_t)OBEM_GEO64 * j, (double)x.x, (double)x.y,
+                              (double)x.z, phi, Fx, Fy, Fz);
+        else
+            tri_closed_form(P.v64 + 9 * (size_t)j, (double)x.x, (double)x.y, (double)x.z, phi, Fx, Fy, Fz);
+        const double kq = OBEM_KC * (double)L.sigma[j];
+        df_put(sh, 4 * t, (float)(kq * Fx));
+        df_put(sh, 4 * t + 1, (float)(kq * Fy));
+        df_put(sh, 4 * t + 2, (float)(kq * Fz));
+        if (WANT_V) df_put(sh, 4 * t + 3, (float)(kq * phi));
+    };
+    u64 D[3][NP], EP[NP];                     // target - centroid, softening of masked pairs
+    auto point = [&](float ox, float oy, float oz, float w) {
+        const u64 OX = pk(ox, ox), OY = pk(oy, oy), OZ = pk(oz, oz), W = pk(w, w);
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const u64 dx = sub2(D[0][p], OX), dy = sub2(D[1][p], OY), dz = sub2(D[2][p], OZ);
+            const u64 r2 = fma2(dz, dz, fma2(dy, dy, fma2(dx, dx, EP[p])));
+            float ra, rb;
+            upk(r2, ra, rb);
+            const u64 inv = pk(rsq(ra), rsq(rb));
+            const u64 s = mul2(W, inv);
+            const u64 s3 = mul2(s, mul2(inv, inv));
+            A[0][p] = fma2(dx, s3, A[0][p]);
+            A[1][p] = fma2(dy, s3, A[1][p]);
+            A[2][p] = fma2(dz, s3, A[2][p]);
+            if (WANT_V) A[3][p] = add2(A[3][p], s);
         }
-        __syncwarp();
     };
     int since = 0;
-    for (int jb = 32 * warp; jb < np; jb += TH) {
-        const bool live = jb + lane < np;
-        const int j = poff + (live ? jb + lane : jb);
+    // the warp's 32 cells (a lane each; live: the lane has one)
+    auto cells32 = [&](int j, bool live) {
         const float4 ca = P.c_a[j], cl = P.c_lo[j], g0 = P.g0_h[j], g1 = P.g1[j], g2 = P.g2[j];
         const float q = live ? ca.w * L.sigma[j] : 0.f;
         const float h2 = g0.w;
         // target - centroid of every pair (exact for nearby targets)
-        u64 D[3][NP], EP[NP];
         unsigned nm = 0u;                     // near targets of this lane's cell
         float dmin = 3e38f;
 #pragma unroll
@@ -172,23 +209,6 @@ direct_cells_kernel(FieldLaunch L, SymBatch SB)
         const float sa = t1 ? 0.f : t3 ? 0.5f : t4 ? 0.4f : t6 ? -0.33784547274789500f : D7_T1;
         const float wb = t4 ? 0.f : t6 ? 0.109951743655322f : D7_W2;
         const float sb = t4 ? 0.f : t6 ? 0.72527135947068800f : D7_T2;
-        auto point = [&](float ox, float oy, float oz, float w) {
-            const u64 OX = pk(ox, ox), OY = pk(oy, oy), OZ = pk(oz, oz), W = pk(w, w);
-#pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                const u64 dx = sub2(D[0][p], OX), dy = sub2(D[1][p], OY), dz = sub2(D[2][p], OZ);
-                const u64 r2 = fma2(dz, dz, fma2(dy, dy, fma2(dx, dx, EP[p])));
-                float ra, rb;
-                upk(r2, ra, rb);
-                const u64 inv = pk(rsq(ra), rsq(rb));
-                const u64 s = mul2(W, inv);
-                const u64 s3 = mul2(s, mul2(inv, inv));
-                A[0][p] = fma2(dx, s3, A[0][p]);
-                A[1][p] = fma2(dy, s3, A[1][p]);
-                A[2][p] = fma2(dz, s3, A[2][p]);
-                if (WANT_V) A[3][p] = add2(A[3][p], s);
-            }
-        };
         if (__any_sync(0xffffffffu, w0 != 0.f)) point(0.f, 0.f, 0.f, q * w0);
         if (__any_sync(0xffffffffu, wa != 0.f)) {
             const float w = q * wa;
@@ -206,7 +226,7 @@ direct_cells_kernel(FieldLaunch L, SymBatch SB)
         unsigned near = __ballot_sync(0xffffffffu, nm != 0u);
         if (near) since = DF_FOLD - 1;                                  // fold their terms at once
         while (near) {
-            const int src = __ffs(near) - 1, jj = poff + jb + src;      // warp-uniform
+            const int src = __ffs(near) - 1, jj = __shfl_sync(0xffffffffu, j, src);      // warp-uniform
             near &= near - 1;
             const unsigned m = __shfl_sync(0xffffffffu, nm, src);
             const float4 c = P.c_a[jj], l = P.c_lo[jj], v0 = P.g0_h[jj], v1 = P.g1[jj], v2 = P.g2[jj];
@@ -227,7 +247,9 @@ direct_cells_kernel(FieldLaunch L, SymBatch SB)
                 if ((closed >> lane) & 1u) s_q[warp][nq + __popc(closed & below)] = ((uint32_t)jj << 3) | (uint32_t)lane;
                 nq += __popc(closed);
                 if (nq >= 32) {
-                    flush(32);
+                    __syncwarp();
+                    closed_pair(s_q[warp][lane]);
+                    __syncwarp();
                     nq -= 32;
                     if (lane < nq) s_q[warp][lane] = s_q[warp][32 + lane];
                     __syncwarp();
@@ -249,11 +271,87 @@ direct_cells_kernel(FieldLaunch L, SymBatch SB)
             df_fold<WANT_V>(sh, A, 1.f);
             since = 0;
         }
+    };
+    if (!GRP) {
+        for (int jb = 32 * warp; jb < np; jb += TH) {
+            const bool live = jb + lane < np;
+            cells32(poff + (live ? jb + lane : jb), live);
+        }
+    } else {
+        float blo[3] = {3e38f, 3e38f, 3e38f}, bhi[3] = {-3e38f, -3e38f, -3e38f};     // box of the targets
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            const float4 x = sh.t[t];
+            blo[0] = fminf(blo[0], x.x); blo[1] = fminf(blo[1], x.y); blo[2] = fminf(blo[2], x.z);
+            bhi[0] = fmaxf(bhi[0], x.x); bhi[1] = fmaxf(bhi[1], x.y); bhi[2] = fmaxf(bhi[2], x.z);
+        }
+        const float4 o = sh.t[0];
+        // group (32 i + lane) NW + warp: neighbours, which are near together, on different warps
+        for (int gb = 0; gb * NW < G.ng; gb += 32) {
+            const int g = (gb + lane) * NW + warp;
+            const bool have = g < G.ng;
+            const float4 cr = G.cr[have ? g : 0];
+            const float gx = fmaxf(fmaxf(blo[0] - cr.x, cr.x - bhi[0]), 0.f),
+                        gy = fmaxf(fmaxf(blo[1] - cr.y, cr.y - bhi[1]), 0.f),
+                        gz = fmaxf(fmaxf(blo[2] - cr.z, cr.z - bhi[2]), 0.f);
+            const bool far = gx * gx + gy * gy + gz * gz >= OBEM_GRP_THETA2 * (cr.w * cr.w);
+            const unsigned fm = __ballot_sync(0xffffffffu, have && far);
+            unsigned nm = __ballot_sync(0xffffffffu, have && !far);
+            __syncwarp();
+            if (have && far) {
+                const int k = __popc(fm & below);
+                s_c[warp][k] = make_float4(cr.x - o.x, cr.y - o.y, cr.z - o.z, cr.w);
+                s_g[warp][k] = g;
+            }
+            __syncwarp();
+            const int nc = __popc(fm) * OBEM_GRP_M;
+            for (int e0 = 0; e0 < nc; e0 += 32) {
+                const int e = e0 + lane;
+                const bool in = e < nc;
+                const int gi = in ? e / OBEM_GRP_M : 0, k = in ? e - gi * OBEM_GRP_M : 0;
+                const float4 c = s_c[warp][gi], u = s_u[k];
+                const float w = in ? G.q[(size_t)s_g[warp][gi] * OBEM_GRP_M + k] : 0.f;
+                const float sx = fmaf(c.w, u.x, c.x), sy = fmaf(c.w, u.y, c.y), sz = fmaf(c.w, u.z, c.z);
+                const u64 SX = pk(sx, sx), SY = pk(sy, sy), SZ = pk(sz, sz), W = pk(w, w);
+#pragma unroll
+                for (int p = 0; p < NP; ++p) {
+                    const u64 dx = sub2(s_rp[0][p], SX), dy = sub2(s_rp[1][p], SY), dz = sub2(s_rp[2][p], SZ);
+                    const u64 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
+                    float ra, rb;
+                    upk(r2, ra, rb);
+                    const u64 inv = pk(rsq(ra), rsq(rb));
+                    const u64 sw = mul2(W, inv);
+                    const u64 s3 = mul2(sw, mul2(inv, inv));
+                    A[0][p] = fma2(dx, s3, A[0][p]);
+                    A[1][p] = fma2(dy, s3, A[1][p]);
+                    A[2][p] = fma2(dz, s3, A[2][p]);
+                    if (WANT_V) A[3][p] = add2(A[3][p], sw);
+                }
+                if (++since == DF_FOLD) {
+                    df_fold<WANT_V>(sh, A, 1.f);
+                    since = 0;
+                }
+            }
+            while (nm) {
+                const int slot = 32 * ((gb + __ffs(nm) - 1) * NW + warp);         // warp-uniform
+                nm &= nm - 1;
+                const bool live = slot + lane < np;
+                cells32(G.perm[live ? slot + lane : slot], live);
+            }
+        }
     }
-    if (nq > 0) flush(nq);
     df_fold<WANT_V>(sh, A, 1.f);
+    // what is left in the warps' queues, together (in warp order): a warp each
+    // for its few would cost as many FP64 instructions as for 32
+    if (lane == 0) s_nq[warp] = nq;
     __syncthreads();
-    df_finish<WANT_V>(L, sh, base, n, 0);
+    {
+        int e = tid, w = 0;
+        while (w < NW && e >= s_nq[w]) e -= s_nq[w++];
+        if (w < NW) closed_pair(s_q[w][e]);
+    }
+    __syncthreads();
+    df_finish<WANT_V>(L, sh, n, 0);
 }
 
 // ---------------------------------------------------------------- charges
@@ -268,7 +366,10 @@ direct_pairs_kernel(FieldLaunch L, SymBatch SB, int add)
     int base, n, s0, s1, cham;
     if (!df_targets<BATCH, T>(L, SB, base, n, s0, s1, cham)) return;
     if (!BATCH) s1 = L.ns_dev ? *L.ns_dev : L.ns;
-    if (tid < T) sh.t[tid] = L.targets[base + min(tid, n - 1)];
+    if (tid < T) {
+        sh.ti[tid] = base + min(tid, n - 1);
+        sh.t[tid] = L.targets[sh.ti[tid]];
+    }
 #pragma unroll
     for (int v = 0; v < 4 * T; ++v) { sh.S[v][tid] = 0.f; sh.C[v][tid] = 0.f; }
     __syncthreads();
@@ -301,27 +402,38 @@ direct_pairs_kernel(FieldLaunch L, SymBatch SB, int add)
     }
     df_fold<WANT_V>(sh, A, DF_VS);
     __syncthreads();
-    df_finish<WANT_V>(L, sh, base, n, add);
+    df_finish<WANT_V>(L, sh, n, add);
 }
 
 // Targets per block: 8 (four packs, 4 warps), 2 (8 warps) for fewer than
 // OBEM_DIRECT_WIDE targets: 2000 targets are 250 blocks of 8, hardly a warp per
 // scheduler, and the cells of a block of 2 cost one iteration per 256.
 
-int obem_launch_direct_cells(obem_ctx *ctx, const FieldLaunch &L, const SymBatch *SB, int slots, cudaStream_t s)
+int obem_launch_direct_cells(obem_ctx *ctx, const FieldLaunch &L, const SymBatch *SB, int slots, const int32_t *perm,
+                             const CellGroups *GR, cudaStream_t s)
 {
     SymBatch none;
     memset(&none, 0, sizeof none);
     const SymBatch &B = SB ? *SB : none;
-    if (slots >= OBEM_DIRECT_WIDE || SB) {
+    CellGroups G;
+    memset(&G, 0, sizeof G);
+    if (GR) G = *GR;
+    if (SB) {
+        direct_cells_kernel<false, true, false, 4, 4><<<(slots + 7) / 8, 128, 0, s>>>(L, B, NULL, G);
+    } else if (slots >= OBEM_DIRECT_WIDE) {
         const int g = (slots + 7) / 8;
-        if (SB) direct_cells_kernel<false, true, 4, 4><<<g, 128, 0, s>>>(L, B);
-        else if (L.want_v) direct_cells_kernel<true, false, 4, 4><<<g, 128, 0, s>>>(L, B);
-        else direct_cells_kernel<false, false, 4, 4><<<g, 128, 0, s>>>(L, B);
+        if (GR) {
+            if (L.want_v) direct_cells_kernel<true, false, true, 4, 4><<<g, 128, 0, s>>>(L, B, perm, G);
+            else direct_cells_kernel<false, false, true, 4, 4><<<g, 128, 0, s>>>(L, B, perm, G);
+        } else if (L.want_v) {
+            direct_cells_kernel<true, false, false, 4, 4><<<g, 128, 0, s>>>(L, B, perm, G);
+        } else {
+            direct_cells_kernel<false, false, false, 4, 4><<<g, 128, 0, s>>>(L, B, perm, G);
+        }
     } else {
         const int g = (slots + 1) / 2;
-        if (L.want_v) direct_cells_kernel<true, false, 1, 8><<<g, 256, 0, s>>>(L, B);
-        else direct_cells_kernel<false, false, 1, 8><<<g, 256, 0, s>>>(L, B);
+        if (L.want_v) direct_cells_kernel<true, false, false, 1, 8><<<g, 256, 0, s>>>(L, B, perm, G);
+        else direct_cells_kernel<false, false, false, 1, 8><<<g, 256, 0, s>>>(L, B, perm, G);
     }
     OBEM_LAUNCH(ctx);
     return OBEM_OK;

@@ -4,7 +4,7 @@
 #pragma once
 #include "field_common.cuh"
 
-#define DF_FOLD 8                   // lane iterations summed in FP32 between compensated folds
+#define DF_FOLD 16                  // lane iterations summed in FP32 between compensated folds
 #define DF_SELF 3.0e38f             // squared distance (x 2^80) given to a target's own charge
 // Charges: positions x 2^40 and k_C q x 2^80 (exact), as in the symmetric
 // kernel, so that close pairs stay finite; the potential carries 2^40
@@ -53,6 +53,7 @@ struct DfShared {
     static constexpr int T = 2 * NP, V = 4 * T, TH = 32 * NW;
     float S[V][TH], C[V][TH];
     float4 t[T];                    // the targets
+    int ti[T];                      // and their indices in E_out
     float red[2][NW][V];
 };
 template <int NP, int NW>

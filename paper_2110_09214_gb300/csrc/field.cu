@@ -253,6 +253,64 @@ static void binsort(const uint32_t *code_in, uint32_t *code, int32_t *perm, uint
     }
 }
 
+// The same order for at most SO_MAX targets in one block: codes and the three
+// radix passes in shared memory (a key is the code above the index), each warp a
+// contiguous stretch of the keys.  Latency-bound, about 10 us for 1e4 targets
+// against 11 launches.
+#define SO_MAX 16384
+#define SO_PER (SO_MAX / 1024)
+#define SO_SMEM (2 * SO_MAX * sizeof(uint32_t) + 32 * RS_RADIX * sizeof(int32_t))
+__global__ void __launch_bounds__(1024) sort_one_kernel(FieldLaunch L, float3 lo, float3 scale, int32_t *perm)
+{
+    extern __shared__ uint32_t so_sm[];
+    __shared__ int32_t s_warp[32];
+    int32_t *cnt = (int32_t *)(so_sm + 2 * SO_MAX);         // [digit][warp]: counts, then first positions
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned below = (1u << lane) - 1u;
+    const int n = L.nt_dev ? *L.nt_dev : L.nt;
+    const int rounds = (n + 1023) / 1024, first = warp * 32 * rounds;      // this warp's stretch
+    for (int i = tid; i < n; i += 1024) so_sm[i] = (bin_code(L.targets[i], lo, scale) << 14) | (uint32_t)i;
+    for (int pass = 0; pass < 3; ++pass) {
+        const uint32_t *in = so_sm + (pass & 1) * SO_MAX;
+        uint32_t *out = so_sm + ((pass & 1) ^ 1) * SO_MAX;
+        __syncthreads();
+        for (int d = lane; d < RS_RADIX; d += 32) cnt[d * 32 + warp] = 0;
+        __syncwarp();
+        uint32_t key[SO_PER];
+        int rank[SO_PER];
+#pragma unroll
+        for (int r = 0; r < SO_PER; ++r) {
+            const int i = first + 32 * r + lane;
+            const bool live = r < rounds && i < n;
+            if (r < rounds) {                              // uniform
+                key[r] = live ? in[i] : 0u;
+                const int dg = live ? (int)(key[r] >> (14 + 6 * pass)) & (RS_RADIX - 1) : RS_RADIX;
+                const unsigned peers = __match_any_sync(0xffffffffu, dg);
+                const int before = live ? cnt[dg * 32 + warp] : 0;
+                __syncwarp();
+                rank[r] = before + __popc(peers & below);
+                if (live && (peers & below) == 0u) cnt[dg * 32 + warp] = before + __popc(peers);
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+        // exclusive scan over (digit, warp): 2048 counts, two per thread
+        const int c0 = cnt[2 * tid], c1 = cnt[2 * tid + 1];
+        const int e = block_scan_1024(c0 + c1, s_warp) - c0 - c1;
+        cnt[2 * tid] = e;
+        cnt[2 * tid + 1] = e + c0;
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < SO_PER; ++r) {
+            const int i = first + 32 * r + lane;
+            if (r < rounds && i < n)
+                out[cnt[((int)(key[r] >> (14 + 6 * pass)) & (RS_RADIX - 1)) * 32 + warp] + rank[r]] = key[r];
+        }
+    }
+    __syncthreads();
+    for (int i = tid; i < n; i += 1024) perm[i] = (int32_t)(so_sm[SO_MAX + i] & (SO_MAX - 1));
+}
+
 // Spatial order of n points for a pass that runs over the cells outermost
 // (the influence of charges on the cells): the Morton bins of the cell box,
 // the stable radix sort and the blocks of at most CT_BLOCK_N points inside a
@@ -1925,6 +1983,8 @@ int obem_sym_grid(int device)
         nbsym_kernel<false, true, 1>, nbsym_kernel<false, true, 4>,
         nbsym_kernel<true, false, SY_CH_SMALL>, nbsym_kernel<false, false, SY_CH_SMALL>,
         nbsym_kernel<true, false, SY_CH_MID>, nbsym_kernel<false, false, SY_CH_MID>};
+    if (cudaFuncSetAttribute(sort_one_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SO_SMEM) != cudaSuccess)
+        return 0;
     const size_t sm[] = {sym_smem(4), sym_smem(3), sym_smem(3), sym_smem(3), sym_smem(3), sym_smem(4), sym_smem(3), sym_smem(4), sym_smem(3)};
     for (int q = 0; q < 9; ++q) {
         if (cudaFuncSetAttribute(ks[q], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm[q]) != cudaSuccess)
@@ -1952,19 +2012,48 @@ __global__ void const_field_kernel(FieldLaunch L)
     if (i < nt) L.E_out[i] = make_float4(L.e_ext.x, L.e_ext.y, L.e_ext.z, 0.f);
 }
 
-// Which kernels evaluate a set of targets (by its capacity: the live count is
-// on the device).  Cells: the direct kernel up to about 1e5 targets, twice that
-// for a mesh of 49k cells and more, where the few blocks of the block kernels
-// run longer: measured block / direct (ms) at 60k and 200k targets, plates of
-// 1024 cells 2.9 / 1.9 and 5.0 / 6.3, plates of 4096 2.9 / 1.7 and 5.3 / 5.4,
-// GEM of 5952 9.8 / 7.2 and 15.7 / 23.2, GEM of 59,968 in groups 40.7 / 13.3
-// and 51.4 / 43.5.
-static bool direct_cells_rule(int targets, int cells)
+// The targets' spatial order into L.perm (Morton codes of the context's cell
+// box, stable radix sort) and, with `blocks`, the block list (L.blocks,
+// L.nblocks).
+static int sort_targets(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets, bool blocks, cudaStream_t s)
 {
-    return targets <= 98304 + 2 * (cells < 49152 ? cells : 49152);
+    float3 lo = make_float3(ctx->bbox_lo[0], ctx->bbox_lo[1], ctx->bbox_lo[2]);
+    float3 sc;
+    sc.x = (float)OBEM_BINS_PER_AXIS / fmaxf(ctx->bbox_hi[0] - ctx->bbox_lo[0], 1e-30f);
+    sc.y = (float)OBEM_BINS_PER_AXIS / fmaxf(ctx->bbox_hi[1] - ctx->bbox_lo[1], 1e-30f);
+    sc.z = (float)OBEM_BINS_PER_AXIS / fmaxf(ctx->bbox_hi[2] - ctx->bbox_lo[2], 1e-30f);
+    if (!blocks && capacity_targets <= SO_MAX) {
+        sort_one_kernel<<<1, 1024, SO_SMEM, s>>>(L, lo, sc, (int32_t *)L.perm);
+        OBEM_LAUNCH(ctx);
+        if (L.events) ctx->launches++;
+        return OBEM_OK;
+    }
+    OBEM_CUDA(ctx, cudaMemsetAsync(ctx->s_hist, 0, sizeof(int32_t) * OBEM_NSUPER, s));
+    const int nb = (capacity_targets + 255) / 256;
+    bin_count_kernel<<<nb, 256, 0, s>>>(L, lo, sc, ctx->s_code, ctx->s_hist);
+    if (blocks) block_list_kernel<<<1, 1024, 0, s>>>(ctx->s_hist, (int2 *)L.blocks, (int32_t *)L.nblocks);
+    binsort(ctx->s_code, ctx->s_code, (int32_t *)L.perm, ctx->s_tk, ctx->s_tv, ctx->s_rh, L.nt, L.nt_dev,
+            capacity_targets, s);
+    OBEM_LAUNCH(ctx);
+    if (L.events) ctx->launches += blocks ? 11 : 10;
+    return OBEM_OK;
 }
-// Charges at themselves: the symmetric kernel takes over between 16,000
-// (558 us, direct 200 us) and 32,000 charges (657 and 714 us).  Charges at
+
+// Which kernels evaluate a set of targets (by its capacity: the live count is
+// on the device).  Cells: the direct kernel up to 2e5 targets, 4.6e5 for meshes
+// of 5000 cells and more, where the few blocks of the block kernels run long,
+// 7.9e5 for many cells in groups: measured block / direct (ms) at 2e5, 4e5 (6e5)
+// and 1e6 targets, plates of 1024 cells (spread out) 12.1 / 4.1 and 23.1 / 19.6
+// at 2e5 and 1e6, plates of 4096 (a cloud) 5.1 / 5.0 and 16.6 / 24.5, in groups
+// GEM of 5952 14.1 / 9.4, 19.4 / 18.2 and 36.7 / 44.8, GEM of 15,888 26.4 / 15.0,
+// 33.3 / 29.1 and 60.4 / 71.4, GEM of 59,968 52.6 / 25.6, 63.8 / 49.1, (80.0 /
+// 72.6) and 111 / 119.
+static bool direct_cells_rule(int targets, int cells, bool grouped)
+{
+    return targets <= (cells < 5000 ? 196608 : grouped && cells >= 32768 ? 786432 : 458752);
+}
+// Charges at themselves: the symmetric kernel takes over at 24,000 charges
+// (356 us, direct 355 us; 16,000: 348 and 173, 32,000: 442 and 627).  Charges at
 // other points: the one-sided kernel from 64,000 points on (20,000 charges:
 // 967 and 875 us at 64,000, 1438 and 1733 us at 128,000), with few charges,
 // whose tiles it reads once per 512 points, from 32,000 (1000 charges: 55 and
@@ -1981,27 +2070,28 @@ int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets,
     const bool cells = L.sigma != NULL && L.panels.np > 0;
     const bool charges = L.sources != NULL;
     const bool add = cells || L.add_init;      // E_out holds a field the all-pairs sum adds to
-    const bool direct_cells = cells && !L.counters && direct_cells_rule(capacity_targets, L.panels.np);
+    // far cells in groups: the context's own cells, one set of targets
+    const bool grouped = ctx->ngrp > 0 && L.panels.c_a == ctx->d_c_a && !L.block_cham;
+    const bool direct_cells = cells && !L.counters && direct_cells_rule(capacity_targets, L.panels.np, grouped);
     if (direct_cells) {
         if (L.events) { cudaEventRecord(L.events[4], s); cudaEventRecord(L.events[5], s); ctx->launches++; }
-        const int rc = obem_launch_direct_cells(ctx, L, NULL, capacity_targets, s);
+        // in spatial order from OBEM_DIRECT_WIDE targets on (blocks of 8): the sort
+        // takes about 10 us, the unordered blocks of a spread-out set or a GEM
+        // twice the time
+        const bool sorted = L.perm && capacity_targets >= OBEM_DIRECT_WIDE;
+        int rc = sorted ? sort_targets(ctx, L, capacity_targets, false, s) : OBEM_OK;
+        CellGroups G;
+        const bool gr = grouped && capacity_targets >= OBEM_DIRECT_GROUPS;
+        int fitted = 0;
+        if (rc == OBEM_OK && gr) rc = obem_cell_groups_fit(ctx, L.sigma, s, &G, &fitted);
+        if (L.events) ctx->launches += fitted;
+        if (rc == OBEM_OK)
+            rc = obem_launch_direct_cells(ctx, L, NULL, capacity_targets, sorted ? L.perm : NULL, gr ? &G : NULL, s);
         if (rc != OBEM_OK) return rc;
     } else if (cells) {
         if (L.perm) {
-            // spatial order of the targets for the cell kernel
-            float3 lo = make_float3(ctx->bbox_lo[0], ctx->bbox_lo[1], ctx->bbox_lo[2]);
-            float3 sc;
-            sc.x = (float)OBEM_BINS_PER_AXIS / fmaxf(ctx->bbox_hi[0] - ctx->bbox_lo[0], 1e-30f);
-            sc.y = (float)OBEM_BINS_PER_AXIS / fmaxf(ctx->bbox_hi[1] - ctx->bbox_lo[1], 1e-30f);
-            sc.z = (float)OBEM_BINS_PER_AXIS / fmaxf(ctx->bbox_hi[2] - ctx->bbox_lo[2], 1e-30f);
-            OBEM_CUDA(ctx, cudaMemsetAsync(ctx->s_hist, 0, sizeof(int32_t) * OBEM_NSUPER, s));
-            const int nb = (capacity_targets + 255) / 256;
-            bin_count_kernel<<<nb, 256, 0, s>>>(L, lo, sc, ctx->s_code, ctx->s_hist);
-            block_list_kernel<<<1, 1024, 0, s>>>(ctx->s_hist, (int2 *)L.blocks, (int32_t *)L.nblocks);
-            binsort(ctx->s_code, ctx->s_code, (int32_t *)L.perm, ctx->s_tk, ctx->s_tv, ctx->s_rh, L.nt, L.nt_dev,
-                    capacity_targets, s);
-            OBEM_LAUNCH(ctx);
-            if (L.events) ctx->launches += 11;
+            const int rc = sort_targets(ctx, L, capacity_targets, true, s);
+            if (rc != OBEM_OK) return rc;
         }
         const int nsuper = capacity_targets < OBEM_NSUPER ? capacity_targets : OBEM_NSUPER;
         dim3 cgrid((capacity_targets + CT_BLOCK - 1) / CT_BLOCK + (L.blocks ? nsuper : 0));
@@ -2014,8 +2104,6 @@ int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets,
             else { near_closed_kernel<false, false><<<cgrid, CT_THREADS, 0, s>>>(L); near_quad_kernel<false, false><<<cgrid, CT_THREADS, 0, s>>>(L); }
         }
         if (L.events) cudaEventRecord(L.events[5], s);
-        // far cells in groups: the context's own cells, one set of targets
-        const bool grouped = ctx->ngrp > 0 && L.panels.c_a == ctx->d_c_a && !L.block_cham;
         if (grouped) {
             CellGroups G;
             int fitted = 0;
@@ -2229,7 +2317,7 @@ int obem_launch_field_batch(obem_ctx *ctx, const FieldBatch &F, const float4 *po
         L.block_cham = F.block_cham;
         L.cham_pan = F.cham_pan;
         if (F.slots <= BT_DIRECT_SLOTS) {
-            const int rc = obem_launch_direct_cells(ctx, L, &F.sym, F.slots, s);
+            const int rc = obem_launch_direct_cells(ctx, L, &F.sym, F.slots, NULL, NULL, s);
             if (rc != OBEM_OK) return rc;
         } else {
             bt_blocks_kernel<<<1, 1024, 0, s>>>(F, F.blocks, F.block_cham, F.nblocks);
