@@ -239,19 +239,30 @@ __global__ void __launch_bounds__(EQ_TH) equilibrate_kernel(float *A, float *LU,
 
 // ------------------------------------------------------------------ panel exchange
 // The CTAs of the pivoting panel (a cooperative launch) meet once per column:
-// each CTA writes its pivot candidate (a 64-bit record and the candidate's
-// row), then arrives on a monotonic counter (zero at the launch) with a
-// release add; a CTA waits for column j until the counter reaches (j + 1) x
-// the CTAs (acquire loads) and then reads every record.  Records and rows go
-// to two buffer sets used by alternate columns: a CTA rewrites a set two
-// columns later, after every CTA has arrived for the column in between, i.e.
-// has finished reading it.  The wait is bounded: after BARRIER_WAIT_NS on
+// each CTA publishes its pivot candidate (a 64-bit record) and the candidate's
+// row, the owner of the row that receives the pivot publishes that row.  What
+// is published carries the column's epoch (its number in the matrix + 1; the
+// buffers are zeroed before the factorisation), so a reader polls the values
+// themselves and no order among them matters.  A column is a chain of two
+// trips through L2, records then the pivot row; with an arrival counter
+// (release add, counter polled, then the records read) it was a chain of
+// four: 3.4 to 2.5 us a column of 60,000 rows, the panels of order 59,968 203 to
+// 147 ms.
+// Records and rows go to two buffer sets used by alternate columns: a CTA
+// rewrites a set two columns later, after it has read every CTA's record of
+// the column in between, which a CTA publishes only after a block barrier
+// behind its reads of the set.  A wait is bounded: after BARRIER_WAIT_NS on
 // the global timer the CTA records OBEM_ERR_TIMEOUT in flag[0] and gives up.
 #define BARRIER_WAIT_NS 2000000000ull
 #define PAN_MAXG 1024           // largest panel grid
-// records [2][PAN_MAXG] (64-bit), gdiag [2][LU_NB], candidate rows [2][PAN_MAXG][LU_NB]
-#define PAN_REC_FLOATS (4 * PAN_MAXG)
-#define PAN_SCRATCH_FLOATS (PAN_REC_FLOATS + 2 * LU_NB + 2 * PAN_MAXG * LU_NB)
+// record: |pivot| bits << 33 | the row in its CTA << 23 | epoch
+#define PAN_ROW_SHIFT 23
+#define PAN_ROW_MASK 0x3ffu
+#define PAN_EPOCH_MASK 0x7fffffu
+static_assert(200 * 1024 / (4 * (LU_NB + 1)) <= PAN_ROW_MASK, "a CTA's rows fit the record");
+// 64-bit words: records [2][PAN_MAXG], gdiag [2][LU_NB], candidate rows [2][PAN_MAXG][LU_NB]
+#define PAN_WORDS (2 * PAN_MAXG + 2 * LU_NB + 2 * PAN_MAXG * LU_NB)
+#define PAN_SCRATCH_FLOATS (2 * PAN_WORDS)
 #define PAN_PLAN_FLOATS 260     // the row swaps' plan (1 + 4 LU_NB ints, padded to 16 bytes)
 
 __device__ __forceinline__ unsigned long long gb_now()
@@ -261,50 +272,76 @@ __device__ __forceinline__ unsigned long long gb_now()
     return t;
 }
 
-// Called by warp 0 only: waits until *count >= target and returns the
-// largest of the G records (in every lane), 0 when the wait ran out (then
-// flag[0] = OBEM_ERR_TIMEOUT).  Lane 0 polls with acquire loads; the warp
-// barrier after it orders the other lanes' reads of the records.
-__device__ unsigned long long pan_wait_records(const unsigned long long *recs, int G, const unsigned *count,
-                                               unsigned target, int *flag)
+__device__ __forceinline__ unsigned long long pan_ld(const unsigned long long *p)
 {
-    const int lane = threadIdx.x & 31;
-    int ok = 1;
-    if (lane == 0) {
-        const unsigned long long t0 = gb_now();
-        for (unsigned it = 1;; ++it) {
-            unsigned v;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
-            if (v >= target) break;
-            if ((it & 63u) == 0u && gb_now() - t0 > BARRIER_WAIT_NS) {
-                ok = 0;
-                atomicExch(flag, OBEM_ERR_TIMEOUT);
-                break;
-            }
-        }
-    }
-    __syncwarp();
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-    unsigned long long best = 0ull;
-    if (ok)
-        for (int t = lane; t < G; t += 32) {
-            const unsigned long long v = __ldcg(recs + t);
-            best = v > best ? v : best;
-        }
-    for (int o = 16; o; o >>= 1) {
-        const unsigned long long v2 = __shfl_xor_sync(0xffffffffu, best, o);
-        best = v2 > best ? v2 : best;
-    }
-    return ok ? (best ? best : 1ull) : 0ull;
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void pan_st(unsigned long long *p, unsigned long long v)
+{
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// Failure-detection self-test: the blocks arrive and wait for one block more
-// than was launched, so every wait runs out after BARRIER_WAIT_NS and records
-// OBEM_ERR_TIMEOUT in flag[0] (flag[1]: the counter, flag[2..]: records).
+// a bounded wait's clock (t0: 0 before its first look, at the 64th poll): true
+// when it ran out (flag[0] = OBEM_ERR_TIMEOUT)
+__device__ __forceinline__ bool pan_late(unsigned it, unsigned long long &t0, int *flag)
+{
+    if ((it & 63u) != 0u) return false;
+    if (t0 == 0ull) t0 = gb_now();
+    if (gb_now() - t0 <= BARRIER_WAIT_NS) return false;
+    atomicExch(flag, OBEM_ERR_TIMEOUT);
+    return true;
+}
+
+// Called by one warp: waits until the G records carry the epoch and returns the
+// largest candidate (in every lane) as |pivot| bits << 32 | ~row (ties to the
+// lower row), 1 when there is none, 0 when the wait ran out.  CTA b's rows
+// start at k + b R.
+__device__ unsigned long long pan_wait_records(const unsigned long long *recs, int G, unsigned epoch, int k, int R,
+                                               int *flag)
+{
+    const int lane = threadIdx.x & 31;
+    unsigned long long t0 = 0ull;
+    unsigned long long best = 1ull;
+    for (int g0 = 0; g0 < G; g0 += 256) {
+        unsigned long long v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = 0ull;
+        for (unsigned it = 1;; ++it) {
+            bool ok = true;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int t = g0 + 32 * q + lane;
+                if (t < G && ((unsigned)v[q] & PAN_EPOCH_MASK) != epoch) v[q] = pan_ld(recs + t);
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                ok = ok && (g0 + 32 * q + lane >= G || ((unsigned)v[q] & PAN_EPOCH_MASK) == epoch);
+            if (__all_sync(0xffffffffu, ok)) break;
+            int late = 0;
+            if (lane == 0) late = pan_late(it, t0, flag);
+            if (__shfl_sync(0xffffffffu, late, 0)) return 0ull;
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const unsigned m = (unsigned)(v[q] >> 33);
+            const int row = k + (g0 + 32 * q + lane) * R + (int)((unsigned)(v[q] >> PAN_ROW_SHIFT) & PAN_ROW_MASK);
+            const unsigned long long key = m ? (unsigned long long)m << 32 | (unsigned)~(unsigned)row : 1ull;
+            best = key > best ? key : best;
+        }
+    }
+    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32));
+    const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32) == hi ? (unsigned)best : 0u);
+    return (unsigned long long)hi << 32 | lo;
+}
+
+// Failure-detection self-test: the blocks wait for a record that nothing
+// publishes, so every wait runs out after BARRIER_WAIT_NS and records
+// OBEM_ERR_TIMEOUT in flag[0] (flag[2..3]: the record).
 __global__ void barrier_timeout_kernel(int *flag)
 {
-    if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"((unsigned *)&flag[1]) : "memory");
-    pan_wait_records((const unsigned long long *)(flag + 2), 1, (const unsigned *)&flag[1], gridDim.x + 1, flag);
+    pan_wait_records((const unsigned long long *)(flag + 2), 1, 1u, 0, 1, flag);
 }
 
 extern "C" int obem_selftest_wait_timeout(obem_ctx *c, obem_stream stream)
@@ -331,10 +368,13 @@ struct PanelArgs {
     float *A;
     int n, k, kb, rows_per_cta;
     int *piv;
-    int *flag;          // [0] status, [1] arrival counter (zero at the launch)
-    unsigned long long *rec;    // [2][PAN_MAXG] CTA b's candidate: |pivot| bits << 32 | ~row, 1: none
-    float *crows;       // [2][PAN_MAXG][LU_NB] the candidate row's panel values
-    float *gdiag;       // [2][LU_NB] the row receiving the pivot, before the swap
+    int *flag;          // [0] status
+    // published (see the panel exchange): CTA b's candidate, |pivot| 0: none;
+    // epoch << 32 | value of the candidate row's panel values and of the row
+    // receiving the pivot, before the swap
+    unsigned long long *rec;    // [2][PAN_MAXG]
+    unsigned long long *crows;  // [2][PAN_MAXG][LU_NB]
+    unsigned long long *gdiag;  // [2][LU_NB]
 };
 
 // best candidate over the CTA, in every thread: v = |a| (-1: none), r = its
@@ -361,22 +401,27 @@ __device__ __forceinline__ void pan_reduce(float &v, int &r, unsigned (*sv)[8], 
     r = bm == 0u ? 0x7fffffff : (int)br;
 }
 
-// Warp 0 publishes the CTA's candidate for column col: the candidate row bi
-// and, from its owner, the row that receives the pivot (both up to date),
-// then the record, then the arrival.  With j >= 0 the two rows' columns
-// j + 2 .. kb - 1 are first brought up to date with the multipliers of
-// column j (the rest of the CTA's rows are updated after the publication);
-// j = -1: no update.
+// Warp 0 publishes the CTA's candidate for column col: its record, the
+// candidate row bi and, from its owner, the row that receives the pivot (both
+// up to date).  With j >= 0 the two rows' columns j + 2 .. kb - 1 are first
+// brought up to date with the multipliers of column j (the rest of the CTA's
+// rows are updated after the publication); j = -1: no update.
 __device__ __forceinline__ void pan_publish(const PanelArgs &a, int col, int j, float bv, int bi, int r0, int rows,
                                             float *sp, int ld, const float *urow)
 {
     const int lane = threadIdx.x & 31, kb = a.kb, b = blockIdx.x;
     const int par = col & 1;
     const int pr = a.k + col;
-    float *crow = a.crows + ((size_t)par * PAN_MAXG + b) * LU_NB;
-    float *gd = a.gdiag + par * LU_NB;
+    const unsigned epoch = (unsigned)(pr + 1) & PAN_EPOCH_MASK;
+    unsigned long long *crow = a.crows + ((size_t)par * PAN_MAXG + b) * LU_NB;
+    unsigned long long *gd = a.gdiag + par * LU_NB;
     const bool has = bi != 0x7fffffff;
     const bool own = pr >= r0 && pr < r0 + rows;
+    if (lane == 0)
+        pan_st(a.rec + (size_t)par * PAN_MAXG + b,
+               (has ? (unsigned long long)__float_as_uint(bv) << 33 | (unsigned long long)(unsigned)(bi - r0) << PAN_ROW_SHIFT
+                    : 0ull) | epoch);
+    const unsigned long long tag = (unsigned long long)epoch << 32;
     for (int c = lane; c < kb; c += 32) {
         if (has) {
             float *row = sp + (size_t)(bi - r0) * ld;
@@ -385,8 +430,8 @@ __device__ __forceinline__ void pan_publish(const PanelArgs &a, int col, int j, 
                 x = fmaf(-row[j], urow[c], x);
                 row[c] = x;
             }
-            crow[c] = x;
-            if (bi == pr) gd[c] = x;
+            pan_st(crow + c, tag | __float_as_uint(x));
+            if (bi == pr) pan_st(gd + c, tag | __float_as_uint(x));
         }
         if (own && bi != pr) {
             float *row = sp + (size_t)(pr - r0) * ld;
@@ -395,33 +440,74 @@ __device__ __forceinline__ void pan_publish(const PanelArgs &a, int col, int j, 
                 x = fmaf(-row[j], urow[c], x);
                 row[c] = x;
             }
-            gd[c] = x;
+            pan_st(gd + c, tag | __float_as_uint(x));
         }
     }
-    if (lane == 0)
-        a.rec[(size_t)par * PAN_MAXG + b] =
-            has ? ((unsigned long long)__float_as_uint(bv) << 32) | (unsigned)(~(unsigned)bi) : 1ull;
-    __syncwarp();
-    // release: the warp's writes above are visible to any CTA that acquires
-    // the counter after this arrival
-    if (lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"((unsigned *)&a.flag[1]) : "memory");
+}
+
+// Warp 0 fetches the pivot row (row p, candidate of CTA q) to urow and swaps:
+// the pivot row to row pr, row pr's old values to row p, where they are the
+// CTA's.  Returns false when the wait ran out.
+__device__ __forceinline__ bool pan_fetch(const PanelArgs &a, int col, int p, int q, int r0, int rows, float *sp, int ld,
+                                          float *urow)
+{
+    static_assert(LU_NB == 64, "two columns per lane");
+    const int lane = threadIdx.x & 31, kb = a.kb;
+    const int par = col & 1, pr = a.k + col;
+    const unsigned epoch = (unsigned)(pr + 1) & PAN_EPOCH_MASK;
+    const unsigned long long *cu = a.crows + ((size_t)par * PAN_MAXG + q) * LU_NB + lane;
+    const unsigned long long *cg = a.gdiag + par * LU_NB + lane;
+    const bool mine = p != pr && p >= r0 && p < r0 + rows;      // warp-uniform
+    const bool h0 = lane < kb, h1 = lane + 32 < kb;
+    const unsigned long long none = (unsigned long long)epoch << 32;
+    unsigned long long u0 = 0ull, u1 = 0ull, g0 = 0ull, g1 = 0ull;
+    if (!h0) u0 = g0 = none;
+    if (!h1) u1 = g1 = none;
+    if (!mine) g0 = g1 = none;
+    unsigned long long t0 = 0ull;
+    for (unsigned it = 1;; ++it) {
+        if ((unsigned)(u0 >> 32) != epoch) u0 = pan_ld(cu);
+        if ((unsigned)(u1 >> 32) != epoch) u1 = pan_ld(cu + 32);
+        if ((unsigned)(g0 >> 32) != epoch) g0 = pan_ld(cg);
+        if ((unsigned)(g1 >> 32) != epoch) g1 = pan_ld(cg + 32);
+        const bool ok = (unsigned)(u0 >> 32) == epoch && (unsigned)(u1 >> 32) == epoch &&
+                        (unsigned)(g0 >> 32) == epoch && (unsigned)(g1 >> 32) == epoch;
+        if (__all_sync(0xffffffffu, ok)) break;
+        int late = 0;
+        if (lane == 0) late = pan_late(it, t0, a.flag);
+        if (__shfl_sync(0xffffffffu, late, 0)) return false;
+    }
+    const float x0 = __uint_as_float((unsigned)u0), x1 = __uint_as_float((unsigned)u1);
+    if (h0) urow[lane] = x0;
+    if (h1) urow[lane + 32] = x1;
+    if (pr >= r0 && pr < r0 + rows) {
+        float *row = sp + (size_t)(pr - r0) * ld;
+        if (h0) row[lane] = x0;
+        if (h1) row[lane + 32] = x1;
+    }
+    if (mine) {
+        float *row = sp + (size_t)(p - r0) * ld;
+        if (h0) row[lane] = __uint_as_float((unsigned)g0);
+        if (h1) row[lane + 32] = __uint_as_float((unsigned)g1);
+    }
+    return true;
 }
 
 // Panel factorisation of A[k:n, k:k+kb] with partial pivoting.  CTA b owns
 // rows k + b*R .. k + (b+1)*R - 1 of the panel in shared memory.  Per column
-// j: wait for every CTA's candidate of column j and take the largest (the
-// same pivot in every CTA), fetch the pivot row, swap, form the multipliers
-// and update column j + 1 of the own rows, find the CTA's candidate for
-// column j + 1 and publish it (warp 0, which then waits for the next
-// column); the other warps update the other columns of the own rows
-// meanwhile.
+// j: warp 0 waits for every CTA's candidate of column j, takes the largest
+// (the same pivot in every CTA), fetches the pivot row and swaps, while the
+// other warps finish column j - 1's update of the own rows (never the rows of
+// the swap: the CTA's candidate and the row that receives the pivot); then
+// the block forms the multipliers, updates column j + 1 of the own rows and
+// finds the CTA's candidate for column j + 1, which warp 0 publishes.
 __global__ void __launch_bounds__(256)
 panel_kernel(PanelArgs a)
 {
     extern __shared__ float sp[];            // [R][kb + 1] (padded against bank conflicts)
     __shared__ unsigned sv[2][8], sr[2][8];
-    __shared__ unsigned long long skey;
-    __shared__ float urow[LU_NB];
+    __shared__ int s_stop;                   // 0, OBEM_ERR_SINGULAR or OBEM_ERR_TIMEOUT
+    __shared__ float s_urow[2][LU_NB];       // pivot rows of alternate columns
     const int R = a.rows_per_cta, kb = a.kb, n = a.n, k = a.k;
     const int ld = kb + 1;
     const int b = blockIdx.x, G = gridDim.x;
@@ -458,40 +544,37 @@ panel_kernel(PanelArgs a)
             if (v > bv) { bv = v; bi = r0 + r; }
         }
         pan_reduce(bv, bi, sv, sr, 0);
-        if (warp == 0) pan_publish(a, 0, -1, bv, bi, r0, rows, sp, ld, urow);
+        if (warp == 0) pan_publish(a, 0, -1, bv, bi, r0, rows, sp, ld, s_urow[0]);
     }
     for (int j = 0; j < kb; ++j) {
         const int par = j & 1;
         const int pr = k + j;                     // row receiving the pivot
+        float *urow = s_urow[par];
         if (warp == 0) {
-            const unsigned long long kw =
-                pan_wait_records(a.rec + (size_t)par * PAN_MAXG, G, (const unsigned *)&a.flag[1],
-                                 (unsigned)(j + 1) * (unsigned)G, a.flag);
-            if (tid == 0) skey = kw;
+            const unsigned long long key = pan_wait_records(a.rec + (size_t)par * PAN_MAXG, G,
+                                                            (unsigned)(pr + 1) & PAN_EPOCH_MASK, k, R, a.flag);
+            const float v = __uint_as_float((unsigned)(key >> 32));
+            const int p = (int)(~(unsigned)(key & 0xffffffffu));
+            int stop = 0;
+            if (key == 0ull) stop = OBEM_ERR_TIMEOUT;
+            else if (key == 1ull || !(v > 0.f)) stop = OBEM_ERR_SINGULAR;
+            else if (!pan_fetch(a, j, p, (p - k) / R, r0, rows, sp, ld, urow)) stop = OBEM_ERR_TIMEOUT;
+            if (tid == 0) {
+                s_stop = stop;
+                if (b == 0 && stop == 0) a.piv[pr] = p;
+            }
         }
         __syncthreads();
-        const unsigned long long key = skey;
-        if (key == 0ull) return;                  // the wait ran out
-        const float v = __uint_as_float((unsigned)(key >> 32));
-        const int p = (int)(~(unsigned)(key & 0xffffffffu));
-        if (key == 1ull || !(v > 0.f)) {
+        if (s_stop) {
             // singular: every CTA stops here; the panel's remaining pivots
             // are set to no swap
-            if (tid == 0) atomicCAS(a.flag, 0, OBEM_ERR_SINGULAR);
-            if (b == 0)
-                for (int jj = j + tid; jj < kb; jj += blockDim.x) a.piv[k + jj] = k + jj;
+            if (s_stop == OBEM_ERR_SINGULAR) {
+                if (tid == 0) atomicCAS(a.flag, 0, OBEM_ERR_SINGULAR);
+                if (b == 0)
+                    for (int jj = j + tid; jj < kb; jj += blockDim.x) a.piv[k + jj] = k + jj;
+            }
             return;
         }
-        const int q = (p - k) / R;                // the CTA holding the pivot row
-        if (tid < kb) {
-            const float u = __ldcg(a.crows + ((size_t)par * PAN_MAXG + q) * LU_NB + tid);
-            const float g = __ldcg(a.gdiag + par * LU_NB + tid);
-            urow[tid] = u;
-            if (pr >= r0 && pr < r0 + rows) sp[(pr - r0) * ld + tid] = u;
-            if (p != pr && p >= r0 && p < r0 + rows) sp[(p - r0) * ld + tid] = g;
-        }
-        if (b == 0 && tid == 0) a.piv[pr] = p;
-        __syncthreads();
         const float inv = 1.0f / urow[j];
         if (j + 1 == kb) {
             for (int r = tid; r < rows; r += blockDim.x)
@@ -517,8 +600,8 @@ panel_kernel(PanelArgs a)
             pan_publish(a, j + 1, j, bv, bi, r0, rows, sp, ld, urow);
         } else {
             // the other rows' columns j + 2 .. kb - 1, while warp 0 waits
-            // for the next column (the barrier after that wait comes before
-            // any of them is read)
+            // for the next column and swaps (the barrier after that comes
+            // before any of them is read)
             const int nx = pr + 1;
             for (int r = tid - 32; r < rows; r += (int)blockDim.x - 32) {
                 const int gr = r0 + r;
@@ -550,8 +633,6 @@ panel_kernel(PanelArgs a)
 #define LS_PLAN_INTS (1 + 4 * LU_NB)        // m, rows[2 LU_NB], src[2 LU_NB]
 __global__ void __launch_bounds__(LU_NB) laswp_plan_kernel(int k, int kb, const int *piv, int *flag, int *plan)
 {
-    // the panel's arrival counter, zeroed for the next panel
-    if (threadIdx.x == 0) flag[1] = 0;
     // a panel that stopped (zero pivot, a wait that ran out) may have left
     // pivots unwritten: no swaps then
     if (*(volatile const int *)flag != 0) {
@@ -1256,7 +1337,7 @@ static int gemm_update(obem_ctx *c, int precision, float *A, int n, int k, int k
 // Pivoting panel factorisation of A[k:n, k:k+kb] (cooperative panel_kernel)
 // followed by its row swaps on every other column.
 struct PanelScratch {
-    float *cval, *crows, *gdiag;    // cval: the 2 x PAN_MAXG 64-bit candidate records
+    unsigned long long *rec, *crows, *gdiag;    // of the panel exchange
     int *plan;                      // the row swaps' plan (LS_PLAN_INTS)
     float *rows;                    // [2 LU_NB][n] the touched rows during the swaps
     int nsm;
@@ -1302,7 +1383,7 @@ static int factor_panel(obem_ctx *c, const PanelScratch &P, int k, int kb, cudaS
     }
     PanelArgs pa;
     pa.A = c->d_LU; pa.n = n; pa.k = k; pa.kb = kb; pa.rows_per_cta = R; pa.piv = c->d_piv;
-    pa.flag = c->d_flag; pa.rec = (unsigned long long *)P.cval; pa.crows = P.crows; pa.gdiag = P.gdiag;
+    pa.flag = c->d_flag; pa.rec = P.rec; pa.crows = P.crows; pa.gdiag = P.gdiag;
     void *args[] = {&pa};
     OBEM_CUDA(c, cudaLaunchCooperativeKernel((void *)panel_kernel, dim3(G), dim3(256), args, smem, s));
     laswp_plan_kernel<<<1, LU_NB, 0, s>>>(k, kb, c->d_piv, c->d_flag, P.plan);
@@ -1514,9 +1595,11 @@ static int factor_system(obem_ctx *c, int precision, cudaStream_t s)
     int nsm = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device);
     PanelScratch PS;
-    PS.cval = c->d_panel;
-    PS.gdiag = c->d_panel + PAN_REC_FLOATS;
-    PS.crows = c->d_panel + PAN_REC_FLOATS + 2 * LU_NB;
+    PS.rec = (unsigned long long *)c->d_panel;
+    PS.gdiag = PS.rec + 2 * PAN_MAXG;
+    PS.crows = PS.gdiag + 2 * LU_NB;
+    // no epoch of an earlier factorisation
+    OBEM_CUDA(c, cudaMemsetAsync(c->d_panel, 0, sizeof(float) * PAN_SCRATCH_FLOATS, s));
     PS.plan = (int *)(c->d_panel + PAN_SCRATCH_FLOATS);
     PS.rows = c->d_panel + PAN_SCRATCH_FLOATS + PAN_PLAN_FLOATS;
     PS.nsm = nsm;
