@@ -1,0 +1,43 @@
+"""The direct cell kernel's sorted targets and groups of cells: the sizes where
+the sort changes (one block up to 16,384 targets) and where groups begin
+(32,768), cells that do not fill the last group, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from gpu_util import FIELD_TOL, guarded_rel_err, potential_err, pts4, to_dev
+from paper_2110_09214_gb300 import inputs, obem
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("nt,cells,flags", [
+    (4096, 33, 0), (16384, 33, 0), (16385, 33, 0),
+    (32767, 1001, obem.OBEM_STEP_CELL_GROUPS), (32768, 31, obem.OBEM_STEP_CELL_GROUPS),
+    (32768, 33, obem.OBEM_STEP_CELL_GROUPS), (32775, 5001, obem.OBEM_STEP_CELL_GROUPS)])
+def test_sorted_and_grouped_targets(nt, cells, flags):
+    rng = np.random.default_rng(nt + cells)
+    m = inputs.parallel_plates(1e-3, 3e-4, max(2, int(np.ceil(np.sqrt(cells / 4)))))
+    mesh = inputs.Mesh(m.tri[:cells], m.kind[:cells], m.group[:cells], m.eps_minus[:cells], m.eps_plus[:cells],
+                       m.group_voltage)
+    cen = mesh.tri.mean(axis=1)
+    sigma = (1e-6 * (1.0 + 0.3 * np.sin(cen[:, 0] / 1e-4)) * np.where(mesh.group % 2 == 0, 1.0, -1.0)).astype(np.float32)
+    pts = rng.uniform([0, 0, 0], [1e-3, 1e-3, 3e-4], (nt, 3)).astype(np.float32)
+    pts[: nt // 3] = pts[0] + 1e-7 * rng.standard_normal((nt // 3, 3)).astype(np.float32)     # a third in one bin
+    ctx = obem.obem_create(capacity=16, dt=1e-12, flags=obem.OBEM_STEP_CELL_FIELD | flags)
+    try:
+        obem.obem_mesh_load(ctx, mesh)
+        out = torch.full((nt, 4), float("nan"), dtype=torch.float32, device="cuda")
+        obem.obem_field_eval(ctx, to_dev(pts4(pts)), out, sigma=to_dev(sigma))
+        torch.cuda.synchronize()
+        got = out.cpu().numpy()
+    finally:
+        obem.obem_destroy(ctx)
+    assert np.all(np.isfinite(got))
+    idx = np.unique(np.concatenate([[0, nt // 3, nt - 1], rng.choice(nt, 509, replace=False)]))
+    x, s = pts[idx].astype(np.float64), sigma.astype(np.float64)
+    E, V = oracle.panel_field(mesh.tri, s, x)
+    _, Vabs = oracle.panel_field(mesh.tri, np.abs(s), x)
+    assert guarded_rel_err(got[idx, :3], E) <= FIELD_TOL
+    assert potential_err(got[idx, 3], V, Vabs) <= FIELD_TOL
