@@ -4,23 +4,24 @@
 //
 //   C[M x N] -= A[M x K] B[K x N]      C, A, B: FP32 row-major sub-blocks
 //
-// The operands are rounded to BF16 (round to nearest even) into K-major
-// scratch (A as is, B transposed), then one CTA per 256 x 256 tile of C (tiles
-// ordered in groups of 8 row tiles for L2 reuse) runs
-// a TMA -> shared memory -> tcgen05.mma pipeline:
-//   warp 0, one lane   TMA producer: 64-wide K slices of A (256 rows) and B
-//                      (256 rows) into a 3-stage ring, 128B-swizzled
-//   warp 1, one lane   MMA issuer: per slice 4 K steps x 2 tcgen05.mma.kind::f16
-//                      (M 128, N 256, K 16), one per half of the tile's rows,
-//                      both on the stage's B; FP32 accumulation in tensor
-//                      memory (two accumulators of 256 columns x 128 lanes: all
-//                      512 columns); tcgen05.commit frees a stage
-//   warps 0-3          epilogue: tcgen05.ld of their 32 lanes of each
-//                      accumulator, through shared memory, C -= D with
-//                      coalesced row accesses
-// The 256-row tile halves the operand bytes each SM fetches per flop against
-// a 128-row one (the 128 x 256 tiles kept the tensor pipe about half busy,
-// fed from L2).
+// Operands are rounded to BF16 (round to nearest even), products accumulated in
+// FP32.  K <= 128: tc_fused_kernel, from the FP32 operands.  Longer K: the
+// operands into K-major scratch (A as is, B transposed; tc_cvt_kernel), then one
+// CTA per 256 x 256 or 128 x 128 tile of C (tiles ordered in groups of 2048 rows
+// for L2 reuse) runs a TMA -> shared memory -> tcgen05.mma pipeline:
+//   warp 0, one lane   TMA producer: 64-wide K slices of A and B into a 3-stage
+//                      ring, 128B-swizzled
+//   warp 1, one lane   MMA issuer: per slice 4 K steps x 1 or 2
+//                      tcgen05.mma.kind::f16 (M 128, N 128 or 256, K 16), one per
+//                      128 rows, all on the stage's B; FP32 accumulation in
+//                      tensor memory; tcgen05.commit frees a stage
+//   warps 0-7          epilogue: tcgen05.ld of their 32 lanes and half the
+//                      columns of each accumulator, through shared memory,
+//                      C -= D with coalesced row accesses
+// Bound: the tensor cores from K 8192 on (2.0 PFLOP/s at 32,768), C's traffic and
+// latency below K 1024 (14 us per call at K 64 in 256 x 256 tiles plus 9 of
+// conversion, 5.5 fused).  The updates of order 59,968 with conversions: 168 to
+// 133 ms.
 // Every wait on an mbarrier is bounded; a wait that runs out records
 // OBEM_ERR_TIMEOUT in *err, the kernel lets its issued copies and MMAs finish
 // (bounded again), frees its tensor memory and returns.
@@ -31,20 +32,22 @@
 
 namespace {
 constexpr int TC_MM = 128;                                        // rows of one MMA and of one accumulator
-constexpr int TC_BM = 256, TC_BN = 256, TC_BK = 64, TC_STAGES = 3, TC_THREADS = 128;
-constexpr int TC_ACC = TC_BM / TC_MM;                             // accumulators per tile
-constexpr uint32_t TC_A_BYTES = TC_BM * TC_BK * 2;               // 32 KB
-constexpr uint32_t TC_B_BYTES = TC_BN * TC_BK * 2;               // 32 KB
-constexpr uint32_t TC_STAGE_BYTES = TC_A_BYTES + TC_B_BYTES;
-constexpr uint32_t TC_TMEM_COLS = TC_ACC * TC_BN;                 // 512: all of the SM's tensor memory
-constexpr int TC_GROUP_M = 8;                                    // row tiles per rasterisation group
-constexpr size_t TC_SMEM = 1024 + (size_t)TC_STAGES * TC_STAGE_BYTES + 256;
+constexpr int TC_BK = 64, TC_STAGES = 3, TC_THREADS = 256;
+constexpr int TC_GROUP_ROWS = 2048;                              // rows of C per rasterisation group
+static_assert((TC_THREADS / 32) * 32 * 33 * 4 <= 3 * 128 * TC_BK * 2, "the epilogue's staging fits the stages of A");
+constexpr int TF_THREADS = 256;                                  // fused kernel
 constexpr unsigned long long TC_WAIT_NS = 2000000000ull;   // 2 s per wait
+// a tile of BM x BN: operand bytes of a stage, shared memory, tensor-memory columns
+__host__ __device__ constexpr uint32_t tc_a_bytes(int bm) { return (uint32_t)bm * TC_BK * 2; }
+__host__ __device__ constexpr uint32_t tc_stage_bytes(int bm, int bn) { return (uint32_t)(bm + bn) * TC_BK * 2; }
+__host__ __device__ constexpr size_t tc_smem_bytes(int bm, int bn) { return 1024 + (size_t)TC_STAGES * tc_stage_bytes(bm, bn) + 256; }
 // instruction descriptor of tcgen05.mma.kind::f16: D FP32 (bits 4-5 = 1),
 // A and B BF16 (bits 7-9 = 1, 10-12 = 1), both K-major (bits 15, 16 = 0),
 // N >> 3 in bits 17-22, M >> 4 in bits 24-28
-constexpr uint32_t TC_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TC_BN >> 3) << 17) |
-                              ((uint32_t)(TC_MM >> 4) << 24);
+__host__ __device__ constexpr uint32_t tc_idesc(int bn)
+{
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(TC_MM >> 4) << 24);
+}
 }
 
 __device__ __forceinline__ uint32_t tc_smem(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -104,12 +107,12 @@ __device__ __forceinline__ uint64_t tc_desc(uint32_t saddr)
            ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
 
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accumulate)
+__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accumulate, uint32_t idesc)
 {
     asm volatile("{\n\t.reg .pred p;\n\t"
                  "setp.ne.b32 p, %3, 0;\n\t"
                  "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %4, p;\n\t}"
-                 ::"r"(d_tmem), "l"(a), "l"(b), "r"(accumulate), "r"(TC_IDESC)
+                 ::"r"(d_tmem), "l"(a), "l"(b), "r"(accumulate), "r"(idesc)
                  : "memory");
 }
 
@@ -137,10 +140,17 @@ __device__ __forceinline__ void tc_tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-__global__ void __launch_bounds__(TC_THREADS, 1)
+// Tiles of 256 x 256 (all 512 columns of tensor memory, one CTA per SM) or of
+// 128 x 128 (two CTAs per SM, so that one's epilogue runs beside the other's
+// main loop, and four times the tiles: updates of short K or few tiles).
+template <int TC_BM, int TC_BN>
+__global__ void __launch_bounds__(TC_THREADS, TC_BM == 256 ? 1 : 2)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, float *__restrict__ C,
                long long ldc, int M, int N, int K, int *err)
 {
+    constexpr int TC_ACC = TC_BM / TC_MM, TC_GROUP_M = TC_GROUP_ROWS / TC_BM;
+    constexpr uint32_t TC_A_BYTES = tc_a_bytes(TC_BM), TC_STAGE_BYTES = tc_stage_bytes(TC_BM, TC_BN),
+                       TC_B_BYTES = TC_STAGE_BYTES - TC_A_BYTES, TC_TMEM_COLS = TC_ACC * TC_BN;
     extern __shared__ uint8_t tc_smem_raw[];
     uint8_t *sm = (uint8_t *)(((uintptr_t)tc_smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *sA = sm;
@@ -191,8 +201,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 
     if (warp >= 2) {
         // the epilogue reads and rewrites this CTA's tile of C: bring it into
-        // L2 while the main loop runs (8 lines of 128 bytes per row)
-        for (int e = threadIdx.x - 64; e < TC_BM * (TC_BN / 32); e += 64) {
+        // L2 while the main loop runs (lines of 128 bytes)
+        for (int e = threadIdx.x - 64; e < TC_BM * (TC_BN / 32); e += TC_THREADS - 64) {
             const int r = m0 + e / (TC_BN / 32), cc = n0 + (e % (TC_BN / 32)) * 32;
             if (r < M && cc < N)
                 asm volatile("prefetch.global.L2 [%0];" ::"l"((unsigned long long)(C + (size_t)r * ldc + cc)));
@@ -236,7 +246,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 for (int a = 0; a < TC_ACC; ++a)
                     if (a == 0 || m0 + a * TC_MM < M)
                         tc_mma(tmem + (uint32_t)(a * TC_BN), tc_desc(a0 + (uint32_t)(a * TC_MM * 128) + 32 * j),
-                               tc_desc(b0 + 32 * j), (kb | j) != 0);
+                               tc_desc(b0 + 32 * j), (kb | j) != 0, tc_idesc(TC_BN));
             tc_commit(&empty[s]);
         }
         // arrives once every MMA issued above has completed (also on failure)
@@ -244,51 +254,52 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
     __syncwarp();
 
-    // epilogue: warp w owns accumulator lanes (rows) 32 w .. 32 w + 31
+    // epilogue: warp w owns accumulator lanes (rows) 32 (w % 4) .. and columns
+    // (w / 4) BN / 2 .. of each accumulator, in chunks of 32 columns; the next
+    // chunk's values of C (the first one's before the wait) are in flight while
+    // a chunk is written back
+    constexpr int CH = TC_BN / 64, NCH = TC_ACC * CH;           // chunks of a warp, accumulator by accumulator
+    const int cbase = n0 + (warp >> 2) * (TC_BN / 2);
+    auto chunk = [&](int q, int &rbase, int &col) {
+        rbase = m0 + (q / CH) * TC_MM + (warp & 3) * 32;
+        col = cbase + (q % CH) * 32 + lane;
+    };
+    float vn[32];
+    auto load_c = [&](int q) {
+        int rbase, col;
+        chunk(q, rbase, col);
+        const int nrow = col < N ? M - rbase : 0;
+        const float *cp = C + (size_t)rbase * ldc + col;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) vn[i] = i < nrow ? __ldcg(cp + (size_t)i * ldc) : 0.f;
+    };
+    load_c(0);
     const bool fine = tc_mbar_wait(done, 0);
     tc_fence_after();
     __syncthreads();
     if (fine && !*(volatile int *)s_fail) {
         float *stage = (float *)sA + warp * 32 * 33;       // pipeline smem is idle now
-        for (int acc = 0; acc < TC_ACC; ++acc) {
-            const int rbase = m0 + acc * TC_MM + warp * 32;
-            if (rbase >= M) break;                          // warp-uniform
-            const int nrow = min(32, M - rbase);
-            // the 32 rows' values of this lane's column, chunk by chunk of 32
-            // columns; the next chunk's loads are in flight while this one is
-            // written back
-            float vn[32];
-            {
-                const int col = n0 + lane;
-                const float *cp = C + (size_t)rbase * ldc + col;
+#pragma unroll 1
+        for (int q = 0; q < NCH; ++q) {
+            float v[32];
 #pragma unroll
-                for (int i = 0; i < 32; ++i) vn[i] = (i < nrow && col < N) ? __ldcg(cp + (size_t)i * ldc) : 0.f;
-            }
-            for (int c = 0; c < TC_BN; c += 32) {
-                if (n0 + c >= N) break;                     // warp-uniform
-                float v[32];
+            for (int i = 0; i < 32; ++i) v[i] = vn[i];
+            if (q + 1 < NCH) load_c(q + 1);
+            int rbase, col;
+            chunk(q, rbase, col);
+            if (rbase >= M || col - lane >= N) continue;    // warp-uniform
+            uint32_t r[32];
+            tc_tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) +
+                             (uint32_t)((q / CH) * TC_BN + (warp >> 2) * (TC_BN / 2) + (q % CH) * 32), r);
 #pragma unroll
-                for (int i = 0; i < 32; ++i) v[i] = vn[i];
-                if (c + 32 < TC_BN && n0 + c + 32 < N) {
-                    const int coln = n0 + c + 32 + lane;
-                    const float *cpn = C + (size_t)rbase * ldc + coln;
+            for (int j = 0; j < 32; ++j) stage[lane * 33 + j] = __uint_as_float(r[j]);
+            __syncwarp();
+            const int nrow = col < N ? M - rbase : 0;
+            float *cp = C + (size_t)rbase * ldc + col;
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) vn[i] = (i < nrow && coln < N) ? __ldcg(cpn + (size_t)i * ldc) : 0.f;
-                }
-                uint32_t r[32];
-                tc_tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(acc * TC_BN + c), r);
-#pragma unroll
-                for (int j = 0; j < 32; ++j) stage[lane * 33 + j] = __uint_as_float(r[j]);
-                __syncwarp();
-                const int col = n0 + c + lane;
-                float *cp = C + (size_t)rbase * ldc + col;
-                if (col < N) {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i)
-                        if (i < nrow) __stcg(cp + (size_t)i * ldc, v[i] - stage[i * 33 + lane]);
-                }
-                __syncwarp();
-            }
+            for (int i = 0; i < 32; ++i)
+                if (i < nrow) __stcg(cp + (size_t)i * ldc, v[i] - stage[i * 33 + lane]);
+            __syncwarp();
         }
     } else if (threadIdx.x == 0) {
         atomicExch(err, OBEM_ERR_TIMEOUT);
@@ -298,6 +309,137 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_TMEM_COLS)
                      : "memory");
+}
+
+// C[M x N] -= A[M x K] B[K x N] for K <= TF_K, from the FP32 operands: a CTA
+// per 128 x BN tile converts its slices of A and B in registers, writes them to
+// shared memory in the layout of the MMA's descriptors and issues the MMAs.  No
+// conversion pass, no BF16 scratch, no ring: with K this short an update is its
+// traffic of C (4 bytes read and written per 2 K flops) and the latency of a
+// launch, and two thirds of a factorisation's updates have K <= 128.
+constexpr int TF_K = 128, TF_BN = 64;
+constexpr size_t tf_smem(int nk)
+{
+    const size_t op = (size_t)nk * tc_stage_bytes(TC_MM, TF_BN), st = (TF_THREADS / 32) * 32 * 33 * sizeof(float);
+    return 1024 + (op > st ? op : st) + 64;
+}
+template <bool VEC>
+__global__ void __launch_bounds__(TF_THREADS, 2)
+tc_fused_kernel(float *__restrict__ C, long long ldc, const float *__restrict__ A, long long lda,
+                const float *__restrict__ B, long long ldb, int M, int N, int K, int *err)
+{
+    constexpr int BN = TF_BN;
+    static_assert(BN == 64, "a chunk of 32 columns per warp");
+    constexpr uint32_t A_BYTES = tc_a_bytes(TC_MM), STAGE = tc_stage_bytes(TC_MM, BN);
+    extern __shared__ uint8_t tc_smem_raw[];
+    __shared__ uint64_t s_done;
+    __shared__ uint32_t s_tmem;
+    uint8_t *sm = (uint8_t *)(((uintptr_t)tc_smem_raw + 1023) & ~(uintptr_t)1023);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int num_m = (M + TC_MM - 1) / TC_MM;
+    const int m0 = (blockIdx.x % num_m) * TC_MM, n0 = (blockIdx.x / num_m) * BN;
+    const int nk = (K + TC_BK - 1) / TC_BK;
+    if (tid == 0) {
+        tc_mbar_init(&s_done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_smem(&s_tmem)),
+                     "r"((uint32_t)BN)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    // the tile of C into L2 (lines of 128 bytes)
+    for (int e = tid; e < TC_MM * (BN / 32); e += TF_THREADS) {
+        const int r = m0 + e / (BN / 32), cc = n0 + (e % (BN / 32)) * 32;
+        if (r < M && cc < N) asm volatile("prefetch.global.L2 [%0];" ::"l"((unsigned long long)(C + (size_t)r * ldc + cc)));
+    }
+    union Pack { __nv_bfloat162 h[4]; uint4 u; };
+    auto put = [](uint8_t *tile, int row, int c, const float (&v)[8]) {        // 16-byte chunk c of a 128-byte row, swizzled
+        Pack o;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) o.h[q] = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
+        *reinterpret_cast<uint4 *>(tile + row * 128 + ((c ^ (row & 7)) << 4)) = o.u;
+    };
+    for (int kc = 0; kc < nk; ++kc) {
+        uint8_t *sA = sm + kc * STAGE, *sB = sA + A_BYTES;
+        float va[4][8], vb[BN / 32][8];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int e = tid + TF_THREADS * q, r = m0 + (e >> 3), k = kc * TC_BK + (e & 7) * 8;
+            const float *p = A + (size_t)r * lda + k;
+            if (VEC && r < M && k + 8 <= K) {
+                const float4 x = *reinterpret_cast<const float4 *>(p), y = *reinterpret_cast<const float4 *>(p + 4);
+                va[q][0] = x.x; va[q][1] = x.y; va[q][2] = x.z; va[q][3] = x.w;
+                va[q][4] = y.x; va[q][5] = y.y; va[q][6] = y.z; va[q][7] = y.w;
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) va[q][i] = r < M && k + i < K ? p[i] : 0.f;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < BN / 32; ++q) {
+            const int e = tid + TF_THREADS * q, n = n0 + e % BN, k = kc * TC_BK + (e / BN) * 8;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) vb[q][i] = n < N && k + i < K ? B[(size_t)(k + i) * ldb + n] : 0.f;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int e = tid + TF_THREADS * q;
+            put(sA, e >> 3, e & 7, va[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < BN / 32; ++q) {
+            const int e = tid + TF_THREADS * q;
+            put(sB, e % BN, e / BN, vb[q]);
+        }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = s_tmem;
+    if (tid == 0) {
+        for (int kc = 0; kc < nk; ++kc) {
+            const uint32_t a0 = tc_smem(sm + kc * STAGE), b0 = a0 + A_BYTES;
+#pragma unroll
+            for (int j = 0; j < TC_BK / 16; ++j)
+                tc_mma(tmem, tc_desc(a0 + 32 * j), tc_desc(b0 + 32 * j), (kc | j) != 0, tc_idesc(BN));
+        }
+        tc_commit(&s_done);
+    }
+    __syncwarp();
+    // epilogue: warp w owns accumulator lanes (rows) 32 (w % 4) .., columns
+    // (w / 4) BN / 2 .. of the tile; its values of C are on the way meanwhile
+    const int rbase = m0 + (warp & 3) * 32, cbase = (warp >> 2) * (BN / 2);
+    const int nrow = min(32, M - rbase);
+    const int col = n0 + cbase + lane;
+    float *cp = C + (size_t)rbase * ldc + col;
+    float v[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = (i < nrow && col < N) ? __ldcg(cp + (size_t)i * ldc) : 0.f;
+    const bool fine = tc_mbar_wait(&s_done, 0);
+    tc_fence_after();
+    __syncthreads();
+    if (fine) {
+        float *stage = (float *)sm + warp * 32 * 33;            // the operands have been read
+        uint32_t r[32];
+        tc_tmem_ld32(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)cbase, r);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) stage[lane * 33 + j] = __uint_as_float(r[j]);
+        __syncwarp();
+        if (col < N) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+                if (i < nrow) __stcg(cp + (size_t)i * ldc, v[i] - stage[i * 33 + lane]);
+        }
+    } else if (tid == 0) {
+        atomicExch(err, OBEM_ERR_TIMEOUT);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)BN) : "memory");
 }
 
 // Both operands of a GEMM to BF16 in one launch: blocks [0, na) round 64 x 64
@@ -431,6 +573,17 @@ void obem_tc_free(obem_ctx *c)
     c->tc_a_bytes = c->tc_b_bytes = 0;
 }
 
+// Tiles of 128 x 128 (else 256 x 256): short K, where a tile is mostly epilogue,
+// and updates whose larger tiles would leave half the SMs idle.  Measured 256 /
+// 128 (us, M x N x K): 30000 x 256 x 256 20.7 / 19.0, 512 x 512 x 512 22.2 / 9.0,
+// 30000 x 1024 x 1024 123 / 95, 4000 x 2048 x 2048 37 / 41, 30000 x 2048 x 2048 282 /
+// 255, 512 x 4096 x 4096 55 / 32, 4000 x 4096 x 4096 116 / 132.
+static bool tc_small_tiles(int M, int N, int K)
+{
+    const long long t256 = (long long)((N + 255) / 256) * ((M + 255) / 256);
+    return K <= 1024 || t256 <= 76 || (K <= 2048 && t256 > 152);
+}
+
 // C[M x N] -= A[M x K] B[K x N] with BF16 operands and FP32 accumulation;
 // C, A, B are FP32 row-major blocks with leading dimensions ldc, lda, ldb.
 // Uses the context's BF16 scratch (obem_tc_reserve grows it); err: device
@@ -439,6 +592,29 @@ int obem_tc_gemm_sub(obem_ctx *c, float *C, long long ldc, const float *A, long 
                      int M, int N, int K, int *err, cudaStream_t s)
 {
     if (M <= 0 || N <= 0 || K <= 0) return OBEM_OK;
+    static unsigned long long attr = 0;   // devices done (a bit each)
+    if (!(attr >> (c->device & 63) & 1ull)) {
+        OBEM_CUDA(c, cudaFuncSetAttribute(tc_gemm_kernel<256, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)tc_smem_bytes(256, 256)));
+        OBEM_CUDA(c, cudaFuncSetAttribute(tc_gemm_kernel<128, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)tc_smem_bytes(128, 128)));
+        OBEM_CUDA(c, cudaFuncSetAttribute(tc_fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)tf_smem(TF_K / TC_BK)));
+        OBEM_CUDA(c, cudaFuncSetAttribute(tc_fused_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)tf_smem(TF_K / TC_BK)));
+        attr |= 1ull << (c->device & 63);
+    }
+    const bool vec = (((uintptr_t)A | (uintptr_t)B) & 15) == 0 && ((lda | ldb) & 3) == 0;
+    const long long t128 = (long long)((N + 127) / 128) * ((M + 127) / 128);
+    if (t128 > 0x3fffffffll) return obem_fail(c, OBEM_ERR_ARG, "tensor-core GEMM: %d x %d exceeds the grid", M, N);
+    if (K <= TF_K) {
+        const int nk = (K + TC_BK - 1) / TC_BK;
+        const unsigned g = (unsigned)((long long)((N + TF_BN - 1) / TF_BN) * ((M + TC_MM - 1) / TC_MM));
+        if (vec) tc_fused_kernel<true><<<g, TF_THREADS, tf_smem(nk), s>>>(C, ldc, A, lda, B, ldb, M, N, K, err);
+        else tc_fused_kernel<false><<<g, TF_THREADS, tf_smem(nk), s>>>(C, ldc, A, lda, B, ldb, M, N, K, err);
+        OBEM_LAUNCH(c);
+        return OBEM_OK;
+    }
     const int ldk = (K + 7) / 8 * 8;                       // 16-byte row pitch for the tensor maps
     int rc = obem_tc_reserve(c, (size_t)M * ldk, (size_t)N * ldk);
     if (rc != OBEM_OK) return rc;
@@ -447,23 +623,22 @@ int obem_tc_gemm_sub(obem_ctx *c, float *C, long long ldc, const float *A, long 
         const int nk = (ldk + CV_T - 1) / CV_T;
         const long long na = (long long)((M + CV_T - 1) / CV_T) * nk, nb = (long long)((N + CV_T - 1) / CV_T) * nk;
         if (na + nb > 0x7fffffffll) return obem_fail(c, OBEM_ERR_ARG, "tensor-core GEMM: operands exceed the grid");
-        const bool vec = (((uintptr_t)A | (uintptr_t)B) & 15) == 0 && ((lda | ldb) & 3) == 0;
         if (vec) tc_cvt_kernel<true><<<(unsigned)(na + nb), 256, 0, s>>>(A, lda, M, K, Ab, B, ldb, N, Bb, ldk, (int)na, nk);
         else tc_cvt_kernel<false><<<(unsigned)(na + nb), 256, 0, s>>>(A, lda, M, K, Ab, B, ldb, N, Bb, ldk, (int)na, nk);
         OBEM_LAUNCH(c);
     }
+    const bool small = tc_small_tiles(M, N, K);
+    const int bt = small ? 128 : 256;
     CUtensorMap ma, mb;
-    rc = tc_map(c, &ma, Ab, M, K, ldk, TC_BM);
-    if (rc == OBEM_OK) rc = tc_map(c, &mb, Bb, N, K, ldk, TC_BN);
+    rc = tc_map(c, &ma, Ab, M, K, ldk, bt);
+    if (rc == OBEM_OK) rc = tc_map(c, &mb, Bb, N, K, ldk, bt);
     if (rc != OBEM_OK) return rc;
-    static unsigned long long attr = 0;   // devices done (a bit each)
-    if (!(attr >> (c->device & 63) & 1ull)) {
-        OBEM_CUDA(c, cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM));
-        attr |= 1ull << (c->device & 63);
+    if (small) {
+        tc_gemm_kernel<128, 128><<<(unsigned)t128, TC_THREADS, tc_smem_bytes(128, 128), s>>>(ma, mb, C, ldc, M, N, K, err);
+    } else {
+        const unsigned g = (unsigned)(((N + 255) / 256) * ((M + 255) / 256));
+        tc_gemm_kernel<256, 256><<<g, TC_THREADS, tc_smem_bytes(256, 256), s>>>(ma, mb, C, ldc, M, N, K, err);
     }
-    const long long tiles = (long long)((N + TC_BN - 1) / TC_BN) * ((M + TC_BM - 1) / TC_BM);
-    if (tiles > 0x7fffffffll) return obem_fail(c, OBEM_ERR_ARG, "tensor-core GEMM: %d x %d exceeds the grid", M, N);
-    tc_gemm_kernel<<<(unsigned)tiles, TC_THREADS, TC_SMEM, s>>>(ma, mb, C, ldc, M, N, K, err);
     OBEM_LAUNCH(c);
     return OBEM_OK;
 }
