@@ -100,7 +100,7 @@ extern "C" int obem_create(obem_ctx **out, const obem_config *cfg)
     ALLOC(c->s_ionkey, sizeof(unsigned long long) * cap);
     ALLOC(c->s_keep, sizeof(int32_t) * cap);
     ALLOC(c->s_nsp, sizeof(int32_t) * cap);
-    ALLOC(c->s_blk, sizeof(int32_t) * 2 * ((size_t)cap / 32 + 8));
+    ALLOC(c->s_blk, sizeof(int32_t) * 2 * ((size_t)cap / 32 + 2048 + 8));   // chunks of 32 and more, of 8 up to 16384 charges
     ALLOC(c->s_rec, sizeof(float4) * OBEM_REC_F4 * ((size_t)cap / 2 + 1));
     ALLOC(c->s_mpart, sizeof(double) * 13 * max_blocks);
     ALLOC(c->s_ctl, sizeof(StepCtl));
