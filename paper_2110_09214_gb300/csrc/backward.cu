@@ -509,11 +509,16 @@ __global__ void __launch_bounds__(32 * BR_WARPS) bw_sigma_kernel(BwLaunch B)
     auto closed_pair = [&](int w, int k) {
         const int t = s_q[w][0][k];
         const float4 x = B.targets[t], g = B.g[t];
-        double phi, fx, fy, fz;
         const size_t jc = (size_t)(j0 + s_q[w][1][k]);
-        tri_closed_form_g(P.v64 + 9 * jc, P.geo + OBEM_GEO64 * jc, (double)x.x, (double)x.y, (double)x.z, phi, fx, fy,
-                          fz);
-        s_v[w][k] = (float)(OBEM_KC * ((double)g.x * fx + (double)g.y * fy + (double)g.z * fz + (double)g.w * phi));
+        Dbf p, a, b, c;
+        if (tri_closed_df(P.geo2 + OBEM_GEO2 * jc, Dbf{x.x, 0.f}, Dbf{x.y, 0.f}, Dbf{x.z, 0.f}, true, p, a, b, c)) {
+            const Dbf s = df_sum(df_sum(df_mulf(a, g.x), df_mulf(b, g.y)), df_sum(df_mulf(c, g.z), df_mulf(p, g.w)));
+            s_v[w][k] = df_mul(Dbf{(float)OBEM_KC, (float)(OBEM_KC - (double)(float)OBEM_KC)}, s).h;
+        } else {
+            double phi, fx, fy, fz;
+            tri_closed_form_g(P.v64 + 9 * jc, P.geo + OBEM_GEO64 * jc, (double)x.x, (double)x.y, (double)x.z, phi, fx, fy, fz);
+            s_v[w][k] = (float)(OBEM_KC * ((double)g.x * fx + (double)g.y * fy + (double)g.z * fz + (double)g.w * phi));
+        }
     };
     // the warp's m queued pairs, evaluated, to their cells' lanes in order
     auto take = [&](int m) {
@@ -964,12 +969,10 @@ __device__ __forceinline__ void if_closed(const PanelsDev &P, int j, const float
     const int lane = threadIdx.x & 31;
     if (lane < n) {
         const float4 x = cq[lane];
-        double phi, fx, fy, fz;
-        tri_closed_form_g(P.v64 + 9 * (size_t)j, P.geo + (size_t)OBEM_GEO64 * j, (double)x.x, (double)x.y, (double)x.z,
-                          phi, fx, fy, fz);
-        const double qk = (double)x.w * OBEM_KC;
-        v[0] += (float)(qk * phi); v[1] += (float)(qk * fx);
-        v[2] += (float)(qk * fy); v[3] += (float)(qk * fz);
+        const float4 r = closed_terms(P.v64 + 9 * (size_t)j, P.geo + (size_t)OBEM_GEO64 * j, P.geo2 + (size_t)OBEM_GEO2 * j,
+                                      x.x, x.y, x.z, x.w);
+        v[0] += r.w; v[1] += r.x;
+        v[2] += r.y; v[3] += r.z;
     }
     __syncwarp();
 }

@@ -269,7 +269,11 @@ static int upload_cells(obem_batch *b)
         BUP(b->d_v64, v64.data(), sizeof(double) * 9 * (size_t)np);
         std::vector<double> geo((size_t)OBEM_GEO64 * np);
         obem_cell_geo64(v64.data(), np, geo.data());
-        BUP(b->d_geo64, geo.data(), sizeof(double) * geo.size());
+        BALLOC(b->d_geo64, obem_geo_bytes(np));
+        if (rc == OBEM_OK &&
+            (cudaMemcpy(b->d_geo64, geo.data(), sizeof(double) * geo.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+             obem_cell_geo2(b->d_v64, b->d_geo64, np) != cudaSuccess))
+            rc = obem_fail(ctx, OBEM_ERR_CUDA, "batch: upload failed");
         BUP(b->d_sigma, sg.data(), sizeof(float) * np);
     }
     if (rc == OBEM_OK &&
@@ -330,6 +334,7 @@ static FieldBatch field_args(obem_batch *b, const obem_state *st)
     F.panels.c_lo = b->d_c_lo;
     F.panels.v64 = b->d_v64;
     F.panels.geo = b->d_geo64;
+    F.panels.geo2 = obem_geo2_of(b->d_geo64, b->np_total);
     F.panels.np = b->np_total;
     F.sigma = b->d_sigma;
     F.cham_pan = b->d_cham_pan;

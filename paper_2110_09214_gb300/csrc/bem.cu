@@ -45,12 +45,13 @@ template <bool B> struct AsBool { static constexpr bool value = B; };
 // in registers and takes the rows two at a time (f32x2), a far entry by the
 // tier of the nearer of the two rows' centroids, evaluated without divergence
 // as up to seven points c, c + a g_k, c + b g_k.  Near entries go to a
-// per-warp queue of the FP64 closed form, 32 at a time: a warp-wide FP64
-// instruction costs the same with one lane as with 32, and with a thread per
-// entry nearly every warp had a near one.  Electrode rows need the potential
+// per-warp queue of the closed form, 32 at a time: a warp-wide instruction
+// costs the same with one lane as with 32, and with a thread per entry nearly
+// every warp had a near one.  Electrode rows need the potential
 // only, dielectric rows the field's component along their normal.
 // Bound: FP32 issue of the far points (5 on average at 60k cells).  Measured at
-// 59,968 cells: 174.2 to 33.0 ms.
+// 59,968 cells: 174.2 to 33.0 ms, 16.5 with the near entries' closed form in pairs
+// of floats.
 __global__ void __launch_bounds__(AS_TH) assemble_kernel(PanelsDev P, const int *kind, const double *em,
                                                          const double *ep, float *A, int n)
 {
@@ -83,20 +84,26 @@ __global__ void __launch_bounds__(AS_TH) assemble_kernel(PanelsDev P, const int 
         if (lane < m) {
             const uint32_t e = s_q[warp][lane];
             const int i = i0 + (int)(e >> 8), jj = j0 + (int)(e & 255u);
-            const double *vi = P.v64 + 9 * (size_t)i;
-            double phi, Fx, Fy, Fz;
-            tri_closed_form_g(P.v64 + 9 * (size_t)jj, P.geo + (size_t)OBEM_GEO64 * jj, (vi[0] + vi[3] + vi[6]) / 3.0,
-                              (vi[1] + vi[4] + vi[7]) / 3.0, (vi[2] + vi[5] + vi[8]) / 3.0, phi, Fx, Fy, Fz);
-            double a;
-            if (kind[i] == OBEM_CELL_ELECTRODE) {
-                a = OBEM_KC * phi;
-            } else if (i == jj) {
-                a = 0.5 * (ep[i] + em[i]);
+            const bool pot = kind[i] == OBEM_CELL_ELECTRODE;
+            const float4 ci = P.c_a[i], li = P.c_lo[i], ni = P.nrm[i];
+            Dbf p, fx, fy, fz;
+            float a;
+            if (!pot && i == jj) {
+                a = (float)(0.5 * (ep[i] + em[i]));
+            } else if (tri_closed_df(P.geo2 + (size_t)OBEM_GEO2 * jj, Dbf{ci.x, li.x}, Dbf{ci.y, li.y}, Dbf{ci.z, li.z}, !pot,
+                                     p, fx, fy, fz)) {
+                const double w = pot ? OBEM_KC : (ep[i] - em[i]) * (1.0 / (4.0 * OBEM_PI));
+                const float wh = (float)w;
+                const Dbf s = pot ? p : df_sum(df_sum(df_mulf(fx, ni.x), df_mulf(fy, ni.y)), df_mulf(fz, ni.z));
+                a = df_mul(Dbf{wh, (float)(w - (double)wh)}, s).h;
             } else {
-                const float4 ni = P.nrm[i];
-                a = (ep[i] - em[i]) / (4.0 * OBEM_PI) * (Fx * ni.x + Fy * ni.y + Fz * ni.z);
+                const double *vi = P.v64 + 9 * (size_t)i;
+                double phi, Fx, Fy, Fz;
+                tri_closed_form_g(P.v64 + 9 * (size_t)jj, P.geo + (size_t)OBEM_GEO64 * jj, (vi[0] + vi[3] + vi[6]) / 3.0,
+                                  (vi[1] + vi[4] + vi[7]) / 3.0, (vi[2] + vi[5] + vi[8]) / 3.0, phi, Fx, Fy, Fz);
+                a = (float)(pot ? OBEM_KC * phi : (ep[i] - em[i]) / (4.0 * OBEM_PI) * (Fx * ni.x + Fy * ni.y + Fz * ni.z));
             }
-            A[(size_t)i * n + jj] = (float)a;
+            A[(size_t)i * n + jj] = a;
         }
         __syncwarp();
     };
@@ -1541,7 +1548,7 @@ int obem_assemble_and_factor(obem_ctx *c, int precision, cudaStream_t s)
     PanelsDev P;
     P.c_a = c->d_c_a; P.g0_h = c->d_g0_h; P.g1 = c->d_g1; P.g2 = c->d_g2; P.nrm = c->d_nrm;
     P.c_lo = c->d_c_lo;
-    P.v64 = c->d_v64; P.geo = c->d_geo64; P.np = n;
+    P.v64 = c->d_v64; P.geo = c->d_geo64; P.geo2 = obem_geo2_of(c->d_geo64, n); P.np = n;
     double *d_em = NULL, *d_ep = NULL;
     struct FreeOnExit { void *p; ~FreeOnExit() { if (p) cudaFree(p); } };
     OBEM_CUDA(c, cudaMalloc((void **)&d_em, sizeof(double) * n));

@@ -148,17 +148,12 @@ direct_cells_kernel(FieldLaunch L, SymBatch SB, const int32_t *perm, CellGroups 
     auto closed_pair = [&](uint32_t e) {
         const int j = (int)(e >> 3), t = (int)(e & 7u);
         const float4 x = sh.t[t];
-        double phi, Fx, Fy, Fz;
-        if (P.geo)
-            tri_closed_form_g(P.v64 + 9 * (size_t)j, P.geo + (size_t)OBEM_GEO64 * j, (double)x.x, (double)x.y,
-                              (double)x.z, phi, Fx, Fy, Fz);
-        else
-            tri_closed_form(P.v64 + 9 * (size_t)j, (double)x.x, (double)x.y, (double)x.z, phi, Fx, Fy, Fz);
-        const double kq = OBEM_KC * (double)L.sigma[j];
-        df_put(sh, 4 * t, (float)(kq * Fx));
-        df_put(sh, 4 * t + 1, (float)(kq * Fy));
-        df_put(sh, 4 * t + 2, (float)(kq * Fz));
-        if (WANT_V) df_put(sh, 4 * t + 3, (float)(kq * phi));
+        const float4 r = closed_terms(P.v64 + 9 * (size_t)j, P.geo ? P.geo + (size_t)OBEM_GEO64 * j : NULL,
+                                      P.geo2 ? P.geo2 + (size_t)OBEM_GEO2 * j : NULL, x.x, x.y, x.z, L.sigma[j]);
+        df_put(sh, 4 * t, r.x);
+        df_put(sh, 4 * t + 1, r.y);
+        df_put(sh, 4 * t + 2, r.z);
+        if (WANT_V) df_put(sh, 4 * t + 3, r.w);
     };
     u64 D[3][NP], EP[NP];                     // target - centroid, softening of masked pairs
     auto point = [&](float ox, float oy, float oz, float w) {

@@ -495,16 +495,6 @@ __device__ __forceinline__ bool cell_is_near(float4 ca, float h2, const BlockFra
     return box_d2(ca.x, ca.y, ca.z, F.lo, F.hi) < TIER_28PT_H2 * h2 || h2 < (FRAME_H * FRAME_H) * F.scale2;
 }
 
-// FP64 closed form of one cell at one target, times k_C sigma (FP32 result)
-__device__ __noinline__ float4 closed_val(const double *v, const double *g, float tx, float ty, float tz, float sg)
-{
-    double phi, Fx, Fy, Fz;
-    if (g) tri_closed_form_g(v, g, (double)tx, (double)ty, (double)tz, phi, Fx, Fy, Fz);
-    else tri_closed_form(v, (double)tx, (double)ty, (double)tz, phi, Fx, Fy, Fz);
-    const double kq = OBEM_KC * (double)sg;
-    return make_float4((float)(kq * Fx), (float)(kq * Fy), (float)(kq * Fz), (float)(kq * phi));
-}
-
 // deterministic compaction of the near cells of [pb, pb + NEAR_CHUNK) of the
 // block's cells into list (as indices of the cell arrays)
 __device__ __forceinline__ int near_list(const FieldLaunch &L, int poff, int np, int pb, const BlockFrame &F,
@@ -531,8 +521,8 @@ __device__ __forceinline__ void diff_exact(float t, float chi, float clo, float 
     d = (t - chi) - clo;
 }
 
-// near cells, targets within h of them: FP64 closed form; E_out = e_ext + that.
-// Few targets of a warp lie within h of a given cell, and a warp-wide FP64
+// near cells, targets within h of them: closed form; E_out = e_ext + that.
+// Few targets of a warp lie within h of a given cell, and a warp-wide
 // instruction costs the same with one lane active as with 32, so the (target,
 // cell) pairs are queued per warp and evaluated 32 at a time.  Queue order is
 // (cell, target slot, lane) and each lane adds its results in queue order:
@@ -545,8 +535,8 @@ __device__ __forceinline__ void nc_flush(const FieldLaunch &L, int n, const floa
     if (lane < n) {
         const float4 e = qp[lane];
         const int j = __float_as_int(e.w);
-        res[lane] = closed_val(L.panels.v64 + 9 * (size_t)j,
-                               L.panels.geo ? L.panels.geo + (size_t)OBEM_GEO64 * j : NULL, e.x, e.y, e.z, L.sigma[j]);
+        res[lane] = closed_terms(L.panels.v64 + 9 * (size_t)j, L.panels.geo ? L.panels.geo + (size_t)OBEM_GEO64 * j : NULL,
+                                 L.panels.geo2 ? L.panels.geo2 + (size_t)OBEM_GEO2 * j : NULL, e.x, e.y, e.z, L.sigma[j]);
     }
     __syncwarp();
     for (int e = 0; e < n; ++e) {
@@ -561,7 +551,7 @@ __device__ __forceinline__ void nc_flush(const FieldLaunch &L, int n, const floa
 }
 
 template <bool WANT_V, bool COUNT>
-__global__ void __launch_bounds__(CT_THREADS)
+__global__ void __launch_bounds__(CT_THREADS, 4)
 near_closed_kernel(FieldLaunch L)
 {
     __shared__ int s_list[NEAR_CHUNK];

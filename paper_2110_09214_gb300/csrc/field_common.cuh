@@ -7,6 +7,7 @@
 #include <math.h>
 
 #include "closed_form.cuh"
+#include "closed_form_df.cuh"
 
 typedef unsigned long long u64;
 
@@ -178,6 +179,27 @@ static __host__ __device__ __noinline__ void tri_closed_form_g(const double *v, 
     Fy = fy + Om * ny;
     Fz = fz + Om * nz;
 }
+
+// w k_C (F, phi) of a cell (FP64 vertices v, geometry g and its pairs of floats
+// g2, both NULL where they are not kept) at a binary32 point, rounded once
+#ifdef __CUDACC__
+static __device__ __noinline__ float4 closed_terms(const double *v, const double *g, const float2 *g2, float x, float y,
+                                                   float z, float w)
+{
+    if (g2) {
+        Dbf p, a, b, c;
+        if (tri_closed_df(g2, Dbf{x, 0.f}, Dbf{y, 0.f}, Dbf{z, 0.f}, true, p, a, b, c)) {
+            const Dbf k = df_mulf(Dbf{(float)OBEM_KC, (float)(OBEM_KC - (double)(float)OBEM_KC)}, w);
+            return make_float4(df_mul(k, a).h, df_mul(k, b).h, df_mul(k, c).h, df_mul(k, p).h);
+        }
+    }
+    double phi, Fx, Fy, Fz;
+    if (g) tri_closed_form_g(v, g, (double)x, (double)y, (double)z, phi, Fx, Fy, Fz);
+    else tri_closed_form(v, (double)x, (double)y, (double)z, phi, Fx, Fy, Fz);
+    const double k = OBEM_KC * (double)w;
+    return make_float4((float)(k * Fx), (float)(k * Fy), (float)(k * Fz), (float)(k * phi));
+}
+#endif
 
 // one FP32 quadrature point of weight w (already k_C sigma A w_i)
 __device__ __forceinline__ void qpoint(float tx, float ty, float tz, float px, float py, float pz,

@@ -419,6 +419,24 @@ void obem_cell_geo64(const double *tri, int np, double *geo)
     }
 }
 
+// the vertices and that geometry as pairs of floats, OBEM_GEO2 per cell, behind
+// the table (an allocation of obem_geo_bytes); returns when they are written
+__global__ void geo2_kernel(const double *v64, const double *geo, int np, float2 *out)
+{
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= np * OBEM_GEO2) return;
+    const int i = e / OBEM_GEO2, k = e % OBEM_GEO2;
+    const double x = k < 9 ? v64[9 * (size_t)i + k] : geo[(size_t)OBEM_GEO64 * i + k - 9];
+    const float h = (float)x;
+    out[e] = make_float2(h, (float)(x - (double)h));
+}
+cudaError_t obem_cell_geo2(const double *d_v64, double *d_geo, int np)
+{
+    geo2_kernel<<<(np * OBEM_GEO2 + 255) / 256, 256>>>(d_v64, d_geo, np, (float2 *)(d_geo + (size_t)OBEM_GEO64 * np));
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? cudaStreamSynchronize(0) : e;
+}
+
 // Cell geometry in the layout of the field kernels (see PanelsDev) from FP64
 // vertices; kind may be NULL (electrode).  Returns the first degenerate cell,
 // or -1.
@@ -524,7 +542,11 @@ extern "C" int obem_mesh_load(obem_ctx *c, int32_t np, const double *tri, const 
         if (!geo) rc = obem_fail(c, OBEM_ERR_ARG, "mesh: host allocation failed");
         else {
             obem_cell_geo64(tri, np, geo);
-            UP(c->d_geo64, geo, sizeof(double) * OBEM_GEO64 * np);
+            if (rc == OBEM_OK &&
+                (cudaMalloc((void **)&c->d_geo64, obem_geo_bytes(np)) != cudaSuccess ||
+                 cudaMemcpy(c->d_geo64, geo, sizeof(double) * OBEM_GEO64 * np, cudaMemcpyHostToDevice) != cudaSuccess ||
+                 obem_cell_geo2(c->d_v64, c->d_geo64, np) != cudaSuccess))
+                rc = obem_fail(c, OBEM_ERR_CUDA, "mesh upload failed");
             free(geo);
         }
     }
@@ -628,6 +650,7 @@ static PanelsDev panels_of(const obem_ctx *c)
     p.c_lo = c->d_c_lo;
     p.v64 = c->d_v64;
     p.geo = c->d_geo64;
+    p.geo2 = obem_geo2_of(c->d_geo64, c->np);
     p.np = c->np;
     return p;
 }

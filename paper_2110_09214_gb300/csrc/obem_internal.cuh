@@ -75,9 +75,16 @@ struct PanelsDev {
     // cell (unit normal, twice the area, unit edge vectors and in-plane edge
     // normals), or NULL (then computed per evaluation)
     const double *geo;
+    // the vertices and that geometry as pairs of floats, OBEM_GEO2 per cell, or
+    // NULL (then FP64; closed_form_df.cuh)
+    const float2 *geo2;
     int np;
 };
 #define OBEM_GEO64 24
+#define OBEM_GEO2 31
+// both tables of np cells in one allocation: bytes, and the second one
+static inline size_t obem_geo_bytes(size_t np) { return sizeof(double) * (OBEM_GEO64 + OBEM_GEO2) * np; }
+static inline const float2 *obem_geo2_of(const double *geo, size_t np) { return geo ? (const float2 *)(geo + OBEM_GEO64 * np) : NULL; }
 
 // Static field map: cell field on a regular grid (valid nx x ny x nz nodes,
 // stored padded to px x py x pz in bricks of 8^3), node (i, j, k) at
@@ -405,6 +412,7 @@ int obem_cell_layout(const double *tri, const int32_t *kind, int np, float4 *ca,
                      float4 *g2, float4 *nr, float4 *cl);
 void obem_energy_lut(const float *grid, int n, uint32_t *lut);
 void obem_cell_geo64(const double *tri, int np, double *geo);
+cudaError_t obem_cell_geo2(const double *d_v64, double *d_geo, int np);
 size_t obem_sym_jpart_floats(int capacity);
 size_t obem_sym_pass_jpart_floats(int capacity);
 size_t obem_sym_pass_ipart_floats(int capacity);
