@@ -85,7 +85,7 @@ __device__ __forceinline__ void df_finish(const FieldLaunch &L, DfShared<NP, NW>
 // distances and weights), the others cell by cell: 60,000 targets in a GEM of
 // 59,968 cells 14.8 to 11.6 ms.
 template <bool WANT_V, bool BATCH, bool GRP, int NP, int NW>
-__global__ void __launch_bounds__(32 * NW, NP == 1 ? 2 : 4)
+__global__ void __launch_bounds__(32 * NW, NW == 8 ? 2 : 4)
 direct_cells_kernel(FieldLaunch L, SymBatch SB, const int32_t *perm, CellGroups G)
 {
     constexpr int T = 2 * NP, TH = 32 * NW;
@@ -400,9 +400,15 @@ direct_pairs_kernel(FieldLaunch L, SymBatch SB, int add)
     df_finish<WANT_V>(L, sh, n, add);
 }
 
-// Targets per block: 8 (four packs, 4 warps), 2 (8 warps) for fewer than
-// OBEM_DIRECT_WIDE targets: 2000 targets are 250 blocks of 8, hardly a warp per
-// scheduler, and the cells of a block of 2 cost one iteration per 256.
+// Targets per block: 8 (four packs, 4 warps), fewer below OBEM_DIRECT_WIDE
+// targets, where blocks of 8 would leave warps idle.  Cells: 2 targets and 8 warps
+// as long as those blocks fit the SMs at once (two per SM), then 2 targets and 4
+// warps (four per SM: no second wave at 1000), 4 targets and 8 warps for many
+// cells, whose loads a block shares.  Measured (us) at 600 and 2000 targets, 2 and
+// 8 / 2 and 4 / 4 and 8: 1024 cells 55 / 68 / 72 and 148 / 125 / 144, 15,888 cells
+// 147 / 202 / 204 and 448 / 437 / 479, 59,968 cells 223 / 326 / 260 and 681 / 718 /
+// 619.
+#define DF_ONE_WAVE 608
 
 int obem_launch_direct_cells(obem_ctx *ctx, const FieldLaunch &L, const SymBatch *SB, int slots, const int32_t *perm,
                              const CellGroups *GR, cudaStream_t s)
@@ -425,10 +431,18 @@ int obem_launch_direct_cells(obem_ctx *ctx, const FieldLaunch &L, const SymBatch
         } else {
             direct_cells_kernel<false, false, false, 4, 4><<<g, 128, 0, s>>>(L, B, perm, G);
         }
-    } else {
+    } else if (slots <= DF_ONE_WAVE) {
         const int g = (slots + 1) / 2;
         if (L.want_v) direct_cells_kernel<true, false, false, 1, 8><<<g, 256, 0, s>>>(L, B, perm, G);
         else direct_cells_kernel<false, false, false, 1, 8><<<g, 256, 0, s>>>(L, B, perm, G);
+    } else if (L.panels.np < 32768) {
+        const int g = (slots + 1) / 2;
+        if (L.want_v) direct_cells_kernel<true, false, false, 1, 4><<<g, 128, 0, s>>>(L, B, perm, G);
+        else direct_cells_kernel<false, false, false, 1, 4><<<g, 128, 0, s>>>(L, B, perm, G);
+    } else {
+        const int g = (slots + 3) / 4;
+        if (L.want_v) direct_cells_kernel<true, false, false, 2, 8><<<g, 256, 0, s>>>(L, B, perm, G);
+        else direct_cells_kernel<false, false, false, 2, 8><<<g, 256, 0, s>>>(L, B, perm, G);
     }
     OBEM_LAUNCH(ctx);
     return OBEM_OK;
