@@ -205,7 +205,7 @@ int obem_bem_solve(obem_ctx *ctx, const double *group_voltage, const float *sigm
  * potential and field of a unit density on cell i; A_i its area; n_i its
  * normal).  sources: device [ns][4] (x, y, z, q), 16-byte aligned; drhs:
  * device [n_panels].  The cell integrals use the quadrature tiers of the
- * field evaluation and the FP64 closed form within one cell size of a charge.
+ * field evaluation and the closed form within one cell size of a charge.
  * OBEM_ERR_STATE without a mesh; OBEM_ERR_TIMEOUT if a bounded wait for a
  * bulk copy of the charges ran out (drhs is then undefined).  Allocates
  * scratch on the first call and whenever ns exceeds every earlier call's;
@@ -470,7 +470,7 @@ int obem_selftest_waits(obem_ctx *ctx, int32_t which, obem_stream stream);
  *   counts[3..5] (block of targets, cell) pairs of the far-cell kernel by
  *   quadrature tier (centroid, 3 to 6 points, 7 or more points; counts[5]
  *   also counts (block, cell) pairs of the near-cell rules),
- *   counts[6] (target, cell) pairs evaluated in the FP64 closed form,
+ *   counts[6] (target, cell) pairs evaluated in the closed form,
  *   counts[7] (target, quadrature point) evaluations of the far- and near-cell
  *   kernels (a separated cell group's equivalent charges count as points),
  *   counts[8] (target, cell) pairs evaluated by quadrature.

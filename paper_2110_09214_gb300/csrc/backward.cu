@@ -12,7 +12,7 @@
 //   w ((d.gE) |d|^-3 + gV |d|^-1).
 // Cells enter through the same point formulas at their quadrature points
 // (tiers by centroid distance in units of the longest edge h) and through the
-// FP64 closed form of F and of its Jacobian near the cell.
+// closed form of F and (FP64) of its Jacobian near the cell.
 //
 // Pair arithmetic is FP32 (rsqrt.approx), two targets per f32x2 instruction;
 // partial sums of a few terms are folded into compensated (TwoSum) binary32
@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(32 * BR_WARPS) bw_sources_kernel(BwLaunch B)
 // A lane per cell, a warp per eighth of the targets; far targets two at a
 // time with the rule of the nearer one (1, 3 or 7 points, as in dL/dx); pairs
 // closer than 3 h are taken by the warp together, a lane per quadrature point,
-// and those within h queue for the FP64 closed form.
+// and those within h queue for the closed form.
 __global__ void __launch_bounds__(32 * BR_WARPS) bw_sigma_kernel(BwLaunch B)
 {
     __shared__ BrTile st;
@@ -649,7 +649,7 @@ __global__ void __launch_bounds__(32 * BR_WARPS) bw_sigma_kernel(BwLaunch B)
 //   infl_near_kernel  one warp per cell over its blocks closer than 3 h, one
 //                     charge per lane with the per-pair tier (points of every
 //                     tier precomputed in shared memory); pairs within h go to
-//                     a per-warp queue of the FP64 closed form, evaluated 32
+//                     a per-warp queue of the closed form, evaluated 32
 //                     at a time.
 // The far pass sums IF_FLUSH charges of a point in FP32 and adds these to a
 // compensated (two-sum) FP32 accumulator, and a cell adds its points' sums to

@@ -6,7 +6,7 @@
 //
 //   assemble_kernel   a thread per column, rows two at a time: Q_ij = k_C
 //                     phi_j(r_i) for electrode rows, W_ij for dielectric
-//                     rows; FP64 closed form for near cells (queued), FP32
+//                     rows; closed form for near cells (queued), FP32
 //                     quadrature (7/3/1 points by distance) for far ones
 //   equilibrate       scale every row by the power of two nearest below
 //                     1 / max |A_ij| (exact; solution unchanged)
@@ -35,7 +35,7 @@ template <bool B> struct AsBool { static constexpr bool value = B; };
 #define LU_NB 64
 #define TS_R 128               // rows of a block row of the one-launch triangular solves
 
-#define AS_CLOSED_H2 16.0f     // d < 4 h: FP64 closed form
+#define AS_CLOSED_H2 16.0f     // d < 4 h: closed form
 #define AS_7PT_H2 1024.0f      // d < 32 h: 7 points
 #define AS_3PT_H2 360000.0f    // d < 600 h: 3 points, else centroid
 #define AS_TH 128              // threads per block: one column (cell) each
@@ -787,27 +787,28 @@ __device__ __forceinline__ void load_block(float (*T)[LU_NB + 1], const float *M
 #define TRSM_LEAF_THREADS 128
 __device__ __forceinline__ unsigned tl_smem(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 template <int M>
-constexpr size_t trsm_leaf_smem() { return sizeof(float) * (size_t)M * (M + TRSM_LEAF_THREADS); }
+constexpr size_t trsm_leaf_smem() { return sizeof(float) * (size_t)M * (M + 4 + TRSM_LEAF_THREADS); }
 template <int M>
 __global__ void __launch_bounds__(TRSM_LEAF_THREADS)
 trsm_leaf_kernel(float *A, int n, int r0, int m, int c0, int nc)
 {
-    extern __shared__ float4 tl_L4[];            // [M][M / 4]: row q = column q of L
+    constexpr int LP = M + 4;                    // pitch (the transposing stores spread over 8 banks)
+    extern __shared__ float4 tl_L4[];            // [M][LP / 4]: row q = column q of L
     float *Lt = (float *)tl_L4;
-    float *Xs = Lt + M * M;                      // [M][TRSM_LEAF_THREADS]
+    float *Xs = Lt + M * LP;                     // [M][TRSM_LEAF_THREADS]
     const int tid = threadIdx.x;
     const int col = blockIdx.x * TRSM_LEAF_THREADS + tid;
     const bool live = col < nc;
     float *x = A + (size_t)r0 * n + c0 + col;
     // every load of the block in flight at once: 4-byte asynchronous copies
-    // into shared memory (a zero-size source writes a zero).  L: lanes take
-    // consecutive rows (conflict-free transposed stores); X: lanes take
-    // consecutive columns (coalesced).
+    // into shared memory (a zero-size source writes a zero), lanes on
+    // consecutive columns (coalesced; with lanes on consecutive rows of L, 32
+    // sectors a load, the 128-row leaf took 35.7 us a call at order 59,968, now 33.8).
     for (int t = tid; t < M * M; t += blockDim.x) {
-        const int r = t % M, q = t / M;
+        const int r = t / M, q = t % M;
         const bool in = r < m && q < r;
         const float *src = in ? A + (size_t)(r0 + r) * n + r0 + q : A;
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(tl_smem(&Lt[q * M + r])), "l"(src),
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(tl_smem(&Lt[q * LP + r])), "l"(src),
                      "r"(in ? 4 : 0)
                      : "memory");
     }
@@ -832,7 +833,7 @@ trsm_leaf_kernel(float *A, int n, int r0, int m, int c0, int nc)
             const float xq = Xs[q * TRSM_LEAF_THREADS + tid];
 #pragma unroll
             for (int r4 = 0; r4 < 64; r4 += 4) {
-                const float4 l = tl_L4[q * (M / 4) + (64 * h + r4) / 4];
+                const float4 l = tl_L4[q * (LP / 4) + (64 * h + r4) / 4];
                 v[r4] = fmaf(-l.x, xq, v[r4]);
                 v[r4 + 1] = fmaf(-l.y, xq, v[r4 + 1]);
                 v[r4 + 2] = fmaf(-l.z, xq, v[r4 + 2]);
@@ -844,7 +845,7 @@ trsm_leaf_kernel(float *A, int n, int r0, int m, int c0, int nc)
             const float xq = v[q];
 #pragma unroll
             for (int r4 = (q + 1) & ~3; r4 < 64; r4 += 4) {
-                const float4 l = tl_L4[(64 * h + q) * (M / 4) + (64 * h + r4) / 4];
+                const float4 l = tl_L4[(64 * h + q) * (LP / 4) + (64 * h + r4) / 4];
                 if (r4 > q) v[r4] = fmaf(-l.x, xq, v[r4]);
                 if (r4 + 1 > q) v[r4 + 1] = fmaf(-l.y, xq, v[r4 + 1]);
                 if (r4 + 2 > q) v[r4 + 2] = fmaf(-l.z, xq, v[r4 + 2]);
@@ -902,19 +903,25 @@ trsm_leaf2_kernel(float *A, int n, int r0, int m, int c0, int nc)
     for (int j = 0; j < TL2_C; ++j)
 #pragma unroll
         for (int i = 0; i < RL; ++i) v[j][i] = Xs[(32 * i + lane) * (TL2_BC + 1) + warp * TL2_C + j];
+    // (four steps unrolled: 127 were 50 KB of code that every block waited for, 15.0
+    // us a call against 13.3)
 #pragma unroll
-    for (int q = 0; q < M - 1; ++q) {
-        float lq[RL];
+    for (int b = 0; b < RL; ++b)
+#pragma unroll 4
+        for (int e = 0; e < 32; ++e) {
+            const int q = 32 * b + e;
+            float lq[RL];
 #pragma unroll
-        for (int i = 0; i < RL; ++i) lq[i] = Ls[(32 * i + lane) * (M + 1) + q];
+            for (int i = b; i < RL; ++i) lq[i] = Ls[(32 * i + lane) * (M + 1) + q];
 #pragma unroll
-        for (int j = 0; j < TL2_C; ++j) {
-            const float xq = __shfl_sync(0xffffffffu, v[j][q / 32], q % 32);
+            for (int j = 0; j < TL2_C; ++j) {
+                const float xq = __shfl_sync(0xffffffffu, v[j][b], e);
+                // (L's upper triangle is stored as zeros; a row's own step must not touch it)
 #pragma unroll
-            for (int i = 0; i < RL; ++i)
-                if (32 * i + 31 > q && 32 * i + lane > q) v[j][i] = fmaf(-lq[i], xq, v[j][i]);
+                for (int i = b; i < RL; ++i)
+                    if (i > b || lane > e) v[j][i] = fmaf(-lq[i], xq, v[j][i]);
+            }
         }
-    }
 #pragma unroll
     for (int j = 0; j < TL2_C; ++j)
 #pragma unroll

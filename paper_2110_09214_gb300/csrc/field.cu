@@ -361,7 +361,7 @@ int obem_point_bins(obem_ctx *ctx, const float4 *pts, int n, void *scratch, int3
 // if its centroid is closer than 1.5 h to the bounding box of the block's
 // targets (or if the block is so spread out that its frame cannot resolve the
 // cell); the test is the same function in all three kernels.
-//   near_closed_kernel  near cells, targets with d < h: FP64 closed form
+//   near_closed_kernel  near cells, targets with d < h: closed form
 //                       (pairs queued per warp, 32 per evaluation); writes
 //                       E_out = e_ext + these terms
 //   near_quad_kernel    near cells, all other targets: 7-point rule on 16

@@ -301,7 +301,7 @@ struct FieldLaunch {
     int want_v;
     // optional counters [OBEM_NCOUNTERS]: charge pairs; (target block, cell)
     // pairs by tier: 1 point, 3-6 points, 7 or more; (target, cell) pairs in
-    // the FP64 closed form; (target, quadrature point) evaluations; (target,
+    // the closed form; (target, quadrature point) evaluations; (target,
     // cell) pairs evaluated by quadrature
     unsigned long long *counters;
     // optional events: [1] after the cell kernels, [2] after the all-pairs kernel,
