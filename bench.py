@@ -794,7 +794,7 @@ def lu_gemm_roofline(dev, n_cells):
     return {"bound": "tensor", "kernel": "tc_gemm_kernel (tcgen05 BF16 GEMM, FP32 accumulation)",
             "shape": [h, h, h], "ms": best, "achieved": tf, "peak": pk["bf16_tflops"], "unit": "TFLOP/s",
             "frac": tf / pk["bf16_tflops"], "peak_source": pk["source"] + ", BF16 burst",
-            "note": "time includes the BF16 rounding of both operands (two conversion kernels)"}
+            "note": "time includes the BF16 rounding of both operands (one conversion kernel)"}
 
 
 def gradient_timing(ctx, mesh, geo, pos_q, sigma, dev, n_probe=4096, reps=2):
