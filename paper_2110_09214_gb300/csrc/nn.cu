@@ -43,17 +43,21 @@ __global__ void nn_bbox_init_kernel(int *bb)
 {
     if (threadIdx.x < 3) bb[threadIdx.x] = 0x7fffffff;              // min
     else if (threadIdx.x < 6) bb[threadIdx.x] = (int)0x80000000;    // max
+    else if (threadIdx.x == 6) bb[6] = 0;                           // largest |q| (bits)
 }
 
+// bounding box of the charges and their largest |q|
 __global__ void nn_bbox_kernel(const float4 *pos, const int32_t *n_dev, int n, int *bb)
 {
     const int nn = n_dev ? *n_dev : n;
-    float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
+    float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY}, mq = 0.f;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nn; i += gridDim.x * blockDim.x) {
         const float4 p = pos[i];
         mn[0] = fminf(mn[0], p.x); mn[1] = fminf(mn[1], p.y); mn[2] = fminf(mn[2], p.z);
         mx[0] = fmaxf(mx[0], p.x); mx[1] = fmaxf(mx[1], p.y); mx[2] = fmaxf(mx[2], p.z);
+        mq = fmaxf(mq, fabsf(p.w));
     }
+    for (int o = 16; o; o >>= 1) mq = fmaxf(mq, __shfl_xor_sync(0xffffffffu, mq, o));
 #pragma unroll
     for (int a = 0; a < 3; ++a)
         for (int o = 16; o; o >>= 1) {
@@ -61,10 +65,12 @@ __global__ void nn_bbox_kernel(const float4 *pos, const int32_t *n_dev, int n, i
             mx[a] = fmaxf(mx[a], __shfl_xor_sync(0xffffffffu, mx[a], o));
         }
     // one atomic per block and bound (per warp they serialised on six words)
-    __shared__ float red[6][NN_THREADS / 32];
+    __shared__ float red[7][NN_THREADS / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0)
+    if (lane == 0) {
         for (int a = 0; a < 3; ++a) { red[a][warp] = mn[a]; red[3 + a][warp] = mx[a]; }
+        red[6][warp] = mq;
+    }
     __syncthreads();
     if (threadIdx.x < 6) {
         float v = red[threadIdx.x][0];
@@ -74,6 +80,10 @@ __global__ void nn_bbox_kernel(const float4 *pos, const int32_t *n_dev, int n, i
             if (threadIdx.x < 3) atomicMin(&bb[threadIdx.x], nn_ford(v));
             else atomicMax(&bb[threadIdx.x], nn_ford(v));
         }
+    } else if (threadIdx.x == 6) {
+        float v = red[6][0];
+        for (int w = 1; w < NN_THREADS / 32; ++w) v = fmaxf(v, red[6][w]);
+        atomicMax(&bb[6], __float_as_int(v));
     }
 }
 
@@ -199,10 +209,15 @@ __global__ void __launch_bounds__(NN_AT) nn_agg_kernel(const float4 *spos, const
 
 // Field at every charge: warp g takes group g.  E_out adds to its initial
 // value when add is set, else starts from e_ext.  A pair at zero distance
-// gives no term: eps2 (x 2^80) is at least that of 1e-19 m.
+// gives no term: eps2 (x 2^80) is at least what keeps k_C q / r^3 of the largest
+// charge (bb[6]) finite, so that its product with the distance is 0.  That is a
+// distance of 2.3e-20 m x (q / e)^(1/3), below 1.5e-4 of any at which
+// k_C q / r^3 itself fits binary32: the other pairs keep their bits.  (A floor
+// without regard to the charges left binary32 from 195 e on; a test of every
+// pair of a cell for it took 3 % of the kernel.)
 __global__ void __launch_bounds__(32 * NN_FW, 4)
 nn_field_kernel(const int32_t *start, const int32_t *occ, const int32_t *grp, const int2 *groups, const int32_t *sorted,
-                const float4 *spos, const float4 *agg, int G, float eps2, float4 *E_out, float3 e_ext, int add)
+                const float4 *spos, const float4 *agg, const int *bb, int G, float eps2, float4 *E_out, float3 e_ext, int add)
 {
     constexpr int NP = NN_T / 2;
     __shared__ DfShared<NP, NN_FW> sh;
@@ -213,6 +228,10 @@ nn_field_kernel(const int32_t *start, const int32_t *occ, const int32_t *grp, co
     const int2 gr = groups[g];
     const int c = gr.x, base = gr.y;
     const int n = min(NN_T, start[c + 1] - base);
+    {
+        const float f = 2.15443469e-13f * cbrtf(fminf((float)OBEM_KC * __int_as_float(bb[6]) * DF_QS, 3.4e38f));   // (1e-38 k_C q)^(1/3)
+        eps2 = fmaxf(eps2, fmaxf(f * f, 1e-30f));
+    }
     u64 TX[NP], TY[NP], TZ[NP], A[4][NP];
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
@@ -284,8 +303,8 @@ int obem_launch_nbody_nn(obem_ctx *c, const float4 *pos, const int32_t *n_dev, i
     nn_agg_kernel<<<nc, NN_AT, 0, s>>>(c->nn_spos, c->nn_start, c->nn_occ, c->nn_grp, c->nn_agg, c->nn_groups);
     const int ng = n / NN_T + (n < nc ? n : nc);
     nn_field_kernel<<<(ng + NN_FW - 1) / NN_FW, 32 * NN_FW, 0, s>>>(
-        c->nn_start, c->nn_occ, c->nn_grp, c->nn_groups, c->nn_sorted, c->nn_spos, c->nn_agg, G,
-        fmaxf(eps2 * DF_QS, 1e-14f), E_out, e_ext, add);
+        c->nn_start, c->nn_occ, c->nn_grp, c->nn_groups, c->nn_sorted, c->nn_spos, c->nn_agg, c->nn_bbox, G,
+        eps2 * DF_QS, E_out, e_ext, add);
     OBEM_LAUNCH(c);
     return OBEM_OK;
 }
