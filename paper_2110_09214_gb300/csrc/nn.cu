@@ -164,8 +164,11 @@ __global__ void nn_scatter_kernel(const float4 *pos, const int32_t *n_dev, int n
     const int32_t c = cell[i];
     const int idx = (((c >> 20) & 1023) * G + ((c >> 10) & 1023)) * G + (c & 1023);
     const int k = atomicAdd(&cursor[idx], 1);
+    const float4 p = pos[i];
     sorted[k] = i;
-    spos[k] = pos[i];
+    // a charge without a position (NaN) gives and gets no term: no charge, and out
+    // of reach (its squared distance to any other is infinite, 1/r 0)
+    spos[k] = isnan(p.x) || isnan(p.y) || isnan(p.z) ? make_float4(1e18f, 1e18f, 1e18f, 0.f) : p;
 }
 
 // per occupied cell: positive and negative charge centres (x, y, z, k_C Q) at

@@ -44,3 +44,17 @@ def test_nn_charges_at_one_point(n, grid, weight, soft):
     got = _gpu_nn(src, grid, soft)
     assert np.all(np.isfinite(got))
     assert guarded_rel_err(got[:, :3], oracle.nbody_nn(src.astype(np.float64), grid, soft)) <= FIELD_TOL
+
+
+@pytest.mark.parametrize("grid", [1, 4, 8])
+def test_nn_charges_without_a_position(grid):
+    """A charge with a NaN coordinate gives no term and gets none; the others
+    see each other as without it."""
+    src = _clouds(3000, 77, 1.0)
+    bad = np.array([0, 7, 8, 9, 1500, 2999])
+    src[bad, np.array([0, 1, 2, 0, 1, 2])] = np.nan
+    src[8, :3] = np.nan
+    got = _gpu_nn(src, grid, 1e-9)
+    rest = np.setdiff1d(np.arange(3000), bad)
+    assert np.all(got[bad] == 0.0)
+    assert guarded_rel_err(got[rest, :3], oracle.nbody_nn(src[rest].astype(np.float64), grid, 1e-9)) <= FIELD_TOL
