@@ -41,6 +41,22 @@ __device__ __forceinline__ bool df_targets(const FieldLaunch &L, const SymBatch 
     return n > 0;
 }
 
+// box of the block's targets (those with a position: fminf and fmaxf pass over a
+// NaN) and its centre
+template <int NP, int NW>
+__device__ __forceinline__ float3 df_box(const DfShared<NP, NW> &sh, float (&lo)[3], float (&hi)[3])
+{
+#pragma unroll
+    for (int c = 0; c < 3; ++c) { lo[c] = 3e38f; hi[c] = -3e38f; }
+#pragma unroll
+    for (int t = 0; t < 2 * NP; ++t) {
+        const float4 x = sh.t[t];
+        lo[0] = fminf(lo[0], x.x); lo[1] = fminf(lo[1], x.y); lo[2] = fminf(lo[2], x.z);
+        hi[0] = fmaxf(hi[0], x.x); hi[1] = fmaxf(hi[1], x.y); hi[2] = fmaxf(hi[2], x.z);
+    }
+    return make_float3(0.5f * (lo[0] + hi[0]), 0.5f * (lo[1] + hi[1]), 0.5f * (lo[2] + hi[2]));
+}
+
 // E_out of the block's targets from the threads' slots
 template <bool WANT_V, int NP, int NW>
 __device__ __forceinline__ void df_finish(const FieldLaunch &L, DfShared<NP, NW> &sh, int n, int add)
@@ -95,9 +111,9 @@ direct_cells_kernel(FieldLaunch L, SymBatch SB, const int32_t *perm, CellGroups 
     __shared__ u64 s_tp[3][NP];               // target packs
     __shared__ int s_nq[NW];
     constexpr int GW = GRP ? NW : 1, GL = GRP ? 32 : 1, GM = GRP ? OBEM_GRP_M : 1;
-    __shared__ float4 s_u[GM], s_c[GW][GL];   // GRP: charges' directions; far groups' centres from target 0, radii
+    __shared__ float4 s_u[GM], s_c[GW][GL];   // GRP: charges' directions; far groups' centres from the box centre, radii
     __shared__ int s_g[GW][GL];               // and numbers
-    __shared__ u64 s_rp[3][NP];               // target packs from target 0
+    __shared__ u64 s_rp[3][NP];               // target packs from the box centre
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned below = (1u << lane) - 1u;
     int base, n, lo, hi, cham;
@@ -130,7 +146,8 @@ direct_cells_kernel(FieldLaunch L, SymBatch SB, const int32_t *perm, CellGroups 
         s_tp[1][tid] = pk(a.y, b.y);
         s_tp[2][tid] = pk(a.z, b.z);
         if (GRP) {
-            const float4 o = sh.t[0];
+            float blo[3], bhi[3];
+            const float3 o = df_box(sh, blo, bhi);
             s_rp[0][tid] = pk(a.x - o.x, b.x - o.x);
             s_rp[1][tid] = pk(a.y - o.y, b.y - o.y);
             s_rp[2][tid] = pk(a.z - o.z, b.z - o.z);
@@ -273,14 +290,8 @@ direct_cells_kernel(FieldLaunch L, SymBatch SB, const int32_t *perm, CellGroups 
             cells32(poff + (live ? jb + lane : jb), live);
         }
     } else {
-        float blo[3] = {3e38f, 3e38f, 3e38f}, bhi[3] = {-3e38f, -3e38f, -3e38f};     // box of the targets
-#pragma unroll
-        for (int t = 0; t < T; ++t) {
-            const float4 x = sh.t[t];
-            blo[0] = fminf(blo[0], x.x); blo[1] = fminf(blo[1], x.y); blo[2] = fminf(blo[2], x.z);
-            bhi[0] = fmaxf(bhi[0], x.x); bhi[1] = fmaxf(bhi[1], x.y); bhi[2] = fmaxf(bhi[2], x.z);
-        }
-        const float4 o = sh.t[0];
+        float blo[3], bhi[3];
+        const float3 o = df_box(sh, blo, bhi);
         // group (32 i + lane) NW + warp: neighbours, which are near together, on different warps
         for (int gb = 0; gb * NW < G.ng; gb += 32) {
             const int g = (gb + lane) * NW + warp;
