@@ -95,7 +95,8 @@ __device__ __forceinline__ void df_finish(const FieldLaunch &L, DfShared<NP, NW>
 // and share few near cells: 1e4 targets in a GEM of 5952 cells 1592 to 677 us),
 // or NULL.
 // GRP: cells in groups of 32.  A warp takes 32 groups at a time, a lane each
-// tests whether the group is far from the block's targets; the far ones enter
+// tests whether the group is far from the block's targets, and these near enough
+// to each other for its smallest cell; the far ones enter
 // as their equivalent charges, a lane per charge of the list of all of them
 // (1.5 points per lane and group, where the cells cost a point and its
 // distances and weights), the others cell by cell: 60,000 targets in a GEM of
@@ -292,6 +293,8 @@ direct_cells_kernel(FieldLaunch L, SymBatch SB, const int32_t *perm, CellGroups 
     } else {
         float blo[3], bhi[3];
         const float3 o = df_box(sh, blo, bhi);
+        const float ex = bhi[0] - o.x, ey = bhi[1] - o.y, ez = bhi[2] - o.z;
+        const float hmin2 = (FRAME_H * FRAME_H) * (ex * ex + ey * ey + ez * ez);
         // group (32 i + lane) NW + warp: neighbours, which are near together, on different warps
         for (int gb = 0; gb * NW < G.ng; gb += 32) {
             const int g = (gb + lane) * NW + warp;
@@ -300,7 +303,7 @@ direct_cells_kernel(FieldLaunch L, SymBatch SB, const int32_t *perm, CellGroups 
             const float gx = fmaxf(fmaxf(blo[0] - cr.x, cr.x - bhi[0]), 0.f),
                         gy = fmaxf(fmaxf(blo[1] - cr.y, cr.y - bhi[1]), 0.f),
                         gz = fmaxf(fmaxf(blo[2] - cr.z, cr.z - bhi[2]), 0.f);
-            const bool far = gx * gx + gy * gy + gz * gz >= OBEM_GRP_THETA2 * (cr.w * cr.w);
+            const bool far = gx * gx + gy * gy + gz * gz >= OBEM_GRP_THETA2 * (cr.w * cr.w) && G.h2min[have ? g : 0] >= hmin2;
             const unsigned fm = __ballot_sync(0xffffffffu, have && far);
             unsigned nm = __ballot_sync(0xffffffffu, have && !far);
             __syncwarp();

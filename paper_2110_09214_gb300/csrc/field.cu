@@ -382,7 +382,6 @@ int obem_point_bins(obem_ctx *ctx, const float4 *pts, int n, void *scratch, int3
 #define NQ_PTS 112
 
 #define TIER_28PT_H2 2.25f          // d >= 1.5 h
-#define FRAME_H 0.05f               // a cell needs h >= FRAME_H * frame scale to be far
 
 
 

@@ -201,6 +201,10 @@ static __device__ __noinline__ float4 closed_terms(const double *v, const double
 }
 #endif
 
+// coordinates relative to a block's frame are rounded to the block's extent: a
+// cell (the smallest of a group) needs h >= FRAME_H * that extent to be far
+#define FRAME_H 0.05f
+
 // one FP32 quadrature point of weight w (already k_C sigma A w_i)
 __device__ __forceinline__ void qpoint(float tx, float ty, float tz, float px, float py, float pz,
                                        float w, float &ax, float &ay, float &az, float &av)

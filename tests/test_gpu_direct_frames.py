@@ -53,3 +53,16 @@ def test_targets_without_a_position(capacity):
     rest = np.setdiff1d(np.arange(NT), bad)
     assert np.all(np.isfinite(got[rest]))
     _check(mesh, sigma, pts, got, rng.choice(rest, 512, replace=False))
+
+
+@pytest.mark.parametrize("capacity", [NT, 16])
+@pytest.mark.parametrize("extent", [1e-2, 10.0])
+def test_targets_far_apart(extent, capacity):
+    """Targets above the mesh, every other one up to `extent` to the side: a
+    block of them cannot resolve a far group relative to its box."""
+    mesh, sigma = _mesh(5001)
+    rng = np.random.default_rng(4)
+    pts = rng.uniform([0, 0, 4e-3], [1e-3, 1e-3, 8e-3], (NT, 3)).astype(np.float32)
+    pts[::2, :2] += extent * rng.uniform(-1, 1, (len(pts[::2]), 2)).astype(np.float32)
+    got = _field(mesh, sigma, pts, capacity)
+    _check(mesh, sigma, pts, got, rng.choice(np.arange(1, NT, 2), 512, replace=False))
