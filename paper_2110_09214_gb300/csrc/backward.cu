@@ -18,7 +18,8 @@
 // partial sums of a few terms are folded into compensated (TwoSum) binary32
 // accumulators, so cancelling terms of both signs lose no more than a few ulps
 // of the largest term.  Pairs at zero distance, and the pair t == p when
-// self_exclude is set, are skipped.
+// self_exclude is set, are skipped; so are charge-target pairs one of which has
+// no position (NaN): its coordinates become 1e18 (fminf), where every term is 0.
 //
 // All three kernels put few rows on a block and split the sum over its lanes
 // or warps: a few thousand probe points then fill the GPU, a far cell's rule
@@ -86,6 +87,9 @@ __device__ __forceinline__ float dens_term(float dx, float dy, float dz, float w
     const float dg = fmaf(dz, g.z, fmaf(dy, g.y, dx * g.x));
     return w * inv * fmaf(dg, inv * inv, g.w);
 }
+
+__device__ __forceinline__ bool no_position(float4 p) { return isnan(p.x) || isnan(p.y) || isnan(p.z); }
+#define BW_FAR 1e18f
 
 // 1 / r of a pack, 0 where r2 is 0
 __device__ __forceinline__ u64 inv_or_0(u64 r2)
@@ -232,8 +236,9 @@ __global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
     const int base = blockIdx.x * T;
     const int n = min(T, B.nt - base);
     if (tid < T) {
-        sh.t[tid] = B.targets[base + min(tid, n - 1)];
-        s_g[tid] = B.g[base + min(tid, n - 1)];
+        const float4 x = B.targets[base + min(tid, n - 1)];
+        sh.t[tid] = x;
+        s_g[tid] = no_position(x) ? make_float4(0.f, 0.f, 0.f, 0.f) : B.g[base + min(tid, n - 1)];
     }
     for (int k = tid; k < BW_NBARY; k += TH) s_b[k] = bary_point(k);
 #pragma unroll
@@ -243,7 +248,8 @@ __global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
         const float4 a = sh.t[2 * p], b = sh.t[2 * p + 1], ga = s_g[2 * p], gb = s_g[2 * p + 1];
-        TX[p] = pk(a.x, b.x); TY[p] = pk(a.y, b.y); TZ[p] = pk(a.z, b.z);
+        TX[p] = pk(fminf(a.x, BW_FAR), fminf(b.x, BW_FAR)); TY[p] = pk(fminf(a.y, BW_FAR), fminf(b.y, BW_FAR));
+        TZ[p] = pk(fminf(a.z, BW_FAR), fminf(b.z, BW_FAR));
         GX[p] = pk(ga.x, gb.x); GY[p] = pk(ga.y, gb.y); GZ[p] = pk(ga.z, gb.z); GV[p] = pk(ga.w, gb.w);
 #pragma unroll
         for (int c = 0; c < 4; ++c) A[c][p] = 0ull;
@@ -258,7 +264,8 @@ __global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
         const int i = ib + lane;
         nx = i + TH < B.ns ? B.sources[i + TH] : none;
         const bool mine = B.self_exclude && ib + 32 > base && ib < base + T;     // warp-uniform
-        const u64 YX = pk(y.x, y.x), YY = pk(y.y, y.y), YZ = pk(y.z, y.z), W = pk(kC * y.w, kC * y.w);
+        const float yx = fminf(y.x, BW_FAR), yy = fminf(y.y, BW_FAR), yz = fminf(y.z, BW_FAR);
+        const u64 YX = pk(yx, yx), YY = pk(yy, yy), YZ = pk(yz, yz), W = pk(kC * y.w, kC * y.w);
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
             const u64 dx = sub2(TX[p], YX), dy = sub2(TY[p], YY), dz = sub2(TZ[p], YZ);
@@ -284,6 +291,11 @@ __global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
             df_put(sh, 4 * t + b, (float)(q * (J[b] * g.x + J[3 + b] * g.y + J[6 + b] * g.z - (double)g.w * F[b])));
     };
     if (B.sigma) {
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {                     // as they are: a NaN is one here
+            const float4 a = sh.t[2 * p], b = sh.t[2 * p + 1];
+            TX[p] = pk(a.x, b.x); TY[p] = pk(a.y, b.y); TZ[p] = pk(a.z, b.z);
+        }
         const PanelsDev &P = B.panels;
         for (int jb = 32 * warp; jb < P.np; jb += TH) {
             const bool live = jb + lane < P.np;
@@ -400,18 +412,22 @@ __global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
 
 // ---------------------------------------------------------------- rows of 32
 // The targets [tb, tb + BR_TILE) as packs in shared memory (positions and g;
-// padding: the last target's position, g = 0)
+// padding: the last target's position, g = 0).  SKIP: a target without a position
+// at 0 and with g = 0, so that it gives no term
 struct BrTile {
     u64 x[3][BR_TILE / 2], g[4][BR_TILE / 2];
 };
+template <bool SKIP>
 __device__ __forceinline__ void br_load(const BwLaunch &B, BrTile &t, int tb)
 {
     __syncthreads();
     for (int l = threadIdx.x; l < BR_TILE / 2; l += blockDim.x) {
         const int a = tb + 2 * l, b = a + 1, last = B.nt - 1;
-        const float4 xa = B.targets[min(a, last)], xb = B.targets[min(b, last)];
+        float4 xa = B.targets[min(a, last)], xb = B.targets[min(b, last)];
         const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-        const float4 ga = a <= last ? B.g[a] : z, gb = b <= last ? B.g[b] : z;
+        float4 ga = a <= last ? B.g[a] : z, gb = b <= last ? B.g[b] : z;
+        if (SKIP && no_position(xa)) xa = ga = z;
+        if (SKIP && no_position(xb)) xb = gb = z;
         t.x[0][l] = pk(xa.x, xb.x); t.x[1][l] = pk(xa.y, xb.y); t.x[2][l] = pk(xa.z, xb.z);
         t.g[0][l] = pk(ga.x, gb.x); t.g[1][l] = pk(ga.y, gb.y); t.g[2][l] = pk(ga.z, gb.z); t.g[3][l] = pk(ga.w, gb.w);
     }
@@ -436,11 +452,12 @@ __global__ void __launch_bounds__(32 * BR_WARPS) bw_sources_kernel(BwLaunch B)
     const int p0 = blockIdx.x * 32, p = p0 + lane;
     const bool live = p < B.ns;
     const float4 y = B.sources[live ? p : p0];
-    const u64 YX = pk(y.x, y.x), YY = pk(y.y, y.y), YZ = pk(y.z, y.z), ONE = pk(1.f, 1.f);
+    const float yx = fminf(y.x, BW_FAR), yy = fminf(y.y, BW_FAR), yz = fminf(y.z, BW_FAR);
+    const u64 YX = pk(yx, yx), YY = pk(yy, yy), YZ = pk(yz, yz), ONE = pk(1.f, 1.f);
     u64 A[4] = {0ull, 0ull, 0ull, 0ull};
     float S[4] = {0.f, 0.f, 0.f, 0.f}, C[4] = {0.f, 0.f, 0.f, 0.f};
     for (int tb = 0; tb < B.nt; tb += BR_TILE) {
-        br_load(B, st, tb);
+        br_load<true>(B, st, tb);
         const int np = (min(BR_TILE, B.nt - tb) + 1) / 2;
         int since = 0;
         for (int l = warp; l < np; l += BR_WARPS) {
@@ -474,7 +491,7 @@ __global__ void __launch_bounds__(32 * BR_WARPS) bw_sources_kernel(BwLaunch B)
         for (int c = 0; c < 4; ++c) {
             float a = 0.f, b = 0.f;
             for (int w = 0; w < BR_WARPS; ++w) df_add(a, b, s_red[0][c][w][lane], s_red[1][c][w][lane]);
-            r[c] = (double)a + (double)b;
+            r[c] = no_position(y) ? 0.0 : (double)a + (double)b;
         }
         const double kq = OBEM_KC * (double)y.w;
         B.dsources[p] = make_float4((float)(-kq * r[0]), (float)(-kq * r[1]), (float)(-kq * r[2]),
@@ -526,7 +543,7 @@ __global__ void __launch_bounds__(32 * BR_WARPS) bw_sigma_kernel(BwLaunch B)
             if (s_q[warp][1][e] == lane) two_sum_acc(S, C, s_v[warp][e]);
     };
     for (int tb = 0; tb < B.nt; tb += BR_TILE) {
-        br_load(B, st, tb);
+        br_load<false>(B, st, tb);
         const int np = (min(BR_TILE, B.nt - tb) + 1) / 2;
         int since = 0;
         for (int l = warp; l < np; l += BR_WARPS) {
