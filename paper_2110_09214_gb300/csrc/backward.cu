@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
 }
 
 // ---------------------------------------------------------------- rows of 32
-// The targets [tb, tb + BR_TILE) as packs in shared memory (positions and g;
+// The live targets of [tb, tb + BR_TILE) as packs in shared memory (positions and g;
 // padding: the last target's position, g = 0).  SKIP: a target without a position
 // at 0 and with g = 0, so that it gives no term
 struct BrTile {
@@ -421,7 +421,8 @@ template <bool SKIP>
 __device__ __forceinline__ void br_load(const BwLaunch &B, BrTile &t, int tb)
 {
     __syncthreads();
-    for (int l = threadIdx.x; l < BR_TILE / 2; l += blockDim.x) {
+    const int np = (min(BR_TILE, B.nt - tb) + 1) / 2;
+    for (int l = threadIdx.x; l < np; l += blockDim.x) {
         const int a = tb + 2 * l, b = a + 1, last = B.nt - 1;
         float4 xa = B.targets[min(a, last)], xb = B.targets[min(b, last)];
         const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -443,15 +444,18 @@ __device__ __forceinline__ void br_fold(u64 &a, float &s, float &c)
 }
 
 // ---------------------------------------------------------------- dL/dy, dL/dq
-// A lane per source, a warp per eighth of the targets.
+// A lane per source.  SPLIT: 32 sources per block, a warp per eighth of the
+// targets; else 256 sources, every warp all targets (no sum over the warps, and a
+// tile of targets for 256 sources: few targets, which leave the eighths nothing to do).
+template <bool SPLIT>
 __global__ void __launch_bounds__(32 * BR_WARPS) bw_sources_kernel(BwLaunch B)
 {
     __shared__ BrTile st;
-    __shared__ float s_red[2][4][BR_WARPS][32];
+    __shared__ float s_red[2][4][SPLIT ? BR_WARPS : 1][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int p0 = blockIdx.x * 32, p = p0 + lane;
+    const int p0 = blockIdx.x * (SPLIT ? 32 : 32 * BR_WARPS) + (SPLIT ? 0 : 32 * warp), p = p0 + lane;
     const bool live = p < B.ns;
-    const float4 y = B.sources[live ? p : p0];
+    const float4 y = B.sources[live ? p : min(p0, B.ns - 1)];
     const float yx = fminf(y.x, BW_FAR), yy = fminf(y.y, BW_FAR), yz = fminf(y.z, BW_FAR);
     const u64 YX = pk(yx, yx), YY = pk(yy, yy), YZ = pk(yz, yz), ONE = pk(1.f, 1.f);
     u64 A[4] = {0ull, 0ull, 0ull, 0ull};
@@ -460,7 +464,7 @@ __global__ void __launch_bounds__(32 * BR_WARPS) bw_sources_kernel(BwLaunch B)
         br_load<true>(B, st, tb);
         const int np = (min(BR_TILE, B.nt - tb) + 1) / 2;
         int since = 0;
-        for (int l = warp; l < np; l += BR_WARPS) {
+        for (int l = SPLIT ? warp : 0; l < np; l += SPLIT ? BR_WARPS : 1) {
             const u64 dx = sub2(st.x[0][l], YX), dy = sub2(st.x[1][l], YY), dz = sub2(st.x[2][l], YZ);
             const u64 gx = st.g[0][l], gy = st.g[1][l], gz = st.g[2][l], gv = st.g[3][l];
             u64 inv = inv_or_0(fma2(dz, dz, fma2(dy, dy, mul2(dx, dx))));
@@ -482,20 +486,24 @@ __global__ void __launch_bounds__(32 * BR_WARPS) bw_sources_kernel(BwLaunch B)
 #pragma unroll
         for (int c = 0; c < 4; ++c) br_fold(A[c], S[c], C[c]);
     }
+    if (SPLIT) {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) { s_red[0][c][warp][lane] = S[c]; s_red[1][c][warp][lane] = C[c]; }
-    __syncthreads();
-    if (warp == 0 && live) {
-        double r[4];
+        for (int c = 0; c < 4; ++c) { s_red[0][c][warp][lane] = S[c]; s_red[1][c][warp][lane] = C[c]; }
+        __syncthreads();
+    }
+    if ((!SPLIT || warp == 0) && live) {
+        // -k_C q and k_C times the sums, in pairs of floats (with few targets the
+        // FP64 products were half the time)
+        const Dbf k = {(float)OBEM_KC, (float)(OBEM_KC - (double)(float)OBEM_KC)}, kq = df_mulf(k, -y.w);
+        float r[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            float a = 0.f, b = 0.f;
-            for (int w = 0; w < BR_WARPS; ++w) df_add(a, b, s_red[0][c][w][lane], s_red[1][c][w][lane]);
-            r[c] = no_position(y) ? 0.0 : (double)a + (double)b;
+            float a = SPLIT ? 0.f : S[c], b = SPLIT ? 0.f : C[c];
+            if (SPLIT)
+                for (int w = 0; w < BR_WARPS; ++w) df_add(a, b, s_red[0][c][w][lane], s_red[1][c][w][lane]);
+            r[c] = no_position(y) ? 0.f : df_mul(c < 3 ? kq : k, df_sum(Dbf{a, 0.f}, Dbf{b, 0.f})).h;
         }
-        const double kq = OBEM_KC * (double)y.w;
-        B.dsources[p] = make_float4((float)(-kq * r[0]), (float)(-kq * r[1]), (float)(-kq * r[2]),
-                                    (float)(OBEM_KC * r[3]));
+        B.dsources[p] = make_float4(r[0], r[1], r[2], r[3]);
     }
 }
 
@@ -1213,6 +1221,12 @@ int obem_launch_influence(obem_ctx *ctx, const float4 *src, int ns, const Panels
     return OBEM_OK;
 }
 
+// 256 sources per block fill the SMs from 262,144 sources on, with few targets from
+// 65,536; measured split / not (us): 1 target 12.7 / 10.7 at 80,000 sources, 83 / 15
+// at 1e6; 128 targets 15.8 / 18.0 at 40,000, 23.2 / 23.9 at 80,000; 1024 targets 215 /
+// 233 at 160,000, 421 / 408 at 320,000, 1294 / 1150 at 1e6.
+static bool bw_split(int ns, int nt) { return ns < 65536 || (ns < 262144 && nt > 128); }
+
 int obem_launch_backward(obem_ctx *ctx, const BwArgs &A, cudaStream_t s)
 {
     BwLaunch B;
@@ -1233,7 +1247,8 @@ int obem_launch_backward(obem_ctx *ctx, const BwArgs &A, cudaStream_t s)
         OBEM_LAUNCH(ctx);
     }
     if (B.dsources && B.ns > 0) {
-        bw_sources_kernel<<<(B.ns + 31) / 32, 32 * BR_WARPS, 0, s>>>(B);
+        if (bw_split(B.ns, B.nt)) bw_sources_kernel<true><<<(B.ns + 31) / 32, 32 * BR_WARPS, 0, s>>>(B);
+        else bw_sources_kernel<false><<<(B.ns + 32 * BR_WARPS - 1) / (32 * BR_WARPS), 32 * BR_WARPS, 0, s>>>(B);
         OBEM_LAUNCH(ctx);
     }
     if (B.dsigma && B.panels.np > 0) {

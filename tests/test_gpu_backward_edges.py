@@ -58,3 +58,19 @@ def test_charges_and_targets_without_a_position(nt, ns):
     assert np.all(dt[bt] == 0.0) and np.all(ds[bs] == 0.0)
     kt, ks = np.setdiff1d(np.arange(nt), bt), np.setdiff1d(np.arange(ns), bs)
     _check(tgt[kt], g[kt], src[ks], dt[kt], ds[ks])
+
+
+@pytest.mark.parametrize("nt,ns", [(1, 31), (17, 255), (1, 65_536), (128, 65_535), (128, 65_537), (129, 65_600),
+                                   (2, 262_143), (129, 262_145)])
+def test_sources_split_or_not(nt, ns):
+    """dL/dy and dL/dq on both sides of the sizes where the targets are no
+    longer split over the warps, blocks of sources partly filled."""
+    tgt, src, g = _inputs(nt, ns, nt + ns)
+    dt, ds = _backward(tgt, g, src)
+    pick = np.unique(np.concatenate([[0, ns - 1], np.random.default_rng(5).choice(ns, min(ns, 2000), replace=False)]))
+    _, _, rs = oracle.field_backward(None, None, tgt.astype(np.float64), src[pick].astype(np.float64), False,
+                                     g.astype(np.float64))
+    _, _, ap, aq = grad_abs_scales(tgt, g, src[pick])
+    assert np.all(np.isfinite(ds))
+    assert grad_err(ds[pick, :3], rs[:, :3], ap) <= FIELD_TOL
+    assert grad_err(ds[pick, 3], rs[:, 3], aq) <= FIELD_TOL
