@@ -1242,7 +1242,9 @@ int obem_launch_backward(obem_ctx *ctx, const BwArgs &A, cudaStream_t s)
     B.dsigma = A.dL_dsigma;
     B.dtargets = (float4 *)A.dL_dtargets;
     B.dsources = (float4 *)A.dL_dsources;
-    if (B.dtargets && B.nt > 0) {
+    if (B.dtargets && B.nt > 0 && !B.ns && !B.sigma) {
+        OBEM_CUDA(ctx, cudaMemsetAsync(B.dtargets, 0, sizeof(float4) * (size_t)B.nt, s));      // nothing acts on them
+    } else if (B.dtargets && B.nt > 0) {
         bw_targets_kernel<<<(B.nt + 2 * BW_NP - 1) / (2 * BW_NP), 32 * BW_NW, 0, s>>>(B);
         OBEM_LAUNCH(ctx);
     }

@@ -74,3 +74,10 @@ def test_sources_split_or_not(nt, ns):
     assert np.all(np.isfinite(ds))
     assert grad_err(ds[pick, :3], rs[:, :3], ap) <= FIELD_TOL
     assert grad_err(ds[pick, 3], rs[:, 3], aq) <= FIELD_TOL
+
+
+@pytest.mark.parametrize("nt", [1, 5, 70_001])
+def test_no_charges_and_no_cells(nt):
+    tgt, _, g = _inputs(nt, 1, nt)
+    dt, _ = _backward(tgt, g, None)
+    assert np.all(dt == 0.0)
