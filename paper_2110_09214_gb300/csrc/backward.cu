@@ -149,25 +149,21 @@ __device__ __noinline__ void tri_closed_jac(const double *v, double rx, double r
         const double wx = ax[i] - lm * tx, wy = ay[i] - lm * ty, wz = az[i] - lm * tz;
         const double p0 = ax[i] * ux + ay[i] * uy + az[i] * uz;
         const double r0sq = p0 * p0 + h * h;
-        double L, cw;
-        if (lm >= 0.0) {
-            L = log((R[j] + lp) / (R[i] + lm));
-            cw = 1.0 / (R[i] * (R[i] + lm)) - 1.0 / (R[j] * (R[j] + lp));
-        } else if (lp <= 0.0) {
-            L = log((R[i] - lm) / (R[j] - lp));
-            cw = 1.0 / (R[j] * (R[j] - lp)) - 1.0 / (R[i] * (R[i] - lm));
-        } else {
-            L = log((R[j] + lp) * (R[i] - lm) / r0sq);
-            cw = (R[i] - lm) / (R[i] * r0sq) - 1.0 / (R[j] * (R[j] + lp));
-        }
+        // (the three cases by selection: the lanes' targets differ in them)
+        const bool fwd = lm >= 0.0, bwd = !fwd && lp <= 0.0, mid = !fwd && !bwd;
+        const double ui = fwd ? R[i] + lm : R[i] - lm, uj = bwd ? R[j] - lp : R[j] + lp;
+        const double L = log((bwd ? ui : mid ? uj * ui : uj) / (bwd ? uj : mid ? r0sq : ui));
+        const double gi = (mid ? ui : 1.0) / (R[i] * (mid ? r0sq : ui)), gj = 1.0 / (R[j] * uj);
+        const double cw = bwd ? gj - gi : gi - gj;
         const double cl = 1.0 / R[i] - 1.0 / R[j];
         const double gx = cl * tx + cw * wx, gy = cl * ty + cw * wy, gz = cl * tz + cw * wz;
         J[0] += ux * gx; J[1] += ux * gy; J[2] += ux * gz;
         J[3] += uy * gx; J[4] += uy * gy; J[5] += uy * gz;
         J[6] += uz * gx; J[7] += uz * gy; J[8] += uz * gz;
         fin[0] += ux * L; fin[1] += uy * L; fin[2] += uz * L;
-        const double c = lm * lp > 0.0 ? (lp * lp - lm * lm) / ((lp * R[i] + lm * R[j]) * R[i] * R[j])
-                                       : (lp / R[j] - lm / R[i]) / r0sq;
+        const bool same = lm * lp > 0.0;
+        const double c = (same ? lp * lp - lm * lm : lp * R[i] - lm * R[j]) /
+                         ((same ? lp * R[i] + lm * R[j] : r0sq) * R[i] * R[j]);
         go[0] += c * (ty * wz - tz * wy);
         go[1] += c * (tz * wx - tx * wz);
         go[2] += c * (tx * wy - ty * wx);
@@ -223,16 +219,21 @@ __device__ __forceinline__ float4 bary_point(int k)
 // points, evaluated as c, c + a g_k, c + b g_k without divergence); pairs
 // closer than 4 h are taken by the warp together, a lane per quadrature point
 // (28 points, 112 below 2 h), and those closer than 1.5 h queue for the FP64
-// Jacobian, 32 at a time.
+// Jacobian: 32 at a time once a warp has more than BW_Q, what is left by all the
+// block's warps together, for the Jacobian of 32 pairs takes a warp 45 us and of a
+// mesh of 32 cells one warp has them all (300 targets of 32 cells 225 us with
+// queues of 32, 98 in a kernel of a warp per target, 76 now).
+#define BW_Q 128
 __global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
 {
     constexpr int NP = BW_NP, T = 2 * NP, TH = 32 * BW_NW;
     __shared__ DfShared<NP, BW_NW> sh;
     __shared__ float4 s_g[T];
     __shared__ float4 s_b[BW_NBARY];
-    __shared__ uint32_t s_q[BW_NW][32];
+    __shared__ uint32_t s_q[BW_NW][BW_Q + 32];
     __shared__ int s_nq[BW_NW];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned below = (1u << lane) - 1u;
     const int base = blockIdx.x * T;
     const int n = min(T, B.nt - base);
     if (tid < T) {
@@ -303,7 +304,7 @@ __global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
             const float4 ca = P.c_a[j], cl = P.c_lo[j], g0 = P.g0_h[j], g1 = P.g1[j], g2 = P.g2[j];
             const float q = live ? ca.w * B.sigma[j] : 0.f, h2 = g0.w;
             u64 D[3][NP], EP[NP];
-            unsigned nm = 0u;
+            unsigned nm = 0u, cm = 0u;                     // near targets of this lane's cell, those for the closed form
             float dmin = 3e38f;
 #pragma unroll
             for (int p = 0; p < NP; ++p) {
@@ -316,10 +317,12 @@ __global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
                 dmin = fminf(dmin, fminf(da, db));
                 const bool na = da < BJ_7PT * h2, nb = db < BJ_7PT * h2;
                 nm |= (na ? 1u << (2 * p) : 0u) | (nb ? 2u << (2 * p) : 0u);
+                cm |= (da < BJ_112PT * h2 ? 1u << (2 * p) : 0u) | (db < BJ_112PT * h2 ? 2u << (2 * p) : 0u);
                 EP[p] = pk(na ? 1e30f : 0.f, nb ? 1e30f : 0.f);     // near pairs: no term here
             }
             if (!live) nm = 0u;
             nm &= (1u << n) - 1u;
+            cm &= nm;
             const bool t1 = dmin >= BJ_1PT * h2, t3 = dmin >= BJ_3PT * h2;
             const float w0 = t1 ? 1.f : t3 ? 0.f : D7_W0, wa = t1 ? 0.f : t3 ? 1.0f / 3.0f : D7_W1,
                         sa = t1 ? 0.f : t3 ? 0.5f : D7_T1, wb = t3 ? 0.f : D7_W2, sb = t3 ? 0.f : D7_T2;
@@ -349,7 +352,16 @@ __global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
             }
             if (__any_sync(0xffffffffu, nm != 0u)) {
                 for (int t = 0; t < n; ++t) {
-                    unsigned bal = __ballot_sync(0xffffffffu, (nm >> t) & 1u);
+                    const unsigned cb = __ballot_sync(0xffffffffu, (cm >> t) & 1u);
+                    if ((cm >> t) & 1u) s_q[warp][nq + __popc(cb & below)] = ((uint32_t)j << 3) | (uint32_t)t;
+                    nq += __popc(cb);
+                    if (nq > BW_Q) {
+                        __syncwarp();
+                        nq -= 32;
+                        closed_pair(s_q[warp][nq + lane]);
+                        __syncwarp();
+                    }
+                    unsigned bal = __ballot_sync(0xffffffffu, ((nm & ~cm) >> t) & 1u);
                     if (!bal) continue;
                     const float4 x = sh.t[t], g = s_g[t];
                     float ax = 0.f, ay = 0.f, az = 0.f;
@@ -359,16 +371,6 @@ __global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
                         const float4 c = P.c_a[jj], l = P.c_lo[jj], v0 = P.g0_h[jj];
                         const float ex = (x.x - c.x) - l.x, ey = (x.y - c.y) - l.y, ez = (x.z - c.z) - l.z;
                         const float d2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
-                        if (d2 < BJ_112PT * v0.w) {
-                            if (lane == 0) s_q[warp][nq] = ((uint32_t)jj << 3) | (uint32_t)t;
-                            if (++nq == 32) {
-                                __syncwarp();
-                                closed_pair(s_q[warp][lane]);
-                                __syncwarp();
-                                nq = 0;
-                            }
-                            continue;
-                        }
                         const float4 v1 = P.g1[jj], v2 = P.g2[jj];
                         const float qq = c.w * B.sigma[jj];
                         const bool coarse = d2 >= BJ_28PT * v0.w;
@@ -391,10 +393,11 @@ __global__ void __launch_bounds__(32 * BW_NW) bw_targets_kernel(BwLaunch B)
     // what is left in the warps' queues, together (in warp order)
     if (lane == 0) s_nq[warp] = nq;
     __syncthreads();
-    {
-        int e = tid, w = 0;
+    for (int k = tid;; k += TH) {
+        int e = k, w = 0;
         while (w < BW_NW && e >= s_nq[w]) e -= s_nq[w++];
-        if (w < BW_NW) closed_pair(s_q[w][e]);
+        if (w == BW_NW) break;
+        closed_pair(s_q[w][e]);
     }
     float s[4 * T], c[4 * T];
 #pragma unroll

@@ -81,3 +81,30 @@ def test_no_charges_and_no_cells(nt):
     tgt, _, g = _inputs(nt, 1, nt)
     dt, _ = _backward(tgt, g, None)
     assert np.all(dt == 0.0)
+
+
+def _near_mesh(cells, rng):
+    """Triangles of about 1 mm whose centroids lie within 0.1 mm: every target
+    near is within 1.5 h of all of them."""
+    from paper_2110_09214_gb300 import inputs
+    tri = rng.normal(0, 5e-4, (cells, 3, 3))
+    tri += rng.normal(0, 3e-5, (cells, 1, 3)) - tri.mean(axis=1, keepdims=True)
+    z = np.zeros(cells, np.int32)
+    return inputs.Mesh(tri, z, z, np.ones(cells), np.ones(cells), np.array([1.0])), \
+        rng.normal(0, 1e-6, cells).astype(np.float32)
+
+
+@pytest.mark.parametrize("nt,cells", [(1, 1), (5, 4), (4, 32), (9, 33), (130, 100), (3, 700), (6, 1300)])
+def test_targets_near_every_cell(nt, cells):
+    """dL/dx where all pairs take the closed form: meshes of a warp's share and
+    less, and queues that are emptied before the end."""
+    rng = np.random.default_rng(nt + cells)
+    mesh, sigma = _near_mesh(cells, rng)
+    tgt = rng.normal(0, 2e-5, (nt, 3)).astype(np.float32)
+    g = (rng.normal(0, 1.0, (nt, 4)) * [1, 1, 1, 1e3]).astype(np.float32)
+    dt, _ = _backward(tgt, g, None, mesh, sigma)
+    _, rt, _ = oracle.field_backward(mesh.tri, sigma.astype(np.float64), tgt.astype(np.float64), None, False,
+                                     g.astype(np.float64))
+    _, at, _, _ = grad_abs_scales(tgt, g, None, mesh.tri, sigma)
+    assert np.all(dt[:, 3] == 0.0)
+    assert grad_err(dt[:, :3], rt, at) <= FIELD_TOL
