@@ -2046,10 +2046,11 @@ static bool direct_cells_rule(int targets, int cells, bool grouped)
 // other points: the one-sided kernel from 64,000 points on (20,000 charges:
 // 967 and 875 us at 64,000, 1438 and 1733 us at 128,000), with few charges,
 // whose tiles it reads once per 512 points, from 32,000 (1000 charges: 55 and
-// 84 us at 64,000).
+// 84 us at 64,000), with a single tile of 256 from 12,288 (1 to 256 charges: 25
+// and 22 to 24 us at 13,000, 25 and 35 to 37 at 32,768; 300 charges 38 and 38).
 static bool direct_pairs_rule(bool self, int targets, int sources)
 {
-    return self ? targets <= 24576 : targets <= (sources < 4096 ? 32768 : 65536);
+    return self ? targets <= 24576 : targets <= (sources <= FT_SRC_TILE ? 12288 : sources < 4096 ? 32768 : 65536);
 }
 
 int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets, cudaStream_t s)
