@@ -91,6 +91,7 @@ __device__ __forceinline__ void df_finish(const FieldLaunch &L, DfShared<NP, NW>
 // the warp evaluates them together, a lane per quadrature point (28 points,
 // 112 below 1.5 h), and pairs within h go to a per-warp queue of the FP64
 // closed form, 32 at a time.  All sums are formed in a fixed order.
+// turn: not 0 where the kernel has the set, or NULL.
 // perm: order of the targets (spatial, so that a block's targets are neighbours
 // and share few near cells: 1e4 targets in a GEM of 5952 cells 1592 to 677 us),
 // or NULL.
@@ -103,8 +104,9 @@ __device__ __forceinline__ void df_finish(const FieldLaunch &L, DfShared<NP, NW>
 // 59,968 cells 14.8 to 11.6 ms.
 template <bool WANT_V, bool BATCH, bool GRP, int NP, int NW>
 __global__ void __launch_bounds__(32 * NW, NW == 8 ? 2 : 4)
-direct_cells_kernel(FieldLaunch L, SymBatch SB, const int32_t *perm, CellGroups G)
+direct_cells_kernel(FieldLaunch L, SymBatch SB, const int32_t *perm, CellGroups G, const int32_t *turn)
 {
+    if (turn && *turn == 0) return;
     constexpr int T = 2 * NP, TH = 32 * NW;
     __shared__ DfShared<NP, NW> sh;
     __shared__ float4 s_b[DF_NBARY];          // near rules: barycentric offsets of the points, weight
@@ -425,7 +427,7 @@ direct_pairs_kernel(FieldLaunch L, SymBatch SB, int add)
 #define DF_ONE_WAVE 608
 
 int obem_launch_direct_cells(obem_ctx *ctx, const FieldLaunch &L, const SymBatch *SB, int slots, const int32_t *perm,
-                             const CellGroups *GR, cudaStream_t s)
+                             const CellGroups *GR, const int32_t *turn, cudaStream_t s)
 {
     SymBatch none;
     memset(&none, 0, sizeof none);
@@ -434,29 +436,29 @@ int obem_launch_direct_cells(obem_ctx *ctx, const FieldLaunch &L, const SymBatch
     memset(&G, 0, sizeof G);
     if (GR) G = *GR;
     if (SB) {
-        direct_cells_kernel<false, true, false, 4, 4><<<(slots + 7) / 8, 128, 0, s>>>(L, B, NULL, G);
+        direct_cells_kernel<false, true, false, 4, 4><<<(slots + 7) / 8, 128, 0, s>>>(L, B, NULL, G, turn);
     } else if (slots >= OBEM_DIRECT_WIDE) {
         const int g = (slots + 7) / 8;
         if (GR) {
-            if (L.want_v) direct_cells_kernel<true, false, true, 4, 4><<<g, 128, 0, s>>>(L, B, perm, G);
-            else direct_cells_kernel<false, false, true, 4, 4><<<g, 128, 0, s>>>(L, B, perm, G);
+            if (L.want_v) direct_cells_kernel<true, false, true, 4, 4><<<g, 128, 0, s>>>(L, B, perm, G, turn);
+            else direct_cells_kernel<false, false, true, 4, 4><<<g, 128, 0, s>>>(L, B, perm, G, turn);
         } else if (L.want_v) {
-            direct_cells_kernel<true, false, false, 4, 4><<<g, 128, 0, s>>>(L, B, perm, G);
+            direct_cells_kernel<true, false, false, 4, 4><<<g, 128, 0, s>>>(L, B, perm, G, turn);
         } else {
-            direct_cells_kernel<false, false, false, 4, 4><<<g, 128, 0, s>>>(L, B, perm, G);
+            direct_cells_kernel<false, false, false, 4, 4><<<g, 128, 0, s>>>(L, B, perm, G, turn);
         }
     } else if (slots <= DF_ONE_WAVE) {
         const int g = (slots + 1) / 2;
-        if (L.want_v) direct_cells_kernel<true, false, false, 1, 8><<<g, 256, 0, s>>>(L, B, perm, G);
-        else direct_cells_kernel<false, false, false, 1, 8><<<g, 256, 0, s>>>(L, B, perm, G);
+        if (L.want_v) direct_cells_kernel<true, false, false, 1, 8><<<g, 256, 0, s>>>(L, B, perm, G, turn);
+        else direct_cells_kernel<false, false, false, 1, 8><<<g, 256, 0, s>>>(L, B, perm, G, turn);
     } else if (L.panels.np < 32768) {
         const int g = (slots + 1) / 2;
-        if (L.want_v) direct_cells_kernel<true, false, false, 1, 4><<<g, 128, 0, s>>>(L, B, perm, G);
-        else direct_cells_kernel<false, false, false, 1, 4><<<g, 128, 0, s>>>(L, B, perm, G);
+        if (L.want_v) direct_cells_kernel<true, false, false, 1, 4><<<g, 128, 0, s>>>(L, B, perm, G, turn);
+        else direct_cells_kernel<false, false, false, 1, 4><<<g, 128, 0, s>>>(L, B, perm, G, turn);
     } else {
         const int g = (slots + 3) / 4;
-        if (L.want_v) direct_cells_kernel<true, false, false, 2, 8><<<g, 256, 0, s>>>(L, B, perm, G);
-        else direct_cells_kernel<false, false, false, 2, 8><<<g, 256, 0, s>>>(L, B, perm, G);
+        if (L.want_v) direct_cells_kernel<true, false, false, 2, 8><<<g, 256, 0, s>>>(L, B, perm, G, turn);
+        else direct_cells_kernel<false, false, false, 2, 8><<<g, 256, 0, s>>>(L, B, perm, G, turn);
     }
     OBEM_LAUNCH(ctx);
     return OBEM_OK;

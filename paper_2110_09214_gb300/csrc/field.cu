@@ -109,6 +109,15 @@ __global__ void bin_count_kernel(FieldLaunch L, float3 lo, float3 scale, uint32_
 // and took 428 us of every field evaluation (a 1000-charge step of 2.68 ms is
 // 2.25 ms without it).
 #define CT_BLOCK_N 512
+// CHOOSE: the launch's cells are evaluated by these blocks or by the direct
+// kernel, whichever suits the targets (direct_turn): nblocks[0] is 0 or
+// nblocks[1] is.
+#define CT_DIRECT_N 196608
+__device__ __forceinline__ bool direct_turn(int targets, int blocks)
+{
+    return targets <= CT_DIRECT_N || 3ll * CT_BLOCK_N * blocks >= 4ll * targets;
+}
+template <bool CHOOSE>
 __global__ void __launch_bounds__(1024) block_list_kernel(const int32_t *hist, int2 *blocks, int32_t *nblocks)
 {
     __shared__ int32_t s_warp[32];
@@ -139,7 +148,11 @@ __global__ void __launch_bounds__(1024) block_list_kernel(const int32_t *hist, i
         a += cnt[q];
         o += nb;
     }
-    if (threadIdx.x == 1023) nblocks[0] = kinc;
+    if (threadIdx.x == 1023) {
+        const bool direct = CHOOSE && direct_turn(a, kinc);          // a: all targets by now
+        nblocks[0] = direct ? 0 : kinc;
+        if (CHOOSE) nblocks[1] = direct;
+    }
 }
 
 // Target order of the cell kernels: a stable LSD radix sort of the bin codes
@@ -349,7 +362,7 @@ int obem_point_bins(obem_ctx *ctx, const float4 *pts, int n, void *scratch, int3
     sc.z = (float)OBEM_BINS_PER_AXIS / fmaxf(ctx->bbox_hi[2] - ctx->bbox_lo[2], 1e-30f);
     OBEM_CUDA(ctx, cudaMemsetAsync(hist, 0, sizeof(int32_t) * OBEM_NSUPER, s));
     bin_count_kernel<<<(n + 255) / 256, 256, 0, s>>>(L, lo, sc, code, hist);
-    block_list_kernel<<<1, 1024, 0, s>>>(hist, *blocks, *nblocks);
+    block_list_kernel<false><<<1, 1024, 0, s>>>(hist, *blocks, *nblocks);
     binsort(code, code, *perm, tk, tv, rh, n, NULL, n, s);
     OBEM_LAUNCH(ctx);
     return OBEM_OK;
@@ -2003,8 +2016,9 @@ __global__ void const_field_kernel(FieldLaunch L)
 
 // The targets' spatial order into L.perm (Morton codes of the context's cell
 // box, stable radix sort) and, with `blocks`, the block list (L.blocks,
-// L.nblocks).
-static int sort_targets(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets, bool blocks, cudaStream_t s)
+// L.nblocks), with `choose` the direct kernel's turn in L.nblocks[1].
+static int sort_targets(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets, bool blocks, bool choose,
+                        cudaStream_t s)
 {
     float3 lo = make_float3(ctx->bbox_lo[0], ctx->bbox_lo[1], ctx->bbox_lo[2]);
     float3 sc;
@@ -2020,7 +2034,8 @@ static int sort_targets(obem_ctx *ctx, const FieldLaunch &L, int capacity_target
     OBEM_CUDA(ctx, cudaMemsetAsync(ctx->s_hist, 0, sizeof(int32_t) * OBEM_NSUPER, s));
     const int nb = (capacity_targets + 255) / 256;
     bin_count_kernel<<<nb, 256, 0, s>>>(L, lo, sc, ctx->s_code, ctx->s_hist);
-    if (blocks) block_list_kernel<<<1, 1024, 0, s>>>(ctx->s_hist, (int2 *)L.blocks, (int32_t *)L.nblocks);
+    if (choose) block_list_kernel<true><<<1, 1024, 0, s>>>(ctx->s_hist, (int2 *)L.blocks, (int32_t *)L.nblocks);
+    else if (blocks) block_list_kernel<false><<<1, 1024, 0, s>>>(ctx->s_hist, (int2 *)L.blocks, (int32_t *)L.nblocks);
     binsort(ctx->s_code, ctx->s_code, (int32_t *)L.perm, ctx->s_tk, ctx->s_tv, ctx->s_rh, L.nt, L.nt_dev,
             capacity_targets, s);
     OBEM_LAUNCH(ctx);
@@ -2029,14 +2044,19 @@ static int sort_targets(obem_ctx *ctx, const FieldLaunch &L, int capacity_target
 }
 
 // Which kernels evaluate a set of targets (by its capacity: the live count is
-// on the device).  Cells: the direct kernel up to 2e5 targets, 4.6e5 for meshes
-// of 5000 cells and more, where the few blocks of the block kernels run long,
-// 7.9e5 for many cells in groups: measured block / direct (ms) at 2e5, 4e5 (6e5)
-// and 1e6 targets, plates of 1024 cells (spread out) 12.1 / 4.1 and 23.1 / 19.6
-// at 2e5 and 1e6, plates of 4096 (a cloud) 5.1 / 5.0 and 16.6 / 24.5, in groups
-// GEM of 5952 14.1 / 9.4, 19.4 / 18.2 and 36.7 / 44.8, GEM of 15,888 26.4 / 15.0,
-// 33.3 / 29.1 and 60.4 / 71.4, GEM of 59,968 52.6 / 25.6, 63.8 / 49.1, (80.0 /
-// 72.6) and 111 / 119.
+// on the device).  Cells: the direct kernel up to 2e5 targets, where it is faster
+// for clouds too (block / direct, ms: clouds of 50 um and less 4.8 / 5.2 on plates of
+// 5040 cells, 6.1 / 6.3 on 8280, 9.9 / 9.7 in a GEM of 5952, 30.8 / 26.5 of 39,904;
+// spread out 12.1 / 4.1 on 1024, 20.7 / 5.6 on 5040).  Above, the block kernels gain
+// on clouds, whose blocks are full (262,144: 4.9 / 6.9, 6.2 / 8.4, 10.4 / 12.9, 31.0 /
+// 35.2), and lose on sets spread over many super-bins (24.8 / 7.3, 32.9 / 8.9, 23.5 /
+// 5.8, 107 / 25.5; a GEM's holes 14.7 / 12.0 and 49.5 / 33.9): from 5000 cells on, up
+// to 4.6e5 targets, 7.9e5 for many cells in groups, the block list decides
+// (direct_turn) by how full its blocks are on average: under three quarters, direct.
+// (Blocks of 512 targets x their number / the targets, and block / direct: 1.00 to
+// 1.13 0.67 to 0.95, 1.26 0.92, 1.41 to 1.47 0.92 to 1.1, 1.56 1.1 to 1.2, 1.7 to 2.2
+// 1.2 to 1.6, above 2.6 2 to 6.)  Smaller meshes, and sets above these lines, take the
+// block kernels.
 static bool direct_cells_rule(int targets, int cells, bool grouped)
 {
     return targets <= (cells < 5000 ? 196608 : grouped && cells >= 32768 ? 786432 : 458752);
@@ -2063,26 +2083,27 @@ int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets,
     // far cells in groups: the context's own cells, one set of targets
     const bool grouped = ctx->ngrp > 0 && L.panels.c_a == ctx->d_c_a && !L.block_cham;
     const bool direct_cells = cells && !L.counters && direct_cells_rule(capacity_targets, L.panels.np, grouped);
-    if (direct_cells) {
-        if (L.events) { cudaEventRecord(L.events[4], s); cudaEventRecord(L.events[5], s); ctx->launches++; }
-        // in spatial order from OBEM_DIRECT_WIDE targets on (blocks of 8): the sort
-        // takes about 10 us, the unordered blocks of a spread-out set or a GEM
-        // twice the time
-        const bool sorted = L.perm && capacity_targets >= OBEM_DIRECT_WIDE;
-        int rc = sorted ? sort_targets(ctx, L, capacity_targets, false, s) : OBEM_OK;
-        CellGroups G;
-        const bool gr = grouped && capacity_targets >= OBEM_DIRECT_GROUPS;
+    // both sides are launched, and the one whose turn it is not returns at once
+    const bool choose = direct_cells && capacity_targets > CT_DIRECT_N && L.perm && L.blocks;
+    CellGroups G;
+    const bool gr = cells && grouped && (!direct_cells || capacity_targets >= OBEM_DIRECT_GROUPS);
+    if (cells) {
+        // in spatial order; the direct kernel from OBEM_DIRECT_WIDE targets on (blocks
+        // of 8): the sort takes about 10 us, the unordered blocks of a spread-out set or
+        // a GEM twice the time
+        const bool sorted = L.perm && (!direct_cells || capacity_targets >= OBEM_DIRECT_WIDE);
+        int rc = sorted ? sort_targets(ctx, L, capacity_targets, !direct_cells || choose, choose, s) : OBEM_OK;
         int fitted = 0;
         if (rc == OBEM_OK && gr) rc = obem_cell_groups_fit(ctx, L.sigma, s, &G, &fitted);
-        if (L.events) ctx->launches += fitted;
-        if (rc == OBEM_OK)
-            rc = obem_launch_direct_cells(ctx, L, NULL, capacity_targets, sorted ? L.perm : NULL, gr ? &G : NULL, s);
+        if (rc == OBEM_OK && direct_cells)
+            rc = obem_launch_direct_cells(ctx, L, NULL, capacity_targets, sorted ? L.perm : NULL, gr ? &G : NULL,
+                                          choose ? L.nblocks + 1 : NULL, s);
+        if (L.events) ctx->launches += fitted + (direct_cells ? 1 : 0);
         if (rc != OBEM_OK) return rc;
+    }
+    if (direct_cells && !choose) {
+        if (L.events) { cudaEventRecord(L.events[4], s); cudaEventRecord(L.events[5], s); }
     } else if (cells) {
-        if (L.perm) {
-            const int rc = sort_targets(ctx, L, capacity_targets, true, s);
-            if (rc != OBEM_OK) return rc;
-        }
         const int nsuper = capacity_targets < OBEM_NSUPER ? capacity_targets : OBEM_NSUPER;
         dim3 cgrid((capacity_targets + CT_BLOCK - 1) / CT_BLOCK + (L.blocks ? nsuper : 0));
         if (L.events) cudaEventRecord(L.events[4], s);
@@ -2094,12 +2115,7 @@ int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets,
             else { near_closed_kernel<false, false><<<cgrid, CT_THREADS, 0, s>>>(L); near_quad_kernel<false, false><<<cgrid, CT_THREADS, 0, s>>>(L); }
         }
         if (L.events) cudaEventRecord(L.events[5], s);
-        if (grouped) {
-            CellGroups G;
-            int fitted = 0;
-            int rc = obem_cell_groups_fit(ctx, L.sigma, s, &G, &fitted);
-            if (rc != OBEM_OK) return rc;
-            if (L.events) ctx->launches += fitted;
+        if (gr) {
             if (L.want_v) {
                 if (L.counters) cell_group_kernel<true, true><<<cgrid, CT_THREADS, 0, s>>>(L, G);
                 else cell_group_kernel<true, false><<<cgrid, CT_THREADS, 0, s>>>(L, G);
@@ -2307,7 +2323,7 @@ int obem_launch_field_batch(obem_ctx *ctx, const FieldBatch &F, const float4 *po
         L.block_cham = F.block_cham;
         L.cham_pan = F.cham_pan;
         if (F.slots <= BT_DIRECT_SLOTS) {
-            const int rc = obem_launch_direct_cells(ctx, L, &F.sym, F.slots, NULL, NULL, s);
+            const int rc = obem_launch_direct_cells(ctx, L, &F.sym, F.slots, NULL, NULL, NULL, s);
             if (rc != OBEM_OK) return rc;
         } else {
             bt_blocks_kernel<<<1, 1024, 0, s>>>(F, F.blocks, F.block_cham, F.nblocks);
@@ -2561,7 +2577,7 @@ extern "C" int obem_field_eval_noalloc(const float *targets, int32_t nt, const f
             return na_fail(err, err_len, OBEM_ERR_CUDA, "cudaMemsetAsync of the histogram failed");
         const int nb = (nt + 255) / 256;
         na_bin_count_kernel<<<nb, 256, 0, s>>>(L, box, code, hist);
-        block_list_kernel<<<1, 1024, 0, s>>>(hist, blocks, nblocks);
+        block_list_kernel<false><<<1, 1024, 0, s>>>(hist, blocks, nblocks);
         binsort(code, code, perm, na_tk, na_tv, na_rh, nt, NULL, nt, s);
         const int nsuper = nt < OBEM_NSUPER ? nt : OBEM_NSUPER;
         dim3 cgrid((nt + CT_BLOCK - 1) / CT_BLOCK + nsuper);

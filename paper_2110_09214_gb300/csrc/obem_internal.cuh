@@ -216,7 +216,7 @@ struct obem_ctx {
     int32_t *s_perm;
     int32_t *s_hist;
     int2 *s_blocks;        // cell-kernel blocks: (first sorted target, count)
-    int32_t *s_nblocks;    // [1] number of blocks, [2..] scan scratch
+    int32_t *s_nblocks;    // number of blocks, the direct kernel's turn, scan scratch
     // symmetric all-pairs kernel (targets == sources): per-item source-side and
     // per-unit target-side partial sums, work counter, persistent grid; NULL
     // when they did not fit the memory budget (the one-sided kernel runs)
@@ -396,9 +396,10 @@ int obem_launch_field_batch(obem_ctx *ctx, const FieldBatch &F, const float4 *po
 // direct.cu: the cell field (E_out = e_ext + cells) and the charges' field of
 // few targets; SB: the batch of chambers, or NULL; slots: capacity of the
 // targets; perm: their spatial order, or NULL; GR: the cells' groups, or NULL
-// (from OBEM_DIRECT_WIDE targets on)
+// (from OBEM_DIRECT_WIDE targets on); turn: on the device, 0 where the block
+// kernels have the set, or NULL
 int obem_launch_direct_cells(obem_ctx *ctx, const FieldLaunch &L, const SymBatch *SB, int slots, const int32_t *perm,
-                             const CellGroups *GR, cudaStream_t s);
+                             const CellGroups *GR, const int32_t *turn, cudaStream_t s);
 // and from which they take the cells in groups: of 59,968 cells 9.8 ms at 65,536
 // targets with the fit (1.7 ms, kept between a context's own densities), 10.2
 // cell by cell, 5.9 and 5.4 at 32,768
