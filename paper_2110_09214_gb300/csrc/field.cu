@@ -417,6 +417,7 @@ struct BlockFrame {
 // false for grid blocks beyond the block list.
 __device__ __forceinline__ bool block_range(const FieldLaunch &L, int nt, int &base, int &end)
 {
+    if (L.block_off && *L.block_off) return false;
     if (L.blocks) {
         if ((int)blockIdx.x >= *L.nblocks) return false;
         const int2 b = L.blocks[blockIdx.x];
@@ -505,6 +506,48 @@ __device__ __forceinline__ void block_targets(const FieldLaunch &L, int end, int
 __device__ __forceinline__ bool cell_is_near(float4 ca, float h2, const BlockFrame &F)
 {
     return box_d2(ca.x, ca.y, ca.z, F.lo, F.hi) < TIER_28PT_H2 * h2 || h2 < (FRAME_H * FRAME_H) * F.scale2;
+}
+
+// Targets in the order given (no scratch to sort them): whether the block kernels
+// take them.  Near cells, 28 points and more each, are what a block of spread-out
+// targets costs; a cloud has few, and there the block kernels are the faster ones
+// from 65,536 targets on (a block per SM).  Block / direct (ms) by the blocks' mean
+// share of near cells: 131,072 targets 0.5 % 2.3 / 3.4 (plates of 4900 cells), 3.9 /
+// 6.5 (GEM of 5952), 1 % 2.8 / 3.5, 2 % 5.2 / 4.7 (plates of 8192), 2.7 % 4.1 / 4.0, 3 %
+// 4.1 / 3.1 (plates of 1600), 5 % 16.1 / 12.1 (GEM of 15,888), all 163 / 10; 458,752: 1 %
+// 7.5 / 12.2, 2.6 % 10.7 / 13.7, 5 % 41.7 / 42.0, 9 % 32 / 22; 65,536: 0.5 % 1.6 / 1.7, 1 % 2.0 /
+// 1.8.  One block with many decides the time alone: its share is limited too.
+struct NearShare {
+    unsigned long long sum;       // near cells of all blocks
+    int most;                     // of one block
+};
+__global__ void __launch_bounds__(CT_THREADS) near_share_kernel(FieldLaunch L, NearShare *out)
+{
+    __shared__ int s_n;
+    int base, end;
+    if (!block_range(L, L.nt, base, end)) return;
+    float tx[CT_TPT], ty[CT_TPT], tz[CT_TPT];
+    int ti[CT_TPT];
+    BlockFrame F;
+    if (threadIdx.x == 0) s_n = 0;
+    block_targets(L, end, base, tx, ty, tz, ti, F);       // (a barrier in it)
+    int n = 0;
+    for (int j = threadIdx.x; j < L.panels.np; j += CT_THREADS) n += cell_is_near(L.panels.c_a[j], L.panels.g0_h[j].w, F);
+    n = (int)__reduce_add_sync(0xffffffffu, (unsigned)n);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&s_n, n);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        atomicAdd(&out->sum, (unsigned long long)s_n);
+        atomicMax(&out->most, s_n);
+    }
+}
+#define CT_UNSORTED_N 65536
+__global__ void near_turn_kernel(const NearShare *in, int nt, int np, int32_t *direct)
+{
+    const long long nb = (nt + CT_BLOCK - 1) / CT_BLOCK;
+    // mean share at most 1/64 per 98,304 targets, the largest four times that
+    const double lim = (double)np / 64.0 * fmax(1.0, (double)nt / 98304.0);
+    *direct = !((double)in->sum <= lim * (double)nb && (double)in->most <= 4.0 * lim);
 }
 
 // deterministic compaction of the near cells of [pb, pb + NEAR_CHUNK) of the
@@ -2073,9 +2116,10 @@ static bool direct_pairs_rule(bool self, int targets, int sources)
     return self ? targets <= 24576 : targets <= (sources <= FT_SRC_TILE ? 12288 : sources < 4096 ? 32768 : 65536);
 }
 
-int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets, cudaStream_t s)
+int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L0, int capacity_targets, cudaStream_t s)
 {
     if (capacity_targets <= 0) return OBEM_OK;
+    FieldLaunch L = L0;
     dim3 grid((capacity_targets + FT_BLOCK_TARGETS - 1) / FT_BLOCK_TARGETS);
     const bool cells = L.sigma != NULL && L.panels.np > 0;
     const bool charges = L.sources != NULL;
@@ -2083,8 +2127,10 @@ int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets,
     // far cells in groups: the context's own cells, one set of targets
     const bool grouped = ctx->ngrp > 0 && L.panels.c_a == ctx->d_c_a && !L.block_cham;
     const bool direct_cells = cells && !L.counters && direct_cells_rule(capacity_targets, L.panels.np, grouped);
-    // both sides are launched, and the one whose turn it is not returns at once
+    // chosen on the device: both sides are launched, and the one whose turn it is not
+    // returns at once
     const bool choose = direct_cells && capacity_targets > CT_DIRECT_N && L.perm && L.blocks;
+    const bool choose_unsorted = direct_cells && capacity_targets >= CT_UNSORTED_N && !L.perm && !L.nt_dev;
     CellGroups G;
     const bool gr = cells && grouped && (!direct_cells || capacity_targets >= OBEM_DIRECT_GROUPS);
     if (cells) {
@@ -2093,15 +2139,25 @@ int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L, int capacity_targets,
         // a GEM twice the time
         const bool sorted = L.perm && (!direct_cells || capacity_targets >= OBEM_DIRECT_WIDE);
         int rc = sorted ? sort_targets(ctx, L, capacity_targets, !direct_cells || choose, choose, s) : OBEM_OK;
+        const int32_t *turn = choose ? L.nblocks + 1 : NULL;
+        if (choose_unsorted) {
+            int32_t *flag = ctx->s_nblocks + 1;
+            NearShare *share = (NearShare *)(ctx->s_nblocks + 2);
+            OBEM_CUDA(ctx, cudaMemsetAsync(share, 0, sizeof *share, s));
+            near_share_kernel<<<(capacity_targets + CT_BLOCK - 1) / CT_BLOCK, CT_THREADS, 0, s>>>(L, share);
+            near_turn_kernel<<<1, 1, 0, s>>>(share, L.nt, L.panels.np, flag);
+            OBEM_LAUNCH(ctx);
+            if (L.events) ctx->launches += 2;
+            L.block_off = turn = flag;
+        }
         int fitted = 0;
         if (rc == OBEM_OK && gr) rc = obem_cell_groups_fit(ctx, L.sigma, s, &G, &fitted);
         if (rc == OBEM_OK && direct_cells)
-            rc = obem_launch_direct_cells(ctx, L, NULL, capacity_targets, sorted ? L.perm : NULL, gr ? &G : NULL,
-                                          choose ? L.nblocks + 1 : NULL, s);
+            rc = obem_launch_direct_cells(ctx, L, NULL, capacity_targets, sorted ? L.perm : NULL, gr ? &G : NULL, turn, s);
         if (L.events) ctx->launches += fitted + (direct_cells ? 1 : 0);
         if (rc != OBEM_OK) return rc;
     }
-    if (direct_cells && !choose) {
+    if (direct_cells && !choose && !choose_unsorted) {
         if (L.events) { cudaEventRecord(L.events[4], s); cudaEventRecord(L.events[5], s); }
     } else if (cells) {
         const int nsuper = capacity_targets < OBEM_NSUPER ? capacity_targets : OBEM_NSUPER;

@@ -216,7 +216,7 @@ struct obem_ctx {
     int32_t *s_perm;
     int32_t *s_hist;
     int2 *s_blocks;        // cell-kernel blocks: (first sorted target, count)
-    int32_t *s_nblocks;    // number of blocks, the direct kernel's turn, scan scratch
+    int32_t *s_nblocks;    // number of blocks, the direct kernel's turn, near cells of unsorted targets
     // symmetric all-pairs kernel (targets == sources): per-item source-side and
     // per-unit target-side partial sums, work counter, persistent grid; NULL
     // when they did not fit the memory budget (the one-sided kernel runs)
@@ -312,6 +312,7 @@ struct FieldLaunch {
     const int32_t *perm;
     const int2 *blocks;
     const int32_t *nblocks;
+    const int32_t *block_off;      // on the device, not 0: the block kernels leave the set to the direct kernel; or NULL
     // E_out already holds a field to add to (e.g. the interpolated map)
     int add_init;
     // > 0: the charges' field by the approximate N-body method on this grid

@@ -77,6 +77,37 @@ def test_many_targets_either_kernel(plates, nt, kind, flags):
     assert potential_err(got[idx, 3], V, Vabs) <= FIELD_TOL
 
 
+@pytest.mark.parametrize("flags", [obem.OBEM_STEP_CELL_FIELD, obem.OBEM_STEP_CELL_FIELD | obem.OBEM_STEP_CELL_GROUPS])
+@pytest.mark.parametrize("kind", ["cloud", "spread", "outlier"])
+@pytest.mark.parametrize("nt", [65_535, 65_536, 131_073, 262_147])
+def test_many_targets_in_the_given_order(plates, nt, kind, flags):
+    """More targets than the context can sort: the near cells of their blocks
+    say which kernels take them (outlier: a cloud with a few far points, whose
+    blocks are near many cells)."""
+    mesh, sigma = plates
+    rng = np.random.default_rng(nt)
+    pts = _points("spread" if kind == "spread" else "cloud", nt, rng).astype(np.float32)
+    if kind == "outlier":
+        pts[[7, nt // 3, nt - 1]] = [[1e-3, 9e-3, 9e-4], [9e-3, 1e-3, 1e-4], [5e-3, 5e-3, 5e-2]]
+    ctx = obem.obem_create(capacity=16, dt=1e-12, flags=flags)
+    try:
+        obem.obem_mesh_load(ctx, mesh)
+        out = torch.full((nt, 4), float("nan"), dtype=torch.float32, device="cuda")
+        obem.obem_field_eval(ctx, to_dev(pts4(pts)), out, sigma=to_dev(sigma))
+        obem.obem_field_eval(ctx, to_dev(pts4(pts)), out, sigma=to_dev(sigma))
+        torch.cuda.synchronize()
+        got = out.cpu().numpy()
+    finally:
+        obem.obem_destroy(ctx)
+    assert np.all(np.isfinite(got))
+    idx = np.unique(np.concatenate([[0, 7, nt // 3, nt - 1], rng.choice(nt, 256, replace=False)]))
+    x, s = pts[idx].astype(np.float64), sigma.astype(np.float64)
+    ref, V = oracle.panel_field(mesh.tri, s, x)
+    _, Vabs = oracle.panel_field(mesh.tri, np.abs(s), x)
+    assert guarded_rel_err(got[idx, :3], ref) <= FIELD_TOL
+    assert potential_err(got[idx, 3], V, Vabs) <= FIELD_TOL
+
+
 def test_live_count_decides(plates):
     """A state of 300,000 slots holding 2000 and 250,000 electrons at rest: the
     cells' field of either kernel moves them (v = (q/m) E dt)."""
