@@ -5,7 +5,7 @@
 //   C[M x N] -= A[M x K] B[K x N]      C, A, B: FP32 row-major sub-blocks
 //
 // Operands are rounded to BF16 (round to nearest even), products accumulated in
-// FP32.  K <= 128: tc_fused_kernel, from the FP32 operands.  Longer K: the
+// FP32.  K <= 128, C not too large: tc_fused_kernel, from the FP32 operands.  Else the
 // operands into K-major scratch (A as is, B transposed; tc_cvt_kernel), then one
 // CTA per 256 x 256 or 128 x 128 tile of C (tiles ordered in groups of 2048 rows
 // for L2 reuse) runs a TMA -> shared memory -> tcgen05.mma pipeline:
@@ -584,6 +584,14 @@ static bool tc_small_tiles(int M, int N, int K)
     return K <= 1024 || t256 <= 76 || (K <= 2048 && t256 > 152);
 }
 
+// From the FP32 operands in one kernel: K up to TF_K, where C is small enough for
+// the latency of a second launch to count; its 64 columns a tile read A again for
+// every 64 columns of C.  Measured fused / converted and 128 x 128 (us, M x N x K):
+// 60000 x 128 x 64 63 / 66 and x 128 65 / 66, 2048 x 2048 x 128 53 / 55, 4096 x 4096 x 64
+// 77 / 71 and x 128 88 / 82, 30000 x 512 x 128 97 / 79, 30000 x 30000 x 64 2138 / 1635 and x
+// 128 2420 / 1689.
+static bool tc_fused(int M, int N, int K) { return K <= TF_K && (long long)M * N <= 10000000ll; }
+
 // C[M x N] -= A[M x K] B[K x N] with BF16 operands and FP32 accumulation;
 // C, A, B are FP32 row-major blocks with leading dimensions ldc, lda, ldb.
 // Uses the context's BF16 scratch (obem_tc_reserve grows it); err: device
@@ -607,7 +615,7 @@ int obem_tc_gemm_sub(obem_ctx *c, float *C, long long ldc, const float *A, long 
     const bool vec = (((uintptr_t)A | (uintptr_t)B) & 15) == 0 && ((lda | ldb) & 3) == 0;
     const long long t128 = (long long)((N + 127) / 128) * ((M + 127) / 128);
     if (t128 > 0x3fffffffll) return obem_fail(c, OBEM_ERR_ARG, "tensor-core GEMM: %d x %d exceeds the grid", M, N);
-    if (K <= TF_K) {
+    if (tc_fused(M, N, K)) {
         const int nk = (K + TC_BK - 1) / TC_BK;
         const unsigned g = (unsigned)((long long)((N + TF_BN - 1) / TF_BN) * ((M + TC_MM - 1) / TC_MM));
         if (vec) tc_fused_kernel<true><<<g, TF_THREADS, tf_smem(nk), s>>>(C, ldc, A, lda, B, ldb, M, N, K, err);
