@@ -23,7 +23,9 @@
 
 #define ST_THREADS 256
 #define ST_CT 128                  // threads of the count and write kernels (4 warps, a chunk of charges each)
-// Charges per chunk: contexts of at most ST_TINY, ST_SMALL, ST_MID charges, more.
+// Charges per chunk: at most ST_TINY, ST_SMALL, ST_MID charges, more; by the live
+// count, on the device (by the capacity, 10,000 charges of a state for 1e6 took
+// 361 us to track, 345 before there were chunks, now 158).
 // Few charges fill the SMs in small chunks and wait for fewer others' trials;
 // larger chunks refill a warp's idle lanes from its list: 10,000 charges (us) 74
 // in chunks of 32, 100,000 240 in chunks of 256 and 145 of 128, 1e6 372 and 385.
@@ -34,6 +36,10 @@
 #define ST_TINY 16384
 #define ST_SMALL 65536
 #define ST_MID 524288
+__host__ __device__ __forceinline__ int step_chunk_len(int n)
+{
+    return n <= ST_TINY ? ST_CHUNK_T : n <= ST_SMALL ? ST_CHUNK_S : n <= ST_MID ? ST_CHUNK_M : ST_CHUNK_L;
+}
 #define ST_MB 1024                 // charges per block of the moments
 #define ST_MB_T 256                // in contexts of at most ST_TINY charges (bound by one SM's FP64: 1000 charges 10.5 us in one block)
 
@@ -807,21 +813,34 @@ __device__ __forceinline__ void step_counts(const StepCounts &n, obem_step_stats
 }
 
 template <int WC>
+__device__ __forceinline__ void count_chunks(const obem_state &st, int n, const GasDev &g, const float4 *E, uint32_t step,
+                                             const u64 *prop, const u64 *ionkey, const StepScratch &W, uint8_t *list,
+                                             StepCounts &sc)
+{
+    const int ch = blockIdx.x * (ST_CT / 32) + (threadIdx.x >> 5);
+    if (ch * WC >= n) return;                            // warp-uniform
+    int nk, ns;
+    step_chunk<WC>(st, g, chamber_of(g), E, step, prop, ionkey, ch * WC, min(WC, n - ch * WC), W, list, nk, ns, sc);
+    if ((threadIdx.x & 31) == 0) { W.blk[2 * ch] = nk; W.blk[2 * ch + 1] = ns; }
+}
+
+// FIX: the chunk length of a context whose capacity leaves no other, or 0 (with the
+// length a variable 1000 charges' step took 1.5 us more; a copy of the chunk's code
+// for each length keeps 1e6 charges at the time of one)
+template <int FIX>
 __global__ void __launch_bounds__(ST_CT) count_kernel(const obem_state st, GasDev g, const float4 *E, uint32_t step,
                                                       const u64 *prop, const u64 *ionkey, StepScratch W,
                                                       obem_step_stats *stats, StepCtl *ctl)
 {
-    __shared__ uint8_t s_list[ST_CT / 32][WC];
-    const int n = cur_n(st);
-    if (blockIdx.x * (WC * (ST_CT / 32)) >= n) return;
-    const int ch = blockIdx.x * (ST_CT / 32) + (threadIdx.x >> 5);
+    __shared__ uint8_t s_list[ST_CT / 32][FIX ? FIX : ST_CHUNK_L];
+    const int n = cur_n(st), len = FIX ? FIX : step_chunk_len(n);
+    if ((int)blockIdx.x * (ST_CT / 32) * len >= n) return;
+    uint8_t *list = s_list[threadIdx.x >> 5];
     StepCounts sc = {0, 0, 0, 0, 0, 0};
-    if (ch * WC < n) {                                   // warp-uniform
-        int nk, ns;
-        step_chunk<WC>(st, g, chamber_of(g), E, step, prop, ionkey, ch * WC, min(WC, n - ch * WC), W,
-                       s_list[threadIdx.x >> 5], nk, ns, sc);
-        if ((threadIdx.x & 31) == 0) { W.blk[2 * ch] = nk; W.blk[2 * ch + 1] = ns; }
-    }
+    if (len == ST_CHUNK_T) count_chunks<ST_CHUNK_T>(st, n, g, E, step, prop, ionkey, W, list, sc);
+    else if (len == ST_CHUNK_S) count_chunks<ST_CHUNK_S>(st, n, g, E, step, prop, ionkey, W, list, sc);
+    else if (len == ST_CHUNK_M) count_chunks<ST_CHUNK_M>(st, n, g, E, step, prop, ionkey, W, list, sc);
+    else count_chunks<ST_CHUNK_L>(st, n, g, E, step, prop, ionkey, W, list, sc);
     step_counts(sc, stats, ctl);
 }
 
@@ -847,10 +866,10 @@ __device__ __forceinline__ void step_scan(int32_t *blk, int nb, int32_t &tk, int
 }
 
 // single block: chunk offsets, totals, capacity and trial checks
-__global__ void __launch_bounds__(1024) scan_kernel(const obem_state st, int32_t *blk, int chunk,
+__global__ void __launch_bounds__(1024) scan_kernel(const obem_state st, int32_t *blk, int fix,
                                                     obem_step_stats *stats, StepCtl *ctl, int cap)
 {
-    const int n = cur_n(st);
+    const int n = cur_n(st), chunk = fix ? fix : step_chunk_len(n);
     int32_t nk, nsp;
     step_scan(blk, (n + chunk - 1) / chunk, nk, nsp);
     if (threadIdx.x == 0) {
@@ -875,7 +894,6 @@ __global__ void __launch_bounds__(1024) scan_kernel(const obem_state st, int32_t
 // order: its records are linked last to first), the charges its cells
 // absorbed to the cells' counts.  Scratch is the only input: the state's
 // arrays can be written in place.
-template <int WC>
 __device__ __forceinline__ void write_chunk(const obem_state &st, uint32_t step, int i0, int m, int off, int n_keep,
                                             uint32_t id0, const int32_t *blk, const StepScratch &W,
                                             unsigned long long *deposit)
@@ -931,15 +949,15 @@ __device__ __forceinline__ void write_chunk(const obem_state &st, uint32_t step,
     }
 }
 
-template <int WC>
+template <int FIX>
 __global__ void __launch_bounds__(ST_CT) write_kernel(const obem_state st, uint32_t step, StepScratch W,
                                                       const StepCtl *ctl, unsigned long long *deposit)
 {
     if (ctl->abort) return;
-    const int n = cur_n(st);
+    const int n = cur_n(st), len = FIX ? FIX : step_chunk_len(n);
     const int ch = blockIdx.x * (ST_CT / 32) + (threadIdx.x >> 5);
-    if (ch * WC >= n) return;
-    write_chunk<WC>(st, step, ch * WC, min(WC, n - ch * WC), 0, ctl->n_keep, *st.next_id, W.blk + 2 * ch, W, deposit);
+    if (ch * len >= n) return;
+    write_chunk(st, step, ch * len, min(len, n - ch * len), 0, ctl->n_keep, *st.next_id, W.blk + 2 * ch, W, deposit);
 }
 
 // free surface density of Eq. (charge-up): e * deposits / area on dielectric
@@ -1196,23 +1214,25 @@ static StepScratch step_scratch(obem_ctx *c)
     W.R.rec = c->s_rec; W.R.count = &c->s_ctl->n_rec; W.R.max = c->cap / 2;
     return W;
 }
-// charges per chunk, by the context's capacity
-static int step_chunk_size(const obem_ctx *c)
+// blocks of the count and write kernels: the most chunks that up to cap charges make
+static int step_chunk_blocks(int cap)
 {
-    return c->cap <= ST_TINY ? ST_CHUNK_T : c->cap <= ST_SMALL ? ST_CHUNK_S : c->cap <= ST_MID ? ST_CHUNK_M : ST_CHUNK_L;
+    int most = 0;
+    for (const int top : {ST_TINY, ST_SMALL, ST_MID, cap}) {
+        const int n = top < cap ? top : cap, len = step_chunk_len(n), ch = (n + len - 1) / len;
+        most = ch > most ? ch : most;
+    }
+    return (most + ST_CT / 32 - 1) / (ST_CT / 32);
 }
 
 static void launch_count(obem_ctx *c, const obem_state &st, const GasDev &g, const float4 *E, uint32_t step,
                          obem_step_stats *stats, cudaStream_t s)
 {
     const StepScratch W = step_scratch(c);
-    const int ch = step_chunk_size(c), per = ch * (ST_CT / 32), nb = (st.capacity + per - 1) / per;
-    typedef void (*K)(const obem_state, GasDev, const float4 *, uint32_t, const u64 *, const u64 *, StepScratch,
-                      obem_step_stats *, StepCtl *);
-    const K k = ch == ST_CHUNK_T ? count_kernel<ST_CHUNK_T> : ch == ST_CHUNK_S ? count_kernel<ST_CHUNK_S>
-              : ch == ST_CHUNK_M ? count_kernel<ST_CHUNK_M> : count_kernel<ST_CHUNK_L>;
-    k<<<nb, ST_CT, 0, s>>>(st, g, E, step, c->s_prop, c->s_ionkey, W, stats, c->s_ctl);
-    scan_kernel<<<1, 1024, 0, s>>>(st, c->s_blk, ch, stats, c->s_ctl, st.capacity < c->cap ? st.capacity : c->cap);
+    const int nb = step_chunk_blocks(st.capacity), fix = st.capacity <= ST_TINY ? ST_CHUNK_T : 0;
+    if (fix) count_kernel<ST_CHUNK_T><<<nb, ST_CT, 0, s>>>(st, g, E, step, c->s_prop, c->s_ionkey, W, stats, c->s_ctl);
+    else count_kernel<0><<<nb, ST_CT, 0, s>>>(st, g, E, step, c->s_prop, c->s_ionkey, W, stats, c->s_ctl);
+    scan_kernel<<<1, 1024, 0, s>>>(st, c->s_blk, fix, stats, c->s_ctl, st.capacity < c->cap ? st.capacity : c->cap);
 }
 
 // write, moments, fold and the new counts
@@ -1220,12 +1240,10 @@ static void launch_write(obem_ctx *c, const obem_state &st, const GasDev &g, uin
                          cudaStream_t s)
 {
     const StepScratch W = step_scratch(c);
-    const int ch = step_chunk_size(c), per = ch * (ST_CT / 32), nb = (st.capacity + per - 1) / per;
     unsigned long long *dep = g.hit_on ? (unsigned long long *)c->d_deposit : NULL;
-    typedef void (*K)(const obem_state, uint32_t, StepScratch, const StepCtl *, unsigned long long *);
-    const K k = ch == ST_CHUNK_T ? write_kernel<ST_CHUNK_T> : ch == ST_CHUNK_S ? write_kernel<ST_CHUNK_S>
-              : ch == ST_CHUNK_M ? write_kernel<ST_CHUNK_M> : write_kernel<ST_CHUNK_L>;
-    k<<<nb, ST_CT, 0, s>>>(st, step, W, c->s_ctl, dep);
+    const int nb = step_chunk_blocks(st.capacity);
+    if (st.capacity <= ST_TINY) write_kernel<ST_CHUNK_T><<<nb, ST_CT, 0, s>>>(st, step, W, c->s_ctl, dep);
+    else write_kernel<0><<<nb, ST_CT, 0, s>>>(st, step, W, c->s_ctl, dep);
     const int m = c->cap <= ST_TINY ? ST_MB_T : ST_MB, mb = (st.capacity + m - 1) / m;
     if (m == ST_MB_T) moments_kernel<ST_MB_T><<<mb, ST_THREADS, 0, s>>>(st, c->s_ctl, stats, c->s_mpart, mb);
     else moments_kernel<ST_MB><<<mb, ST_THREADS, 0, s>>>(st, c->s_ctl, stats, c->s_mpart, mb);
@@ -1526,7 +1544,7 @@ __global__ void __launch_bounds__(ST_CT) bt_write_kernel(const obem_state st, St
     if (*B.abort) return;
     const BtChunk q = bt_chunk<WC>(B);
     if (q.m <= 0) return;
-    write_chunk<WC>(st, *B.step, q.i0, q.m, q.off, B.ctl[q.c].n_keep, B.next_id[q.c], W.blk + 2 * q.ch, W, NULL);
+    write_chunk(st, *B.step, q.i0, q.m, q.off, B.ctl[q.c].n_keep, B.next_id[q.c], W.blk + 2 * q.ch, W, NULL);
 }
 
 // per chamber: new counts (or, when any chamber failed, the chambers that did
