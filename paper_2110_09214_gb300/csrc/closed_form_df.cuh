@@ -174,7 +174,7 @@ static __host__ __device__ __noinline__ bool tri_closed_df(const float2 *g2, Dbf
         a[i][1] = df_dif(num(3 * i + 1), ry);
         a[i][2] = df_dif(num(3 * i + 2), rz);
         const Dbf s = df_dot(a[i], a[i]);
-        ok = ok && s.h > 1e-24f && s.h < 1e12f;
+        ok = ok && s.h > 1e-22f && s.h < 1e12f;      // (products of three below 1e-33 lose their low parts)
         R[i] = df_sqrt(s);
     }
     const Dbf h = df_neg(df_dot(a[0], n)), h2 = df_mul(h, h);
