@@ -1712,7 +1712,7 @@ int obem_selftest_solve_wait(obem_ctx *c, cudaStream_t s)
 {
     if (!c->factored || c->nsys < 2 * TS_R)
         return obem_fail(c, OBEM_ERR_STATE, "wait self-test: needs the factors of a system of >= %d rows", 2 * TS_R);
-    const int n = c->nsys, nbk = (n + TS_R - 1) / TS_R;
+    const int n = c->nsys;
     int *ticket = (int *)(c->d_trsv + n), *err = ticket + 2;
     const int one = 1;
     OBEM_CUDA(c, cudaMemsetAsync(ticket, 0, sizeof(int) * 3, s));

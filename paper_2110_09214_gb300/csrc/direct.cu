@@ -367,16 +367,16 @@ direct_cells_kernel(FieldLaunch L, SymBatch SB, const int32_t *perm, CellGroups 
 
 // ---------------------------------------------------------------- charges
 // A lane takes every (32 NW)-th charge; add: on top of E_out (else e_ext).
-template <bool WANT_V, bool BATCH, int NP, int NW>
+template <bool WANT_V, int NP, int NW>
 __global__ void __launch_bounds__(32 * NW, NP == 1 ? 2 : 4)
-direct_pairs_kernel(FieldLaunch L, SymBatch SB, int add)
+direct_pairs_kernel(FieldLaunch L, int add)
 {
     constexpr int T = 2 * NP, TH = 32 * NW;
     __shared__ DfShared<NP, NW> sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    int base, n, s0, s1, cham;
-    if (!df_targets<BATCH, T>(L, SB, base, n, s0, s1, cham)) return;
-    if (!BATCH) s1 = L.ns_dev ? *L.ns_dev : L.ns;
+    const int base = blockIdx.x * T, n = min(T, (L.nt_dev ? *L.nt_dev : L.nt) - base);
+    if (n <= 0) return;
+    const int ns = L.ns_dev ? *L.ns_dev : L.ns;
     if (tid < T) {
         sh.ti[tid] = base + min(tid, n - 1);
         sh.t[tid] = L.targets[sh.ti[tid]];
@@ -399,11 +399,11 @@ direct_pairs_kernel(FieldLaunch L, SymBatch SB, int add)
     const int own = L.self_exclude ? base + L.self_off : 0x7fffffff - T;
     int since = 0;
     const float4 none = make_float4(1e6f, 1e6f, 1e6f, 0.f);
-    float4 nx = s0 + tid < s1 ? L.sources[s0 + tid] : none;
-    for (int ib = s0 + 32 * warp; ib < s1; ib += TH) {
+    float4 nx = tid < ns ? L.sources[tid] : none;
+    for (int ib = 32 * warp; ib < ns; ib += TH) {
         const float4 src = nx;
         const int i = ib + lane;
-        nx = i + TH < s1 ? L.sources[i + TH] : none;
+        nx = i + TH < ns ? L.sources[i + TH] : none;
         if (ib + 32 > own && ib < own + T) df_source<WANT_V, true>(TX, TY, TZ, src, kC, eps2, i - own, A);   // uniform
         else df_source<WANT_V, false>(TX, TY, TZ, src, kC, eps2, 0, A);
         if (++since == DF_FOLD) {
@@ -464,21 +464,16 @@ int obem_launch_direct_cells(obem_ctx *ctx, const FieldLaunch &L, const SymBatch
     return OBEM_OK;
 }
 
-int obem_launch_direct_pairs(obem_ctx *ctx, const FieldLaunch &L, const SymBatch *SB, int slots, int add,
-                             cudaStream_t s)
+int obem_launch_direct_pairs(obem_ctx *ctx, const FieldLaunch &L, int slots, int add, cudaStream_t s)
 {
-    SymBatch none;
-    memset(&none, 0, sizeof none);
-    const SymBatch &B = SB ? *SB : none;
-    if (slots >= OBEM_DIRECT_WIDE || SB) {
+    if (slots >= OBEM_DIRECT_WIDE) {
         const int g = (slots + 7) / 8;
-        if (SB) direct_pairs_kernel<false, true, 4, 4><<<g, 128, 0, s>>>(L, B, add);
-        else if (L.want_v) direct_pairs_kernel<true, false, 4, 4><<<g, 128, 0, s>>>(L, B, add);
-        else direct_pairs_kernel<false, false, 4, 4><<<g, 128, 0, s>>>(L, B, add);
+        if (L.want_v) direct_pairs_kernel<true, 4, 4><<<g, 128, 0, s>>>(L, add);
+        else direct_pairs_kernel<false, 4, 4><<<g, 128, 0, s>>>(L, add);
     } else {
         const int g = (slots + 1) / 2;
-        if (L.want_v) direct_pairs_kernel<true, false, 1, 8><<<g, 256, 0, s>>>(L, B, add);
-        else direct_pairs_kernel<false, false, 1, 8><<<g, 256, 0, s>>>(L, B, add);
+        if (L.want_v) direct_pairs_kernel<true, 1, 8><<<g, 256, 0, s>>>(L, add);
+        else direct_pairs_kernel<false, 1, 8><<<g, 256, 0, s>>>(L, add);
     }
     OBEM_LAUNCH(ctx);
     return OBEM_OK;

@@ -2270,7 +2270,7 @@ int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L0, int capacity_targets
             }
             if (L.events) ctx->launches += 4 + 2 * npass;
         } else if (direct) {
-            const int rc = obem_launch_direct_pairs(ctx, L, NULL, capacity_targets, add ? 1 : 0, s);
+            const int rc = obem_launch_direct_pairs(ctx, L, capacity_targets, add ? 1 : 0, s);
             if (rc != OBEM_OK) return rc;
         } else if (L.want_v) {
             if (add) nbody_kernel<true, true><<<grid, FT_THREADS, 0, s>>>(L);

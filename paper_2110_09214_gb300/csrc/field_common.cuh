@@ -205,21 +205,6 @@ static __device__ __noinline__ float4 closed_terms(const double *v, const double
 // cell (the smallest of a group) needs h >= FRAME_H * that extent to be far
 #define FRAME_H 0.05f
 
-// one FP32 quadrature point of weight w (already k_C sigma A w_i)
-__device__ __forceinline__ void qpoint(float tx, float ty, float tz, float px, float py, float pz,
-                                       float w, float &ax, float &ay, float &az, float &av)
-{
-    float dx = tx - px, dy = ty - py, dz = tz - pz;
-    float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-    float inv = rsq(r2);
-    float s = w * inv;
-    float s3 = s * (inv * inv);
-    ax = fmaf(dx, s3, ax);
-    ay = fmaf(dy, s3, ay);
-    az = fmaf(dz, s3, az);
-    av += s;
-}
-
 // Dunavant degree-5 rule, points c + t (v_k - c)
 #define D7_W0 0.225f
 #define D7_W1 0.132394152788506f

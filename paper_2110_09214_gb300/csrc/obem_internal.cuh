@@ -405,8 +405,7 @@ int obem_launch_direct_cells(obem_ctx *ctx, const FieldLaunch &L, const SymBatch
 // targets with the fit (1.7 ms, kept between a context's own densities), 10.2
 // cell by cell, 5.9 and 5.4 at 32,768
 #define OBEM_DIRECT_GROUPS 32768
-int obem_launch_direct_pairs(obem_ctx *ctx, const FieldLaunch &L, const SymBatch *SB, int slots, int add,
-                             cudaStream_t s);
+int obem_launch_direct_pairs(obem_ctx *ctx, const FieldLaunch &L, int slots, int add, cudaStream_t s);
 int obem_sym_batch_ch(long long items);
 long long obem_sym_items(int capacity);
 size_t obem_sym_sizes(int capacity, int ch, size_t *ipart_floats);

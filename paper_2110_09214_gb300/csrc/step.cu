@@ -658,19 +658,6 @@ __device__ __forceinline__ bool recombined(int i, uint8_t s, const u64 *prop, co
     return false;
 }
 
-template <typename T>
-__device__ __forceinline__ T block_sum(T v, T *sh)
-{
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    T t = 0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
-    return t;   // valid in thread 0
-}
-
 // ---------------------------------------------------------------- simulate
 // The new state of a chunk of charges, in scratch at the charges' own indices.
 struct StepScratch {
