@@ -517,10 +517,16 @@ __device__ __forceinline__ bool cell_is_near(float4 ca, float h2, const BlockFra
 // 4.1 / 3.1 (plates of 1600), 5 % 16.1 / 12.1 (GEM of 15,888), all 163 / 10; 458,752: 1 %
 // 7.5 / 12.2, 2.6 % 10.7 / 13.7, 5 % 41.7 / 42.0, 9 % 32 / 22; 65,536: 0.5 % 1.6 / 1.7, 1 % 2.0 /
 // 1.8.  One block with many decides the time alone: its share is limited too.
+// The counts and the decision lie in a slot of the context's scratch, another for
+// every call: such calls use no other scratch, so they may overlap on several streams.
 struct NearShare {
     unsigned long long sum;       // near cells of all blocks
     int most;                     // of one block
+    int32_t direct;               // the decision: not 0 for the direct kernel
+    int pad[4];
 };
+#define NEAR_SLOTS (OBEM_NSUPER / 8)
+static_assert(sizeof(NearShare) == 32, "eight words a slot");
 __global__ void __launch_bounds__(CT_THREADS) near_share_kernel(FieldLaunch L, NearShare *out)
 {
     __shared__ int s_n;
@@ -542,12 +548,12 @@ __global__ void __launch_bounds__(CT_THREADS) near_share_kernel(FieldLaunch L, N
     }
 }
 #define CT_UNSORTED_N 65536
-__global__ void near_turn_kernel(const NearShare *in, int nt, int np, int32_t *direct)
+__global__ void near_turn_kernel(NearShare *in, int nt, int np)
 {
     const long long nb = (nt + CT_BLOCK - 1) / CT_BLOCK;
     // mean share at most 1/64 per 98,304 targets, the largest four times that
     const double lim = (double)np / 64.0 * fmax(1.0, (double)nt / 98304.0);
-    *direct = !((double)in->sum <= lim * (double)nb && (double)in->most <= 4.0 * lim);
+    in->direct = !((double)in->sum <= lim * (double)nb && (double)in->most <= 4.0 * lim);
 }
 
 // deterministic compaction of the near cells of [pb, pb + NEAR_CHUNK) of the
@@ -2141,14 +2147,13 @@ int obem_launch_field(obem_ctx *ctx, const FieldLaunch &L0, int capacity_targets
         int rc = sorted ? sort_targets(ctx, L, capacity_targets, !direct_cells || choose, choose, s) : OBEM_OK;
         const int32_t *turn = choose ? L.nblocks + 1 : NULL;
         if (choose_unsorted) {
-            int32_t *flag = ctx->s_nblocks + 1;
-            NearShare *share = (NearShare *)(ctx->s_nblocks + 2);
+            NearShare *share = (NearShare *)(ctx->s_nblocks + 8) + __sync_fetch_and_add(&ctx->near_slot, 1u) % NEAR_SLOTS;
             OBEM_CUDA(ctx, cudaMemsetAsync(share, 0, sizeof *share, s));
             near_share_kernel<<<(capacity_targets + CT_BLOCK - 1) / CT_BLOCK, CT_THREADS, 0, s>>>(L, share);
-            near_turn_kernel<<<1, 1, 0, s>>>(share, L.nt, L.panels.np, flag);
+            near_turn_kernel<<<1, 1, 0, s>>>(share, L.nt, L.panels.np);
             OBEM_LAUNCH(ctx);
             if (L.events) ctx->launches += 2;
-            L.block_off = turn = flag;
+            L.block_off = turn = &share->direct;
         }
         int fitted = 0;
         if (rc == OBEM_OK && gr) rc = obem_cell_groups_fit(ctx, L.sigma, s, &G, &fitted);

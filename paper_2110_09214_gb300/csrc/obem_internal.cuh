@@ -216,7 +216,8 @@ struct obem_ctx {
     int32_t *s_perm;
     int32_t *s_hist;
     int2 *s_blocks;        // cell-kernel blocks: (first sorted target, count)
-    int32_t *s_nblocks;    // number of blocks, the direct kernel's turn, near cells of unsorted targets
+    int32_t *s_nblocks;    // number of blocks, the direct kernel's turn; from [8] on slots for unsorted targets
+    unsigned near_slot;    // the next of these slots
     // symmetric all-pairs kernel (targets == sources): per-item source-side and
     // per-unit target-side partial sums, work counter, persistent grid; NULL
     // when they did not fit the memory budget (the one-sided kernel runs)

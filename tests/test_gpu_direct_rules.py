@@ -108,6 +108,38 @@ def test_many_targets_in_the_given_order(plates, nt, kind, flags):
     assert potential_err(got[idx, 3], V, Vabs) <= FIELD_TOL
 
 
+def test_unsorted_calls_on_two_streams(plates):
+    """A cloud and a spread-out set alternating on two streams of one context:
+    each call has its own decision."""
+    mesh, sigma = plates
+    rng = np.random.default_rng(12)
+    nt = 65_536
+    sets = [_points(kind, nt, rng).astype(np.float32) for kind in ("cloud", "spread")]
+    sg = to_dev(sigma)
+    x = [to_dev(pts4(p)) for p in sets]
+    ctx = obem.obem_create(capacity=16, dt=1e-12, flags=obem.OBEM_STEP_CELL_FIELD)
+    try:
+        obem.obem_mesh_load(ctx, mesh)
+        want = []
+        for k in range(2):
+            o = torch.full((nt, 4), float("nan"), dtype=torch.float32, device="cuda")
+            obem.obem_field_eval(ctx, x[k], o, sigma=sg)
+            torch.cuda.synchronize()
+            want.append(o)
+        streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+        out = [[torch.full((nt, 4), float("nan"), dtype=torch.float32, device="cuda") for _ in range(12)] for _ in range(2)]
+        torch.cuda.synchronize()
+        for r in range(12):
+            for k in range(2):
+                obem.obem_field_eval(ctx, x[k], out[k][r], sigma=sg, stream=streams[k])
+        torch.cuda.synchronize()
+        for k in range(2):
+            for o in out[k]:
+                assert torch.equal(o, want[k])
+    finally:
+        obem.obem_destroy(ctx)
+
+
 def test_live_count_decides(plates):
     """A state of 300,000 slots holding 2000 and 250,000 electrons at rest: the
     cells' field of either kernel moves them (v = (q/m) E dt)."""
