@@ -378,7 +378,7 @@ def run_ours(a, ws, rank, local):
     traffic = nbody_traffic_per_launch(ch.n)
     # whole-step and cell-stage FP32 rates: 18 flops per ordered charge pair
     # and per (target, quadrature point) evaluation of the cell kernels (the
-    # same pair formula); the FP64 closed form of targets within one cell size
+    # same pair formula); the closed form of targets within one cell size
     # is not counted in FP32 flops
     cell_s = prof["cell_ms"] / 1e3
     step_flops = FLOPS_PER_PAIR * (pairs + prof["cell_points"])
@@ -475,7 +475,7 @@ def run_ours(a, ws, rank, local):
                      "step": {"achieved": step_rate, "frac": step_rate / peak_meas if peak_meas else None,
                               "unit": "TFLOP/s",
                               "note": "whole fused step (ms_per_step): 18 flops per ordered charge pair and per "
-                                      "(target, quadrature point) of the cell kernels; FP64 closed form not "
+                                      "(target, quadrature point) of the cell kernels; closed form not "
                                       "counted"},
                      "cells": {"achieved": cell_rate, "frac": cell_rate / peak_meas if peak_meas else None,
                                "unit": "TFLOP/s", "note": "cell stage (binning, near and far kernels): 18 flops "

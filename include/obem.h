@@ -260,7 +260,9 @@ int obem_field_eval(obem_ctx *ctx, const float *targets, int32_t nt, const float
  * source-role gradients of a charge are returned separately (add them for
  * the total).  Pairs at zero distance are skipped.  Cells near a target
  * (closer than 1.5 longest edges for dL_dtargets, 1 for dL_dsigma) use the
- * FP64 closed form and its Jacobian; farther cells use quadrature tiers.
+ * closed form and its (FP64) Jacobian; farther cells use quadrature tiers.
+ * Charges and targets without a position (a NaN coordinate) give each other no
+ * term.
  * Errors: OBEM_ERR_ARG for negative sizes, missing inputs, self_exclude
  * without sources of size nt, dL_dsources without sources, or arrays not
  * 16-byte aligned; OBEM_ERR_STATE for sigma or dL_dsigma without a mesh.
@@ -307,6 +309,8 @@ int obem_surface_charge(obem_ctx *ctx, float *sigma_free, int64_t *counts, int32
  * largest extent); a charge's cell is floor((x - lo) * (grid / W)) per axis in
  * binary32.  pos_q: device [n][4] (x, y, z, q); E_out: device [n][4]
  * (Ex, Ey, Ez, 0).  grid: 1..OBEM_NN_GMAX.  softening: Plummer length (m).
+ * Charges at one point give each other no term; a charge without a position (a
+ * NaN coordinate) gives none and gets 0.
  * Repeatable to binary32 rounding, not bit for bit: the charges of a cell
  * are summed in the order a counting sort with atomics leaves them (the exact
  * all-pairs field is bit-reproducible).  Allocates nothing, does not
@@ -454,11 +458,13 @@ int obem_selftest_waits(obem_ctx *ctx, int32_t which, obem_stream stream);
 /* Stage timing of obem_step, for measurement (not part of the method).
  * obem_profile(ctx, 1) starts recording CUDA events on the step's stream
  * around its stages (up to 256 steps are kept; older ones are dropped) and
- * counting the evaluations below (the cell kernels then run in their counting
- * variants, a few per cent slower); obem_profile(ctx, OBEM_PROFILE_TIMES)
- * records the events only (counts[2..6] stay 0; sets of up to about 1e5
- * charges then take the single cell kernel, as without a profile, which has no
- * separate near part);
+ * counting the evaluations below.  The block kernels then run in their counting
+ * variants, also for the sets that the direct kernels take otherwise: the counts
+ * and stage times of such sets (up to 1e5 to 5e5 charges) are those of the block
+ * kernels, not of an ordinary step.  obem_profile(ctx, OBEM_PROFILE_TIMES)
+ * records the events only (counts[2..6] stay 0; the kernels are those of an
+ * ordinary step, and sets of up to 1e5 to 5e5 charges take the direct cell
+ * kernel, which has no separate near part);
  * obem_stage_times() waits for the recorded events and returns, summed over
  * the recorded steps:
  *   ms[0] cell field (binning + near + far kernels), ms[1] all-pairs field
@@ -551,6 +557,8 @@ int obem_field_eval_noalloc(const float *targets, int32_t nt, const float *sourc
  * obem_batch_autotune: times the field for cell-kernel blocks of 128, 256 and
  *   512 targets on the current charges (best of reps runs each) and keeps the
  *   fastest; out host [4]: chosen size, its time (ms), the time at 512, 0.
+ *   Batches of at most 98,304 slots take the direct cell kernel, which has no such
+ *   blocks: their times differ by noise only, and the size has no effect.
  *   The size changes the field by rounding only (the quadrature tier of a cell
  *   is chosen per block).  obem_batch_set_block sets it directly (32..512). */
 typedef struct obem_batch obem_batch;

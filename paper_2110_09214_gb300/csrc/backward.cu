@@ -994,8 +994,8 @@ __device__ __forceinline__ float if_reduce4(const float (&v)[4])
     return c;
 }
 
-// the queued charges [0, n) of the closed-form queue, one per lane (FP64,
-// result rounded to FP32 into the lane's sums)
+// the queued charges [0, n) of the closed-form queue, one per lane (its result
+// rounded to binary32 into the lane's sums)
 __device__ __forceinline__ void if_closed(const PanelsDev &P, int j, const float4 *cq, int n, float (&v)[4])
 {
     const int lane = threadIdx.x & 31;

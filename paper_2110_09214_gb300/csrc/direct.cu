@@ -89,7 +89,7 @@ __device__ __forceinline__ void df_finish(const FieldLaunch &L, DfShared<NP, NW>
 // the 1-, 3-, 4-, 6- or 7-point tier; a group of points that no lane of the
 // warp needs is skipped.  Pairs closer than 3 h, by the target's own distance:
 // the warp evaluates them together, a lane per quadrature point (28 points,
-// 112 below 1.5 h), and pairs within h go to a per-warp queue of the FP64
+// 112 below 1.5 h), and pairs within h go to a per-warp queue of the
 // closed form, 32 at a time.  All sums are formed in a fixed order.
 // turn: not 0 where the kernel has the set, or NULL.
 // perm: order of the targets (spatial, so that a block's targets are neighbours
@@ -353,7 +353,7 @@ direct_cells_kernel(FieldLaunch L, SymBatch SB, const int32_t *perm, CellGroups 
     }
     df_fold<WANT_V>(sh, A, 1.f);
     // what is left in the warps' queues, together (in warp order): a warp each
-    // for its few would cost as many FP64 instructions as for 32
+    // for its few would cost as many instructions as for 32
     if (lane == 0) s_nq[warp] = nq;
     __syncthreads();
     {

@@ -17,7 +17,7 @@
 // the cells or charges instead; the rules stand at obem_launch_field.
 //
 // Cells.  Targets are ordered along a 64^3 Morton grid (stable radix sort) and
-// cut into blocks of <= 512; per block, cells near its box get the FP64
+// cut into blocks of <= 512; per block, cells near its box get the
 // closed form (targets within h) and a 112- or 28-point rule, the others one
 // of the quadrature tiers of field_common.cuh (TIER_*_H2, far_point),
 // emitted as point sources into the same packed loop as the charges.
